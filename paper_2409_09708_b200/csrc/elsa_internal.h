@@ -185,6 +185,12 @@ bool attention_suits(int tokens, int heads, int dim);
 elsa_status launch_attention(const uint16_t* qkv, int images, int tokens, int heads, int dim, elsa_dtype dtype,
                              uint16_t* out, uint32_t* dev_status, cudaStream_t stream, const float* bias = nullptr,
                              const float* mask = nullptr, int n_masks = 0, int bias_pitch = 0);
+// The same for windows that fit a warp's registers (head dimension 32, at most 64 tokens); arguments as checked by
+// launch_attention, which calls it.
+bool window_attention_suits(int tokens, int heads, int dim);
+elsa_status launch_window_attention(const uint16_t* qkv, int windows, int tokens, int heads, int dim, elsa_dtype dtype, uint16_t* out,
+                                    uint32_t* dev_status, cudaStream_t stream, const float* bias, const float* mask, int n_masks,
+                                    int bias_pitch, const DeviceInfo& dev);
 // Operand forms of the backward pass.  transpose16: src [R][C] -> dst [C][Rp] with the tail R..Rp zero (C, Rp
 // multiples of 8).  colsum: db [C] = column sums of src [R][C], through ceil(R / 512) * C floats of scratch.
 elsa_status launch_transpose16(const uint16_t* src, uint16_t* dst, int R, int C, int Rp, cudaStream_t stream);
