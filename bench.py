@@ -36,7 +36,7 @@ if ROOT not in sys.path:
 
 METRIC = "sparse-GEMM dense-equivalent TFLOP/s over the ViT linear stack"
 UNIT = "TFLOP/s"
-GEMM_KERNELS = ("linear_tc_dense", "linear_tc_pair", "linear_tc_sp24", "linear_tc_sp24_pair", "linear_tc_sp24_ws", "linear_tc_sp24_st")   # forms of the tcgen05 GEMM
+GEMM_KERNELS = ("linear_small", "linear_tc_dense", "linear_tc_pair", "linear_tc_sp24", "linear_tc_sp24_pair", "linear_tc_sp24_ws", "linear_tc_sp24_st")   # forms of the tcgen05 GEMM
 
 # Recorded DRAM traffic (ncu, one-pass captures) lives in profiles/dram_traffic.json: per workload and kernel
 # the bytes of one step, the command that captured them and a hash of the kernel sources at that time.

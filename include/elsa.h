@@ -74,8 +74,10 @@ typedef enum {
     ELSA_VARIANT_TC_SPARSE_PAIR = 5, /* the same on CTA pairs (256 features x 224 rows per pair) */
     ELSA_VARIANT_TC_SPARSE_WS = 6, /* N <= 2, in % 128 == 0, in <= 1024: CTA pairs that keep their 256-feature
                                     * weight block and its metadata in tensor memory for a whole layer */
-    ELSA_VARIANT_TC_SPARSE_ST = 7  /* N <= 2, in % 128 == 0, any length: the weight block streams through
+    ELSA_VARIANT_TC_SPARSE_ST = 7, /* N <= 2, in % 128 == 0, any length: the weight block streams through
                                     * tensor memory in K chunks of 256, shared memory carries activations only */
+    ELSA_VARIANT_TC_SMALL = 8      /* few token rows: weight tiles expanded on their way to shared memory, the
+                                    * reduction cut over the CTAs of a cluster where tiles alone leave SMs idle */
 } elsa_variant;
 
 /* Sizes of the packed form (host-only arithmetic; 0 on invalid arguments). */
@@ -276,7 +278,8 @@ typedef enum {
     ELSA_KERNEL_INT8_FORMAT = 12,       /* INT8 compress / unpack */
     ELSA_KERNEL_BLOCK_ROWWISE = 13,     /* LayerNorm, residual add, GELU, column copy of the chained block */
     ELSA_KERNEL_BACKWARD_FORMAT = 14,   /* transposes, column sums and mask of the backward pass */
-    ELSA_KERNEL_ATTENTION = 15          /* multi-head self-attention of the chained block */
+    ELSA_KERNEL_ATTENTION = 15,         /* multi-head self-attention of the chained block */
+    ELSA_KERNEL_LINEAR_SMALL = 16       /* linear with few token rows, straight from the packed weight */
 } elsa_kernel_id;
 
 typedef struct {

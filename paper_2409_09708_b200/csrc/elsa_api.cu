@@ -163,7 +163,7 @@ elsa_status side_pipe(int device, SidePipe** pipe)
     return ELSA_OK;
 }
 
-enum LinearKind { KIND_SIMT, KIND_DENSE_ONE, KIND_DENSE_PAIR, KIND_SPARSE_ONE, KIND_SPARSE_PAIR, KIND_SPARSE_WS, KIND_SPARSE_ST };
+enum LinearKind { KIND_SIMT, KIND_SMALL, KIND_DENSE_ONE, KIND_DENSE_PAIR, KIND_SPARSE_ONE, KIND_SPARSE_PAIR, KIND_SPARSE_WS, KIND_SPARSE_ST };
 
 // Form of the 2-of-4 weight image each sparse kernel reads.
 int sp24_layout_of(LinearKind kind)
@@ -179,6 +179,7 @@ elsa_status pick_kind(int rows, int out, int in, int N, int M, int sm_count, Lin
     switch (variant) {
     case ELSA_VARIANT_SIMT: *kind = KIND_SIMT; return ELSA_OK;
     case ELSA_VARIANT_TC_DENSE: *kind = KIND_DENSE_ONE; return ELSA_OK;
+    case ELSA_VARIANT_TC_SMALL: *kind = KIND_SMALL; return ELSA_OK;
     case ELSA_VARIANT_TC_PAIR: *kind = KIND_DENSE_PAIR; return ELSA_OK;
     case ELSA_VARIANT_TC_SPARSE:
     case ELSA_VARIANT_TC_SPARSE_PAIR:
@@ -214,14 +215,23 @@ elsa_status pick_kind(int rows, int out, int in, int N, int M, int sm_count, Lin
         *kind = ws ? KIND_SPARSE_WS : st ? KIND_SPARSE_ST : KIND_SPARSE_PAIR;
     }
     else
-        *kind = linear_tc_pair_suits(rows, out, sm_count) ? KIND_DENSE_PAIR : KIND_DENSE_ONE;
+        *kind = linear_tc_pair_suits(rows, out, sm_count) ? KIND_DENSE_PAIR : KIND_SMALL;
     return ELSA_OK;
 }
 
-// After validation: enqueue one layer.
+SmallJob small_job(const void* X, int rows, const void* w, const uint32_t* idx, const void* bias, int out, int in, int N, int M,
+                   void* Y, bool masked = false)
+{
+    SmallJob j;
+    j.X = (const uint16_t*)X; j.w = (const uint16_t*)w; j.idx = idx; j.bias = (const uint16_t*)bias; j.Y = (uint16_t*)Y;
+    j.rows = rows; j.in = in; j.out = out; j.N = N; j.M = M; j.masked = masked;
+    return j;
+}
+
+// After validation: enqueue one layer.  small_splits: how the few-rows kernel cuts the reduction (0: its own choice).
 elsa_status run_linear(const void* X, int rows, const void* vals, const uint32_t* idx, const void* bias, int out,
                        int in, int N, int M, elsa_dtype dtype, void* Y, void* workspace, uint32_t* dev_status,
-                       cudaStream_t stream)
+                       cudaStream_t stream, int small_splits = 0)
 {
     DeviceInfo dev;
     elsa_status st = device_info(&dev);
@@ -231,6 +241,11 @@ elsa_status run_linear(const void* X, int rows, const void* vals, const uint32_t
     if (kind == KIND_SIMT)
         return launch_linear_simt((const uint16_t*)X, rows, (const uint16_t*)vals, idx, (const uint16_t*)bias, out,
                                   in, N, M, dtype, (uint16_t*)Y, stream);
+    if (kind == KIND_SMALL) {
+        const SmallJob job = small_job(X, rows, vals, idx, bias, out, in, N, M, Y);
+        if (small_splits == 0) small_splits = linear_small_splits(&job, 1, dev.sm_count);
+        return launch_linear_small_group(&job, 1, small_splits, false, dtype, dev_status, stream);
+    }
     if (kind == KIND_SPARSE_ONE)
         return launch_linear_tc_sparse((const uint16_t*)X, rows, (const uint16_t*)vals, idx, (const uint16_t*)bias, out,
                                        in, N, M, dtype, (uint16_t*)Y, workspace, dev_status, stream);
@@ -379,6 +394,10 @@ elsa_status elsa_nm_linear_masked(const void* X, int rows, const void* W_sup, co
     if ((st = pick_kind(rows, out, in, N, M, dev.sm_count, &kind)) != ELSA_OK) return st;
     if (kind == KIND_SIMT || kind == KIND_SPARSE_ONE)
         return fail(ELSA_ERR_NM, "the forced variant has no mask-on-load form");
+    if (kind == KIND_SMALL) {
+        const SmallJob job = small_job(X, rows, W_sup, nullptr, bias, out, in, N, M, Y, N != M);
+        return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, dev.sm_count), false, dtype, dev_status, stream);
+    }
     if (kind == KIND_SPARSE_PAIR || kind == KIND_SPARSE_WS || kind == KIND_SPARSE_ST) {
         uint8_t* meta = (uint8_t*)workspace + sp24_meta_offset(out, in);
         if ((st = launch_dense_to_sp24((const uint16_t*)W_sup, out, in, N, M, 128, sp24_layout_of(kind), (uint16_t*)workspace, meta,
@@ -485,12 +504,22 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
     const bool grouped = g_grouping.load(std::memory_order_relaxed) &&
                          g_variant.load(std::memory_order_relaxed) == ELSA_VARIANT_AUTO &&
                          workspace_bytes >= elsa_vit_workspace_bytes(cfg, n_layers, dtype);
+    std::vector<LinearKind> kind(n_layers);
+    std::vector<SmallJob> small;
+    for (int l = 0; l < n_layers; ++l) {
+        const elsa_layer& c = cfg[l];
+        if ((st = pick_kind(c.rows, c.out, c.in, c.N, c.M, dev.sm_count, &kind[l])) != ELSA_OK) return layer_fail(st, l);
+        if (kind[l] == KIND_SMALL)
+            small.push_back(small_job(c.X, c.rows, c.vals, c.N == c.M ? nullptr : c.idx, c.bias, c.out, c.in, c.N, c.M, c.Y));
+    }
+    // cut as they are in shared launches, so that results do not depend on the scratch given
+    const int small_splits = small.empty() ? 0 : linear_small_splits(small.data(), (int)small.size(), dev.sm_count);
     if (!grouped) {
         for (int l = 0; l < n_layers; ++l) {
             const elsa_layer& c = cfg[l];
             set_profile_layer(l);
             st = run_linear(c.X, c.rows, c.vals, c.N == c.M ? nullptr : c.idx, c.bias, c.out, c.in, c.N, c.M, dtype,
-                            c.Y, workspace, dev_status, stream);
+                            c.Y, workspace, dev_status, stream, small_splits);
             if (st != ELSA_OK) return layer_fail(st, l);
         }
         set_profile_layer(-1);
@@ -502,12 +531,10 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
     // one CTA per SM.  Everything else waits for the images.
     SidePipe* side = nullptr;
     if ((st = side_pipe(dev.device, &side)) != ELSA_OK) return st;
-    std::vector<LinearKind> kind(n_layers);
     std::vector<uint8_t*> region(n_layers);
     size_t off = 0;
     for (int l = 0; l < n_layers; ++l) {
         const elsa_layer& c = cfg[l];
-        if ((st = pick_kind(c.rows, c.out, c.in, c.N, c.M, dev.sm_count, &kind[l])) != ELSA_OK) return layer_fail(st, l);
         region[l] = (uint8_t*)workspace + off;
         off += round_up(elsa_workspace_bytes(c.rows, c.in, c.out, c.N, c.M, dtype), 256);
     }
@@ -549,7 +576,7 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
         table.total_units = 0;
         for (int l = 0; l < n_layers; ++l) {
             const elsa_layer& c = cfg[l];
-            if (c.N != c.M) {
+            if (c.N != c.M && kind[l] != KIND_SMALL) {
                 if (kind[l] == KIND_SPARSE_PAIR || kind[l] == KIND_SPARSE_WS || kind[l] == KIND_SPARSE_ST) {
                     uint8_t* meta = region[l] + sp24_meta_offset(c.out, c.in);
                     batch_add_to_sp24(&table, (const uint16_t*)c.vals, c.idx, c.out, c.in, c.N, c.M, 128,
@@ -643,17 +670,11 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
             }
         }
     }
-    // small layers: one CTA per tile, one launch each
-    for (int l = 0; l < n_layers; ++l) {
-        if (kind[l] != KIND_DENSE_ONE) continue;
-        const elsa_layer& c = cfg[l];
-        set_profile_layer(l);
-        const uint16_t* Wd = c.N == c.M ? (const uint16_t*)c.vals : (const uint16_t*)region[l];
-        st = launch_linear_tc_dense((const uint16_t*)c.X, c.rows, Wd, (const uint16_t*)c.bias, c.out, c.in, dtype,
-                                    (uint16_t*)c.Y, dev_status, stream);
-        if (st != ELSA_OK) return layer_fail(st, l);
+    // layers with few rows, straight from their packed weights, in groups
+    for (size_t at = 0; at < small.size(); at += (size_t)linear_small_group_max()) {
+        const int n = (int)(small.size() - at) < linear_small_group_max() ? (int)(small.size() - at) : linear_small_group_max();
+        if ((st = launch_linear_small_group(small.data() + at, n, small_splits, false, dtype, dev_status, stream)) != ELSA_OK) return st;
     }
-    set_profile_layer(-1);
     return ELSA_OK;
 }
 
@@ -824,6 +845,7 @@ struct BlockLinear {
     LinearKind kind;
     void* ws;          // this linear's part of region WORKSPACE
     bool image_ready;  // its weight image has been enqueued already
+    bool first;        // no kernel of the same call runs before it
 };
 
 struct BlockPlan {
@@ -895,6 +917,7 @@ elsa_status block_check(const void* x, int rows, int dim, int mlp_dim, const els
         lin[l].out = outs[l];
         lin[l].ws = (uint8_t*)scratch + plan->ws_off[l];
         lin[l].image_ready = false;
+        lin[l].first = false;
         elsa_status st = pick_kind(rows, outs[l], ins[l], src[l]->N, src[l]->M, dev.sm_count, &lin[l].kind);
         if (st != ELSA_OK) return st;
     }
@@ -938,6 +961,14 @@ elsa_status block_linear(BlockLinear& L, const uint16_t* X, int rows, elsa_dtype
         job.rows = rows; job.in = L.in; job.out = L.out;
         job.act = act; job.residual = residual;
         return launch_linear_tc_pair_group(&job, 1, dtype, dev_status, stream);
+    }
+    if (L.kind == KIND_SMALL) {
+        SmallJob job = small_job(X, rows, w.vals, w.N == w.M ? nullptr : w.idx, w.bias, L.out, L.in, w.N, w.M, Y);
+        job.act = act; job.residual = residual;
+        DeviceInfo dev;
+        if ((st = device_info(&dev)) != ELSA_OK) return st;
+        // after another kernel of the same call the weights are older than that kernel's start
+        return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, dev.sm_count), !L.first, dtype, dev_status, stream);
     }
     *residual_left = residual != nullptr;
     uint16_t* dst = residual ? tmp : Y;
@@ -1058,6 +1089,7 @@ elsa_status elsa_vit_block_rest(const void* x, int rows, int dim, int mlp_dim, c
     BlockLinear lin[4];
     if ((st = block_check(x, rows, dim, mlp_dim, w, dtype, y, true, scratch, scratch_bytes, &plan, lin, dev)) != ELSA_OK)
         return st;
+    lin[1].first = true;
     return block_rest((const uint16_t*)x, rows, dim, mlp_dim, w, dtype, (uint16_t*)y, (uint8_t*)scratch, plan, lin,
                       dev_status, (cudaStream_t)stream);
 }
@@ -1365,9 +1397,11 @@ elsa_status dense_product(const uint16_t* A, int m, const uint16_t* B, int n, in
                           uint32_t* dev_status, cudaStream_t stream, int sm_count)
 {
     const int variant = g_variant.load(std::memory_order_relaxed);
-    const bool pair = variant == ELSA_VARIANT_TC_PAIR || (variant != ELSA_VARIANT_TC_DENSE && linear_tc_pair_suits(m, n, sm_count));
-    return pair ? launch_linear_tc_pair(A, m, B, nullptr, n, k, dtype, Y, dev_status, stream)
-                : launch_linear_tc_dense(A, m, B, nullptr, n, k, dtype, Y, dev_status, stream);
+    if (variant == ELSA_VARIANT_TC_DENSE) return launch_linear_tc_dense(A, m, B, nullptr, n, k, dtype, Y, dev_status, stream);
+    if (variant == ELSA_VARIANT_TC_PAIR || (variant != ELSA_VARIANT_TC_SMALL && linear_tc_pair_suits(m, n, sm_count)))
+        return launch_linear_tc_pair(A, m, B, nullptr, n, k, dtype, Y, dev_status, stream);
+    const SmallJob job = small_job(A, m, B, nullptr, nullptr, n, k, 8, 8, Y);
+    return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, sm_count), false, dtype, dev_status, stream);
 }
 
 }  // namespace
@@ -1443,7 +1477,7 @@ elsa_status elsa_set_linear_variant(elsa_variant v)
 {
     if (v != ELSA_VARIANT_AUTO && v != ELSA_VARIANT_SIMT && v != ELSA_VARIANT_TC_DENSE && v != ELSA_VARIANT_TC_PAIR &&
         v != ELSA_VARIANT_TC_SPARSE && v != ELSA_VARIANT_TC_SPARSE_PAIR && v != ELSA_VARIANT_TC_SPARSE_WS &&
-        v != ELSA_VARIANT_TC_SPARSE_ST)
+        v != ELSA_VARIANT_TC_SPARSE_ST && v != ELSA_VARIANT_TC_SMALL)
         return fail(ELSA_ERR_SHAPE, "unknown variant %d", (int)v);
     g_variant.store((int)v, std::memory_order_relaxed);
     return ELSA_OK;

@@ -94,6 +94,26 @@ elsa_status launch_linear_tc_dense(const uint16_t* X, int rows, const uint16_t* 
                                    const uint16_t* bias, int out, int in, elsa_dtype dtype,
                                    uint16_t* Y, uint32_t* dev_status, cudaStream_t stream);
 
+// Few token rows: the product straight from the packed weight (or the dense shared weight projected on the fly), one
+// launch for up to linear_small_group_max() independent layers.  early: the weights are older than the call's first
+// kernel, so their expansion may start before the predecessor kernel has ended.
+struct SmallJob {
+    const uint16_t* X;
+    const uint16_t* w;        // packed values (N == M: the weight itself); masked: the dense shared weight
+    const uint32_t* idx;
+    const uint16_t* bias;
+    uint16_t* Y;
+    int rows, in, out, N, M;
+    bool masked = false;
+    int act = 0;                          // 0 none, 1 GELU
+    const uint16_t* residual = nullptr;   // [rows][out], added after the activation, before the one rounding
+};
+int linear_small_group_max();
+// Ranges the reductions of these jobs are cut into when they run together.  A result depends on it in its last bits.
+int linear_small_splits(const SmallJob* jobs, int n, int sm_count);
+elsa_status launch_linear_small_group(const SmallJob* jobs, int n, int splits, bool early, elsa_dtype dtype, uint32_t* dev_status,
+                                      cudaStream_t stream);
+
 // The same GEMM on CTA pairs (cluster of two, tcgen05 cta_group::2); for large row counts.
 elsa_status launch_linear_tc_pair(const uint16_t* X, int rows, const uint16_t* Wd, const uint16_t* bias,
                                   int out, int in, elsa_dtype dtype, uint16_t* Y, uint32_t* dev_status,

@@ -507,6 +507,160 @@ __device__ __forceinline__ void unpack_group(const uint16_t* __restrict__ vals, 
     }
 }
 
+// ---- eight consecutive positions of a packed row as one 16-byte unit (groups of 4: two groups, groups of 8: one),
+// in two halves so that a caller can have the loads of several units in flight before it expands the first.
+struct PackedUnit {
+    uint32_t v[4];      // the unit's kept values in order, two per word
+    uint32_t fields;    // their index fields, first value lowest
+};
+
+// NC: the level's N as a compile-time constant (0 = take `N_runtime`).  N < M.  Reads go past L1, which is not known to be
+// clean of older contents while a predecessor kernel still runs (see `early` in elsa_linear_small.cu).
+template <int M, int NC>
+__device__ __forceinline__ PackedUnit load_packed_unit(const uint16_t* __restrict__ vals_row, const uint32_t* __restrict__ idx_row,
+                                                       int N_runtime, int unit)
+{
+    static_assert(M == 4 || M == 8, "groups of 16 hold two units: expand_unit16");
+    constexpr int B = M == 4 ? 2 : 3;
+    const int N = NC ? NC : N_runtime;
+    const int count = (8 / M) * N;              // values of the unit
+    PackedUnit p;
+    p.v[0] = p.v[1] = p.v[2] = p.v[3] = 0u;
+    const uint16_t* v = vals_row + (size_t)unit * count;
+    if ((count & 3) == 0) {                     // 4 values at most (8 would be the dense level)
+        const uint2 t = __ldcg(reinterpret_cast<const uint2*>(v));
+        p.v[0] = t.x; p.v[1] = t.y;
+    } else if ((count & 1) == 0) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (q < (count >> 1)) p.v[q] = __ldcg(reinterpret_cast<const uint32_t*>(v) + q);
+    } else {
+#pragma unroll
+        for (int t = 0; t < 7; ++t)
+            if (t < count) p.v[t >> 1] |= (uint32_t)__ldcg(v + t) << (16 * (t & 1));
+    }
+    const int bit0 = unit * count * B, w0 = bit0 >> 5, sh = bit0 & 31;
+    const uint32_t lo = __ldcg(idx_row + w0);
+    const uint32_t hi = (sh + count * B > 32) ? __ldcg(idx_row + w0 + 1) : 0u;
+    p.fields = __funnelshift_r(lo, hi, sh);
+    return p;
+}
+
+// shl that gives 0 for shifts of 32 and more (negative ones included)
+__device__ __forceinline__ uint32_t shl_or_zero(uint32_t v, uint32_t s)
+{
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));
+    return r;
+}
+
+// Up to two values (the halves of w) at the positions of a group of 8 or 4: byte-permute selectors that start as "zero
+// byte" (bytes of the permute's second operand) and get the value's two bytes at its position, 8 selector bits apiece.
+template <bool kTwo>
+__device__ __forceinline__ uint4 place_in_8(uint32_t w, uint32_t fields)
+{
+    const uint32_t a0 = (fields << 3) & 0x38u, a1 = fields & 0x38u;
+    uint32_t lo = 0x44444444u ^ shl_or_zero(0x54u, a0), hi = 0x44444444u ^ shl_or_zero(0x54u, a0 - 32u);
+    if constexpr (kTwo) {
+        lo ^= shl_or_zero(0x76u, a1);
+        hi ^= shl_or_zero(0x76u, a1 - 32u);
+    }
+    return make_uint4(prmt(w, 0u, lo), prmt(w, 0u, lo >> 16), prmt(w, 0u, hi), prmt(w, 0u, hi >> 16));
+}
+
+// kTwo: both halves of w; otherwise its low (kHigh: high) half alone.
+template <bool kTwo, bool kHigh>
+__device__ __forceinline__ uint2 place_in_4(uint32_t w, uint32_t fields)
+{
+    uint32_t sel = 0x44444444u ^ ((kHigh ? 0x76u : 0x54u) << ((fields << 3) & 0x18u));
+    if constexpr (kTwo) sel ^= 0x76u << ((fields << 1) & 0x18u);
+    return make_uint2(prmt(w, 0u, sel), prmt(w, 0u, sel >> 16));
+}
+
+// The unit's eight positions: values at theirs, +0.0 elsewhere.  The common levels place one or two values per permute;
+// the others split the values into a plane of low bytes and one of high bytes, scatter those by byte permutes
+// (selector nibble of a position = slot of its value; slot 7 is zero because fewer than eight values are kept) and
+// re-interleave.
+template <int M, int NC>
+__device__ __forceinline__ uint4 expand_packed_unit(const PackedUnit& p, int N_runtime)
+{
+    if constexpr (M == 8 && NC == 1) return place_in_8<false>(p.v[0], p.fields);
+    if constexpr (M == 8 && NC == 2) return place_in_8<true>(p.v[0], p.fields);
+    if constexpr (M == 8 && NC == 4) {
+        const uint4 a = place_in_8<true>(p.v[0], p.fields), b = place_in_8<true>(p.v[1], p.fields >> 6);
+        return make_uint4(a.x | b.x, a.y | b.y, a.z | b.z, a.w | b.w);
+    }
+    if constexpr (M == 4 && NC == 1) {
+        const uint2 a = place_in_4<false, false>(p.v[0], p.fields), b = place_in_4<false, true>(p.v[0], p.fields >> 2);
+        return make_uint4(a.x, a.y, b.x, b.y);
+    }
+    if constexpr (M == 4 && NC == 2) {
+        const uint2 a = place_in_4<true, false>(p.v[0], p.fields), b = place_in_4<true, false>(p.v[1], p.fields >> 4);
+        return make_uint4(a.x, a.y, b.x, b.y);
+    }
+    constexpr int B = M == 4 ? 2 : 3;
+    const int N = NC ? NC : N_runtime;
+    uint32_t sel = 0x77777777u;
+#pragma unroll
+    for (int t = 0; t < 7; ++t)
+        if (t < (8 / M) * N) {
+            uint32_t pos = (p.fields >> (t * B)) & (uint32_t)(M - 1);
+            if (M == 4 && t >= N) pos += 4u;
+            sel ^= (uint32_t)(7 ^ t) << (4u * pos);      // positions are distinct: the nibble is still 7
+        }
+    const uint32_t l0 = prmt(p.v[0], p.v[1], 0x6420u), l1 = prmt(p.v[2], p.v[3], 0x6420u);
+    const uint32_t h0 = prmt(p.v[0], p.v[1], 0x7531u), h1 = prmt(p.v[2], p.v[3], 0x7531u);
+    const uint32_t pl03 = prmt(l0, l1, sel & 0xFFFFu), pl47 = prmt(l0, l1, sel >> 16);
+    const uint32_t ph03 = prmt(h0, h1, sel & 0xFFFFu), ph47 = prmt(h0, h1, sel >> 16);
+    return make_uint4(prmt(pl03, ph03, 0x5140u), prmt(pl03, ph03, 0x7362u), prmt(pl47, ph47, 0x5140u), prmt(pl47, ph47, 0x7362u));
+}
+
+// A unit of a packed row with groups of 16: half of group unit / 2.
+__device__ __forceinline__ uint4 expand_unit16(const uint16_t* __restrict__ vals_row, const uint32_t* __restrict__ idx_row, int N, int unit)
+{
+    const int g = unit >> 1, bit0 = g * N * 4, w0 = bit0 >> 5, sh = bit0 & 31;
+    unsigned long long fields = __ldcg(idx_row + w0);
+    if (sh + 4 * N > 32) fields |= (unsigned long long)__ldcg(idx_row + w0 + 1) << 32;
+    fields >>= sh;
+    if (sh + 4 * N > 64) fields |= (unsigned long long)__ldcg(idx_row + w0 + 2) << (64 - sh);
+    const uint16_t* v = vals_row + (size_t)g * N;
+    unsigned long long lo = 0, hi = 0;
+    for (int t = 0; t < N; ++t) {
+        const uint32_t pos = (uint32_t)(fields >> (4 * t)) & 15u;
+        if ((int)(pos >> 3) != (unit & 1)) continue;
+        const unsigned long long x = (unsigned long long)__ldcg(v + t) << (16u * (pos & 3u));
+        if (pos & 4u) hi |= x; else lo |= x;
+    }
+    return make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
+}
+
+// Eight consecutive positions of a DENSE row projected onto level N:M, from the 16 bytes of the unit (groups of 16:
+// from the whole group w, w16, with `half` saying which eight are wanted).
+template <int M>
+__device__ __forceinline__ uint4 mask_unit(const uint4& w, const uint4& w16, int half, int N)
+{
+    uint32_t keep = 0, a[4] = {w.x, w.y, w.z, w.w};
+    if constexpr (M == 16) {
+        const uint32_t b[8] = {w.x, w.y, w.z, w.w, w16.x, w16.y, w16.z, w16.w};
+        uint16_t h[16];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) { h[2 * q] = (uint16_t)(b[q] & 0xFFFFu); h[2 * q + 1] = (uint16_t)(b[q] >> 16); }
+        keep = keep_mask<16>(group_ranks<16>(h), N) >> (8 * half);
+        if (half) { a[0] = w16.x; a[1] = w16.y; a[2] = w16.z; a[3] = w16.w; }
+    } else {
+#pragma unroll
+        for (int gl = 0; gl < 8 / M; ++gl) {
+            uint32_t h[M];
+#pragma unroll
+            for (int i = 0; i < M; ++i) h[i] = (a[(gl * M + i) >> 1] >> (16 * (i & 1))) & 0xFFFFu;
+            keep |= keep_mask_sorted<M>(h, N) << (gl * M);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] &= ((keep >> (2 * q)) & 1u ? 0xFFFFu : 0u) | ((keep >> (2 * q + 1)) & 1u ? 0xFFFF0000u : 0u);
+    return make_uint4(a[0], a[1], a[2], a[3]);
+}
+
 // One thread per (weight row, 16 consecutive k): rebuilds those 16 positions from the packed form,
 // then emits, per aligned chunk of 4, two values with ascending positions (i0 < i1).  Pruned
 // positions are zero in the rebuilt segment, so a chunk with fewer than two kept weights simply
