@@ -171,6 +171,19 @@ int sp24_layout_of(LinearKind kind)
     return kind == KIND_SPARSE_WS ? SP24_PERMUTED : kind == KIND_SPARSE_ST ? SP24_TILED : SP24_ROWS;
 }
 
+// The weight image that a layer's kernel reads, built in `region`.
+ImageJob image_job(LinearKind kind, const void* vals, const uint32_t* idx, int out, int in, int N, int M, void* region)
+{
+    ImageJob j;
+    j.src = (const uint16_t*)vals; j.idx = idx; j.dst = (uint16_t*)region; j.out = out; j.in = in; j.N = N; j.M = M;
+    if (kind == KIND_SPARSE_PAIR || kind == KIND_SPARSE_WS || kind == KIND_SPARSE_ST) {
+        j.kind = IMAGE_SP24;
+        j.meta = (uint8_t*)region + sp24_meta_offset(out, in);
+        j.layout = sp24_layout_of(kind);
+    }
+    return j;
+}
+
 // Which kernel a layer runs on.  AUTO is the product rule; a forced variant is honoured where it applies.
 elsa_status pick_kind(int rows, int out, int in, int N, int M, int sm_count, LinearKind* kind)
 {
@@ -398,11 +411,13 @@ elsa_status elsa_nm_linear_masked(const void* X, int rows, const void* W_sup, co
         const SmallJob job = small_job(X, rows, W_sup, nullptr, bias, out, in, N, M, Y, N != M);
         return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, dev.sm_count), false, dtype, dev_status, stream);
     }
+    ImageJob image;
+    image.src = (const uint16_t*)W_sup; image.dst = (uint16_t*)workspace; image.out = out; image.in = in; image.N = N; image.M = M;
     if (kind == KIND_SPARSE_PAIR || kind == KIND_SPARSE_WS || kind == KIND_SPARSE_ST) {
-        uint8_t* meta = (uint8_t*)workspace + sp24_meta_offset(out, in);
-        if ((st = launch_dense_to_sp24((const uint16_t*)W_sup, out, in, N, M, 128, sp24_layout_of(kind), (uint16_t*)workspace, meta,
-                                       stream)) != ELSA_OK)
-            return st;
+        image.kind = IMAGE_MASK_SP24;
+        image.meta = (uint8_t*)workspace + sp24_meta_offset(out, in);
+        image.layout = sp24_layout_of(kind);
+        if ((st = launch_images(&image, 1, stream)) != ELSA_OK) return st;
         SparseJob job;
         job.X = (const uint16_t*)X; job.bias = (const uint16_t*)bias; job.Y = (uint16_t*)Y; job.workspace = workspace;
         job.rows = rows; job.in = in; job.out = out;
@@ -412,7 +427,8 @@ elsa_status elsa_nm_linear_masked(const void* X, int rows, const void* W_sup, co
     }
     const uint16_t* Wd = (const uint16_t*)W_sup;     // the dense level multiplies the shared weight as it is
     if (N != M) {
-        if ((st = launch_mask((const uint16_t*)W_sup, out, in, N, M, (uint16_t*)workspace, stream)) != ELSA_OK) return st;
+        image.kind = IMAGE_MASK;
+        if ((st = launch_images(&image, 1, stream)) != ELSA_OK) return st;
         Wd = (const uint16_t*)workspace;
     }
     if (kind == KIND_DENSE_PAIR)
@@ -569,28 +585,13 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
     cudaStream_t image_stream = forked ? side->stream : stream;
     // weight images of all layers, one launch per 256 layers
     {
-        static BatchTable table;          // host staging of the kernel parameters
-        static std::mutex table_mutex;
-        std::lock_guard<std::mutex> lock(table_mutex);
-        table.n = 0;
-        table.total_units = 0;
+        std::vector<ImageJob> jobs;
         for (int l = 0; l < n_layers; ++l) {
             const elsa_layer& c = cfg[l];
-            if (c.N != c.M && kind[l] != KIND_SMALL) {
-                if (kind[l] == KIND_SPARSE_PAIR || kind[l] == KIND_SPARSE_WS || kind[l] == KIND_SPARSE_ST) {
-                    uint8_t* meta = region[l] + sp24_meta_offset(c.out, c.in);
-                    batch_add_to_sp24(&table, (const uint16_t*)c.vals, c.idx, c.out, c.in, c.N, c.M, 128,
-                                      sp24_layout_of(kind[l]), (uint16_t*)region[l], meta);
-                } else {
-                    batch_add_unpack(&table, (const uint16_t*)c.vals, c.idx, c.out, c.in, c.N, c.M, (uint16_t*)region[l]);
-                }
-            }
-            if (table.n == kBatchMax || (l == n_layers - 1 && table.n > 0)) {
-                if ((st = launch_image_batch(table, image_stream)) != ELSA_OK) return st;
-                table.n = 0;
-                table.total_units = 0;
-            }
+            if (c.N != c.M && kind[l] != KIND_SMALL)
+                jobs.push_back(image_job(kind[l], c.vals, c.idx, c.out, c.in, c.N, c.M, region[l]));
         }
+        if (!jobs.empty() && (st = launch_images(jobs.data(), (int)jobs.size(), image_stream)) != ELSA_OK) return st;
     }
     if (forked) {
         cudaError_t e = cudaEventRecord(side->join, side->stream);
@@ -924,23 +925,24 @@ elsa_status block_check(const void* x, int rows, int dim, int mlp_dim, const els
     return ELSA_OK;
 }
 
-// The weight image of a linear whose kernel takes it ready-made (the others build theirs when they run).
-elsa_status block_image(BlockLinear& L, cudaStream_t stream)
+// Whether a linear's kernel takes a ready-made weight image (the others build theirs when they run, or need none).
+bool takes_image(const BlockLinear& L)
 {
-    const elsa_block_linear& w = *L.w;
-    elsa_status st = ELSA_OK;
-    if (w.N == w.M) return ELSA_OK;
-    if (L.kind == KIND_DENSE_PAIR)
-        st = launch_unpack((const uint16_t*)w.vals, w.idx, L.out, L.in, w.N, w.M, (uint16_t*)L.ws, stream);
-    else if (L.kind == KIND_SPARSE_WS)
-        st = launch_linear_tc_sparse_pair_prepare((const uint16_t*)w.vals, w.idx, L.out, L.in, w.N, w.M, SP24_PERMUTED,
-                                                  L.ws, stream);
-    else if (L.kind == KIND_SPARSE_ST)
-        st = launch_nm_to_sp24((const uint16_t*)w.vals, w.idx, L.out, L.in, w.N, w.M, 128, SP24_TILED, (uint16_t*)L.ws,
-                               (uint8_t*)L.ws + sp24_meta_offset(L.out, L.in), stream);
-    else
-        return ELSA_OK;
-    L.image_ready = st == ELSA_OK;
+    return L.w->N != L.w->M && (L.kind == KIND_DENSE_PAIR || L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST);
+}
+
+// The images of the linears that take one, in one launch.
+elsa_status block_images(BlockLinear* lin, int n, cudaStream_t stream)
+{
+    ImageJob jobs[4];
+    int count = 0;
+    for (int l = 0; l < n; ++l)
+        if (takes_image(lin[l]) && !lin[l].image_ready)
+            jobs[count++] = image_job(lin[l].kind, lin[l].w->vals, lin[l].w->idx, lin[l].out, lin[l].in, lin[l].w->N, lin[l].w->M, lin[l].ws);
+    if (count == 0) return ELSA_OK;
+    const elsa_status st = launch_images(jobs, count, stream);
+    if (st == ELSA_OK)
+        for (int l = 0; l < n; ++l) lin[l].image_ready = takes_image(lin[l]);
     return st;
 }
 
@@ -954,7 +956,7 @@ elsa_status block_linear(BlockLinear& L, const uint16_t* X, int rows, elsa_dtype
     elsa_status st = ELSA_OK;
     *residual_left = false;
     if (L.kind == KIND_DENSE_PAIR) {
-        if (w.N != w.M && !L.image_ready && (st = block_image(L, stream)) != ELSA_OK) return st;
+        if ((st = block_images(&L, 1, stream)) != ELSA_OK) return st;
         PairJob job;
         job.X = X; job.Wd = w.N == w.M ? (const uint16_t*)w.vals : (const uint16_t*)L.ws;
         job.bias = (const uint16_t*)w.bias; job.Y = Y;
@@ -973,7 +975,7 @@ elsa_status block_linear(BlockLinear& L, const uint16_t* X, int rows, elsa_dtype
     *residual_left = residual != nullptr;
     uint16_t* dst = residual ? tmp : Y;
     if (L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST) {
-        if (!L.image_ready && (st = block_image(L, stream)) != ELSA_OK) return st;
+        if ((st = block_images(&L, 1, stream)) != ELSA_OK) return st;
         SparseJob job;
         job.X = X; job.bias = (const uint16_t*)w.bias; job.Y = dst; job.workspace = L.ws;
         job.rows = rows; job.in = L.in; job.out = L.out; job.act = act;
@@ -1116,16 +1118,14 @@ elsa_status run_block(const void* x, int rows, int dim, int mlp_dim, const elsa_
     // The four weight images do not depend on x: they are built on the library's side stream while the first
     // LayerNorm runs on the caller's, which waits for them before the first linear.
     bool any_image = false;
-    for (int l = 0; l < 4; ++l)
-        any_image = any_image || (lin[l].w->N != lin[l].w->M && (lin[l].kind == KIND_DENSE_PAIR ||
-                                                                  lin[l].kind == KIND_SPARSE_WS || lin[l].kind == KIND_SPARSE_ST));
+    for (int l = 0; l < 4; ++l) any_image = any_image || takes_image(lin[l]);
     SidePipe* side = nullptr;
     if (any_image) {
         if ((st = side_pipe(dev.device, &side)) != ELSA_OK) return st;
         cudaError_t e = cudaEventRecord(side->fork, stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(side->stream, side->fork, 0);
         if (e != cudaSuccess) return fail(ELSA_ERR_CUDA, "forking the image stream: %s", cudaGetErrorString(e));
-        for (int l = 0; l < 4 && st == ELSA_OK; ++l) st = block_image(lin[l], side->stream);
+        st = block_images(lin, 4, side->stream);
         e = cudaEventRecord(side->join, side->stream);   // joined even after a failed launch: the fork must not dangle
         if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, side->join, 0);
         if (st != ELSA_OK) return st;

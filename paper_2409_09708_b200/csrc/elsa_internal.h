@@ -141,6 +141,19 @@ enum Sp24Layout { SP24_ROWS = 0, SP24_PERMUTED = 1, SP24_TILED = 2 };
 // packed weight -> 2-of-4 image + metadata blocks of 2 KB per (128 features, block_k of K), block_k = 64 or 128.
 elsa_status launch_nm_to_sp24(const uint16_t* vals, const uint32_t* idx, int out, int in, int N, int M, int block_k,
                               int layout, uint16_t* a_img, uint8_t* meta, cudaStream_t stream);
+// Any number of weight images, one launch per 256: the dense masked weight or its 2-of-4 form, from the packed weight
+// or from the dense shared weight projected onto its level (src then holds the dense weight, idx is unused).
+enum ImageKind { IMAGE_UNPACK = 0, IMAGE_SP24 = 1, IMAGE_MASK = 2, IMAGE_MASK_SP24 = 3 };
+struct ImageJob {
+    int kind = IMAGE_UNPACK;
+    const uint16_t* src = nullptr;
+    const uint32_t* idx = nullptr;
+    uint16_t* dst = nullptr;
+    uint8_t* meta = nullptr;      // 2-of-4 forms
+    int out = 0, in = 0, N = 0, M = 0;
+    int layout = SP24_ROWS, block_k = 128;
+};
+elsa_status launch_images(const ImageJob* jobs, int n, cudaStream_t stream);
 // Where the metadata blocks start in a layer's scratch: after the image, whose rows are rounded up to 32.
 inline size_t sp24_meta_offset(int out, int in) { return round_up((size_t)((out + 31) / 32 * 32) * (size_t)in, 256); }
 // The same on CTA pairs (256 features x 224 rows per pair, K blocks of 128).
@@ -220,7 +233,7 @@ elsa_status launch_mask_apply(uint16_t* dW, const uint32_t* idx, int out, int in
 // dW [out][in] = mask .* round16(sum over ranges of partial [splits][out][in]); idx NULL (N == M) keeps everything.
 elsa_status launch_wgrad_finish(const float* partial, int splits, const uint32_t* idx, int out, int in, int N, int M,
                                 elsa_dtype dtype, uint16_t* dW, cudaStream_t stream);
-// Several levels of one weight in one pass, and the dense projections used by the mask-on-load linear.
+// Several levels of one weight in one pass.
 constexpr int kMaxLevels = 16;
 struct LevelTable {
     int n;
@@ -229,19 +242,14 @@ struct LevelTable {
     uint32_t* idx[kMaxLevels];
 };
 elsa_status launch_compress_levels(const uint16_t* W, int out, int in, int M, const LevelTable& t, cudaStream_t stream);
-elsa_status launch_mask(const uint16_t* W, int out, int in, int N, int M, uint16_t* Wm, cudaStream_t stream);
-elsa_status launch_dense_to_sp24(const uint16_t* W, int out, int in, int N, int M, int block_k, int layout,
-                                 uint16_t* a_img, uint8_t* meta, cudaStream_t stream);
 
-// Batched weight-format kernels: one launch over a table of weights (kernel-parameter space).
-enum BatchKind { BATCH_COMPRESS = 0, BATCH_UNPACK = 1, BATCH_TO_SP24 = 2 };
+// Batched compress: one launch over a table of weights (kernel-parameter space).
 struct BatchItem {
     const void* src;
-    const void* src2;
     void* dst;
     void* dst2;
     long long first_unit;   // prefix sum of work units over the table
-    int out, in, N, M, wpr, aux, aux2, aux3, kind;
+    int out, in, N, M, wpr, segs_per_row;
 };
 constexpr int kBatchMax = 256;
 struct BatchTable {
@@ -250,12 +258,7 @@ struct BatchTable {
     int n;
 };
 void batch_add_compress(BatchTable* t, const uint16_t* W, int out, int in, int N, int M, uint16_t* vals, uint32_t* idx);
-void batch_add_unpack(BatchTable* t, const uint16_t* vals, const uint32_t* idx, int out, int in, int N, int M,
-                      uint16_t* Wm);
-void batch_add_to_sp24(BatchTable* t, const uint16_t* vals, const uint32_t* idx, int out, int in, int N, int M,
-                       int block_k, int layout, uint16_t* a_img, uint8_t* meta);
 elsa_status launch_compress_batch(const BatchTable& t, cudaStream_t stream);
-elsa_status launch_image_batch(const BatchTable& t, cudaStream_t stream);
 
 // Several dense-rate layers in one persistent launch of the CTA-pair kernel (at most
 // linear_tc_pair_group_max() of them): their tiles form one sequence.

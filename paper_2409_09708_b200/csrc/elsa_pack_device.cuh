@@ -371,142 +371,6 @@ __device__ __forceinline__ void compress_segment(const uint16_t* __restrict__ W,
     compress_segment_levels<M>(W, in, 1, &N, &vals_one, &idx_one, segs_per_row, seg_id, words);
 }
 
-// One thread projects one group of the dense weight onto level N:M: kept values stay, the others
-// become +0.0 (the "dynamic masking" of Sec. 3.1 applied to the shared weight, with no packed form).
-template <int M>
-__device__ __forceinline__ void mask_group(const uint16_t* __restrict__ W, int N, uint16_t* __restrict__ Wm, long long gid)
-{
-    uint16_t w[M];
-    load_group<M>(W + (size_t)gid * M, w);
-    const uint32_t keep = keep_mask<M>(group_ranks<M>(w), N);
-    uint16_t* dst = Wm + (size_t)gid * M;
-    if constexpr (M == 4) {
-        uint2 r;
-        r.x = (keep & 1u ? w[0] : 0u) | ((uint32_t)(keep & 2u ? w[1] : 0u) << 16);
-        r.y = (keep & 4u ? w[2] : 0u) | ((uint32_t)(keep & 8u ? w[3] : 0u) << 16);
-        *reinterpret_cast<uint2*>(dst) = r;
-    } else {
-#pragma unroll
-        for (int q = 0; q < M / 8; ++q) {
-            uint32_t x[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int i = 8 * q + 2 * k;
-                x[k] = ((keep >> i) & 1u ? (uint32_t)w[i] : 0u) | (((keep >> (i + 1)) & 1u ? (uint32_t)w[i + 1] : 0u) << 16);
-            }
-            reinterpret_cast<uint4*>(dst)[q] = make_uint4(x[0], x[1], x[2], x[3]);
-        }
-    }
-}
-
-// One thread rebuilds one group: N values scattered to their positions, +0.0 elsewhere.
-template <int M>
-__device__ __forceinline__ void unpack_group(const uint16_t* __restrict__ vals, const uint32_t* __restrict__ idx,
-                                             int in, int N, uint16_t* __restrict__ Wm, int words_per_row,
-                                             long long gid)
-{
-    constexpr int B = (M == 4) ? 2 : (M == 8) ? 3 : 4;
-    const int groups_per_row = in / M;
-    const int o = (int)(gid / groups_per_row);
-    const int g = (int)(gid % groups_per_row);
-
-    const uint16_t* v = vals + (size_t)o * ((size_t)groups_per_row * N) + (size_t)g * N;
-    if constexpr (M != 16) {
-        // Groups of 4 and 8 with N < M: the kept values are loaded with the widest access their alignment
-        // allows, split into a plane of low bytes and a plane of high bytes, scattered to their positions by
-        // byte permutes (selector nibble of position i = slot holding its value; unused positions point at
-        // slot M-1, which is zero because N < M), and re-interleaved.
-        if (words_per_row) {
-            constexpr int R = M / 2;
-            const uint32_t* row = idx + (size_t)o * words_per_row;
-            const int bit0 = g * N * B;
-            const int w0 = bit0 >> 5, sh = bit0 & 31;
-            const uint32_t lo = row[w0];
-            const uint32_t hi = (sh + N * B > 32) ? row[w0 + 1] : 0u;
-            const uint32_t fields = __funnelshift_r(lo, hi, sh);
-            uint32_t vr[R];
-#pragma unroll
-            for (int q = 0; q < R; ++q) vr[q] = 0;
-            if ((N & 3) == 0) {                                   // N = 4 (M = 8)
-                const uint2 t = *reinterpret_cast<const uint2*>(v);
-                vr[0] = t.x; vr[1] = t.y;
-            } else if ((N & 1) == 0) {
-#pragma unroll
-                for (int q = 0; q < R; ++q)
-                    if (q < (N >> 1)) vr[q] = reinterpret_cast<const uint32_t*>(v)[q];
-            } else {
-#pragma unroll
-                for (int t = 0; t < M; ++t)
-                    if (t < N) vr[t >> 1] |= (uint32_t)v[t] << (16 * (t & 1));
-            }
-            uint32_t inv = (M == 8) ? 0x77777777u : 0x3333u;
-#pragma unroll
-            for (int t = 0; t < M - 1; ++t)
-                if (t < N) {
-                    const uint32_t pos4 = ((fields >> (t * B)) & (uint32_t)(M - 1)) * 4u;
-                    inv = (inv & ~(0xFu << pos4)) | ((uint32_t)t << pos4);
-                }
-            uint16_t* dst = Wm + (size_t)o * in + (size_t)g * M;
-            if constexpr (M == 4) {
-                const uint32_t pl = prmt(prmt(vr[0], vr[1], 0x6420u), 0u, inv);
-                const uint32_t ph = prmt(prmt(vr[0], vr[1], 0x7531u), 0u, inv);
-                *reinterpret_cast<uint2*>(dst) = make_uint2(prmt(pl, ph, 0x5140u), prmt(pl, ph, 0x7362u));
-            } else {
-                const uint32_t l0 = prmt(vr[0], vr[1], 0x6420u), l1 = prmt(vr[2], vr[3], 0x6420u);
-                const uint32_t h0 = prmt(vr[0], vr[1], 0x7531u), h1 = prmt(vr[2], vr[3], 0x7531u);
-                const uint32_t pl03 = prmt(l0, l1, inv & 0xFFFFu), pl47 = prmt(l0, l1, inv >> 16);
-                const uint32_t ph03 = prmt(h0, h1, inv & 0xFFFFu), ph47 = prmt(h0, h1, inv >> 16);
-                *reinterpret_cast<uint4*>(dst) = make_uint4(prmt(pl03, ph03, 0x5140u), prmt(pl03, ph03, 0x7362u),
-                                                            prmt(pl47, ph47, 0x5140u), prmt(pl47, ph47, 0x7362u));
-            }
-            return;
-        }
-    }
-    unsigned long long fields;
-    if (words_per_row) {
-        const uint32_t* row = idx + (size_t)o * words_per_row;
-        const long long bit0 = (long long)g * N * B;
-        const int w0 = (int)(bit0 >> 5), sh = (int)(bit0 & 31);
-        const int nbits = N * B;
-        unsigned long long lo = row[w0];
-        if (sh + nbits > 32) lo |= (unsigned long long)row[w0 + 1] << 32;
-        fields = lo >> sh;
-        if (sh + nbits > 64) fields |= (unsigned long long)row[w0 + 2] << (64 - sh);
-    } else {
-        fields = 0;  // N == M: position t holds value t
-#pragma unroll
-        for (int t = 0; t < M; ++t) fields |= (unsigned long long)t << (t * B);
-    }
-
-    uint16_t w[M];
-#pragma unroll
-    for (int i = 0; i < M; ++i) w[i] = 0;
-    for (int t = 0; t < N; ++t) {
-        const int pos = (int)((fields >> (t * B)) & (M - 1));
-        const uint16_t val = v[t];
-#pragma unroll
-        for (int i = 0; i < M; ++i) w[i] = (i == pos) ? val : w[i];
-    }
-
-    uint16_t* dst = Wm + (size_t)o * in + (size_t)g * M;
-    if constexpr (M == 4) {
-        uint2 r;
-        r.x = w[0] | ((uint32_t)w[1] << 16);
-        r.y = w[2] | ((uint32_t)w[3] << 16);
-        *reinterpret_cast<uint2*>(dst) = r;
-    } else {
-#pragma unroll
-        for (int q = 0; q < M / 8; ++q) {
-            uint4 r;
-            r.x = w[8 * q + 0] | ((uint32_t)w[8 * q + 1] << 16);
-            r.y = w[8 * q + 2] | ((uint32_t)w[8 * q + 3] << 16);
-            r.z = w[8 * q + 4] | ((uint32_t)w[8 * q + 5] << 16);
-            r.w = w[8 * q + 6] | ((uint32_t)w[8 * q + 7] << 16);
-            reinterpret_cast<uint4*>(dst)[q] = r;
-        }
-    }
-}
-
 // ---- eight consecutive positions of a packed row as one 16-byte unit (groups of 4: two groups, groups of 8: one),
 // in two halves so that a caller can have the loads of several units in flight before it expands the first.
 struct PackedUnit {
@@ -659,144 +523,6 @@ __device__ __forceinline__ uint4 mask_unit(const uint4& w, const uint4& w16, int
 #pragma unroll
     for (int q = 0; q < 4; ++q) a[q] &= ((keep >> (2 * q)) & 1u ? 0xFFFFu : 0u) | ((keep >> (2 * q + 1)) & 1u ? 0xFFFF0000u : 0u);
     return make_uint4(a[0], a[1], a[2], a[3]);
-}
-
-// One thread per (weight row, 16 consecutive k): rebuilds those 16 positions from the packed form,
-// then emits, per aligned chunk of 4, two values with ascending positions (i0 < i1).  Pruned
-// positions are zero in the rebuilt segment, so a chunk with fewer than two kept weights simply
-// borrows a zero from another position.
-// Second half of the 2-of-4 re-encoding: given 16 consecutive positions of a weight row with the pruned
-// ones already zero (d) and the kept set (keep), emits two values per aligned chunk of 4 (ascending
-// positions, a zero borrowed where fewer than two are kept) and the chunk nibbles as tensor memory wants them.
-// In the permuted forms (Sp24Layout) weight row o lands in image row (o & ~31) | (4 * (o % 8) + (o % 32) / 8), so
-// that row r of a block of 32 holds feature 8 * (r % 4) + r / 4: the order in which the transposing stores of the
-// tensor-memory-fed kernels want the features in tensor-memory lanes.  The tiled form also interleaves the
-// 16-byte units of the 32 rows of a block inside every 256 k.  The image has its rows rounded up to 32; rows
-// past `out` are written as zeros.
-__device__ __forceinline__ void sp24_emit(const uint16_t (&d)[16], uint32_t keep, bool real, int o_src, int seg, int k0, int in,
-                                          int out, uint16_t* __restrict__ a_img, uint16_t* __restrict__ meta16, int k_blocks,
-                                          int steps_per_block, int layout)
-{
-    const int o = layout != SP24_ROWS ? ((o_src & ~31) | (4 * (o_src & 7) + ((o_src & 31) >> 3))) : o_src;
-    constexpr int kFeatTile = 128;
-    uint32_t nibbles = 0;
-    uint16_t sel[8];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const uint32_t m4 = (keep >> (4 * c)) & 15u;
-        const int cnt = __popc(m4);
-        int i0, i1;
-        if (cnt >= 2) { i0 = __ffs(m4) - 1; i1 = 31 - __clz(m4); }
-        else if (cnt == 1) { const int p = __ffs(m4) - 1; i0 = (p == 3) ? 0 : p; i1 = 3; }
-        else { i0 = 0; i1 = 1; }
-        nibbles |= (uint32_t)(i0 | (i1 << 2)) << (4 * c);
-        uint16_t v0 = d[4 * c], v1 = d[4 * c];
-#pragma unroll
-        for (int i = 1; i < 4; ++i) {
-            v0 = (i == i0) ? d[4 * c + i] : v0;
-            v1 = (i == i1) ? d[4 * c + i] : v1;
-        }
-        sel[2 * c] = v0;
-        sel[2 * c + 1] = v1;
-    }
-
-    if (k0 < in && o_src < ((out + 31) & ~31)) {      // `d` is all zero where the row or the segment is padding
-        uint4 r;
-        r.x = sel[0] | ((uint32_t)sel[1] << 16);
-        r.y = sel[2] | ((uint32_t)sel[3] << 16);
-        r.z = sel[4] | ((uint32_t)sel[5] << 16);
-        r.w = sel[6] | ((uint32_t)sel[7] << 16);
-        size_t at = (size_t)o * (size_t)in + (size_t)k0;        // byte offset of (row o, k0) in the row-major forms
-        if (layout == SP24_TILED)
-            at = (size_t)(o >> 5) * 32 * (size_t)in + (size_t)(k0 >> 8) * 8192 + (size_t)((((k0 & 255) >> 4) * 32 + (o & 31)) * 16);
-        *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(a_img) + at) = r;
-    }
-    // metadata half-word: block (feature tile, k block) -> lane -> 4 words, one per K step of 32; a
-    // block covers steps_per_block (2 or 4) steps and leaves the other words zero
-    const int ftile = o / kFeatTile, m = o % kFeatTile;
-    const int kb = seg / (2 * steps_per_block), step = (seg / 2) % steps_per_block, k1 = seg % 2;
-    const int lane = (m % 8) + 8 * k1 + 16 * (m / 16);
-    const int hi = (m / 8) % 2;
-    const size_t word = (((size_t)ftile * k_blocks + kb) * 128 + lane) * 4 + step;
-    meta16[2 * word + hi] = (uint16_t)nibbles;
-    if (steps_per_block == 2) meta16[2 * (word + 2) + hi] = 0;
-}
-
-
-
-// One thread per (weight row, 16 consecutive k) of a PACKED weight: rebuilds those 16 positions, then
-// emits their 2-of-4 form.
-template <int M>
-__device__ __forceinline__ void to_sp24_segment(const uint16_t* __restrict__ vals, const uint32_t* __restrict__ idx,
-                                                int out, int in, int N, int words_per_row,
-                                                uint16_t* __restrict__ a_img, uint16_t* __restrict__ meta16,
-                                                int k_blocks, int steps_per_block, int layout, long long tid)
-{
-    constexpr int B = (M == 4) ? 2 : (M == 8) ? 3 : 4;
-    constexpr int G = 16 / M;                         // groups per 16-k segment
-    const int segs = k_blocks * steps_per_block * 2;  // 16-k segments per (padded) row
-    const int o = (int)(tid / segs);                  // padded row index
-    const int seg = (int)(tid % segs);
-    const int k0 = seg * 16;
-
-    uint16_t d[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) d[i] = 0;
-    uint32_t keep = 0;
-    const bool real = o < out && k0 < in;             // in is a multiple of 16 on this path
-    if (real) {
-        const int groups_per_row = in / M;
-        const uint16_t* v = vals + (size_t)o * ((size_t)groups_per_row * N);
-        const uint32_t* row = idx + (size_t)o * words_per_row;
-#pragma unroll
-        for (int gl = 0; gl < G; ++gl) {
-            const int g = k0 / M + gl;
-            for (int t = 0; t < N; ++t) {
-                const long long bit = ((long long)g * N + t) * B;
-                const int w0 = (int)(bit >> 5), sh = (int)(bit & 31);
-                uint32_t f = row[w0] >> sh;
-                if (sh + B > 32) f |= row[w0 + 1] << (32 - sh);
-                const int pos = gl * M + (int)(f & (uint32_t)(M - 1));
-                const uint16_t val = v[(size_t)g * N + t];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) d[i] = (i == pos) ? val : d[i];
-                keep |= 1u << pos;
-            }
-        }
-    }
-    sp24_emit(d, keep, real, o, seg, k0, in, out, a_img, meta16, k_blocks, steps_per_block, layout);
-}
-
-// The same from the DENSE shared weight: the 16 positions are projected onto level N:M on the fly
-// (N <= 2), so the supernet's forward needs no packed copy of the weight.
-template <int M>
-__device__ __forceinline__ void dense_to_sp24_segment(const uint16_t* __restrict__ W, int out, int in, int N,
-                                                      uint16_t* __restrict__ a_img, uint16_t* __restrict__ meta16,
-                                                      int k_blocks, int steps_per_block, int layout, long long tid)
-{
-    constexpr int G = 16 / M;
-    const int segs = k_blocks * steps_per_block * 2;
-    const int o = (int)(tid / segs);
-    const int seg = (int)(tid % segs);
-    const int k0 = seg * 16;
-
-    uint16_t d[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) d[i] = 0;
-    uint32_t keep = 0;
-    const bool real = o < out && k0 < in;
-    if (real) {
-#pragma unroll
-        for (int gl = 0; gl < G; ++gl) {
-            uint16_t w[M];
-            load_group<M>(W + (size_t)o * in + k0 + gl * M, w);
-            const uint32_t kg = keep_mask<M>(group_ranks<M>(w), N);
-#pragma unroll
-            for (int i = 0; i < M; ++i) d[gl * M + i] = ((kg >> i) & 1u) ? w[i] : (uint16_t)0;
-            keep |= kg << (gl * M);
-        }
-    }
-    sp24_emit(d, keep, real, o, seg, k0, in, out, a_img, meta16, k_blocks, steps_per_block, layout);
 }
 
 }  // namespace

@@ -21,7 +21,6 @@
 // row m + 8; nibble c of a half-word describes chunk c: position of the first stored value in bits
 // 0-1, of the second in bits 2-3 (first < second).
 
-#include "elsa_pack_device.cuh"
 #include <atomic>
 
 #include "elsa_tc_common.cuh"
@@ -50,34 +49,6 @@ constexpr int kStagingTotal = kEpiWarps * 2 * kStagingBytes;
 constexpr int kBarrierBytes = 256;
 
 static_assert(kStageBytes % 1024 == 0, "stages keep the 1024-byte alignment of the swizzled tiles");
-
-// ------------------------------------------------------------------ re-encoding
-
-// (the per-segment device code is in elsa_pack_device.cuh)
-template <int M>
-__global__ void __launch_bounds__(256)
-nm_to_sp24_kernel(const uint16_t* __restrict__ vals, const uint32_t* __restrict__ idx, int out, int in, int N,
-                  int words_per_row, uint16_t* __restrict__ a_img, uint16_t* __restrict__ meta16, int out_tiles,
-                  int k_blocks, int steps_per_block, int layout)
-{
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    pdl_wait_for_predecessors();
-    pdl_release_successors();
-    if (tid >= (long long)out_tiles * kFeatTile * k_blocks * steps_per_block * 2) return;
-    to_sp24_segment<M>(vals, idx, out, in, N, words_per_row, a_img, meta16, k_blocks, steps_per_block, layout, tid);
-}
-
-template <int M>
-__global__ void __launch_bounds__(256)
-dense_to_sp24_kernel(const uint16_t* __restrict__ W, int out, int in, int N, uint16_t* __restrict__ a_img,
-                     uint16_t* __restrict__ meta16, int out_tiles, int k_blocks, int steps_per_block, int layout)
-{
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    pdl_wait_for_predecessors();
-    pdl_release_successors();
-    if (tid >= (long long)out_tiles * kFeatTile * k_blocks * steps_per_block * 2) return;
-    dense_to_sp24_segment<M>(W, out, in, N, a_img, meta16, k_blocks, steps_per_block, layout, tid);
-}
 
 // ------------------------------------------------------------------ GEMM
 
@@ -270,51 +241,6 @@ linear_tc_sp24_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
 }
 
 }  // namespace
-
-elsa_status launch_nm_to_sp24(const uint16_t* vals, const uint32_t* idx, int out, int in, int N, int M, int block_k,
-                              int layout, uint16_t* a_img, uint8_t* meta, cudaStream_t stream)
-{
-    const int perm = layout;
-    const int tiles_f = (out + kFeatTile - 1) / kFeatTile;
-    const int k_blocks = (in + block_k - 1) / block_k;
-    const int steps = block_k / kSpUmmaK;
-    const long long threads = (long long)tiles_f * kFeatTile * k_blocks * steps * 2;
-    const unsigned grid = (unsigned)((threads + 255) / 256);
-    const int wpr = (int)index_words_per_row(in, N, M);
-    ProfileScope scope(ELSA_KERNEL_NM_TO_SP24, stream);
-    if (M == 4)
-        launch_pdl(nm_to_sp24_kernel<4>, dim3(grid), dim3(256), 0, stream, 1, vals, idx, out, in, N, wpr, a_img,
-                   (uint16_t*)meta, tiles_f, k_blocks, steps, perm);
-    else if (M == 8)
-        launch_pdl(nm_to_sp24_kernel<8>, dim3(grid), dim3(256), 0, stream, 1, vals, idx, out, in, N, wpr, a_img,
-                   (uint16_t*)meta, tiles_f, k_blocks, steps, perm);
-    else
-        launch_pdl(nm_to_sp24_kernel<16>, dim3(grid), dim3(256), 0, stream, 1, vals, idx, out, in, N, wpr, a_img,
-                   (uint16_t*)meta, tiles_f, k_blocks, steps, perm);
-    return launched("nm_to_sp24");
-}
-
-elsa_status launch_dense_to_sp24(const uint16_t* W, int out, int in, int N, int M, int block_k, int layout,
-                                 uint16_t* a_img, uint8_t* meta, cudaStream_t stream)
-{
-    const int perm = layout;
-    const int tiles_f = (out + kFeatTile - 1) / kFeatTile;
-    const int k_blocks = (in + block_k - 1) / block_k;
-    const int steps = block_k / kSpUmmaK;
-    const long long threads = (long long)tiles_f * kFeatTile * k_blocks * steps * 2;
-    const unsigned grid = (unsigned)((threads + 255) / 256);
-    ProfileScope scope(ELSA_KERNEL_NM_TO_SP24, stream);
-    if (M == 4)
-        launch_pdl(dense_to_sp24_kernel<4>, dim3(grid), dim3(256), 0, stream, 1, W, out, in, N, a_img, (uint16_t*)meta,
-                   tiles_f, k_blocks, steps, perm);
-    else if (M == 8)
-        launch_pdl(dense_to_sp24_kernel<8>, dim3(grid), dim3(256), 0, stream, 1, W, out, in, N, a_img, (uint16_t*)meta,
-                   tiles_f, k_blocks, steps, perm);
-    else
-        launch_pdl(dense_to_sp24_kernel<16>, dim3(grid), dim3(256), 0, stream, 1, W, out, in, N, a_img, (uint16_t*)meta,
-                   tiles_f, k_blocks, steps, perm);
-    return launched("dense_to_sp24");
-}
 
 bool linear_tc_sparse_suits(int in, int N)
 {

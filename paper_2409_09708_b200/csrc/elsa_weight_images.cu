@@ -1,0 +1,401 @@
+// Weight images: what the tensor-core kernels read in place of the packed weight (Sec. 2, Fig. 2 of the ELSA paper: the
+// indices give each kept value's position).  Four kinds, from the packed form or from a dense shared weight projected
+// onto its level on the way (Sec. 3.1):
+//   IMAGE_UNPACK, IMAGE_MASK        the dense masked weight [out][in]
+//   IMAGE_SP24, IMAGE_MASK_SP24     N <= 2: two values per aligned chunk of 4 and the metadata of the 2:4 sparse MMA
+// One kernel for any number of weights: a block of 256 threads works on one weight, at a level known at compile time
+// for the common ones, and every thread has the loads of all its units in flight before it expands the first.  The
+// images are a few MB, so what bounds a launch is latency, and what bounds a large table is the traffic through L2.
+// Against one thread per 8 or 16 positions with a loop over the kept values: image and GEMM of 3152 x 768 -> 3072 at 2:4
+// 20.6 -> 17.1 us back to back (the 2-of-4 image about 6 -> 2.5), of 197 x 768 -> 2304 on the dense image 8.2 -> 7.5; the
+// four images of a DeiT-B block in one launch 22 -> 12.6 us between events.
+
+#include "elsa_pack_device.cuh"
+
+namespace elsa {
+namespace {
+
+constexpr int kImageThreads = 256;
+constexpr int kUnitsPerThread = 4;        // dense images: units of 8 positions
+
+struct ImageItem {
+    const uint16_t* src;
+    const uint32_t* idx;
+    uint16_t* dst;
+    uint16_t* meta;
+    int first_block;
+    int out, in, N, M, words_per_row, kind, layout;
+    int k_blocks, steps;                  // 2-of-4 forms: metadata blocks along K, K steps of 32 per block (2 or 4)
+};
+
+template <int kMax>
+struct ImageTable {
+    ImageItem item[kMax];
+    int n;
+};
+
+// ---------------------------------------------------------------- dense images
+
+template <typename Raw, typename Load, typename Finish>
+__device__ __forceinline__ void dense_image_block(const ImageItem& it, int block, Load load, Finish finish)
+{
+    const uint32_t units_per_row = (uint32_t)it.in >> 3, units = (uint32_t)it.out * units_per_row;
+    const uint32_t base = (uint32_t)block * (kImageThreads * kUnitsPerThread) + threadIdx.x;
+    Raw raw[kUnitsPerThread];
+    uint32_t row[kUnitsPerThread], u[kUnitsPerThread];
+#pragma unroll
+    for (int i = 0; i < kUnitsPerThread; ++i) {
+        const uint32_t unit = base + (uint32_t)(i * kImageThreads);
+        row[i] = unit / units_per_row;
+        u[i] = unit - row[i] * units_per_row;
+        if (unit < units) raw[i] = load((int)row[i], (int)u[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < kUnitsPerThread; ++i) {
+        if (base + (uint32_t)(i * kImageThreads) >= units) break;
+        reinterpret_cast<uint4*>(it.dst)[(size_t)row[i] * units_per_row + u[i]] = finish(raw[i], (int)u[i]);
+    }
+}
+
+template <int M, int NC>
+__device__ __forceinline__ void unpack_block(const ImageItem& it, int block)
+{
+    const int N = it.N, vpr = it.in / M * N, wpr = it.words_per_row;
+    dense_image_block<PackedUnit>(
+        it, block, [&](int row, int u) { return load_packed_unit<M, NC>(it.src + (size_t)row * vpr, it.idx + (size_t)row * wpr, N, u); },
+        [&](const PackedUnit& p, int) { return expand_packed_unit<M, NC>(p, N); });
+}
+
+struct DenseGroup16 { uint4 a, b; };
+
+// ---------------------------------------------------------------- 2-of-4 images
+
+// The kept values (N <= 2 per group) of 16 consecutive positions of a row, in order, and their index fields.
+struct Segment {
+    uint32_t v[4];
+    uint32_t fields;
+};
+
+template <int M, int N>
+__device__ __forceinline__ Segment load_segment(const uint16_t* __restrict__ vals_row, const uint32_t* __restrict__ idx_row, int seg)
+{
+    constexpr int B = M == 4 ? 2 : M == 8 ? 3 : 4;
+    constexpr int count = 16 / M * N;
+    Segment s;
+    s.v[0] = s.v[1] = s.v[2] = s.v[3] = 0u;
+    const uint16_t* v = vals_row + (size_t)seg * count;
+    if constexpr (count == 8) {
+        const uint4 t = __ldg(reinterpret_cast<const uint4*>(v));
+        s.v[0] = t.x; s.v[1] = t.y; s.v[2] = t.z; s.v[3] = t.w;
+    } else if constexpr (count == 4) {
+        const uint2 t = __ldg(reinterpret_cast<const uint2*>(v));
+        s.v[0] = t.x; s.v[1] = t.y;
+    } else if constexpr (count == 2) {
+        s.v[0] = __ldg(reinterpret_cast<const uint32_t*>(v));
+    } else {
+        s.v[0] = __ldg(v);
+    }
+    const int bit0 = seg * count * B, w0 = bit0 >> 5, sh = bit0 & 31;
+    const uint32_t lo = __ldg(idx_row + w0);
+    const uint32_t hi = (sh + count * B > 32) ? __ldg(idx_row + w0 + 1) : 0u;
+    s.fields = __funnelshift_r(lo, hi, sh);
+    return s;
+}
+
+// Value at a position of a group of 8 given as four words.
+__device__ __forceinline__ uint32_t half_at(const uint32_t (&a)[4], uint32_t pos)
+{
+    const uint32_t lo = pos & 2u ? a[1] : a[0], hi = pos & 2u ? a[3] : a[2];
+    const uint32_t w = pos & 4u ? hi : lo;
+    return (pos & 1u ? w >> 16 : w) & 0xFFFFu;
+}
+
+// The same from 16 dense positions (words a[8]), projected onto level N:M (the N of largest magnitude, lowest position
+// first among equals).
+template <int M, int N>
+__device__ __forceinline__ Segment pick_segment(const uint4& x, const uint4& y)
+{
+    const uint32_t a[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+    Segment s;
+    s.v[0] = s.v[1] = s.v[2] = s.v[3] = 0u;
+    s.fields = 0;
+    if constexpr (M == 16) {
+        uint16_t h[16];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) { h[2 * q] = (uint16_t)(a[q] & 0xFFFFu); h[2 * q + 1] = (uint16_t)(a[q] >> 16); }
+        const uint32_t keep = keep_mask<16>(group_ranks<16>(h), N);
+        const uint32_t p0 = (uint32_t)__ffs((int)keep) - 1u, p1 = 31u - (uint32_t)__clz((int)keep);
+        const uint32_t lo[4] = {a[0], a[1], a[2], a[3]}, hi[4] = {a[4], a[5], a[6], a[7]};
+        s.v[0] = half_at(p0 & 8u ? hi : lo, p0 & 7u);
+        s.fields = p0;
+        if constexpr (N == 2) {
+            s.v[0] |= half_at(p1 & 8u ? hi : lo, p1 & 7u) << 16;
+            s.fields |= p1 << 4;
+        }
+    } else if constexpr (M == 8) {
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            uint32_t h[8], w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) { w[q] = a[4 * g + q]; h[2 * q] = w[q] & 0xFFFFu; h[2 * q + 1] = w[q] >> 16; }
+            const uint32_t keep = keep_mask_sorted<8>(h, N);
+            const uint32_t p0 = (uint32_t)__ffs((int)keep) - 1u, p1 = 31u - (uint32_t)__clz((int)keep);
+            if constexpr (N == 1) {
+                s.v[0] |= half_at(w, p0) << (16 * g);
+                s.fields |= p0 << (3 * g);
+            } else {
+                s.v[g] = half_at(w, p0) | (half_at(w, p1) << 16);
+                s.fields |= (p0 | (p1 << 3)) << (6 * g);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            uint32_t h[4] = {a[2 * g] & 0xFFFFu, a[2 * g] >> 16, a[2 * g + 1] & 0xFFFFu, a[2 * g + 1] >> 16};
+            const uint32_t keep = keep_mask_sorted<4>(h, N);
+            const uint32_t p0 = (uint32_t)__ffs((int)keep) - 1u, p1 = 31u - (uint32_t)__clz((int)keep);
+            const uint32_t w0 = p0 & 2u ? a[2 * g + 1] : a[2 * g], w1 = p1 & 2u ? a[2 * g + 1] : a[2 * g];
+            const uint32_t v0 = (p0 & 1u ? w0 >> 16 : w0) & 0xFFFFu, v1 = (p1 & 1u ? w1 >> 16 : w1) & 0xFFFFu;
+            if constexpr (N == 1) {
+                s.v[g >> 1] |= v0 << (16 * (g & 1));
+                s.fields |= p0 << (2 * g);
+            } else {
+                s.v[g] = v0 | (v1 << 16);
+                s.fields |= (p0 | (p1 << 2)) << (4 * g);
+            }
+        }
+    }
+    return s;
+}
+
+// The 2-of-4 form of a segment: per aligned chunk of 4 two values with ascending positions i0 < i1 and the metadata
+// nibble i0 | i1 << 2.  A chunk with one kept value takes position 3 as the second (0 as the first where the value itself
+// is at 3), one with none takes 0 and 1; the values borrowed there are zero.
+template <int M, int N>
+__device__ __forceinline__ uint4 sp24_words(const Segment& s, uint32_t& nibbles)
+{
+    uint32_t w[4], nib = 0;
+    // one value (low half of v) at position l of chunk c, if `here`
+    auto single = [&](bool here, uint32_t v, uint32_t l, int c) {
+        w[c] = here ? (l == 3u ? v << 16 : v) : 0u;
+        nib |= (here ? (l == 3u ? 0xCu : (l | 0xCu)) : 4u) << (4 * c);
+    };
+    if constexpr (M == 4 && N == 2) {
+        w[0] = s.v[0]; w[1] = s.v[1]; w[2] = s.v[2]; w[3] = s.v[3];
+        nib = s.fields & 0xFFFFu;
+    } else if constexpr (M == 4) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) single(true, (s.v[c >> 1] >> (16 * (c & 1))) & 0xFFFFu, (s.fields >> (2 * c)) & 3u, c);
+    } else {
+        constexpr int B = M == 8 ? 3 : 4, kChunks = M / 4;
+#pragma unroll
+        for (int g = 0; g < 16 / M; ++g) {
+            const uint32_t f = s.fields >> (g * N * B);
+            const uint32_t p0 = f & (uint32_t)(M - 1);
+            if constexpr (N == 1) {
+                const uint32_t v = M == 8 ? (s.v[0] >> (16 * g)) & 0xFFFFu : s.v[0];
+#pragma unroll
+                for (int c = 0; c < kChunks; ++c) single((p0 >> 2) == (uint32_t)c, v, p0 & 3u, g * kChunks + c);
+            } else {
+                const uint32_t p1 = (f >> B) & (uint32_t)(M - 1), v = s.v[g];
+#pragma unroll
+                for (int c = 0; c < kChunks; ++c) {
+                    const bool h0 = (p0 >> 2) == (uint32_t)c, h1 = (p1 >> 2) == (uint32_t)c;
+                    if (h0 && h1) {
+                        w[g * kChunks + c] = v;
+                        nib |= ((p0 & 3u) | ((p1 & 3u) << 2)) << (4 * (g * kChunks + c));
+                    } else {
+                        single(h0 || h1, h0 ? v & 0xFFFFu : v >> 16, (h0 ? p0 : p1) & 3u, g * kChunks + c);
+                    }
+                }
+            }
+        }
+    }
+    nibbles = nib;
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// A thread has 16 positions of image rows m and m + 8 of a block of 16 rows: the two share a metadata word.  Eight lanes
+// cover the eight row pairs, four groups of lanes four consecutive 16-position segments.
+// Image row o holds feature o_src: in the permuted forms (Sp24Layout) row r of a block of 32 holds feature
+// 8 * (r % 4) + r / 4.  Rows are padded to 128 for the metadata (zero), to 32 for the values.
+template <int M, int N, bool kMask>
+__device__ __forceinline__ void sp24_block(const ImageItem& it, int block)
+{
+    const int out = it.out, in = it.in, steps = it.steps, k_blocks = it.k_blocks;
+    const int segs = k_blocks * steps * 2;                         // per row, padding included
+    const int seg_groups = segs >> 2;
+    const int slot = block * (kImageThreads / 32) + (int)(threadIdx.x >> 5);      // (16 rows, 4 segments) of this warp
+    const int rows16 = slot / seg_groups;
+    if (rows16 >= (out + 127) / 128 * 8) return;
+    const int lane = threadIdx.x & 31;
+    const int seg = (slot - rows16 * seg_groups) * 4 + (lane >> 3);
+    const int o0 = rows16 * 16 + (lane & 7);
+    const int k0 = seg * 16;
+    int src_row[2];
+    Segment s[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int o = o0 + 8 * i, r = o & 31;
+        src_row[i] = it.layout != SP24_ROWS ? (o & ~31) | (8 * (r & 3) + (r >> 2)) : o;
+        if (src_row[i] < out && k0 < in) {
+            if constexpr (kMask) {
+                const uint4* g = reinterpret_cast<const uint4*>(it.src + (size_t)src_row[i] * in + k0);
+                s[i] = pick_segment<M, N>(__ldg(g), __ldg(g + 1));
+            } else {
+                s[i] = load_segment<M, N>(it.src + (size_t)src_row[i] * (in / M * N), it.idx + (size_t)src_row[i] * it.words_per_row, seg);
+            }
+        }
+    }
+    uint32_t word = 0;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        uint32_t nib = 0x4444u;                                    // four empty chunks
+        if (src_row[i] < out && k0 < in) v = sp24_words<M, N>(s[i], nib);
+        word |= nib << (16 * i);
+        if (k0 < in && src_row[i] < ((out + 31) & ~31)) {
+            const int o = o0 + 8 * i;
+            size_t at = (size_t)o * (size_t)in + (size_t)k0;       // byte offset of (row o, k0) in the row-major forms
+            if (it.layout == SP24_TILED)
+                at = (size_t)(o >> 5) * 32 * (size_t)in + (size_t)(k0 >> 8) * 8192 + (size_t)((((k0 & 255) >> 4) * 32 + (o & 31)) * 16);
+            *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(it.dst) + at) = v;
+        }
+    }
+    // metadata: block (128 features, k block) -> tensor-memory lane -> 4 words, one per K step of 32; a block of 64 k
+    // leaves the last two zero
+    const int kb = seg / (2 * steps), step = (seg >> 1) % steps, k1 = seg & 1;
+    const int tm_lane = (lane & 7) + 8 * k1 + 16 * (rows16 & 7);
+    uint32_t* meta = reinterpret_cast<uint32_t*>(it.meta) + (((size_t)(rows16 >> 3) * k_blocks + kb) * 128 + tm_lane) * 4 + step;
+    meta[0] = word;
+    if (steps == 2) meta[2] = 0u;
+}
+
+// Blocks of a weight.
+int image_blocks(const ImageJob& j)
+{
+    if (j.kind == IMAGE_UNPACK || j.kind == IMAGE_MASK) {
+        const long long units = (long long)j.out * (j.in / 8);
+        return (int)((units + kImageThreads * kUnitsPerThread - 1) / (kImageThreads * kUnitsPerThread));
+    }
+    const long long segs = (long long)((j.in + j.block_k - 1) / j.block_k) * (j.block_k / 32) * 2;
+    const long long warps = (long long)((j.out + 127) / 128 * 8) * (segs / 4);
+    return (int)((warps + kImageThreads / 32 - 1) / (kImageThreads / 32));
+}
+
+template <int kMax>
+__global__ void __launch_bounds__(kImageThreads) weight_image_kernel(const __grid_constant__ ImageTable<kMax> t)
+{
+    pdl_wait_for_predecessors();
+    pdl_release_successors();
+    int cur = 0;
+    if constexpr (kMax > 1) {
+        int hi = t.n - 1;
+        while (cur < hi) {
+            const int mid = (cur + hi + 1) >> 1;
+            if (t.item[mid].first_block <= (int)blockIdx.x) cur = mid; else hi = mid - 1;
+        }
+    }
+    const ImageItem& it = t.item[cur];
+    const int block = (int)blockIdx.x - it.first_block;
+    const int N = it.N, M = it.M;
+    if (it.kind == IMAGE_SP24) {
+        if (M == 4) { if (N == 2) sp24_block<4, 2, false>(it, block); else sp24_block<4, 1, false>(it, block); }
+        else if (M == 8) { if (N == 2) sp24_block<8, 2, false>(it, block); else sp24_block<8, 1, false>(it, block); }
+        else { if (N == 2) sp24_block<16, 2, false>(it, block); else sp24_block<16, 1, false>(it, block); }
+    } else if (it.kind == IMAGE_MASK_SP24) {
+        if (M == 4) { if (N == 2) sp24_block<4, 2, true>(it, block); else sp24_block<4, 1, true>(it, block); }
+        else if (M == 8) { if (N == 2) sp24_block<8, 2, true>(it, block); else sp24_block<8, 1, true>(it, block); }
+        else { if (N == 2) sp24_block<16, 2, true>(it, block); else sp24_block<16, 1, true>(it, block); }
+    } else if (it.kind == IMAGE_UNPACK) {
+        if (N == M) {
+            dense_image_block<uint4>(it, block, [&](int row, int u) { return __ldg(reinterpret_cast<const uint4*>(it.src + (size_t)row * it.in) + u); },
+                                     [](const uint4& v, int) { return v; });
+        } else if (M == 8) {
+            if (N == 1) unpack_block<8, 1>(it, block);
+            else if (N == 2) unpack_block<8, 2>(it, block);
+            else if (N == 4) unpack_block<8, 4>(it, block);
+            else unpack_block<8, 0>(it, block);
+        } else if (M == 4) {
+            if (N == 1) unpack_block<4, 1>(it, block);
+            else if (N == 2) unpack_block<4, 2>(it, block);
+            else unpack_block<4, 0>(it, block);
+        } else {
+            const int vpr = it.in / 16 * N, wpr = it.words_per_row;
+            dense_image_block<int>(it, block, [](int row, int) { return row; },
+                                   [&](int row, int u) { return expand_unit16(it.src + (size_t)row * vpr, it.idx + (size_t)row * wpr, N, u); });
+        }
+    } else {
+        if (M == 16) {
+            dense_image_block<DenseGroup16>(it, block,
+                                            [&](int row, int u) {
+                                                const uint4* g = reinterpret_cast<const uint4*>(it.src + (size_t)row * it.in) + (u & ~1);
+                                                return DenseGroup16{__ldg(g), __ldg(g + 1)};
+                                            },
+                                            [&](const DenseGroup16& g, int u) { return mask_unit<16>(g.a, g.b, u & 1, N); });
+        } else {
+            dense_image_block<uint4>(it, block, [&](int row, int u) { return __ldg(reinterpret_cast<const uint4*>(it.src + (size_t)row * it.in) + u); },
+                                     [&](const uint4& v, int) { return M == 8 ? mask_unit<8>(v, v, 0, N) : mask_unit<4>(v, v, 0, N); });
+        }
+    }
+}
+
+template <int kMax>
+elsa_status launch_table(const ImageJob* jobs, int n, cudaStream_t stream)
+{
+    ImageTable<kMax> t;      // on the stack: several threads may launch at once
+    int blocks = 0;
+    for (int i = 0; i < n; ++i) {
+        const ImageJob& j = jobs[i];
+        ImageItem& it = t.item[i];
+        it.src = j.src; it.idx = j.idx; it.dst = j.dst; it.meta = (uint16_t*)j.meta;
+        it.first_block = blocks;
+        it.out = j.out; it.in = j.in; it.N = j.N; it.M = j.M; it.kind = j.kind; it.layout = j.layout;
+        it.words_per_row = (int)index_words_per_row(j.in, j.N, j.M);
+        it.k_blocks = (j.in + j.block_k - 1) / j.block_k;
+        it.steps = j.block_k / 32;
+        blocks += image_blocks(j);
+    }
+    t.n = n;
+    const int k = n > 1 || jobs[0].kind == IMAGE_MASK ? ELSA_KERNEL_WEIGHT_IMAGES : jobs[0].kind == IMAGE_UNPACK ? ELSA_KERNEL_UNPACK : ELSA_KERNEL_NM_TO_SP24;
+    ProfileScope scope(k, stream);
+    cudaError_t e = launch_pdl(weight_image_kernel<kMax>, dim3((unsigned)blocks), dim3(kImageThreads), 0, stream, 1, t);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return fail(ELSA_ERR_CUDA, "launch of the weight images failed: %s", cudaGetErrorString(e));
+    }
+    return launched("weight images");
+}
+
+}  // namespace
+
+elsa_status launch_images(const ImageJob* jobs, int n, cudaStream_t stream)
+{
+    constexpr int kMost = 256;       // items per launch (kernel parameters are limited to 32 KB)
+    for (int at = 0; at < n; at += kMost) {
+        const int count = n - at < kMost ? n - at : kMost;
+        const elsa_status st = count == 1   ? launch_table<1>(jobs + at, count, stream)
+                               : count <= 8 ? launch_table<8>(jobs + at, count, stream)
+                                            : launch_table<kMost>(jobs + at, count, stream);
+        if (st != ELSA_OK) return st;
+    }
+    return ELSA_OK;
+}
+
+elsa_status launch_unpack(const uint16_t* vals, const uint32_t* idx, int out, int in, int N, int M, uint16_t* Wm, cudaStream_t stream)
+{
+    ImageJob j;
+    j.kind = IMAGE_UNPACK; j.src = vals; j.idx = idx; j.dst = Wm; j.out = out; j.in = in; j.N = N; j.M = M;
+    return launch_images(&j, 1, stream);
+}
+
+elsa_status launch_nm_to_sp24(const uint16_t* vals, const uint32_t* idx, int out, int in, int N, int M, int block_k, int layout,
+                              uint16_t* a_img, uint8_t* meta, cudaStream_t stream)
+{
+    ImageJob j;
+    j.kind = IMAGE_SP24; j.src = vals; j.idx = idx; j.dst = a_img; j.meta = meta; j.out = out; j.in = in; j.N = N; j.M = M;
+    j.layout = layout; j.block_k = block_k;
+    return launch_images(&j, 1, stream);
+}
+
+}  // namespace elsa

@@ -1,0 +1,59 @@
+"""The weight images behind the tensor-core kernels: with X = I the product is the masked weight itself, rounded once, so
+a position or metadata mistake of any image shows exactly.  Rows below, at and past the 16- and 128-row units of the
+2-of-4 form, fewer and more than a block's worth of units, every level with N <= 2 (and some above for the dense image),
+from the packed weight and from the dense shared weight.
+"""
+import numpy as np
+import pytest
+import torch
+
+from oracle import elsa_oracle as eo
+from paper_2409_09708_b200 import synth
+
+LEVELS = [(1, 4), (2, 4), (1, 8), (2, 8), (1, 16), (2, 16)]
+CASES = [(8, 128), (136, 256), (40, 384), (1000, 640)]
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_2409_09708_b200 import binding
+    return binding
+
+
+def masked(W, N, M):
+    vals, idx, mask = eo.nm_compress(synth.bits(W), N, M)
+    return W.double().numpy() * mask
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("variant", ["tc_sparse", "tc_sparse_pair", "tc_sparse_ws", "tc_sparse_st", "tc_pair", "tc_dense"])
+@pytest.mark.parametrize("level", LEVELS, ids=["%dof%d" % l for l in LEVELS])
+def test_identity_product_is_the_masked_weight(lib, level, variant):
+    N, M = level
+    for out, in_ in CASES:
+        W = synth.randn((out, in_), 3 * out + in_ + N, synth.W_STD, torch.float16)
+        X = torch.eye(in_, dtype=torch.float16, device="cuda")
+        Wd = W.cuda()
+        vals, idx = lib.elsa_nm_compress(Wd, N, M)
+        lib.elsa_set_linear_variant(getattr(lib, "VARIANT_" + variant.upper()))
+        try:
+            Y = lib.elsa_nm_linear(X, vals, idx, None, out, in_, N, M)
+            Y_masked = Y if variant == "tc_sparse" else lib.elsa_nm_linear_masked(X, Wd, None, N, M)
+            torch.cuda.synchronize()
+        finally:
+            lib.elsa_set_linear_variant(lib.VARIANT_AUTO)
+        ref = masked(W, N, M).T
+        assert np.array_equal(Y.double().cpu().numpy(), ref), (out, in_)
+        assert np.array_equal(Y_masked.double().cpu().numpy(), ref), (out, in_)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("level", [(1, 4), (2, 4), (3, 4), (4, 4), (1, 8), (2, 8), (3, 8), (4, 8), (7, 8), (5, 16), (16, 16)],
+                         ids=lambda l: "%dof%d" % l)
+def test_unpack_around_a_block_of_units(lib, level):
+    N, M = level
+    for out, in_ in [(8, 16), (64, 128), (65 * 8, 16), (24, 16 * 23)]:          # 16 units, exactly 1024, one more row, ragged
+        W = synth.randn((out, in_), out + in_ + N, synth.W_STD, torch.bfloat16)
+        vals, idx = lib.elsa_nm_compress(W.cuda(), N, M)
+        got = lib.elsa_nm_unpack(vals, idx, out, in_, N, M)
+        assert np.array_equal(got.double().cpu().numpy(), masked(W, N, M)), (out, in_)
