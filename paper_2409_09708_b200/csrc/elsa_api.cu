@@ -136,34 +136,73 @@ elsa_status check_linear(const void* X, int rows, const void* vals, const uint32
     return ELSA_OK;
 }
 
-// Side stream of elsa_vit_linears (weight images beside the dense layers), created once per device.
+// A side stream with its fork and join events, for the weight images that are built beside a call's other kernels.  A
+// call takes one from the device's pool and hands it back when all it enqueued is joined into the caller's stream, so
+// calls of several threads never share events; the pool holds as many as calls have ever overlapped.
 struct SidePipe {
+    int device;
     cudaStream_t stream;
     cudaEvent_t fork, join;
-    bool ready;
 };
-SidePipe g_side[64];
+std::vector<SidePipe> g_side[64];
 std::mutex g_side_mutex;
 
-elsa_status side_pipe(int device, SidePipe** pipe)
-{
-    std::lock_guard<std::mutex> lock(g_side_mutex);
-    SidePipe& p = g_side[device & 63];
-    if (!p.ready) {
-        const bool ok = cudaStreamCreateWithFlags(&p.stream, cudaStreamNonBlocking) == cudaSuccess &&
-                        cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming) == cudaSuccess &&
-                        cudaEventCreateWithFlags(&p.join, cudaEventDisableTiming) == cudaSuccess;
-        if (!ok) {
-            cudaError_t e = cudaGetLastError();
-            return fail(ELSA_ERR_CUDA, "creating the image stream: %s", cudaGetErrorString(e));
-        }
-        p.ready = true;
+class SideStream {
+public:
+    ~SideStream()
+    {
+        if (!have_) return;
+        std::lock_guard<std::mutex> lock(g_side_mutex);
+        g_side[pipe_.device & 63].push_back(pipe_);
     }
-    *pipe = &p;
-    return ELSA_OK;
-}
+    // Takes a pipe (once); the side stream then starts where `from` stands now.
+    elsa_status fork(int device, cudaStream_t from)
+    {
+        if (!have_) {
+            std::lock_guard<std::mutex> lock(g_side_mutex);
+            std::vector<SidePipe>& pool = g_side[device & 63];
+            if (!pool.empty()) {
+                pipe_ = pool.back();
+                pool.pop_back();
+            } else {
+                pipe_.device = device;
+                const bool ok = cudaStreamCreateWithFlags(&pipe_.stream, cudaStreamNonBlocking) == cudaSuccess &&
+                                cudaEventCreateWithFlags(&pipe_.fork, cudaEventDisableTiming) == cudaSuccess &&
+                                cudaEventCreateWithFlags(&pipe_.join, cudaEventDisableTiming) == cudaSuccess;
+                if (!ok) {
+                    cudaError_t e = cudaGetLastError();
+                    return fail(ELSA_ERR_CUDA, "creating the image stream: %s", cudaGetErrorString(e));
+                }
+            }
+            have_ = true;
+        }
+        cudaError_t e = cudaEventRecord(pipe_.fork, from);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(pipe_.stream, pipe_.fork, 0);
+        if (e != cudaSuccess) { cudaGetLastError(); return fail(ELSA_ERR_CUDA, "forking the image stream: %s", cudaGetErrorString(e)); }
+        forked_ = true;
+        return ELSA_OK;
+    }
+    // `into` waits for what the side stream holds (nothing to do without a fork).  Also after a failed launch: a fork
+    // must not dangle.
+    elsa_status join(cudaStream_t into)
+    {
+        if (!forked_) return ELSA_OK;
+        forked_ = false;
+        cudaError_t e = cudaEventRecord(pipe_.join, pipe_.stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(into, pipe_.join, 0);
+        if (e != cudaSuccess) { cudaGetLastError(); return fail(ELSA_ERR_CUDA, "joining the image stream: %s", cudaGetErrorString(e)); }
+        return ELSA_OK;
+    }
+    bool forked() const { return forked_; }
+    cudaStream_t stream() const { return pipe_.stream; }
 
-enum LinearKind { KIND_SIMT, KIND_SMALL, KIND_DENSE_ONE, KIND_DENSE_PAIR, KIND_SPARSE_ONE, KIND_SPARSE_PAIR, KIND_SPARSE_WS, KIND_SPARSE_ST };
+private:
+    bool have_ = false, forked_ = false;
+    SidePipe pipe_;
+};
+
+// KIND_SMALL expands a packed weight itself; KIND_SMALL_IMAGE is the same kernel on the dense image of the weight.
+enum LinearKind { KIND_SIMT, KIND_SMALL, KIND_SMALL_IMAGE, KIND_DENSE_ONE, KIND_DENSE_PAIR, KIND_SPARSE_ONE, KIND_SPARSE_PAIR, KIND_SPARSE_WS, KIND_SPARSE_ST };
 
 // Form of the 2-of-4 weight image each sparse kernel reads.
 int sp24_layout_of(LinearKind kind)
@@ -184,8 +223,13 @@ ImageJob image_job(LinearKind kind, const void* vals, const uint32_t* idx, int o
     return j;
 }
 
+// What a layer is part of: a call of its own, a table whose layers share persistent launches, or a chained block, where
+// the images are built off the critical path and an epilogue that takes GELU or the residual saves a pass.
+enum LinearUse { USE_SINGLE, USE_TABLE, USE_CHAIN };
+
 // Which kernel a layer runs on.  AUTO is the product rule; a forced variant is honoured where it applies.
-elsa_status pick_kind(int rows, int out, int in, int N, int M, int sm_count, LinearKind* kind)
+// gelu: the layer's epilogue applies GELU (USE_CHAIN).
+elsa_status pick_kind(LinearUse use, int rows, int out, int in, int N, int M, int sm_count, LinearKind* kind, bool gelu = false)
 {
     const int variant = g_variant.load(std::memory_order_relaxed);
     const bool sparse_ok = N != M && linear_tc_sparse_suits(in, N);
@@ -213,22 +257,54 @@ elsa_status pick_kind(int rows, int out, int in, int N, int M, int sm_count, Lin
         return ELSA_OK;
     default: break;
     }
-    // Levels with N <= 2 fit the 2:4 sparse MMA.  Measured on B200 it beats the dense-rate kernels from K = 256
-    // up once there are enough tiles to fill the CTA pairs; K = 128 layers are pure streaming problems and
-    // stay on the dense-rate path.
-    if (sparse_ok && in >= 256 && (long long)((rows + 223) / 224) * ((out + 255) / 256) >= sm_count / 4) {
-        // With the weight block resident in tensor memory the activations are the only shared-memory
-        // traffic: every layer whose reduction fits (in <= 896) and that has at least two blocks of 256
-        // features goes there.
-        const bool ws = linear_tc_sparse_ws_suits(in, out, N, sm_count) && in <= 896 && out >= 512 &&
-                        rows >= 256 * (sm_count / 2) / ((out + 255) / 256);
-        // Longer reductions do not fit tensor memory whole: the weight streams through it chunk by chunk, which
-        // still keeps it out of shared memory (measured against staging it there for every row tile).
-        const bool st = !ws && in > 768 && linear_tc_sparse_st_suits(in, N);
-        *kind = ws ? KIND_SPARSE_WS : st ? KIND_SPARSE_ST : KIND_SPARSE_PAIR;
+    // Times below: us back to back, weight image included, at 2:8 unless noted.
+    const int k_blocks = (in + 63) / 64;
+    const long long tiles_small = (long long)((rows + 127) / 128) * ((out + 63) / 64);
+    const long long tiles_f = (out + 255) / 256, pairs = sm_count / 2;
+    const bool pair_full = linear_tc_pair_suits(rows, out, sm_count);
+    const bool ws_ok = sparse_ok && linear_tc_sparse_ws_suits(in, out, N, sm_count) && out >= 512;
+    const bool st_ok = sparse_ok && linear_tc_sparse_st_suits(in, N);
+    // With at least 900 rows per SM pair the weight-stationary kernel's set-up (its block goes to tensor memory first) is
+    // paid back by activations being its only shared-memory traffic: 768 -> 3072, 6304 rows 23.2 against 23.1 on the
+    // sparse pair kernel, 12608 rows 35.0 against 38.8, 3152 rows 17.3 against 16.4; 1024 -> 4096, 12608 rows 53.8
+    // against 58.8 on the streaming kernel; 256 -> 1024 at the dense rate, 25216 rows 20.5 against 18.7.
+    const bool ws_large = ws_ok && (long long)rows * tiles_f >= 900 * pairs;
+    if (use == USE_TABLE) {
+        // Layers of a table share launches, so a layer need not fill the chip by itself and what counts is throughput:
+        // N <= 2 goes to the sparse MMA from K = 256 and a quarter wave of tiles up (K = 128 layers are pure streaming
+        // problems), weight-stationary where the reduction fits beside wide accumulators, streaming where it does not.
+        if (sparse_ok && in >= 256 && (long long)((rows + 223) / 224) * tiles_f >= sm_count / 4) {
+            const bool ws = ws_large || (ws_ok && in <= 896 && rows >= 256 * pairs / tiles_f);
+            *kind = ws ? KIND_SPARSE_WS : in > 768 && st_ok ? KIND_SPARSE_ST : KIND_SPARSE_PAIR;
+        } else {
+            *kind = pair_full ? KIND_DENSE_PAIR : KIND_SMALL_IMAGE;
+        }
+        return ELSA_OK;
     }
-    else
-        *kind = linear_tc_pair_suits(rows, out, sm_count) ? KIND_DENSE_PAIR : KIND_SMALL;
+    if (tiles_small <= sm_count) {
+        // One wave of 128 x 64 tiles: latency.
+        if (use == USE_CHAIN) { *kind = KIND_SMALL_IMAGE; return ELSA_OK; }
+        int ranges = 1;
+        {
+            SmallJob j;
+            j.rows = rows; j.out = out; j.in = in;
+            ranges = linear_small_splits(&j, 1, sm_count);
+        }
+        // Expanding in the kernel saves a launch on the host and costs ~0.3 us of device time per K block and CTA: taken
+        // up to 6 blocks (197 rows, 768 -> 768: 7.8 against 7.6; 3072 -> 768 would be 13.7 against 10).
+        if (N != M && ranges >= 2 && k_blocks <= 6 * ranges) *kind = KIND_SMALL;
+        // A cut reduction pays from 16 K blocks up (4:4, 197 rows: 3072 -> 768 7.4 against 12.2, 768 -> 768 5.3 both).
+        else *kind = ranges >= 2 && k_blocks >= 16 ? KIND_SMALL_IMAGE : KIND_DENSE_ONE;
+        return ELSA_OK;
+    }
+    // More than a wave of small tiles.  Below K = 512 the sparse kernels do not beat the pair kernel until the
+    // weight-stationary one does (384 -> 384, 6304 rows: 8.2 against 8.8); from there up the sparse pair kernel leads,
+    // and from about 5M outputs the streaming one (3072 -> 768: 6304 rows 24.5 against 25.0, 12608 rows 38.7 against 36.6).
+    // Only the streaming and weight-stationary ones take GELU in their epilogue.
+    if (ws_large) *kind = KIND_SPARSE_WS;
+    else if (sparse_ok && in >= 512 && st_ok && (gelu || (long long)rows * out >= 5000000LL)) *kind = KIND_SPARSE_ST;
+    else if (sparse_ok && in >= 512 && !gelu) *kind = KIND_SPARSE_PAIR;
+    else *kind = KIND_DENSE_PAIR;
     return ELSA_OK;
 }
 
@@ -241,16 +317,20 @@ SmallJob small_job(const void* X, int rows, const void* w, const uint32_t* idx, 
     return j;
 }
 
+// The few-rows kernel on a weight that lies dense in memory (the dense level, or a weight image).
+SmallJob small_dense_job(const void* X, int rows, const void* Wd, const void* bias, int out, int in, void* Y)
+{
+    return small_job(X, rows, Wd, nullptr, bias, out, in, 4, 4, Y);
+}
+
 // After validation: enqueue one layer.  small_splits: how the few-rows kernel cuts the reduction (0: its own choice).
-elsa_status run_linear(const void* X, int rows, const void* vals, const uint32_t* idx, const void* bias, int out,
+elsa_status run_linear(LinearKind kind, const void* X, int rows, const void* vals, const uint32_t* idx, const void* bias, int out,
                        int in, int N, int M, elsa_dtype dtype, void* Y, void* workspace, uint32_t* dev_status,
                        cudaStream_t stream, int small_splits = 0)
 {
     DeviceInfo dev;
     elsa_status st = device_info(&dev);
     if (st != ELSA_OK) return st;
-    LinearKind kind;
-    if ((st = pick_kind(rows, out, in, N, M, dev.sm_count, &kind)) != ELSA_OK) return st;
     if (kind == KIND_SIMT)
         return launch_linear_simt((const uint16_t*)X, rows, (const uint16_t*)vals, idx, (const uint16_t*)bias, out,
                                   in, N, M, dtype, (uint16_t*)Y, stream);
@@ -282,6 +362,11 @@ elsa_status run_linear(const void* X, int rows, const void* vals, const uint32_t
     if (kind == KIND_DENSE_PAIR)
         return launch_linear_tc_pair((const uint16_t*)X, rows, Wd, (const uint16_t*)bias, out, in, dtype,
                                      (uint16_t*)Y, dev_status, stream);
+    if (kind == KIND_SMALL_IMAGE) {
+        const SmallJob job = small_dense_job(X, rows, Wd, bias, out, in, Y);
+        if (small_splits == 0) small_splits = linear_small_splits(&job, 1, dev.sm_count);
+        return launch_linear_small_group(&job, 1, small_splits, false, dtype, dev_status, stream);
+    }
     return launch_linear_tc_dense((const uint16_t*)X, rows, Wd, (const uint16_t*)bias, out, in, dtype,
                                   (uint16_t*)Y, dev_status, stream);
 }
@@ -358,7 +443,9 @@ elsa_status elsa_nm_linear(const void* X, int rows, const void* vals, const uint
     if (st != ELSA_OK) return st;
     DeviceInfo dev;
     if ((st = device_info(&dev)) != ELSA_OK) return st;
-    return run_linear(X, rows, vals, N == M ? nullptr : idx, bias, out, in, N, M, dtype, Y, workspace, dev_status,
+    LinearKind kind;
+    if ((st = pick_kind(USE_SINGLE, rows, out, in, N, M, dev.sm_count, &kind)) != ELSA_OK) return st;
+    return run_linear(kind, X, rows, vals, N == M ? nullptr : idx, bias, out, in, N, M, dtype, Y, workspace, dev_status,
                       (cudaStream_t)stream);
 }
 
@@ -404,7 +491,7 @@ elsa_status elsa_nm_linear_masked(const void* X, int rows, const void* W_sup, co
     if ((st = device_info(&dev)) != ELSA_OK) return st;
     cudaStream_t stream = (cudaStream_t)stream_;
     LinearKind kind;
-    if ((st = pick_kind(rows, out, in, N, M, dev.sm_count, &kind)) != ELSA_OK) return st;
+    if ((st = pick_kind(USE_SINGLE, rows, out, in, N, M, dev.sm_count, &kind)) != ELSA_OK) return st;
     if (kind == KIND_SIMT || kind == KIND_SPARSE_ONE)
         return fail(ELSA_ERR_NM, "the forced variant has no mask-on-load form");
     if (kind == KIND_SMALL) {
@@ -434,6 +521,10 @@ elsa_status elsa_nm_linear_masked(const void* X, int rows, const void* W_sup, co
     if (kind == KIND_DENSE_PAIR)
         return launch_linear_tc_pair((const uint16_t*)X, rows, Wd, (const uint16_t*)bias, out, in, dtype, (uint16_t*)Y,
                                      dev_status, stream);
+    if (kind == KIND_SMALL_IMAGE) {
+        const SmallJob job = small_dense_job(X, rows, Wd, bias, out, in, Y);
+        return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, dev.sm_count), false, dtype, dev_status, stream);
+    }
     return launch_linear_tc_dense((const uint16_t*)X, rows, Wd, (const uint16_t*)bias, out, in, dtype, (uint16_t*)Y,
                                   dev_status, stream);
 }
@@ -524,9 +615,9 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
     std::vector<SmallJob> small;
     for (int l = 0; l < n_layers; ++l) {
         const elsa_layer& c = cfg[l];
-        if ((st = pick_kind(c.rows, c.out, c.in, c.N, c.M, dev.sm_count, &kind[l])) != ELSA_OK) return layer_fail(st, l);
-        if (kind[l] == KIND_SMALL)
-            small.push_back(small_job(c.X, c.rows, c.vals, c.N == c.M ? nullptr : c.idx, c.bias, c.out, c.in, c.N, c.M, c.Y));
+        if ((st = pick_kind(USE_TABLE, c.rows, c.out, c.in, c.N, c.M, dev.sm_count, &kind[l])) != ELSA_OK) return layer_fail(st, l);
+        if (kind[l] == KIND_SMALL_IMAGE || kind[l] == KIND_SMALL)
+            small.push_back(small_dense_job(c.X, c.rows, c.vals, c.bias, c.out, c.in, c.Y));
     }
     // cut as they are in shared launches, so that results do not depend on the scratch given
     const int small_splits = small.empty() ? 0 : linear_small_splits(small.data(), (int)small.size(), dev.sm_count);
@@ -534,7 +625,7 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
         for (int l = 0; l < n_layers; ++l) {
             const elsa_layer& c = cfg[l];
             set_profile_layer(l);
-            st = run_linear(c.X, c.rows, c.vals, c.N == c.M ? nullptr : c.idx, c.bias, c.out, c.in, c.N, c.M, dtype,
+            st = run_linear(kind[l], c.X, c.rows, c.vals, c.N == c.M ? nullptr : c.idx, c.bias, c.out, c.in, c.N, c.M, dtype,
                             c.Y, workspace, dev_status, stream, small_splits);
             if (st != ELSA_OK) return layer_fail(st, l);
         }
@@ -545,18 +636,18 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
     // The weight images are built on a side stream while the dense layers, which need none, already run on
     // the caller's: the image kernel is a small streaming kernel whose blocks fit beside the persistent GEMM's
     // one CTA per SM.  Everything else waits for the images.
-    SidePipe* side = nullptr;
-    if ((st = side_pipe(dev.device, &side)) != ELSA_OK) return st;
+    SideStream side;
     std::vector<uint8_t*> region(n_layers);
-    size_t off = 0;
+    size_t off = 0, n_small = 0;
     for (int l = 0; l < n_layers; ++l) {
         const elsa_layer& c = cfg[l];
         region[l] = (uint8_t*)workspace + off;
+        if (kind[l] == KIND_SMALL_IMAGE && c.N != c.M) small[n_small].w = (const uint16_t*)region[l];
+        n_small += kind[l] == KIND_SMALL_IMAGE;
         off += round_up(elsa_workspace_bytes(c.rows, c.in, c.out, c.N, c.M, dtype), 256);
     }
     // dense-rate layers that multiply the stored values as they are (N = M), on CTA pairs, in groups: launched
     // first, the weight images are built beside them
-    bool forked = false;
     {
         std::vector<PairJob> jobs;
         for (int l = 0; l <= n_layers; ++l) {
@@ -569,34 +660,31 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
                 jobs.push_back(j);
             }
             if (!jobs.empty() && (l == n_layers || (int)jobs.size() == linear_tc_pair_group_max())) {
-                if (!forked) {
-                    // the side stream starts where the caller's stream stands now (after the compress kernels)
-                    cudaError_t e = cudaEventRecord(side->fork, stream);
-                    if (e == cudaSuccess) e = cudaStreamWaitEvent(side->stream, side->fork, 0);
-                    if (e != cudaSuccess) { cudaGetLastError(); return fail(ELSA_ERR_CUDA, "forking the image stream: %s", cudaGetErrorString(e)); }
-                    forked = true;
-                }
-                if ((st = launch_linear_tc_pair_group(jobs.data(), (int)jobs.size(), dtype, dev_status, stream)) != ELSA_OK)
+                // the side stream starts where the caller's stream stands now (after the compress kernels)
+                if (!side.forked() && (st = side.fork(dev.device, stream)) != ELSA_OK) return st;
+                if ((st = launch_linear_tc_pair_group(jobs.data(), (int)jobs.size(), dtype, dev_status, stream)) != ELSA_OK) {
+                    side.join(stream);
                     return st;
+                }
                 jobs.clear();
             }
         }
     }
-    cudaStream_t image_stream = forked ? side->stream : stream;
+    cudaStream_t image_stream = side.forked() ? side.stream() : stream;
     // weight images of all layers, one launch per 256 layers
     {
         std::vector<ImageJob> jobs;
         for (int l = 0; l < n_layers; ++l) {
             const elsa_layer& c = cfg[l];
-            if (c.N != c.M && kind[l] != KIND_SMALL)
+            if (c.N != c.M)
                 jobs.push_back(image_job(kind[l], c.vals, c.idx, c.out, c.in, c.N, c.M, region[l]));
         }
-        if (!jobs.empty() && (st = launch_images(jobs.data(), (int)jobs.size(), image_stream)) != ELSA_OK) return st;
+        if (!jobs.empty()) st = launch_images(jobs.data(), (int)jobs.size(), image_stream);
     }
-    if (forked) {
-        cudaError_t e = cudaEventRecord(side->join, side->stream);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, side->join, 0);
-        if (e != cudaSuccess) { cudaGetLastError(); return fail(ELSA_ERR_CUDA, "joining the image stream: %s", cudaGetErrorString(e)); }
+    {
+        const elsa_status joined = side.join(stream);
+        if (st != ELSA_OK) return st;
+        if (joined != ELSA_OK) return joined;
     }
     // sparse-rate layers, in groups
     {
@@ -671,7 +759,7 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
             }
         }
     }
-    // layers with few rows, straight from their packed weights, in groups
+    // layers with few rows, in groups
     for (size_t at = 0; at < small.size(); at += (size_t)linear_small_group_max()) {
         const int n = (int)(small.size() - at) < linear_small_group_max() ? (int)(small.size() - at) : linear_small_group_max();
         if ((st = launch_linear_small_group(small.data() + at, n, small_splits, false, dtype, dev_status, stream)) != ELSA_OK) return st;
@@ -814,7 +902,9 @@ elsa_status elsa_vit_linears_host(const elsa_host_layer* cfg, int n_layers, elsa
         if (e == cudaSuccess && l >= 2) e = cudaStreamWaitEvent(stream, pipe->out_done[slot], 0);
         if (e != cudaSuccess) return cuda_fail(e, l, "ordering the kernels");
         if ((st = launch_compress((const uint16_t*)dW, c.out, c.in, c.N, c.M, (uint16_t*)dV, dI, stream)) != ELSA_OK) return st;
-        if ((st = run_linear(dX, c.rows, dV, dI, dB, c.out, c.in, c.N, c.M, dtype, dY, base + plan.ws, dev_status,
+        LinearKind kind;
+        if ((st = pick_kind(USE_SINGLE, c.rows, c.out, c.in, c.N, c.M, dev.sm_count, &kind)) != ELSA_OK) return st;
+        if ((st = run_linear(kind, dX, c.rows, dV, dI, dB, c.out, c.in, c.N, c.M, dtype, dY, base + plan.ws, dev_status,
                              stream)) != ELSA_OK)
             return st;
         e = cudaEventRecord(pipe->compute_done[slot], stream);
@@ -878,10 +968,11 @@ bool block_plan(int rows, int dim, int mlp_dim, const elsa_block_weights* w, els
     return true;
 }
 
-// Validation shared by the three entry points; fills the four linears' descriptions.
+// Validation shared by the entry points; fills the four linears' descriptions.  images: where their weight images go
+// when not in region WORKSPACE of the scratch.
 elsa_status block_check(const void* x, int rows, int dim, int mlp_dim, const elsa_block_weights* w, elsa_dtype dtype,
                         const void* y, bool need_y, void* scratch, size_t scratch_bytes, BlockPlan* plan,
-                        BlockLinear (&lin)[4], const DeviceInfo& dev)
+                        BlockLinear (&lin)[4], const DeviceInfo& dev, uint8_t* images = nullptr)
 {
     if (!x || !w || !scratch || (need_y && !y)) return fail(ELSA_ERR_NULL, "x, w, y and scratch must not be NULL");
     if (rows <= 0 || dim <= 0 || mlp_dim <= 0) return fail(ELSA_ERR_SHAPE, "non-positive size (rows=%d, dim=%d, mlp_dim=%d)", rows, dim, mlp_dim);
@@ -916,10 +1007,10 @@ elsa_status block_check(const void* x, int rows, int dim, int mlp_dim, const els
         lin[l].w = src[l];
         lin[l].in = ins[l];
         lin[l].out = outs[l];
-        lin[l].ws = (uint8_t*)scratch + plan->ws_off[l];
+        lin[l].ws = images ? images + (plan->ws_off[l] - plan->off[ELSA_BLOCK_WORKSPACE]) : (uint8_t*)scratch + plan->ws_off[l];
         lin[l].image_ready = false;
         lin[l].first = false;
-        elsa_status st = pick_kind(rows, outs[l], ins[l], src[l]->N, src[l]->M, dev.sm_count, &lin[l].kind);
+        elsa_status st = pick_kind(USE_CHAIN, rows, outs[l], ins[l], src[l]->N, src[l]->M, dev.sm_count, &lin[l].kind, l == 2);
         if (st != ELSA_OK) return st;
     }
     return ELSA_OK;
@@ -928,7 +1019,7 @@ elsa_status block_check(const void* x, int rows, int dim, int mlp_dim, const els
 // Whether a linear's kernel takes a ready-made weight image (the others build theirs when they run, or need none).
 bool takes_image(const BlockLinear& L)
 {
-    return L.w->N != L.w->M && (L.kind == KIND_DENSE_PAIR || L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST);
+    return L.w->N != L.w->M && (L.kind == KIND_DENSE_PAIR || L.kind == KIND_SMALL_IMAGE || L.kind == KIND_SPARSE_PAIR || L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST);
 }
 
 // The images of the linears that take one, in one launch.
@@ -964,25 +1055,30 @@ elsa_status block_linear(BlockLinear& L, const uint16_t* X, int rows, elsa_dtype
         job.act = act; job.residual = residual;
         return launch_linear_tc_pair_group(&job, 1, dtype, dev_status, stream);
     }
-    if (L.kind == KIND_SMALL) {
-        SmallJob job = small_job(X, rows, w.vals, w.N == w.M ? nullptr : w.idx, w.bias, L.out, L.in, w.N, w.M, Y);
+    if (L.kind == KIND_SMALL || L.kind == KIND_SMALL_IMAGE) {
+        const bool ready = L.image_ready;       // built and joined before an earlier kernel of this call
+        if ((st = block_images(&L, 1, stream)) != ELSA_OK) return st;
+        SmallJob job = L.kind == KIND_SMALL ? small_job(X, rows, w.vals, w.N == w.M ? nullptr : w.idx, w.bias, L.out, L.in, w.N, w.M, Y)
+                                            : small_dense_job(X, rows, w.N == w.M ? w.vals : L.ws, w.bias, L.out, L.in, Y);
         job.act = act; job.residual = residual;
         DeviceInfo dev;
         if ((st = device_info(&dev)) != ELSA_OK) return st;
         // after another kernel of the same call the weights are older than that kernel's start
-        return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, dev.sm_count), !L.first, dtype, dev_status, stream);
+        const bool early = !L.first && (L.kind == KIND_SMALL || w.N == w.M || ready);
+        return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, dev.sm_count), early, dtype, dev_status, stream);
     }
     *residual_left = residual != nullptr;
     uint16_t* dst = residual ? tmp : Y;
-    if (L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST) {
+    if (L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST || (L.kind == KIND_SPARSE_PAIR && act == 0)) {
         if ((st = block_images(&L, 1, stream)) != ELSA_OK) return st;
         SparseJob job;
         job.X = X; job.bias = (const uint16_t*)w.bias; job.Y = dst; job.workspace = L.ws;
         job.rows = rows; job.in = L.in; job.out = L.out; job.act = act;
-        return L.kind == KIND_SPARSE_WS ? launch_linear_tc_sparse_ws_group(&job, 1, dtype, dev_status, stream)
-                                        : launch_linear_tc_sparse_st_group(&job, 1, dtype, dev_status, stream);
+        return L.kind == KIND_SPARSE_WS   ? launch_linear_tc_sparse_ws_group(&job, 1, dtype, dev_status, stream)
+               : L.kind == KIND_SPARSE_ST ? launch_linear_tc_sparse_st_group(&job, 1, dtype, dev_status, stream)
+                                          : launch_linear_tc_sparse_pair_group(&job, 1, dtype, dev_status, stream);
     }
-    st = run_linear(X, rows, w.vals, w.N == w.M ? nullptr : w.idx, w.bias, L.out, L.in, w.N, w.M, dtype, dst, L.ws,
+    st = run_linear(L.kind, X, rows, w.vals, w.N == w.M ? nullptr : w.idx, w.bias, L.out, L.in, w.N, w.M, dtype, dst, L.ws,
                     dev_status, stream);
     if (st != ELSA_OK) return st;
     return launch_act_inplace(dst, (long long)rows * L.out, act, dtype, stream);
@@ -995,11 +1091,19 @@ struct BlockCarry {
     const uint16_t* r = nullptr;   // x2
 };
 
+// The side stream's part in a block: joined between the first LayerNorm and the first linear, where the images of the
+// block itself must be ready; those of the next block (or NULL) are started there, beside this block's kernels.
+struct BlockSide {
+    SideStream* side;
+    BlockLinear* next;
+    int device;
+};
+
 // carry (or NULL) + x_sum: the block's input is carry->t + carry->r, written to x_sum; otherwise it is x.
 elsa_status block_qkv(const uint16_t* x, int rows, int dim, const elsa_block_weights* w, elsa_dtype dtype,
                       uint8_t* scratch, const BlockPlan& plan, BlockLinear (&lin)[4], uint32_t* dev_status,
                       cudaStream_t stream, const BlockCarry* carry = nullptr, uint16_t* x_sum = nullptr,
-                      const elsa_swin_attn* swin = nullptr)
+                      const elsa_swin_attn* swin = nullptr, const BlockSide* beside = nullptr)
 {
     uint16_t* x1 = (uint16_t*)(scratch + plan.off[ELSA_BLOCK_X1]);
     uint16_t* qkv = (uint16_t*)(scratch + plan.off[ELSA_BLOCK_QKV]);
@@ -1009,6 +1113,17 @@ elsa_status block_qkv(const uint16_t* x, int rows, int dim, const elsa_block_wei
     elsa_status st = launch_layer_norm(add ? carry->t : x, add ? carry->r : nullptr, add ? x_sum : nullptr,
                                        (const uint16_t*)w->ln1_gain, (const uint16_t*)w->ln1_bias,
                                        x1, rows, dim, w->eps, dtype, stream, swin ? &out_map : nullptr);
+    if (beside != nullptr) {
+        const elsa_status joined = beside->side->join(stream);
+        if (st == ELSA_OK) st = joined;
+        if (st == ELSA_OK && beside->next != nullptr) {
+            bool any = false;
+            for (int l = 0; l < 4; ++l) any = any || takes_image(beside->next[l]);
+            if (any && (st = beside->side->fork(beside->device, stream)) == ELSA_OK)
+                st = block_images(beside->next, 4, beside->side->stream());
+            if (st != ELSA_OK) beside->side->join(stream);
+        }
+    }
     if (st != ELSA_OK) return st;
     bool left = false;
     return block_linear(lin[0], x1, rows, dtype, qkv, 0, nullptr, nullptr, &left, dev_status, stream);
@@ -1101,38 +1216,23 @@ elsa_status elsa_vit_block_rest(const void* x, int rows, int dim, int mlp_dim, c
 namespace elsa {
 namespace {
 
-// The whole block; tokens == 0 runs the stand-in a = V, otherwise the attention kernel over images of `tokens` rows.
-elsa_status run_block(const void* x, int rows, int dim, int mlp_dim, const elsa_block_weights* w, elsa_dtype dtype,
-                      void* y, void* scratch, size_t scratch_bytes, uint32_t* dev_status, void* stream_, int tokens, int heads,
-                      const BlockCarry* carry = nullptr, uint16_t* x_sum = nullptr, BlockCarry* defer = nullptr,
-                      const elsa_swin_attn* swin = nullptr)
-{
-    DeviceInfo dev;
-    elsa_status st = device_info(&dev);
-    if (st != ELSA_OK) return st;
+struct PreparedBlock {
     BlockPlan plan;
     BlockLinear lin[4];
-    if ((st = block_check(x, rows, dim, mlp_dim, w, dtype, y, true, scratch, scratch_bytes, &plan, lin, dev)) != ELSA_OK)
-        return st;
-    cudaStream_t stream = (cudaStream_t)stream_;
-    // The four weight images do not depend on x: they are built on the library's side stream while the first
-    // LayerNorm runs on the caller's, which waits for them before the first linear.
-    bool any_image = false;
-    for (int l = 0; l < 4; ++l) any_image = any_image || takes_image(lin[l]);
-    SidePipe* side = nullptr;
-    if (any_image) {
-        if ((st = side_pipe(dev.device, &side)) != ELSA_OK) return st;
-        cudaError_t e = cudaEventRecord(side->fork, stream);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(side->stream, side->fork, 0);
-        if (e != cudaSuccess) return fail(ELSA_ERR_CUDA, "forking the image stream: %s", cudaGetErrorString(e));
-        st = block_images(lin, 4, side->stream);
-        e = cudaEventRecord(side->join, side->stream);   // joined even after a failed launch: the fork must not dangle
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, side->join, 0);
-        if (st != ELSA_OK) return st;
-        if (e != cudaSuccess) return fail(ELSA_ERR_CUDA, "joining the image stream: %s", cudaGetErrorString(e));
-    }
+};
+
+// A validated block's kernels; tokens == 0 runs the stand-in a = V, otherwise the attention kernel over images of
+// `tokens` rows.  The block's images are on beside->side already, or built where they are used.
+elsa_status run_prepared(const void* x, int rows, int dim, int mlp_dim, const elsa_block_weights* w, elsa_dtype dtype,
+                         void* y, void* scratch, PreparedBlock& block, const BlockSide* beside, uint32_t* dev_status, cudaStream_t stream,
+                         int tokens, int heads, const BlockCarry* carry = nullptr, uint16_t* x_sum = nullptr,
+                         BlockCarry* defer = nullptr, const elsa_swin_attn* swin = nullptr)
+{
+    const BlockPlan& plan = block.plan;
+    BlockLinear (&lin)[4] = block.lin;
+    elsa_status st;
     uint8_t* s8 = (uint8_t*)scratch;
-    if ((st = block_qkv((const uint16_t*)x, rows, dim, w, dtype, s8, plan, lin, dev_status, stream, carry, x_sum, swin)) != ELSA_OK)
+    if ((st = block_qkv((const uint16_t*)x, rows, dim, w, dtype, s8, plan, lin, dev_status, stream, carry, x_sum, swin, beside)) != ELSA_OK)
         return st;
     if (carry != nullptr && carry->t != nullptr) x = x_sum;      // the block's input, as just stored
     if (swin) {
@@ -1154,8 +1254,36 @@ elsa_status run_block(const void* x, int rows, int dim, int mlp_dim, const elsa_
     return block_rest((const uint16_t*)x, rows, dim, mlp_dim, w, dtype, (uint16_t*)y, s8, plan, lin, dev_status, stream, defer, swin);
 }
 
+// One block on its own: its images do not depend on x and are built beside the first LayerNorm.
+elsa_status run_block(const void* x, int rows, int dim, int mlp_dim, const elsa_block_weights* w, elsa_dtype dtype,
+                      void* y, void* scratch, size_t scratch_bytes, uint32_t* dev_status, void* stream_, int tokens, int heads,
+                      const elsa_swin_attn* swin = nullptr)
+{
+    DeviceInfo dev;
+    elsa_status st = device_info(&dev);
+    if (st != ELSA_OK) return st;
+    PreparedBlock block;
+    if ((st = block_check(x, rows, dim, mlp_dim, w, dtype, y, true, scratch, scratch_bytes, &block.plan, block.lin, dev)) != ELSA_OK)
+        return st;
+    cudaStream_t stream = (cudaStream_t)stream_;
+    SideStream side;
+    bool any = false;
+    for (int l = 0; l < 4; ++l) any = any || takes_image(block.lin[l]);
+    if (any) {
+        if ((st = side.fork(dev.device, stream)) == ELSA_OK) st = block_images(block.lin, 4, side.stream());
+        if (st != ELSA_OK) {
+            side.join(stream);
+            return st;
+        }
+    }
+    const BlockSide beside = {&side, nullptr, dev.device};
+    return run_prepared(x, rows, dim, mlp_dim, w, dtype, y, scratch, block, &beside, dev_status, stream, tokens, heads, nullptr, nullptr,
+                        nullptr, swin);
+}
+
 struct EncoderPlan {
     size_t block_bytes;   // scratch of the largest block
+    size_t images;        // a second place for weight images: block b + 1's are built while block b runs
     size_t buf[2];        // byte offsets of the two activation buffers the blocks alternate between
     size_t total;
 };
@@ -1164,16 +1292,21 @@ bool encoder_plan(int rows, int dim, int mlp_dim, const elsa_block_weights* bloc
 {
     if (!blocks || n_blocks <= 0) return false;
     p->block_bytes = 0;
+    size_t image_bytes = 0;
     for (int b = 0; b < n_blocks; ++b) {
         BlockPlan plan;
         if (!block_plan(rows, dim, mlp_dim, blocks + b, dtype, &plan)) return false;
         if (plan.total > p->block_bytes) p->block_bytes = plan.total;
+        const size_t images = plan.total - plan.off[ELSA_BLOCK_WORKSPACE];
+        if (images > image_bytes) image_bytes = images;
     }
     size_t at = round_up(p->block_bytes, 256);
     for (int i = 0; i < 2; ++i) {
         p->buf[i] = at;
         at += round_up((size_t)rows * dim * 2, 256);
     }
+    p->images = at;
+    at += image_bytes;
     p->total = at;
     return true;
 }
@@ -1219,10 +1352,11 @@ elsa_status elsa_vit_encoder(const void* x, int images, int tokens, int heads, i
     uint8_t* s8 = (uint8_t*)scratch;
     uint16_t* buf[2] = {(uint16_t*)(s8 + plan.buf[0]), (uint16_t*)(s8 + plan.buf[1])};
     // every block is validated before the first launch
+    std::vector<PreparedBlock> prepared(n_blocks);
     for (int b = 0; b < n_blocks; ++b) {
-        BlockPlan bp;
-        BlockLinear lin[4];
-        if ((st = block_check(x, rows, dim, mlp_dim, blocks + b, dtype, buf[0], true, scratch, plan.block_bytes, &bp, lin, dev)) != ELSA_OK) {
+        PreparedBlock& p = prepared[b];
+        if ((st = block_check(x, rows, dim, mlp_dim, blocks + b, dtype, buf[0], true, scratch, plan.block_bytes, &p.plan, p.lin, dev,
+                              b & 1 ? s8 + plan.images : nullptr)) != ELSA_OK) {
             char msg[400];
             snprintf(msg, sizeof msg, "%s", elsa_last_error());
             return fail(st, "block %d: %s", b, msg);
@@ -1230,15 +1364,30 @@ elsa_status elsa_vit_encoder(const void* x, int images, int tokens, int heads, i
     }
     // Block b reads its input from buf[b % 2] (block 0: from x) and writes its output to buf[(b + 1) % 2]; where a
     // block's last residual is still to be added, the next block's first LayerNorm does it while it normalises.
+    // The weight images of block b + 1 are built on a side stream while block b runs, alternating between two places.
+    SideStream side;
+    bool any = false;
+    for (int l = 0; l < 4; ++l) any = any || takes_image(prepared[0].lin[l]);
+    if (any) {
+        if ((st = side.fork(dev.device, (cudaStream_t)stream)) == ELSA_OK) st = block_images(prepared[0].lin, 4, side.stream());
+        if (st != ELSA_OK) {
+            side.join((cudaStream_t)stream);
+            return st;
+        }
+    }
     BlockCarry carry;
     const void* in = x;
     for (int b = 0; b < n_blocks; ++b) {
         const bool last = b + 1 == n_blocks;
         void* out = (last && final_gain == nullptr) ? y : (void*)buf[(b + 1) & 1];
         BlockCarry next;
-        st = run_block(in, rows, dim, mlp_dim, blocks + b, dtype, out, scratch, plan.block_bytes, dev_status, stream, tokens, heads,
-                       &carry, buf[b & 1], last && final_gain == nullptr ? nullptr : &next);
-        if (st != ELSA_OK) return st;
+        const BlockSide beside = {&side, last ? nullptr : prepared[b + 1].lin, dev.device};
+        st = run_prepared(in, rows, dim, mlp_dim, blocks + b, dtype, out, scratch, prepared[b], &beside, dev_status, (cudaStream_t)stream,
+                          tokens, heads, &carry, buf[b & 1], last && final_gain == nullptr ? nullptr : &next);
+        if (st != ELSA_OK) {
+            side.join((cudaStream_t)stream);
+            return st;
+        }
         carry = next;
         in = buf[(b + 1) & 1];
     }
@@ -1329,7 +1478,7 @@ elsa_status elsa_swin_block(const void* x, int images, int heads, int dim, int m
     if (attn->bias_pitch < T) return fail(ELSA_ERR_SHAPE, "bias_pitch=%d is below the %d tokens of a window", attn->bias_pitch, T);
     if ((long long)images * attn->H * attn->W > 0x7fffffffLL) return fail(ELSA_ERR_SHAPE, "images * H * W does not fit an int");
     return run_block(x, images * attn->H * attn->W, dim, mlp_dim, w, dtype, y, scratch, scratch_bytes, dev_status, stream, T, heads,
-                     nullptr, nullptr, nullptr, attn);
+                     attn);
 }
 
 elsa_status elsa_window_attention(const void* qkv, int windows, int tokens, int heads, int dim, const float* bias,
@@ -1397,11 +1546,14 @@ elsa_status dense_product(const uint16_t* A, int m, const uint16_t* B, int n, in
                           uint32_t* dev_status, cudaStream_t stream, int sm_count)
 {
     const int variant = g_variant.load(std::memory_order_relaxed);
-    if (variant == ELSA_VARIANT_TC_DENSE) return launch_linear_tc_dense(A, m, B, nullptr, n, k, dtype, Y, dev_status, stream);
-    if (variant == ELSA_VARIANT_TC_PAIR || (variant != ELSA_VARIANT_TC_SMALL && linear_tc_pair_suits(m, n, sm_count)))
-        return launch_linear_tc_pair(A, m, B, nullptr, n, k, dtype, Y, dev_status, stream);
-    const SmallJob job = small_job(A, m, B, nullptr, nullptr, n, k, 8, 8, Y);
-    return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, sm_count), false, dtype, dev_status, stream);
+    const SmallJob job = small_dense_job(A, m, B, nullptr, n, k, Y);
+    LinearKind kind;       // the dense level's rule
+    const elsa_status st = pick_kind(USE_SINGLE, m, n, k, 4, 4, sm_count, &kind);
+    if (st != ELSA_OK || variant == ELSA_VARIANT_TC_DENSE || kind == KIND_DENSE_ONE)
+        return launch_linear_tc_dense(A, m, B, nullptr, n, k, dtype, Y, dev_status, stream);
+    if (kind == KIND_SMALL || kind == KIND_SMALL_IMAGE)
+        return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, sm_count), false, dtype, dev_status, stream);
+    return launch_linear_tc_pair(A, m, B, nullptr, n, k, dtype, Y, dev_status, stream);
 }
 
 }  // namespace

@@ -1,0 +1,71 @@
+"""Calls that build weight images on a side stream, made from several threads on streams of their own at once: every result
+equals the one of the same call made alone (a call whose images were ordered after another call's work would not)."""
+import threading
+
+import pytest
+import torch
+
+from paper_2409_09708_b200 import synth
+
+
+@pytest.mark.gpu
+def test_encoders_and_tables_of_several_threads_do_not_disturb_each_other():
+    from paper_2409_09708_b200 import binding as lib
+    dtype, dim, tokens, heads = torch.bfloat16, 256, 65, 4
+    code = lib.dtype_code(dtype)
+    levels = [(2, 4), (1, 8), (4, 8), (4, 4), (2, 8)]
+
+    def case(seed):
+        blocks, keep = [], []
+        for b in range(4):
+            lin = {}
+            for i, (name, k, o) in enumerate((("qkv", dim, 3 * dim), ("proj", dim, dim), ("fc1", dim, 4 * dim), ("fc2", 4 * dim, dim))):
+                N, M = levels[(seed + b + i) % 5]
+                W = synth.randn((o, k), 100 * seed + 10 * b + i, 0.05, dtype, "cuda")
+                lin[name] = lib.elsa_nm_compress(W, N, M) + (synth.randn((o,), 7 + i, 0.02, dtype, "cuda"), N, M)
+            ln = [synth.randn((dim,), 50 + i, 0.1, dtype, "cuda") + (1.0 if i % 2 == 0 else 0.0) for i in range(4)]
+            w, k = lib.make_block_weights(*[t.to(dtype) for t in ln], lin)
+            blocks.append(w)
+            keep.append(k)
+        images = 3 + 20 * (seed % 3)                                 # one wave of small tiles, and more
+        x = synth.randn((images * tokens, dim), seed, 1.0, dtype, "cuda")
+        layers = []
+        for i, (N, M) in enumerate([(4, 4), (2, 4), (1, 8), (4, 8)]):
+            layer = synth.Layer("l", 9000, 512, 512, N, M, 3 * i + seed, 3 * i + 1, 3 * i + 2)
+            X, W, bias = synth.layer_tensors(layer, dtype, device="cuda")
+            vals, idx = lib.elsa_nm_compress(W, N, M)
+            layers.append(dict(X=X, vals=vals, idx=idx, bias=bias, N=N, M=M, Y=torch.empty((9000, 512), dtype=dtype, device="cuda")))
+        table = lib.make_layer_table(layers)
+        ws = lib.alloc_workspace(lib.elsa_vit_workspace_bytes(table, code))
+        return dict(x=x, table=lib.make_encoder_table(blocks), keep=(keep, layers), layers=table, Y=[l["Y"] for l in layers], ws=ws)
+
+    def run(c):
+        y, c["scratch"] = lib.elsa_vit_encoder(c["x"], tokens, heads, 4 * dim, c["table"], scratch=c.get("scratch"))
+        for t in c["Y"]:
+            t.zero_()
+        lib.elsa_vit_linears(c["layers"], code, c["ws"])
+        return [y.clone()] + [t.clone() for t in c["Y"]]
+
+    cases = [case(s) for s in range(4)]
+    alone = [run(c) for c in cases]
+    torch.cuda.synchronize()
+    wrong, errors = [], []
+
+    def work(i):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(10):
+                    got = run(cases[i])
+                    torch.cuda.current_stream().synchronize()
+                    if not all(torch.equal(a, b) for a, b in zip(got, alone[i])):
+                        wrong.append(i)
+        except Exception as e:                                       # a failed call fails the test, not the thread alone
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
+    assert not wrong, wrong
