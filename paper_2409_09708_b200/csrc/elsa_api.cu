@@ -1022,16 +1022,21 @@ bool takes_image(const BlockLinear& L)
     return L.w->N != L.w->M && (L.kind == KIND_DENSE_PAIR || L.kind == KIND_SMALL_IMAGE || L.kind == KIND_SPARSE_PAIR || L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST);
 }
 
-// The images of the linears that take one, in one launch.
-elsa_status block_images(BlockLinear* lin, int n, cudaStream_t stream)
+// Adds the images that n linears take to `jobs`.
+void add_images(const BlockLinear* lin, int n, std::vector<ImageJob>* jobs)
 {
-    ImageJob jobs[4];
-    int count = 0;
     for (int l = 0; l < n; ++l)
         if (takes_image(lin[l]) && !lin[l].image_ready)
-            jobs[count++] = image_job(lin[l].kind, lin[l].w->vals, lin[l].w->idx, lin[l].out, lin[l].in, lin[l].w->N, lin[l].w->M, lin[l].ws);
-    if (count == 0) return ELSA_OK;
-    const elsa_status st = launch_images(jobs, count, stream);
+            jobs->push_back(image_job(lin[l].kind, lin[l].w->vals, lin[l].w->idx, lin[l].out, lin[l].in, lin[l].w->N, lin[l].w->M, lin[l].ws));
+}
+
+// The images of n linears that take one, in one launch.
+elsa_status block_images(BlockLinear* lin, int n, cudaStream_t stream)
+{
+    std::vector<ImageJob> jobs;
+    add_images(lin, n, &jobs);
+    if (jobs.empty()) return ELSA_OK;
+    const elsa_status st = launch_images(jobs.data(), (int)jobs.size(), stream);
     if (st == ELSA_OK)
         for (int l = 0; l < n; ++l) lin[l].image_ready = takes_image(lin[l]);
     return st;
@@ -1056,7 +1061,7 @@ elsa_status block_linear(BlockLinear& L, const uint16_t* X, int rows, elsa_dtype
         return launch_linear_tc_pair_group(&job, 1, dtype, dev_status, stream);
     }
     if (L.kind == KIND_SMALL || L.kind == KIND_SMALL_IMAGE) {
-        const bool ready = L.image_ready;       // built and joined before an earlier kernel of this call
+        const bool ready = L.image_ready;       // enqueued before an earlier kernel of this call, which waited for it
         if ((st = block_images(&L, 1, stream)) != ELSA_OK) return st;
         SmallJob job = L.kind == KIND_SMALL ? small_job(X, rows, w.vals, w.N == w.M ? nullptr : w.idx, w.bias, L.out, L.in, w.N, w.M, Y)
                                             : small_dense_job(X, rows, w.N == w.M ? w.vals : L.ws, w.bias, L.out, L.in, Y);
@@ -1091,19 +1096,11 @@ struct BlockCarry {
     const uint16_t* r = nullptr;   // x2
 };
 
-// The side stream's part in a block: joined between the first LayerNorm and the first linear, where the images of the
-// block itself must be ready; those of the next block (or NULL) are started there, beside this block's kernels.
-struct BlockSide {
-    SideStream* side;
-    BlockLinear* next;
-    int device;
-};
-
 // carry (or NULL) + x_sum: the block's input is carry->t + carry->r, written to x_sum; otherwise it is x.
 elsa_status block_qkv(const uint16_t* x, int rows, int dim, const elsa_block_weights* w, elsa_dtype dtype,
                       uint8_t* scratch, const BlockPlan& plan, BlockLinear (&lin)[4], uint32_t* dev_status,
                       cudaStream_t stream, const BlockCarry* carry = nullptr, uint16_t* x_sum = nullptr,
-                      const elsa_swin_attn* swin = nullptr, const BlockSide* beside = nullptr)
+                      const elsa_swin_attn* swin = nullptr)
 {
     uint16_t* x1 = (uint16_t*)(scratch + plan.off[ELSA_BLOCK_X1]);
     uint16_t* qkv = (uint16_t*)(scratch + plan.off[ELSA_BLOCK_QKV]);
@@ -1113,17 +1110,6 @@ elsa_status block_qkv(const uint16_t* x, int rows, int dim, const elsa_block_wei
     elsa_status st = launch_layer_norm(add ? carry->t : x, add ? carry->r : nullptr, add ? x_sum : nullptr,
                                        (const uint16_t*)w->ln1_gain, (const uint16_t*)w->ln1_bias,
                                        x1, rows, dim, w->eps, dtype, stream, swin ? &out_map : nullptr);
-    if (beside != nullptr) {
-        const elsa_status joined = beside->side->join(stream);
-        if (st == ELSA_OK) st = joined;
-        if (st == ELSA_OK && beside->next != nullptr) {
-            bool any = false;
-            for (int l = 0; l < 4; ++l) any = any || takes_image(beside->next[l]);
-            if (any && (st = beside->side->fork(beside->device, stream)) == ELSA_OK)
-                st = block_images(beside->next, 4, beside->side->stream());
-            if (st != ELSA_OK) beside->side->join(stream);
-        }
-    }
     if (st != ELSA_OK) return st;
     bool left = false;
     return block_linear(lin[0], x1, rows, dtype, qkv, 0, nullptr, nullptr, &left, dev_status, stream);
@@ -1222,9 +1208,9 @@ struct PreparedBlock {
 };
 
 // A validated block's kernels; tokens == 0 runs the stand-in a = V, otherwise the attention kernel over images of
-// `tokens` rows.  The block's images are on beside->side already, or built where they are used.
+// `tokens` rows.  The block's images have been enqueued already, or are built where they are used.
 elsa_status run_prepared(const void* x, int rows, int dim, int mlp_dim, const elsa_block_weights* w, elsa_dtype dtype,
-                         void* y, void* scratch, PreparedBlock& block, const BlockSide* beside, uint32_t* dev_status, cudaStream_t stream,
+                         void* y, void* scratch, PreparedBlock& block, uint32_t* dev_status, cudaStream_t stream,
                          int tokens, int heads, const BlockCarry* carry = nullptr, uint16_t* x_sum = nullptr,
                          BlockCarry* defer = nullptr, const elsa_swin_attn* swin = nullptr)
 {
@@ -1232,7 +1218,7 @@ elsa_status run_prepared(const void* x, int rows, int dim, int mlp_dim, const el
     BlockLinear (&lin)[4] = block.lin;
     elsa_status st;
     uint8_t* s8 = (uint8_t*)scratch;
-    if ((st = block_qkv((const uint16_t*)x, rows, dim, w, dtype, s8, plan, lin, dev_status, stream, carry, x_sum, swin, beside)) != ELSA_OK)
+    if ((st = block_qkv((const uint16_t*)x, rows, dim, w, dtype, s8, plan, lin, dev_status, stream, carry, x_sum, swin)) != ELSA_OK)
         return st;
     if (carry != nullptr && carry->t != nullptr) x = x_sum;      // the block's input, as just stored
     if (swin) {
@@ -1254,7 +1240,8 @@ elsa_status run_prepared(const void* x, int rows, int dim, int mlp_dim, const el
     return block_rest((const uint16_t*)x, rows, dim, mlp_dim, w, dtype, (uint16_t*)y, s8, plan, lin, dev_status, stream, defer, swin);
 }
 
-// One block on its own: its images do not depend on x and are built beside the first LayerNorm.
+// One block on its own.  Its images are one launch ahead of the first LayerNorm: a fork to a side stream and back costs
+// about 7 us in events and lost launch overlap, the launch 3 to 6.
 elsa_status run_block(const void* x, int rows, int dim, int mlp_dim, const elsa_block_weights* w, elsa_dtype dtype,
                       void* y, void* scratch, size_t scratch_bytes, uint32_t* dev_status, void* stream_, int tokens, int heads,
                       const elsa_swin_attn* swin = nullptr)
@@ -1266,24 +1253,14 @@ elsa_status run_block(const void* x, int rows, int dim, int mlp_dim, const elsa_
     if ((st = block_check(x, rows, dim, mlp_dim, w, dtype, y, true, scratch, scratch_bytes, &block.plan, block.lin, dev)) != ELSA_OK)
         return st;
     cudaStream_t stream = (cudaStream_t)stream_;
-    SideStream side;
-    bool any = false;
-    for (int l = 0; l < 4; ++l) any = any || takes_image(block.lin[l]);
-    if (any) {
-        if ((st = side.fork(dev.device, stream)) == ELSA_OK) st = block_images(block.lin, 4, side.stream());
-        if (st != ELSA_OK) {
-            side.join(stream);
-            return st;
-        }
-    }
-    const BlockSide beside = {&side, nullptr, dev.device};
-    return run_prepared(x, rows, dim, mlp_dim, w, dtype, y, scratch, block, &beside, dev_status, stream, tokens, heads, nullptr, nullptr,
+    if ((st = block_images(block.lin, 4, stream)) != ELSA_OK) return st;
+    return run_prepared(x, rows, dim, mlp_dim, w, dtype, y, scratch, block, dev_status, stream, tokens, heads, nullptr, nullptr,
                         nullptr, swin);
 }
 
 struct EncoderPlan {
     size_t block_bytes;   // scratch of the largest block
-    size_t images;        // a second place for weight images: block b + 1's are built while block b runs
+    size_t images;        // the weight images of every block
     size_t buf[2];        // byte offsets of the two activation buffers the blocks alternate between
     size_t total;
 };
@@ -1297,8 +1274,7 @@ bool encoder_plan(int rows, int dim, int mlp_dim, const elsa_block_weights* bloc
         BlockPlan plan;
         if (!block_plan(rows, dim, mlp_dim, blocks + b, dtype, &plan)) return false;
         if (plan.total > p->block_bytes) p->block_bytes = plan.total;
-        const size_t images = plan.total - plan.off[ELSA_BLOCK_WORKSPACE];
-        if (images > image_bytes) image_bytes = images;
+        image_bytes += plan.total - plan.off[ELSA_BLOCK_WORKSPACE];
     }
     size_t at = round_up(p->block_bytes, 256);
     for (int i = 0; i < 2; ++i) {
@@ -1353,41 +1329,34 @@ elsa_status elsa_vit_encoder(const void* x, int images, int tokens, int heads, i
     uint16_t* buf[2] = {(uint16_t*)(s8 + plan.buf[0]), (uint16_t*)(s8 + plan.buf[1])};
     // every block is validated before the first launch
     std::vector<PreparedBlock> prepared(n_blocks);
+    std::vector<ImageJob> image_jobs;
+    uint8_t* image_at = s8 + plan.images;
     for (int b = 0; b < n_blocks; ++b) {
         PreparedBlock& p = prepared[b];
         if ((st = block_check(x, rows, dim, mlp_dim, blocks + b, dtype, buf[0], true, scratch, plan.block_bytes, &p.plan, p.lin, dev,
-                              b & 1 ? s8 + plan.images : nullptr)) != ELSA_OK) {
+                              image_at)) != ELSA_OK) {
             char msg[400];
             snprintf(msg, sizeof msg, "%s", elsa_last_error());
             return fail(st, "block %d: %s", b, msg);
         }
+        image_at += p.plan.total - p.plan.off[ELSA_BLOCK_WORKSPACE];
+        add_images(p.lin, 4, &image_jobs);
+        for (int l = 0; l < 4; ++l) p.lin[l].image_ready = takes_image(p.lin[l]);
     }
+    // The weight images of all blocks in one launch ahead of the chain (170 MB for a dense DeiT-B: 25 us once, against
+    // about 7 us a block for building them beside the block before on a side stream).
+    if (!image_jobs.empty() && (st = launch_images(image_jobs.data(), (int)image_jobs.size(), (cudaStream_t)stream)) != ELSA_OK) return st;
     // Block b reads its input from buf[b % 2] (block 0: from x) and writes its output to buf[(b + 1) % 2]; where a
     // block's last residual is still to be added, the next block's first LayerNorm does it while it normalises.
-    // The weight images of block b + 1 are built on a side stream while block b runs, alternating between two places.
-    SideStream side;
-    bool any = false;
-    for (int l = 0; l < 4; ++l) any = any || takes_image(prepared[0].lin[l]);
-    if (any) {
-        if ((st = side.fork(dev.device, (cudaStream_t)stream)) == ELSA_OK) st = block_images(prepared[0].lin, 4, side.stream());
-        if (st != ELSA_OK) {
-            side.join((cudaStream_t)stream);
-            return st;
-        }
-    }
     BlockCarry carry;
     const void* in = x;
     for (int b = 0; b < n_blocks; ++b) {
         const bool last = b + 1 == n_blocks;
         void* out = (last && final_gain == nullptr) ? y : (void*)buf[(b + 1) & 1];
         BlockCarry next;
-        const BlockSide beside = {&side, last ? nullptr : prepared[b + 1].lin, dev.device};
-        st = run_prepared(in, rows, dim, mlp_dim, blocks + b, dtype, out, scratch, prepared[b], &beside, dev_status, (cudaStream_t)stream,
+        st = run_prepared(in, rows, dim, mlp_dim, blocks + b, dtype, out, scratch, prepared[b], dev_status, (cudaStream_t)stream,
                           tokens, heads, &carry, buf[b & 1], last && final_gain == nullptr ? nullptr : &next);
-        if (st != ELSA_OK) {
-            side.join((cudaStream_t)stream);
-            return st;
-        }
+        if (st != ELSA_OK) return st;
         carry = next;
         in = buf[(b + 1) & 1];
     }
