@@ -139,7 +139,7 @@ elsa_status elsa_vit_compress(const elsa_weight* w, int n_weights, elsa_dtype dt
 
 /*
  * Sec. 3.1, subset-superset relation: all levels N:M of a supernet layer share one weight, and the
- * magnitude ranks inside a group do not depend on N.  This call reads W once and writes the packed
+ * magnitude ranks inside a group do not depend on N.  This call writes, in one launch, the packed
  * form of every requested level N_list[l]:M (same M), each bit-identical to what elsa_nm_compress
  * writes for that level.  `N_list`, `vals` and `idx` are HOST arrays of n_levels entries holding
  * device pointers (idx[l] may be NULL iff N_list[l] == M); n_levels <= 16.

@@ -456,8 +456,7 @@ elsa_status elsa_nm_compress_levels(const void* W, int out, int in, int M, const
     if (n_levels < 1 || n_levels > kMaxLevels)
         return fail(ELSA_ERR_SHAPE, "n_levels=%d is outside 1..%d", n_levels, kMaxLevels);
     if (!aligned16(W)) return fail(ELSA_ERR_ALIGN, "W must be 16-byte aligned");
-    LevelTable t;
-    t.n = n_levels;
+    CompressJob jobs[kMaxLevels];
     for (int l = 0; l < n_levels; ++l) {
         elsa_status st = check_level(out, in, N_list[l], M, dtype);
         if (st == ELSA_OK && !vals[l]) st = fail(ELSA_ERR_NULL, "vals must not be NULL");
@@ -469,14 +468,12 @@ elsa_status elsa_nm_compress_levels(const void* W, int out, int in, int M, const
             snprintf(msg, sizeof msg, "%s", elsa_last_error());
             return fail(st, "level %d: %s", l, msg);
         }
-        t.N[l] = N_list[l];
-        t.vals[l] = (uint16_t*)vals[l];
-        t.idx[l] = N_list[l] == M ? nullptr : idx[l];
+        jobs[l] = {(const uint16_t*)W, (uint16_t*)vals[l], N_list[l] == M ? nullptr : idx[l], out, in, N_list[l], M};
     }
     DeviceInfo dev;
     elsa_status st = device_info(&dev);
     if (st != ELSA_OK) return st;
-    return launch_compress_levels((const uint16_t*)W, out, in, M, t, (cudaStream_t)stream);
+    return launch_compress_jobs(jobs, n_levels, (cudaStream_t)stream);
 }
 
 elsa_status elsa_nm_linear_masked(const void* X, int rows, const void* W_sup, const void* bias, int out, int in,
@@ -550,22 +547,12 @@ elsa_status elsa_vit_compress(const elsa_weight* w, int n_weights, elsa_dtype dt
     DeviceInfo dev;
     elsa_status st = device_info(&dev);
     if (st != ELSA_OK) return st;
-    static BatchTable table;              // host staging of the kernel parameters
-    static std::mutex table_mutex;
-    std::lock_guard<std::mutex> lock(table_mutex);
-    table.n = 0;
-    table.total_units = 0;
+    std::vector<CompressJob> jobs(n_weights);
     for (int i = 0; i < n_weights; ++i) {
         const elsa_weight& c = w[i];
-        batch_add_compress(&table, (const uint16_t*)c.W, c.out, c.in, c.N, c.M, (uint16_t*)c.vals,
-                           c.N == c.M ? nullptr : c.idx);
-        if (table.n == kBatchMax || i == n_weights - 1) {
-            if ((st = launch_compress_batch(table, (cudaStream_t)stream)) != ELSA_OK) return st;
-            table.n = 0;
-            table.total_units = 0;
-        }
+        jobs[i] = {(const uint16_t*)c.W, (uint16_t*)c.vals, c.N == c.M ? nullptr : c.idx, c.out, c.in, c.N, c.M};
     }
-    return ELSA_OK;
+    return launch_compress_jobs(jobs.data(), n_weights, (cudaStream_t)stream);
 }
 
 size_t elsa_vit_workspace_bytes(const elsa_layer* cfg, int n_layers, elsa_dtype dtype)

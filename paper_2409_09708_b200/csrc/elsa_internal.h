@@ -233,32 +233,15 @@ elsa_status launch_mask_apply(uint16_t* dW, const uint32_t* idx, int out, int in
 // dW [out][in] = mask .* round16(sum over ranges of partial [splits][out][in]); idx NULL (N == M) keeps everything.
 elsa_status launch_wgrad_finish(const float* partial, int splits, const uint32_t* idx, int out, int in, int N, int M,
                                 elsa_dtype dtype, uint16_t* dW, cudaStream_t stream);
-// Several levels of one weight in one pass.
+// Any number of (weight, level) pairs, one launch per 256.
+struct CompressJob {
+    const uint16_t* W;
+    uint16_t* vals;
+    uint32_t* idx;
+    int out, in, N, M;
+};
+elsa_status launch_compress_jobs(const CompressJob* jobs, int n, cudaStream_t stream);
 constexpr int kMaxLevels = 16;
-struct LevelTable {
-    int n;
-    int N[kMaxLevels];
-    uint16_t* vals[kMaxLevels];
-    uint32_t* idx[kMaxLevels];
-};
-elsa_status launch_compress_levels(const uint16_t* W, int out, int in, int M, const LevelTable& t, cudaStream_t stream);
-
-// Batched compress: one launch over a table of weights (kernel-parameter space).
-struct BatchItem {
-    const void* src;
-    void* dst;
-    void* dst2;
-    long long first_unit;   // prefix sum of work units over the table
-    int out, in, N, M, wpr, segs_per_row;
-};
-constexpr int kBatchMax = 256;
-struct BatchTable {
-    BatchItem item[kBatchMax];
-    long long total_units;
-    int n;
-};
-void batch_add_compress(BatchTable* t, const uint16_t* W, int out, int in, int N, int M, uint16_t* vals, uint32_t* idx);
-elsa_status launch_compress_batch(const BatchTable& t, cudaStream_t stream);
 
 // Several dense-rate layers in one persistent launch of the CTA-pair kernel (at most
 // linear_tc_pair_group_max() of them): their tiles form one sequence.

@@ -63,15 +63,13 @@ __device__ __forceinline__ uint32_t keep_mask(unsigned long long ranks, int N)
     return keep;
 }
 
-// One warp compresses 32 consecutive groups of one row, one group per lane, to each of `n_levels`
-// levels N_list[l]:M (one read of W, ranks computed once).  The 32 groups own exactly N*b whole index
-// words of the row's bitstream, so the warp assembles its words in shared memory and writes them with
-// one coalesced store.
+// One warp compresses 32 consecutive groups of one row, one group per lane, at any level N < M: the form for the levels
+// that have none of their own (elsa_compress.cu).  The 32 groups own exactly N*b whole index words of the row's
+// bitstream, so the warp assembles its words in shared memory and writes them with one coalesced store.
 template <int M>
-__device__ __forceinline__ void compress_segment_levels(const uint16_t* __restrict__ W, int in, int n_levels,
-                                                        const int* N_list, uint16_t* const* vals_list,
-                                                        uint32_t* const* idx_list, int segs_per_row, long long seg_id,
-                                                        uint32_t (*words)[kMaxIndexWordsPerSegment])
+__device__ __forceinline__ void compress_segment(const uint16_t* __restrict__ W, int in, int N, uint16_t* __restrict__ vals,
+                                                 uint32_t* __restrict__ idx, int segs_per_row, int words_per_row, long long seg_id,
+                                                 uint32_t (*words)[kMaxIndexWordsPerSegment])
 {
     constexpr int B = (M == 4) ? 2 : (M == 8) ? 3 : 4;
     const int lane = threadIdx.x & 31;
@@ -81,86 +79,41 @@ __device__ __forceinline__ void compress_segment_levels(const uint16_t* __restri
     const int seg = (int)(seg_id % segs_per_row);
     const int groups_per_row = in / M;
     const int g = seg * 32 + lane;
-    const bool valid = g < groups_per_row;
+    const int seg_words = N * B;  // index words this segment owns
 
-    uint16_t w[M];
-    unsigned long long ranks = 0;
-    if (valid) {
+    for (int k = lane; k < seg_words; k += 32) words[warp][k] = 0;
+    __syncwarp();
+    if (g < groups_per_row) {
+        uint16_t w[M];
         load_group<M>(W + (size_t)o * in + (size_t)g * M, w);
-        ranks = group_ranks<M>(w);
-    }
-
-    for (int l = 0; l < n_levels; ++l) {
-        const int N = N_list[l];
-        uint16_t* vals = vals_list[l];
-        uint32_t* idx = idx_list[l];
-        const int words_per_row = (N == M) ? 0 : (groups_per_row * N * B + 31) / 32;
-        const int seg_words = N * B;  // index words this segment owns (when N < M)
-
-        if (words_per_row) {
-            for (int k = lane; k < seg_words; k += 32) words[warp][k] = 0;
-            __syncwarp();
-        }
-        if (valid) {
-            const uint32_t keep = keep_mask<M>(ranks, N);
-            uint16_t* v = vals + (size_t)o * ((size_t)groups_per_row * N) + (size_t)g * N;
-            unsigned long long fields = 0;
-            int t = 0;
-#pragma unroll
-            for (int i = 0; i < M; ++i) {
-                if ((keep >> i) & 1u) {
-                    v[t] = w[i];
-                    fields |= (unsigned long long)i << (t * B);
-                    ++t;
-                }
-            }
-            if (words_per_row) {
-                const int bit0 = lane * seg_words;  // bit offset of this group's fields in the segment
-                const int w0 = bit0 >> 5, sh = bit0 & 31;
-                // up to 60 bits shifted by up to 31: three words at most
-                const uint32_t lo = (uint32_t)(fields << sh);
-                const uint32_t mid = (uint32_t)(fields >> (32 - sh));
-                const uint32_t hi = sh ? (uint32_t)(fields >> (64 - sh)) : 0u;
-                // a zero part may lie past the segment's last word and is skipped
-                if (lo) atomicOr(&words[warp][w0], lo);
-                if (mid) atomicOr(&words[warp][w0 + 1], mid);
-                if (hi) atomicOr(&words[warp][w0 + 2], hi);
-            }
-        }
-        if (words_per_row) {
-            __syncwarp();
-            const int first = seg * seg_words;
-            uint32_t* row = idx + (size_t)o * words_per_row;
-            for (int k = lane; k < seg_words && first + k < words_per_row; k += 32) row[first + k] = words[warp][k];
-            __syncwarp();
-        }
-    }
-}
-
-// ---- single-level fast path for M = 4 and M = 8 (the levels of the ViT tables) -------------------
-//
-// Same result as compress_segment_levels with one level, in about a third of the instructions:
-//   * every position gets a unique key (magnitude bits above, M-1-position below), so "the N of largest
-//     magnitude, lowest position first among equals" is "key >= the N-th largest key";
-//   * the N-th largest key comes from a sorting network (5 / 19 compare-exchanges);
-//   * kept values are compacted with byte permutes driven by a small table in shared memory: for each
-//     keep mask, the kept positions in ascending order as 4-bit fields (the permute selectors) and as
-//     log2(M)-bit fields (the index bits to store);
-//   * one vector store per group for the values.
-struct CompactEntry { uint32_t order4; uint32_t fields; };
-
-template <int M>
-__device__ __forceinline__ void build_compact_table(CompactEntry* table)
-{
-    constexpr int B = (M == 4) ? 2 : 3;
-    for (int m = threadIdx.x; m < (1 << M); m += blockDim.x) {
-        uint32_t o4 = 0, f = 0;
+        const uint32_t keep = keep_mask<M>(group_ranks<M>(w), N);
+        uint16_t* v = vals + (size_t)o * ((size_t)groups_per_row * N) + (size_t)g * N;
+        unsigned long long fields = 0;
         int t = 0;
-        for (int i = 0; i < M; ++i)
-            if ((m >> i) & 1) { o4 |= (uint32_t)i << (4 * t); f |= (uint32_t)i << (B * t); ++t; }
-        table[m].order4 = o4;
-        table[m].fields = f;
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            if ((keep >> i) & 1u) {
+                v[t] = w[i];
+                fields |= (unsigned long long)i << (t * B);
+                ++t;
+            }
+        }
+        const int bit0 = lane * seg_words;  // bit offset of this group's fields in the segment
+        const int w0 = bit0 >> 5, sh = bit0 & 31;
+        // up to 60 bits shifted by up to 31: three words at most
+        const uint32_t lo = (uint32_t)(fields << sh);
+        const uint32_t mid = (uint32_t)(fields >> (32 - sh));
+        const uint32_t hi = sh ? (uint32_t)(fields >> (64 - sh)) : 0u;
+        // a zero part may lie past the segment's last word and is skipped
+        if (lo) atomicOr(&words[warp][w0], lo);
+        if (mid) atomicOr(&words[warp][w0 + 1], mid);
+        if (hi) atomicOr(&words[warp][w0 + 2], hi);
     }
+    __syncwarp();
+    const int first = seg * seg_words;
+    uint32_t* row = idx + (size_t)o * words_per_row;
+    for (int k = lane; k < seg_words && first + k < words_per_row; k += 32) row[first + k] = words[warp][k];
+    __syncwarp();
 }
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
@@ -232,143 +185,65 @@ __device__ __forceinline__ uint32_t keep_mask_sorted(const uint32_t (&h)[M], int
     return keep;
 }
 
-// Split in two so that a warp can have the loads of several segments in flight before it works on the
-// first: one 16-byte load per lane is too little outstanding memory traffic to cover its own latency.
-template <int M>
-__device__ __forceinline__ void compress_fast_load(const uint16_t* __restrict__ W, int in, int o, int seg,
-                                                   uint32_t (&r)[M / 2])
+// The 16 bits at position `pos` of consecutive positions packed two to a word.
+template <int kWords>
+__device__ __forceinline__ uint32_t half_of(const uint32_t (&a)[kWords], uint32_t pos)
 {
-    constexpr int R = M / 2;                      // 32-bit registers per group
-    const int lane = threadIdx.x & 31;
-    const int g = seg * 32 + lane;
-#pragma unroll
-    for (int q = 0; q < R; ++q) r[q] = 0;
-    if (g < in / M) {
-        const uint16_t* src = W + (size_t)o * in + (size_t)g * M;
-        if constexpr (M == 4) { const uint2 v = *reinterpret_cast<const uint2*>(src); r[0] = v.x; r[1] = v.y; }
-        else { const uint4 v = *reinterpret_cast<const uint4*>(src); r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w; }
+    uint32_t w;
+    if constexpr (kWords == 2) w = pos & 2u ? a[1] : a[0];
+    else if constexpr (kWords == 4) w = pos & 4u ? (pos & 2u ? a[3] : a[2]) : (pos & 2u ? a[1] : a[0]);
+    else {
+        const uint32_t lo = pos & 4u ? (pos & 2u ? a[3] : a[2]) : (pos & 2u ? a[1] : a[0]);
+        const uint32_t hi = pos & 4u ? (pos & 2u ? a[7] : a[6]) : (pos & 2u ? a[5] : a[4]);
+        w = pos & 8u ? hi : lo;
     }
+    return (pos & 1u ? w >> 16 : w) & 0xFFFFu;
 }
 
-// NC: the level's N as a compile-time constant (0 = take `N_runtime`): with N known every branch on it folds.
-template <int M, int NC>
-__device__ __forceinline__ void compress_fast_emit(const uint32_t (&r)[M / 2], int in, int N_runtime,
-                                                   uint16_t* __restrict__ vals, uint32_t* __restrict__ idx,
-                                                   int o, int seg,
-                                                   uint32_t (*words)[kMaxIndexWordsPerSegment],
-                                                   const CompactEntry* table)
+// Keep mask of a group of 16 (words of two positions), N <= 8.  The even and the odd positions' magnitudes are sorted side
+// by side, two to an instruction; the N-th largest of the two sorted lists A, B is the largest of the minima of A's i-th
+// and B's (N - i)-th.  What exceeds it is kept, and of what equals it the lowest positions that are still needed.  (768 x
+// 768 at 2:16 1.8 us against 5.8 by ranks; groups of 8 and 4 are 5 to 20 % quicker by keep_mask_sorted.)
+template <int N>
+__device__ __forceinline__ uint32_t keep_mask16(const uint32_t (&a)[8])
 {
-    static_assert(M == 4 || M == 8, "fast path for groups of 4 and 8");
-    constexpr int B = (M == 4) ? 2 : 3;
-    constexpr int R = M / 2;
-    const int N = NC ? NC : N_runtime;
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int groups_per_row = in / M;
-    const int g = seg * 32 + lane;
-    const bool valid = g < groups_per_row;
-    const int words_per_row = (N == M) ? 0 : (groups_per_row * N * B + 31) / 32;
-    const int seg_words = N * B;
-
-    uint16_t* dst = vals + (size_t)o * ((size_t)groups_per_row * N) + (size_t)g * N;
-    if (N == M) {                                 // dense level: the values are the weight
-        if (valid) {
-            if constexpr (M == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(r[0], r[1]);
-            else *reinterpret_cast<uint4*>(dst) = make_uint4(r[0], r[1], r[2], r[3]);
-        }
-        return;
+    static_assert(N >= 1 && N <= 8, "candidates from two lists of eight");
+    uint32_t k[8], s[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s[q] = k[q] = a[q] & 0x7FFF7FFFu;
+    auto sort2 = [&](int x, int y) {
+        const uint32_t hi = __vmaxu2(s[x], s[y]), lo = __vminu2(s[x], s[y]);
+        s[x] = hi; s[y] = lo;
+    };
+    sort2(0, 1); sort2(2, 3); sort2(4, 5); sort2(6, 7);
+    sort2(0, 2); sort2(1, 3); sort2(4, 6); sort2(5, 7);
+    sort2(1, 2); sort2(5, 6);
+    sort2(0, 4); sort2(1, 5); sort2(2, 6); sort2(3, 7);
+    sort2(2, 4); sort2(3, 5);
+    sort2(1, 2); sort2(3, 4); sort2(5, 6);
+    uint32_t thr = 0;
+#pragma unroll
+    for (int i = 0; i <= N; ++i) {       // i of A and N - i of B lie at or above the candidate
+        const uint32_t x = i > 0 ? s[i > 0 ? i - 1 : 0] & 0xFFFFu : 0xFFFFu, y = i < N ? s[i < N ? N - i - 1 : 0] >> 16 : 0xFFFFu;
+        thr = max(thr, min(x, y));
     }
-    for (int k = lane; k < seg_words; k += 32) words[warp][k] = 0;
-    __syncwarp();
-    if (valid) {
-        uint32_t h[M];
+    const uint32_t thr2 = thr | (thr << 16);
+    uint32_t above = 0, least = 0;       // magnitudes > thr, >= thr (15-bit values: a borrow clears the half's top bit)
 #pragma unroll
-        for (int q = 0; q < R; ++q) { h[2 * q] = r[q] & 0xFFFFu; h[2 * q + 1] = r[q] >> 16; }
-        const uint32_t keep = keep_mask_sorted<M>(h, N);
-        const CompactEntry e = table[keep];
-        // low and high bytes of the halfwords as two planes, compacted by the position list, re-interleaved
-        uint32_t w[R];
-        if constexpr (M == 4) {
-            const uint32_t lo = prmt(prmt(r[0], r[1], 0x6420u), 0u, e.order4);
-            const uint32_t hi = prmt(prmt(r[0], r[1], 0x7531u), 0u, e.order4);
-            w[0] = prmt(lo, hi, 0x5140u);
-            w[1] = prmt(lo, hi, 0x7362u);
-        } else {
-            const uint32_t l0 = prmt(r[0], r[1], 0x6420u), l1 = prmt(r[2], r[3], 0x6420u);
-            const uint32_t h0 = prmt(r[0], r[1], 0x7531u), h1 = prmt(r[2], r[3], 0x7531u);
-            const uint32_t lo03 = prmt(l0, l1, e.order4 & 0xFFFFu), lo47 = prmt(l0, l1, e.order4 >> 16);
-            const uint32_t hi03 = prmt(h0, h1, e.order4 & 0xFFFFu), hi47 = prmt(h0, h1, e.order4 >> 16);
-            w[0] = prmt(lo03, hi03, 0x5140u);
-            w[1] = prmt(lo03, hi03, 0x7362u);
-            w[2] = prmt(lo47, hi47, 0x5140u);
-            w[3] = prmt(lo47, hi47, 0x7362u);
-        }
-        // the group's N values are contiguous: the widest store their common alignment allows
-        if ((N & 3) == 0) {
-            *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);          // N = 4 (M = 8)
-        } else if ((N & 1) == 0) {
-#pragma unroll
-            for (int q = 0; q < R; ++q)
-                if (q < (N >> 1)) reinterpret_cast<uint32_t*>(dst)[q] = w[q];
-        } else {
-#pragma unroll
-            for (int t = 0; t < M; ++t)
-                if (t < N) dst[t] = (uint16_t)(w[t >> 1] >> (16 * (t & 1)));
-        }
-        // index bits: at most 21 (M = 8) or 6 (M = 4) bits at bit offset lane * N * B of the segment
-        const int bit0 = lane * seg_words;
-        const int w0 = bit0 >> 5, sh = bit0 & 31;
-        const uint32_t lo = e.fields << sh;
-        const uint32_t hi = sh ? (e.fields >> (32 - sh)) : 0u;
-        if (lo) atomicOr(&words[warp][w0], lo);
-        if (hi) atomicOr(&words[warp][w0 + 1], hi);
+    for (int q = 0; q < 8; ++q) {
+        const uint32_t g = ~((thr2 | 0x80008000u) - k[q]) & 0x80008000u, e = ((k[q] | 0x80008000u) - thr2) & 0x80008000u;
+        above |= (((g >> 15) | (g >> 30)) & 3u) << (2 * q);
+        least |= (((e >> 15) | (e >> 30)) & 3u) << (2 * q);
     }
-    __syncwarp();
-    const int first = seg * seg_words;
-    uint32_t* row = idx + (size_t)o * words_per_row;
-    for (int k = lane; k < seg_words && first + k < words_per_row; k += 32) row[first + k] = words[warp][k];
-    __syncwarp();
-}
-
-template <int M, int NC = 0>
-__device__ __forceinline__ void compress_segment_fast(const uint16_t* __restrict__ W, int in, int N,
-                                                      uint16_t* __restrict__ vals, uint32_t* __restrict__ idx,
-                                                      int segs_per_row, long long seg_id,
-                                                      uint32_t (*words)[kMaxIndexWordsPerSegment],
-                                                      const CompactEntry* table)
-{
-    // a weight has far fewer than 2^32 segments: 32-bit division
-    const uint32_t o = (uint32_t)seg_id / (uint32_t)segs_per_row;
-    const uint32_t seg = (uint32_t)seg_id - o * (uint32_t)segs_per_row;
-    uint32_t r[M / 2];
-    compress_fast_load<M>(W, in, (int)o, (int)seg, r);
-    compress_fast_emit<M, NC>(r, in, N, vals, idx, (int)o, (int)seg, words, table);
-}
-
-// The same with the 16 bytes of the group already in registers (requested one unit ahead by the caller).
-template <int M, int NC = 0>
-__device__ __forceinline__ void compress_segment_fast_preloaded(const uint32_t (&r4)[4], int in, int N,
-                                                                uint16_t* __restrict__ vals, uint32_t* __restrict__ idx,
-                                                                int o, int seg, uint32_t (*words)[kMaxIndexWordsPerSegment],
-                                                                const CompactEntry* table)
-{
-    uint32_t r[M / 2];
-#pragma unroll
-    for (int q = 0; q < M / 2; ++q) r[q] = r4[q];
-    compress_fast_emit<M, NC>(r, in, N, vals, idx, o, seg, words, table);
-}
-
-// Single level: the form elsa_nm_compress uses.
-template <int M>
-__device__ __forceinline__ void compress_segment(const uint16_t* __restrict__ W, int in, int N,
-                                                 uint16_t* __restrict__ vals, uint32_t* __restrict__ idx,
-                                                 int segs_per_row, int words_per_row, long long seg_id,
-                                                 uint32_t (*words)[kMaxIndexWordsPerSegment])
-{
-    (void)words_per_row;
-    uint16_t* vals_one = vals;
-    uint32_t* idx_one = idx;
-    compress_segment_levels<M>(W, in, 1, &N, &vals_one, &idx_one, segs_per_row, seg_id, words);
+    uint32_t equal = least & ~above;
+    int need = N - __popc(above);
+    if (__popc(equal) == need) return least;
+    uint32_t keep = above;
+    for (; need > 0; --need) {
+        keep |= equal & (0u - equal);
+        equal &= equal - 1u;
+    }
+    return keep;
 }
 
 // ---- eight consecutive positions of a packed row as one 16-byte unit (groups of 4: two groups, groups of 8: one),

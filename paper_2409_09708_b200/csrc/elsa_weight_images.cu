@@ -102,14 +102,6 @@ __device__ __forceinline__ Segment load_segment(const uint16_t* __restrict__ val
     return s;
 }
 
-// Value at a position of a group of 8 given as four words.
-__device__ __forceinline__ uint32_t half_at(const uint32_t (&a)[4], uint32_t pos)
-{
-    const uint32_t lo = pos & 2u ? a[1] : a[0], hi = pos & 2u ? a[3] : a[2];
-    const uint32_t w = pos & 4u ? hi : lo;
-    return (pos & 1u ? w >> 16 : w) & 0xFFFFu;
-}
-
 // The same from 16 dense positions (words a[8]), projected onto level N:M (the N of largest magnitude, lowest position
 // first among equals).
 template <int M, int N>
@@ -120,42 +112,39 @@ __device__ __forceinline__ Segment pick_segment(const uint4& x, const uint4& y)
     s.v[0] = s.v[1] = s.v[2] = s.v[3] = 0u;
     s.fields = 0;
     if constexpr (M == 16) {
-        uint16_t h[16];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) { h[2 * q] = (uint16_t)(a[q] & 0xFFFFu); h[2 * q + 1] = (uint16_t)(a[q] >> 16); }
-        const uint32_t keep = keep_mask<16>(group_ranks<16>(h), N);
+        const uint32_t keep = keep_mask16<N>(a);
         const uint32_t p0 = (uint32_t)__ffs((int)keep) - 1u, p1 = 31u - (uint32_t)__clz((int)keep);
-        const uint32_t lo[4] = {a[0], a[1], a[2], a[3]}, hi[4] = {a[4], a[5], a[6], a[7]};
-        s.v[0] = half_at(p0 & 8u ? hi : lo, p0 & 7u);
+        s.v[0] = half_of(a, p0);
         s.fields = p0;
         if constexpr (N == 2) {
-            s.v[0] |= half_at(p1 & 8u ? hi : lo, p1 & 7u) << 16;
+            s.v[0] |= half_of(a, p1) << 16;
             s.fields |= p1 << 4;
         }
     } else if constexpr (M == 8) {
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
-            uint32_t h[8], w[4];
+            const uint32_t w[4] = {a[4 * g], a[4 * g + 1], a[4 * g + 2], a[4 * g + 3]};
+            uint32_t h[8];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) { w[q] = a[4 * g + q]; h[2 * q] = w[q] & 0xFFFFu; h[2 * q + 1] = w[q] >> 16; }
+            for (int i = 0; i < 8; ++i) h[i] = (w[i >> 1] >> (16 * (i & 1))) & 0xFFFFu;
             const uint32_t keep = keep_mask_sorted<8>(h, N);
             const uint32_t p0 = (uint32_t)__ffs((int)keep) - 1u, p1 = 31u - (uint32_t)__clz((int)keep);
             if constexpr (N == 1) {
-                s.v[0] |= half_at(w, p0) << (16 * g);
+                s.v[0] |= half_of(w, p0) << (16 * g);
                 s.fields |= p0 << (3 * g);
             } else {
-                s.v[g] = half_at(w, p0) | (half_at(w, p1) << 16);
+                s.v[g] = half_of(w, p0) | (half_of(w, p1) << 16);
                 s.fields |= (p0 | (p1 << 3)) << (6 * g);
             }
         }
     } else {
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
-            uint32_t h[4] = {a[2 * g] & 0xFFFFu, a[2 * g] >> 16, a[2 * g + 1] & 0xFFFFu, a[2 * g + 1] >> 16};
+            const uint32_t w[2] = {a[2 * g], a[2 * g + 1]};
+            const uint32_t h[4] = {w[0] & 0xFFFFu, w[0] >> 16, w[1] & 0xFFFFu, w[1] >> 16};
             const uint32_t keep = keep_mask_sorted<4>(h, N);
             const uint32_t p0 = (uint32_t)__ffs((int)keep) - 1u, p1 = 31u - (uint32_t)__clz((int)keep);
-            const uint32_t w0 = p0 & 2u ? a[2 * g + 1] : a[2 * g], w1 = p1 & 2u ? a[2 * g + 1] : a[2 * g];
-            const uint32_t v0 = (p0 & 1u ? w0 >> 16 : w0) & 0xFFFFu, v1 = (p1 & 1u ? w1 >> 16 : w1) & 0xFFFFu;
+            const uint32_t v0 = half_of(w, p0), v1 = half_of(w, p1);
             if constexpr (N == 1) {
                 s.v[g >> 1] |= v0 << (16 * (g & 1));
                 s.fields |= p0 << (2 * g);
@@ -284,7 +273,7 @@ int image_blocks(const ImageJob& j)
 }
 
 template <int kMax>
-__global__ void __launch_bounds__(kImageThreads) weight_image_kernel(const __grid_constant__ ImageTable<kMax> t)
+__global__ void __launch_bounds__(kImageThreads, 4) weight_image_kernel(const __grid_constant__ ImageTable<kMax> t)
 {
     pdl_wait_for_predecessors();
     pdl_release_successors();

@@ -57,3 +57,21 @@ def test_unpack_around_a_block_of_units(lib, level):
         vals, idx = lib.elsa_nm_compress(W.cuda(), N, M)
         got = lib.elsa_nm_unpack(vals, idx, out, in_, N, M)
         assert np.array_equal(got.double().cpu().numpy(), masked(W, N, M)), (out, in_)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16], ids=["f16", "bf16"])
+def test_ties_of_many_kinds_compress_as_the_oracle(lib, dtype):
+    """Few distinct magnitudes, so most groups have ties around the threshold: every level, rows whose index bits do and do
+    not fill whole words, one segment per warp and four."""
+    rng = np.random.default_rng(11)
+    for out, in_ in [(8, 48), (24, 16 * 23), (2400, 1024)]:
+        W = torch.from_numpy(rng.integers(-3, 4, (out, in_)).astype(np.float32)).to(dtype)
+        Wd, Wb = W.cuda(), synth.bits(W)
+        for M in (4, 8, 16):
+            levels = [n for n in (1, 2, 3, 4, 5, 8, 11) if n <= M]
+            for N, (vals, idx) in zip(levels, lib.elsa_nm_compress_levels(Wd, levels, M)):
+                ovals, oidx, _ = eo.nm_compress(Wb, N, M)
+                assert (synth.bits(vals) == ovals).all(), (out, in_, N, M)
+                if N < M:
+                    assert (idx.cpu().numpy().view(np.uint32) == oidx).all(), (out, in_, N, M)
