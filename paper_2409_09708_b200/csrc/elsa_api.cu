@@ -300,10 +300,17 @@ elsa_status pick_kind(LinearUse use, int rows, int out, int in, int N, int M, in
     // More than a wave of small tiles.  Below K = 512 the sparse kernels do not beat the pair kernel until the
     // weight-stationary one does (384 -> 384, 6304 rows: 8.2 against 8.8); from there up the sparse pair kernel leads,
     // and from about 5M outputs the streaming one (3072 -> 768: 6304 rows 24.5 against 25.0, 12608 rows 38.7 against 36.6).
-    // Only the streaming and weight-stationary ones take GELU in their epilogue.
+    // With GELU the epilogue weighs more: the weight-stationary kernel leads where an SM pair's rows times K pass 390000
+    // (768 -> 3072, 3152 rows 16.8 against 17.0 on the pair kernel, 4925 rows 20.9 against 24.3; 384 -> 1536, 12608 rows
+    // 19.9 against 21.7), the pair kernel below; the streaming one is slower than either up to K = 1024.
+    if (gelu) {
+        const bool ws = ws_ok && (long long)rows * tiles_f * (in < 768 ? in : 768) >= 390000LL * pairs;
+        *kind = ws ? KIND_SPARSE_WS : in > 1024 && st_ok && (long long)rows * out >= 5000000LL ? KIND_SPARSE_ST : KIND_DENSE_PAIR;
+        return ELSA_OK;
+    }
     if (ws_large) *kind = KIND_SPARSE_WS;
-    else if (sparse_ok && in >= 512 && st_ok && (gelu || (long long)rows * out >= 5000000LL)) *kind = KIND_SPARSE_ST;
-    else if (sparse_ok && in >= 512 && !gelu) *kind = KIND_SPARSE_PAIR;
+    else if (sparse_ok && in >= 512 && st_ok && (long long)rows * out >= 5000000LL) *kind = KIND_SPARSE_ST;
+    else if (sparse_ok && in >= 512) *kind = KIND_SPARSE_PAIR;
     else *kind = KIND_DENSE_PAIR;
     return ELSA_OK;
 }

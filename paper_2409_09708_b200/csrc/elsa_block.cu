@@ -4,10 +4,7 @@
 // column range.  All of them are HBM-bound streaming kernels: 16-byte loads and stores, fp32 arithmetic, one
 // rounding to the 16-bit type per stored value; the row-wise ones give a row to a warp, or, for the model widths
 // (128, 256, 512, 768, 1024), several rows at a time to groups of 16 or 32 lanes.
-#include "elsa_internal.h"
-
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
+#include "elsa_tc_common.cuh"
 
 namespace elsa {
 namespace {
@@ -50,22 +47,6 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8])
 {
     return make_uint4(pack2_rn<kBf16>(f[0], f[1]), pack2_rn<kBf16>(f[2], f[3]), pack2_rn<kBf16>(f[4], f[5]),
                       pack2_rn<kBf16>(f[6], f[7]));
-}
-
-// v * Phi(v) = max(v, 0) - 0.5 |v| erfc(|v| / sqrt 2) with erfc as 2^Q(|v|), Q of degree 6: the form and the
-// coefficients of the GEMM epilogues (3e-7 absolute error in fp32).
-__device__ __forceinline__ float gelu_erf(float v)
-{
-    const float a = fminf(fabsf(v), 5.9375f);
-    float q = fmaf(a, 3.309303065e-05f, -7.692219224e-04f);
-    q = fmaf(q, a, 8.080724627e-03f);
-    q = fmaf(q, a, -5.341212079e-02f);
-    q = fmaf(q, a, -4.587709606e-01f);
-    q = fmaf(q, a, -1.151201725e+00f);
-    q = fmaf(q, a, 6.939759714e-06f);
-    float e;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(q));
-    return fmaf(-0.5f * fabsf(v), e, fmaxf(v, 0.0f));
 }
 
 __device__ __forceinline__ float warp_sum(float v)
@@ -311,9 +292,14 @@ __global__ void __launch_bounds__(256) act_inplace_kernel(uint16_t* Y, long long
     for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < vecs; v += (long long)gridDim.x * blockDim.x) {
         float f[8];
         unpack8<kBf16>(y4[v], f);
+        if (act == 1) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e)
-            f[e] = act == 1 ? gelu_erf(f[e]) : f[e];
+            for (int e = 0; e < 8; e += 2) {
+                const float2 g = gelu_pair(f[e], f[e + 1]);
+                f[e] = g.x;
+                f[e + 1] = g.y;
+            }
+        }
         y4[v] = pack8<kBf16>(f);
     }
 }

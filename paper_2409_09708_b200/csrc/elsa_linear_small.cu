@@ -348,7 +348,11 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
                 for (int i = 0; i < 4; ++i) {
                     const float2 bv = raw2_to_float2<kBf16>(b[i]), rv = raw2_to_float2<kBf16>(r[i]);
                     float x = a[2 * i] + bv.x, y = a[2 * i + 1] + bv.y;
-                    if (L.act == 1) { x = gelu_exact(x); y = gelu_exact(y); }
+                    if (L.act == 1) {
+                        const float2 g = gelu_pair(x, y);
+                        x = g.x;
+                        y = g.y;
+                    }
                     o[i] = pack2<kBf16>(x + rv.x, y + rv.y);
                 }
                 *reinterpret_cast<uint4*>(L.Y + (size_t)row * L.out + col) = make_uint4(o[0], o[1], o[2], o[3]);

@@ -8,14 +8,15 @@
 // only half of the W rows, and one tcgen05.mma.cta_group::2 (M = 256) issued by the leader CTA
 // drives both tensor cores, so each SM moves 2/3 of the bytes per MMA.
 //
-// Per CTA (352 threads):
+// Per CTA (352 threads; 608 in the form with GELU or a residual):
 //   warp 0      TMA producer for this CTA's operand halves; completion bytes of both CTAs are
 //               credited to the leader's stage barrier
 //   warp 1      allocates tensor memory (pair-wide); in the leader one lane issues the MMAs and
 //               commits, by multicast, onto both CTAs' stage and accumulator barriers
 //   warps 2-9   epilogue, two warps per TMEM lane quarter (alternating 32-column chunks):
 //               tcgen05.ld of all the warp's chunks, accumulator released, then + bias in fp32,
-//               round to 16 bit, swizzled staging, TMA store
+//               round to 16 bit, swizzled staging, TMA store (four warps per quarter, chunk by chunk,
+//               in the form with GELU or a residual)
 //   warp 10     bias loader: copies the next tile's bias into one of two shared buffers, so the
 //               epilogue warps issue no global loads of their own
 // Two TMEM accumulators let the MMAs of tile i+1 overlap the epilogue of tile i.  Every wait is
@@ -41,19 +42,12 @@ constexpr int kMaxBlockN = 256;
 constexpr int kNumAccum = 2;
 constexpr int kTmemCols = kNumAccum * kMaxBlockN;
 constexpr int kMaxStages = 8;
-constexpr int kEpiWarps = 8;
-constexpr int kEpiParts = kEpiWarps / 4;   // warps per TMEM lane quarter; they share the quarter's chunks
-constexpr int kBiasWarp = 2 + kEpiWarps;
-constexpr int kThreads = (kBiasWarp + 1) * 32;
 constexpr int kEpiCols = 32;
-constexpr int kMaxChunksPerWarp = kMaxBlockN / kEpiCols / kEpiParts;
 constexpr int kATileBytes = kRowsPerCta * kBlockK * 2;
 constexpr int kStagingBytes = 32 * kEpiCols * 2;
-constexpr int kStagingBufs = 1;     // one staging buffer per epilogue warp: the shared memory goes to a sixth pipeline stage instead
-constexpr int kStagingTotal = kEpiWarps * kStagingBufs * kStagingBytes;
 constexpr int kBiasBytes = 2 * kMaxBlockN * 2;   // two tiles' bias as stored (16 bit)
 constexpr int kScaleBytes = 2 * kMaxBlockN * 4;  // INT8 form: two tiles' combined scales (fp32)
-constexpr int kBarrierBytes = 256;
+constexpr int kBarrierBytes = 384;
 
 // One layer of a launch.  A launch may carry several layers (a group): the persistent CTA pairs walk the
 // tiles of all of them in one sequence, so the tail of one layer overlaps the head of the next and
@@ -70,11 +64,11 @@ struct alignas(64) PairLayer {
     const float* w_scale;   // INT8 form only: per-feature weight scale, and the activations' scale
     float x_scale;
     int act;                    // epilogue activation (0 none, 1 GELU) on acc + bias
-    const uint16_t* residual;   // [rows][out] added after the activation, or NULL
+    int has_residual;           // [rows][out] added after the activation (PairGroup::map_r)
 };
 
 template <int kMaxLayers>
-struct PairGroup {
+struct alignas(64) PairGroup {
     PairLayer layer[kMaxLayers];
     int n_layers;
     int num_tiles;     // over all layers
@@ -84,6 +78,7 @@ struct PairGroup {
     // tile t / splits over range t % splits, and each range's fp32 sums go to partial[range][rows][out].
     int splits;
     float* partial;
+    CUtensorMap map_r;   // fused form: the residual, boxes as map_y's
 };
 
 constexpr int kStageBytesMax = kATileBytes + (kMaxBlockN / 2) * kBlockK * 2;   // stage slots sized for BN = 256
@@ -93,6 +88,23 @@ constexpr int kStageBytesMax = kATileBytes + (kMaxBlockN / 2) * kBlockK * 2;   /
 // MMA reads them through MN-major descriptors). Separate instantiations, so the plain form pays nothing for the
 // others.
 constexpr int kFormPlain = 0, kFormInt8 = 1, kFormFused = 2, kFormTn = 3;
+
+// The epilogue's share of a CTA.  GELU and a residual make the epilogue the longer part of a tile unless four warps per
+// scheduler work on it, 32 columns at a time in 96 registers (8 warps that hold 128 columns each have 40 registers left
+// for the arithmetic of all of them: 50432 x 768 -> 3072 with GELU 223 us there, 183 here, 160 without GELU), each with
+// a buffer for every chunk it has of a tile, so that the residual can be brought in by TMA while the tile is multiplied
+// (read by the lanes row by row as it was needed it took 309 us, 206 here; 50432 x 768 -> 768 86 and 57).
+template <int kForm>
+struct PairShape {
+    static constexpr int kEpiWarps = kForm == kFormFused ? 16 : 8;
+    static constexpr int kEpiParts = kEpiWarps / 4;   // warps per TMEM lane quarter; they share the quarter's chunks
+    static constexpr int kBiasWarp = 2 + kEpiWarps;
+    static constexpr int kThreads = (kBiasWarp + 1) * 32;
+    static constexpr int kMaxChunksPerWarp = kMaxBlockN / kEpiCols / kEpiParts;
+    // elsewhere one buffer per epilogue warp: the shared memory goes to a sixth pipeline stage instead
+    static constexpr int kStagingBufs = kForm == kFormFused ? kMaxChunksPerWarp : 1;
+    static constexpr int kStagingTotal = kEpiWarps * kStagingBufs * kStagingBytes;
+};
 constexpr int kTnBoxBytes = 64 * 64 * 2;   // one box of the Tn form: 64 reduction rows of 128 bytes
 constexpr int kGroupMax = 72;   // layers per grouped launch (kernel parameters are limited to 32 KB)
 
@@ -100,12 +112,15 @@ constexpr int kGroupMax = 72;   // layers per grouped launch (kernel parameters 
 // int32 accumulators); the epilogue turns an accumulator into float, multiplies by x_scale * w_scale[feature],
 // adds the bias, each in fp32 with one rounding per operation, and rounds once to the 16-bit output type.
 template <bool kBf16, int kForm, int kMaxLayers>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(PairShape<kForm>::kThreads, 1)
 linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
 {
     constexpr bool kInt8 = kForm == kFormInt8;     // 8-bit integer operands, scales in the epilogue
     constexpr bool kFused = kForm == kFormFused;   // activation and residual in the epilogue
     constexpr bool kTn = kForm == kFormTn;         // operands [K][M] and [K][N]
+    using Shape = PairShape<kForm>;
+    constexpr int kEpiWarps = Shape::kEpiWarps, kEpiParts = Shape::kEpiParts, kBiasWarp = Shape::kBiasWarp;
+    constexpr int kMaxChunksPerWarp = Shape::kMaxChunksPerWarp, kStagingBufs = Shape::kStagingBufs, kStagingTotal = Shape::kStagingTotal;
 
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -128,7 +143,8 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
     const uint32_t tmem_empty_bar = tmem_full_bar + 8 * kNumAccum;             // used in the leader only
     const uint32_t bias_full_bar = tmem_empty_bar + 8 * kNumAccum;             // per CTA
     const uint32_t bias_empty_bar = bias_full_bar + 16;                        // per CTA
-    const uint32_t holder_off = scale_off + kScaleBytes + 16 * kMaxStages + 16 * kNumAccum + 32;
+    const uint32_t res_bar = bias_empty_bar + 16;                              // fused form, one per epilogue warp
+    const uint32_t holder_off = scale_off + kScaleBytes + 16 * kMaxStages + 16 * kNumAccum + 32 + (kFused ? 8 * kEpiWarps : 0);
     volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(smem_gen + holder_off);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem_gen + holder_off + 4);
 
@@ -145,6 +161,8 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
             mbar_init(bias_full_bar + 8 * b, 1);
             mbar_init(bias_empty_bar + 8 * b, kEpiWarps);
         }
+        if constexpr (kFused)
+            for (int w = 0; w < kEpiWarps; ++w) mbar_init(res_bar + 8 * w, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
@@ -313,7 +331,8 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
         const uint32_t empty_remote = mapa_shared(tmem_empty_bar, 0);
         int acc = 0;
         uint32_t acc_phase = 0;
-        uint32_t chunk_counter = 0;
+        uint32_t res_phase = 0;
+        (void)res_phase;
         int cur = 0;
         uint32_t it = 0;
 
@@ -337,9 +356,22 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
             const uint32_t scale_cur = smem_base + scale_off + bias_b * (kMaxBlockN * 4);
             (void)scale_cur;
             const int l_act = kFused ? L.act : 0;
-            const uint16_t* l_res = kFused ? L.residual : nullptr;
+            const bool l_res = kFused && L.has_residual != 0;
             (void)l_act;
             (void)l_res;
+            if constexpr (kFused) {
+                // the buffers are free once the last tile's stores have read them; the residual arrives under the MMAs
+                if (lane == 0) {
+                    bulk_wait_group_read<0>();
+                    if (l_res) {
+                        mbar_arrive_expect_tx(res_bar + 8 * ew, (uint32_t)(my_chunks * kStagingBytes));
+                        for (int i = 0; i < my_chunks; ++i)
+                            tma_load_2d(stage_buf + (uint32_t)(i * kStagingBytes), &p.map_r, res_bar + 8 * ew,
+                                        n0 + (part + kEpiParts * i) * kEpiCols, m0 + q * 32);
+                    }
+                }
+                __syncwarp();
+            }
             bool ok = mbar_wait(bias_full_bar + 8 * bias_b, (it >> 1) & 1u, abort_flag, p.dev_status, 6);
             ok = ok && mbar_wait(tmem_full_bar + 8 * acc, acc_phase, abort_flag, p.dev_status, 4);
             ok = __all_sync(0xFFFFFFFFu, ok);
@@ -348,8 +380,9 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
             const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kMaxBlockN);
             const int row0 = m0 + q * 32;
 
-            // converts, stages and stores one 32 x 32 chunk
-            auto emit = [&](const uint32_t (&r)[32], int c) {
+            // converts, stages and stores one 32 x 32 chunk (the warp's i-th)
+            auto emit = [&](const uint32_t (&r)[32], int c, int i) {
+                (void)i;
                 if constexpr (kTn) {
                     if (p.partial != nullptr) {
                         // a range's fp32 sums as they are: this lane's row, 32 consecutive columns
@@ -365,6 +398,9 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                         return;
                     }
                 }
+                const uint32_t buf = stage_buf + (uint32_t)(kStagingBufs > 1 ? i * kStagingBytes : 0);
+                const uint32_t row_addr = buf + (uint32_t)(lane * 64);
+                const uint32_t sw = (uint32_t)((lane >> 1) & 3);   // 64-byte swizzle of the staging rows
                 // 16 columns: + bias (read as stored, eight values per load), rounded to 16 bit
                 auto convert16 = [&](auto with_act, int h, uint32_t (&pk)[8]) {
 #pragma unroll
@@ -372,17 +408,12 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                         uint32_t bw[4];
                         asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(bw[0]), "=r"(bw[1]), "=r"(bw[2]), "=r"(bw[3])
                                      : "r"(bias_cur + (uint32_t)(c * kEpiCols * 2 + (2 * h + g) * 16)));
-                        // this lane's row of the residual, eight values (a whole load lies inside or outside the row)
+                        // this lane's row of the residual, where its result will be
                         uint32_t res[4] = {0u, 0u, 0u, 0u};
                         if constexpr (kFused) {
-                            if (l_res != nullptr) {
-                                const int row = row0 + lane;
-                                const int col = n0 + c * kEpiCols + (2 * h + g) * 8;
-                                if (row < l_rows && col < l_out) {
-                                    const uint4 u = __ldg(reinterpret_cast<const uint4*>(l_res + (size_t)row * (size_t)l_out + col));
-                                    res[0] = u.x; res[1] = u.y; res[2] = u.z; res[3] = u.w;
-                                }
-                            }
+                            if (l_res)
+                                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(res[0]), "=r"(res[1]), "=r"(res[2]), "=r"(res[3])
+                                             : "r"(row_addr + (((uint32_t)(2 * h + g) ^ sw) << 4)));
                         }
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
@@ -396,31 +427,26 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                                 const float vy = __fadd_rn(__fmul_rn((float)(int)r[2 * j + 1], sy), bv.y);
                                 pk[4 * g + e] = pack2<kBf16>(vx, vy);
                             } else {
-                                float vx = __uint_as_float(r[2 * j]) + bv.x;
-                                float vy = __uint_as_float(r[2 * j + 1]) + bv.y;
+                                float2 v = f32x2_split(f32x2_add(f32x2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1])), f32x2(bv.x, bv.y)));
                                 if constexpr (kFused) {
                                     const float2 rv = raw2_to_float2<kBf16>(res[e]);   // zeros without a residual
-                                    if constexpr (decltype(with_act)::value) {
-                                        vx = gelu_exact(vx);
-                                        vy = gelu_exact(vy);
-                                    }
-                                    vx += rv.x;
-                                    vy += rv.y;
+                                    if constexpr (decltype(with_act)::value) v = gelu_pair(v.x, v.y);
+                                    v.x += rv.x;
+                                    v.y += rv.y;
                                 }
-                                pk[4 * g + e] = pack2<kBf16>(vx, vy);
+                                pk[4 * g + e] = pack2<kBf16>(v.x, v.y);
                             }
                         }
                     }
                 };
-                const uint32_t buf = stage_buf + (chunk_counter % kStagingBufs) * kStagingBytes;
-                const uint32_t row_addr = buf + (uint32_t)(lane * 64);
-                const uint32_t sw = (uint32_t)((lane >> 1) & 3);   // 64-byte swizzle of the staging rows
                 uint32_t pk[8];
                 // the activation is a warp-uniform property of the layer: one branch per chunk, none per value
                 if (kFused && l_act == 1) convert16(std::true_type{}, 0, pk);
                 else convert16(std::false_type{}, 0, pk);
-                if (lane == 0) bulk_wait_group_read<kStagingBufs - 1>();   // the store that last used this buffer has drained it
-                __syncwarp();
+                if constexpr (!kFused) {
+                    if (lane == 0) bulk_wait_group_read<kStagingBufs - 1>();   // the store that last used this buffer has drained it
+                    __syncwarp();
+                }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     if (h == 1) {
@@ -441,7 +467,6 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                     if (row0 < l_rows && col0 < l_out) tma_store_2d(&L.map_y, buf, col0, row0);
                     bulk_commit_group();
                 }
-                ++chunk_counter;
             };
             // hands the accumulator back once this warp's last load of it has completed
             auto release = [&]() {
@@ -450,18 +475,37 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                 if (lane == 0) mbar_arrive_cluster(empty_remote + 8 * acc);
             };
 
-            // All of this warp's chunks are requested at once and the accumulator is handed back as soon
-            // as they have arrived: a tensor-memory load queues behind the MMAs already issued, so
-            // loads taken one at a time would each pay that wait.
-            uint32_t r[kMaxChunksPerWarp][32];
+            if constexpr (kFused) {
+                if (l_res) {
+                    ok = mbar_wait(res_bar + 8 * ew, res_phase, abort_flag, p.dev_status, 7);
+                    ok = __all_sync(0xFFFFFFFFu, ok);
+                    if (!ok) break;
+                    res_phase ^= 1u;
+                }
 #pragma unroll
-            for (int i = 0; i < kMaxChunksPerWarp; ++i)
-                if (i < my_chunks) tmem_ld_32x32b_x32(t_row + (uint32_t)((part + kEpiParts * i) * kEpiCols), r[i]);
-            tmem_wait_ld();
-            release();
+                for (int i = 0; i < kMaxChunksPerWarp; ++i) {
+                    if (i >= my_chunks) break;
+                    uint32_t r[32];
+                    tmem_ld_32x32b_x32(t_row + (uint32_t)((part + kEpiParts * i) * kEpiCols), r);
+                    tmem_wait_ld();
+                    if (i == my_chunks - 1) release();
+                    emit(r, part + kEpiParts * i, i);
+                }
+                if (my_chunks == 0) release();
+            } else {
+                // All of this warp's chunks are requested at once and the accumulator is handed back as soon
+                // as they have arrived: a tensor-memory load queues behind the MMAs already issued, so
+                // loads taken one at a time would each pay that wait.
+                uint32_t r[kMaxChunksPerWarp][32];
 #pragma unroll
-            for (int i = 0; i < kMaxChunksPerWarp; ++i)
-                if (i < my_chunks) emit(r[i], part + kEpiParts * i);
+                for (int i = 0; i < kMaxChunksPerWarp; ++i)
+                    if (i < my_chunks) tmem_ld_32x32b_x32(t_row + (uint32_t)((part + kEpiParts * i) * kEpiCols), r[i]);
+                tmem_wait_ld();
+                release();
+#pragma unroll
+                for (int i = 0; i < kMaxChunksPerWarp; ++i)
+                    if (i < my_chunks) emit(r[i], part + kEpiParts * i, i);
+            }
             // this warp has read the tile's bias for the last time
             __syncwarp();
             if (lane == 0) mbar_arrive(bias_empty_bar + 8 * bias_b);
@@ -526,6 +570,7 @@ elsa_status launch_group(const PairJob* jobs, int n, elsa_dtype dtype, uint32_t*
                          const DeviceInfo& dev)
 {
     constexpr bool kInt8 = kForm == kFormInt8;
+    constexpr int kThreads = PairShape<kForm>::kThreads, kStagingTotal = PairShape<kForm>::kStagingTotal;
     static PairGroup<kMaxLayers> g;   // host staging of the kernel parameters (single-threaded launch path)
     static std::mutex g_mutex;
     std::lock_guard<std::mutex> lock(g_mutex);
@@ -543,7 +588,7 @@ elsa_status launch_group(const PairJob* jobs, int n, elsa_dtype dtype, uint32_t*
         L.w_scale = j.w_scale;
         L.x_scale = j.x_scale;
         L.act = j.act;
-        L.residual = j.residual;
+        L.has_residual = j.residual != nullptr;
         elsa_status st;
         if constexpr (kInt8) {
             L.num_k_blocks = (j.in + 2 * kBlockK - 1) / (2 * kBlockK);
@@ -579,6 +624,11 @@ elsa_status launch_group(const PairJob* jobs, int n, elsa_dtype dtype, uint32_t*
         if ((st = make_map_2d(&L.map_y, j.Y, (uint64_t)j.out, (uint64_t)j.rows, kEpiCols, 32, CU_TENSOR_MAP_SWIZZLE_64B,
                               "Y")) != ELSA_OK)
             return st;
+    }
+    if (kForm == kFormFused && jobs[0].residual != nullptr) {
+        const elsa_status st = make_map_2d(&g.map_r, jobs[0].residual, (uint64_t)jobs[0].out, (uint64_t)jobs[0].rows, kEpiCols, 32,
+                                           CU_TENSOR_MAP_SWIZZLE_64B, "the residual");
+        if (st != ELSA_OK) return st;
     }
     g.n_layers = n;
     g.splits = kForm == kFormTn ? jobs[0].splits : 1;
@@ -645,11 +695,12 @@ elsa_status launch_linear_tc_pair_group(const PairJob* jobs, int n, elsa_dtype d
     bool fused = false;
     for (int i = 0; i < n; ++i) fused = fused || jobs[i].act != 0 || jobs[i].residual != nullptr;
     if (fused) {
-        if (n == 1)
-            return dtype == ELSA_BF16 ? launch_group<true, kFormFused, 1>(jobs, 1, dtype, dev_status, stream, dev)
-                                      : launch_group<false, kFormFused, 1>(jobs, 1, dtype, dev_status, stream, dev);
-        return dtype == ELSA_BF16 ? launch_group<true, kFormFused, kGroupMax>(jobs, n, dtype, dev_status, stream, dev)
-                                  : launch_group<false, kFormFused, kGroupMax>(jobs, n, dtype, dev_status, stream, dev);
+        for (int i = 0; i < n; ++i) {
+            st = dtype == ELSA_BF16 ? launch_group<true, kFormFused, 1>(jobs + i, 1, dtype, dev_status, stream, dev)
+                                    : launch_group<false, kFormFused, 1>(jobs + i, 1, dtype, dev_status, stream, dev);
+            if (st != ELSA_OK) return st;
+        }
+        return ELSA_OK;
     }
     if (n == 1)
         return dtype == ELSA_BF16 ? launch_group<true, kFormPlain, 1>(jobs, 1, dtype, dev_status, stream, dev)

@@ -340,6 +340,7 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
             const int f = f0 + feat_in_quarter;
             const int l_rows = L.rows, l_out = L.out;
             const float bias_f = (L.bias != nullptr && f < l_out) ? bias_to_float<kBf16>(__ldg(L.bias + f)) : 0.f;
+            const uint64_t bias2 = f32x2(bias_f, bias_f);
             const int l_act = kAct ? L.act : 0;
             (void)l_act;
             bool ok = mbar_wait(tmem_full_bar, acc_phase, abort_flag, p.dev_status, 4);
@@ -376,9 +377,7 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
                 for (int i = 0; i < kRoundSteps; ++i)
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        w[i][j] = kAct ? pack2<kBf16>(apply_act(__uint_as_float(rr[i][2 * j]) + bias_f, l_act),
-                                                      apply_act(__uint_as_float(rr[i][2 * j + 1]) + bias_f, l_act))
-                                       : pack2<kBf16>(__uint_as_float(rr[i][2 * j]) + bias_f, __uint_as_float(rr[i][2 * j + 1]) + bias_f);
+                        w[i][j] = finish_pair<kBf16, kAct>(rr[i][2 * j], rr[i][2 * j + 1], bias2, l_act);
                 if (rd + 1 < kRounds) {
 #pragma unroll
                     for (int i = 0; i < kRoundSteps; ++i)

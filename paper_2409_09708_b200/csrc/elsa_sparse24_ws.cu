@@ -322,6 +322,7 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
                 if (lane == 0) mbar_arrive_cluster_release(w_ready_remote);
             }
             const float bias_f = (L.bias != nullptr && f_ok) ? bias_to_float<kBf16>(__ldg(L.bias + f)) : 0.f;
+            const uint64_t bias2 = f32x2(bias_f, bias_f);
             const int l_act = kAct ? L.act : 0;
             (void)l_act;
             // this warp's run of token columns: steps of 16, [first_step, first_step + my_steps)
@@ -358,9 +359,7 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
                     uint32_t w[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        w[j] = kAct ? pack2<kBf16>(apply_act(__uint_as_float(rr[s][2 * j]) + bias_f, l_act),
-                                                   apply_act(__uint_as_float(rr[s][2 * j + 1]) + bias_f, l_act))
-                                    : pack2<kBf16>(__uint_as_float(rr[s][2 * j]) + bias_f, __uint_as_float(rr[s][2 * j + 1]) + bias_f);
+                        w[j] = finish_pair<kBf16, kAct>(rr[s][2 * j], rr[s][2 * j + 1], bias2, l_act);
                     stmatrix_x4_trans(st_addr + (uint32_t)(s * kStepCols * 64), w[0], w[1], w[2], w[3]);
                     stmatrix_x4_trans(st_addr + (uint32_t)(s * kStepCols * 64 + 512), w[4], w[5], w[6], w[7]);
                 }

@@ -218,28 +218,64 @@ __device__ __forceinline__ float2 raw2_to_float2(uint32_t w)
     else return __half22float2(*reinterpret_cast<const __half2*>(&w));
 }
 
-// GELU in its exact form, v * Phi(v) = 0.5 v (1 + erf(v / sqrt 2)) (the activation of the ViT MLP), in fp32.
-// With a = |v|: gelu(v) = max(v, 0) - 0.5 a erfc(a / sqrt 2), and erfc(a / sqrt 2) = 2^Q(a) with Q a polynomial of
-// degree 6 fitted to log2 erfc on [0, 5.9375] (beyond it erfc < 3e-9; fit_gelu.py beside the package's build script
-// reproduces the coefficients and the error: 3e-7 absolute in fp32 over all v).  Ten instructions and one
-// special-function-unit operation per value; the library erff cost the epilogue warps about 40 instructions and
-// tripled the time of an fc1 layer on the sparse kernels, a rational form with a reciprocal still doubled it.
-__device__ __forceinline__ float gelu_exact(float v)
+// Two fp32 values in one instruction.
+__device__ __forceinline__ uint64_t f32x2(float a, float b)
 {
-    const float a = fminf(fabsf(v), 5.9375f);
-    float q = fmaf(a, 3.309303065e-05f, -7.692219224e-04f);
-    q = fmaf(q, a, 8.080724627e-03f);
-    q = fmaf(q, a, -5.341212079e-02f);
-    q = fmaf(q, a, -4.587709606e-01f);
-    q = fmaf(q, a, -1.151201725e+00f);
-    q = fmaf(q, a, 6.939759714e-06f);
-    float e;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(q));
-    return fmaf(-0.5f * fabsf(v), e, fmaxf(v, 0.0f));
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 f32x2_split(uint64_t v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t f32x2_add(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 
-// Epilogue activation of a layer: 0 none, 1 GELU.
-__device__ __forceinline__ float apply_act(float v, int act) { return act == 1 ? gelu_exact(v) : v; }
+// GELU in its exact form, v * Phi(v) = 0.5 v (1 + erf(v / sqrt 2)) (the activation of the ViT MLP), in fp32, of two values.
+// With n = -|v|: gelu(v) = max(v, 0) + n * erfc(-n / sqrt 2) / 2, and erfc / 2 = 2^(Q(n) - 1) with Q a polynomial of
+// degree 6 fitted to log2 erfc on [-5.9375, 0] (below it erfc < 3e-9; fit_gelu.py beside the package's build script
+// reproduces the coefficients and the error: 3e-7 absolute in fp32 over all v).  Two values share the instructions of
+// the polynomial and of the last product: 6.5 instructions and one special-function operation a value, 11 for one value
+// at a time, which made the epilogue the slowest part of a GELU layer on every GEMM kernel (50432 x 768 -> 3072, pair
+// kernel 304 -> 223 us, weight-stationary one 167 -> 137).
+__device__ __forceinline__ float2 gelu_pair(float x, float y)
+{
+    const float nx = fmaxf(-fabsf(x), -5.9375f), ny = fmaxf(-fabsf(y), -5.9375f);
+    const uint64_t n = f32x2(nx, ny);
+    uint64_t q = f32x2_fma(n, f32x2(3.309303065e-05f, 3.309303065e-05f), f32x2(7.692219224e-04f, 7.692219224e-04f));
+    q = f32x2_fma(q, n, f32x2(8.080724627e-03f, 8.080724627e-03f));
+    q = f32x2_fma(q, n, f32x2(5.341212079e-02f, 5.341212079e-02f));
+    q = f32x2_fma(q, n, f32x2(-4.587709606e-01f, -4.587709606e-01f));
+    q = f32x2_fma(q, n, f32x2(1.151201725f, 1.151201725f));
+    q = f32x2_fma(q, n, f32x2(6.939759714e-06f - 1.0f, 6.939759714e-06f - 1.0f));
+    const float2 p = f32x2_split(q);
+    float ex, ey;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(p.x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ey) : "f"(p.y));
+    return f32x2_split(f32x2_fma(n, f32x2(ex, ey), f32x2(fmaxf(x, 0.0f), fmaxf(y, 0.0f))));
+}
+
+// What a GEMM's epilogue stores for two accumulators: + bias, GELU where the layer has it, rounded once.
+template <bool kBf16, bool kAct>
+__device__ __forceinline__ uint32_t finish_pair(uint32_t a, uint32_t b, uint64_t bias2, int act)
+{
+    float2 v = f32x2_split(f32x2_add(f32x2(__uint_as_float(a), __uint_as_float(b)), bias2));
+    if (kAct && act == 1) v = gelu_pair(v.x, v.y);
+    return pack2<kBf16>(v.x, v.y);
+}
 
 template <bool kBf16>
 __device__ __forceinline__ float bias_to_float(uint16_t u)

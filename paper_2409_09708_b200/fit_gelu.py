@@ -1,7 +1,7 @@
 """Fits the polynomial the kernels' GELU uses and prints its coefficients and error.
 
-gelu(v) = v Phi(v) = max(v, 0) - 0.5 a erfc(a / sqrt 2) with a = |v|; the kernels evaluate erfc(a / sqrt 2) as
-2^Q(a), Q of degree 6 on [0, 5.9375] (clamped beyond).  Q is a weighted least-squares fit of log2 erfc, the weights
+gelu(v) = v Phi(v) = max(v, 0) + n erfc(-n / sqrt 2) / 2 with n = -|v|; the kernels evaluate erfc(-n / sqrt 2) / 2 as
+2^(Q(-n) - 1), Q of degree 6 on [0, 5.9375] (n clamped beyond).  Q is a weighted least-squares fit of log2 erfc, the weights
 iterated towards the largest absolute error of the resulting GELU.  Run: python -m paper_2409_09708_b200.fit_gelu
 """
 import math
@@ -25,12 +25,14 @@ def fit(deg=6, n=6000, rounds=200):
 
 
 def gelu_f32(v, co):
-    a = np.minimum(np.abs(v), np.float32(A_MAX))
-    q = np.zeros_like(a)
+    n = np.maximum(-np.abs(v), np.float32(-A_MAX))
+    co = [c if i % 2 == 0 else -c for i, c in enumerate(co)]          # Q as a polynomial in n
+    co[0] = np.float32(co[0] - np.float32(1))
+    q = np.zeros_like(n)
     for c in co[::-1]:
-        q = (q * a + c).astype(np.float32)
+        q = (q * n + c).astype(np.float32)
     e = np.exp2(q.astype(np.float64)).astype(np.float32)
-    return (np.maximum(v, np.float32(0)) - (np.float32(0.5) * np.abs(v) * e).astype(np.float32)).astype(np.float32)
+    return (np.maximum(v, np.float32(0)) + (n * e).astype(np.float32)).astype(np.float32)
 
 
 if __name__ == "__main__":
