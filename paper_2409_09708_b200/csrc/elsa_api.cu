@@ -1478,7 +1478,7 @@ namespace elsa {
 namespace {
 
 struct BackwardPlan {
-    size_t wm, wmt, partial, sums, total;   // byte offsets of the regions
+    size_t wmt, partial, sums, total;   // byte offsets of the regions
 };
 
 // Upper bound, from host arithmetic alone, of the ranges the dW product may be cut into: what a device of 256 SMs
@@ -1495,10 +1495,13 @@ BackwardPlan backward_plan(int rows, int in, int out)
 {
     BackwardPlan p;
     size_t at = 0;
-    p.wm = at;      at += round_up((size_t)out * in * 2, 256);                      // masked weight [out][in]
-    p.wmt = at;     at += round_up((size_t)out * in * 2, 256);                      // its transpose [in][out]
-    p.partial = at; at += round_up((size_t)((rows + 511) / 512) * out * 4, 256);    // column sums of dY per 512 rows
-    const int bound = wgrad_splits_bound(in, out);                                  // fp32 sums of dW per range of rows
+    p.wmt = at;     at += round_up((size_t)out * in * 2, 256);                      // transposed masked weight [in][out]
+    const int bound = wgrad_splits_bound(in, out);
+    int parts = (rows + 511) / 512;                                                 // parts of the column sums of dY:
+    if (parts < linear_tc_pair_tn_sums_parts(in, 1)) parts = linear_tc_pair_tn_sums_parts(in, 1);   // 512 rows each, or
+    if (parts < linear_tc_pair_tn_sums_parts(in, bound)) parts = linear_tc_pair_tn_sums_parts(in, bound);   // from dW's product
+    p.partial = at; at += round_up((size_t)parts * out * 4, 256);
+    // fp32 sums of dW per range of rows
     p.sums = at;    at += bound > 1 ? round_up((size_t)bound * out * in * 4, 256) : 0;
     p.total = at;
     return p;
@@ -1556,17 +1559,12 @@ elsa_status elsa_nm_linear_backward(const void* dY, const void* X, int rows, con
     const uint16_t* dy = (const uint16_t*)dY;
     if (dX) {
         // dX = dY Wm: the forward GEMM with the transposed masked weight, reduction over `out`
-        uint16_t* wm = (uint16_t*)(ws + plan.wm);
         uint16_t* wmt = (uint16_t*)(ws + plan.wmt);
-        const uint16_t* dense = (const uint16_t*)vals;
-        if (N != M) {
-            if ((st = launch_unpack((const uint16_t*)vals, idx, out, in, N, M, wm, stream)) != ELSA_OK) return st;
-            dense = wm;
-        }
-        if ((st = launch_transpose16(dense, wmt, out, in, out, stream)) != ELSA_OK) return st;
+        if ((st = launch_transpose_packed((const uint16_t*)vals, idx, wmt, out, in, N, M, stream)) != ELSA_OK) return st;
         if ((st = dense_product(dy, rows, wmt, in, out, dtype, (uint16_t*)dX, dev_status, stream, dev.sm_count)) != ELSA_OK) return st;
     }
-    if (db && (st = launch_colsum(dy, rows, out, (float*)(ws + plan.partial), (uint16_t*)db, dtype, stream)) != ELSA_OK) return st;
+    float* db_sums = (float*)(ws + plan.partial);
+    int db_parts = 0;
     if (dW) {
         // dW = dY^T X, reduction over the token rows: both operands are read as they are stored (reduction index
         // outermost), then the mask
@@ -1574,14 +1572,19 @@ elsa_status elsa_nm_linear_backward(const void* dY, const void* X, int rows, con
         int splits = linear_tc_pair_tn_splits(out, in, rows, dev.sm_count);
         if (splits > wgrad_splits_bound(in, out)) splits = wgrad_splits_bound(in, out);
         float* sums = (float*)(ws + plan.sums);
-        if ((st = launch_linear_tc_pair_tn(dy, (const uint16_t*)X, out, in, rows, dtype, (uint16_t*)dW, splits, sums, dev_status,
-                                           stream)) != ELSA_OK)
+        if ((st = launch_linear_tc_pair_tn(dy, (const uint16_t*)X, out, in, rows, dtype, (uint16_t*)dW, splits, sums,
+                                           db ? db_sums : nullptr, &db_parts, dev_status, stream)) != ELSA_OK)
             return st;
-        st = splits > 1 ? launch_wgrad_finish(sums, splits, idx, out, in, N, M, dtype, (uint16_t*)dW, stream)
-                        : launch_mask_apply((uint16_t*)dW, idx, out, in, N, M, stream);
-        if (st != ELSA_OK) return st;
+        if (splits > 1) {
+            st = launch_wgrad_finish(sums, splits, idx, out, in, N, M, dtype, (uint16_t*)dW, db_sums, db_parts, (uint16_t*)db, stream);
+            if (st != ELSA_OK || db_parts > 0) return st;
+        } else if ((st = launch_mask_apply((uint16_t*)dW, idx, out, in, N, M, stream)) != ELSA_OK) {
+            return st;
+        }
     }
-    return ELSA_OK;
+    if (!db) return ELSA_OK;
+    return db_parts > 0 ? launch_colsum_finish(db_sums, db_parts, out, (uint16_t*)db, dtype, stream)
+                        : launch_colsum(dy, rows, out, db_sums, (uint16_t*)db, dtype, stream);
 }
 
 }  // extern "C"

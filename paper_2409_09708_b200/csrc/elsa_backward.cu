@@ -2,10 +2,12 @@
 // sparse weights derived from the shared weight; for Y = X Wm^T + b that is dX = dY Wm, dW = mask .* dY^T X,
 // db = column sums of dY).  The two contractions run on the dense tensor-core GEMM of the forward path, which
 // wants both operands with the reduction index contiguous; these kernels bring the operands into that form:
-//   transpose16    [R][C] -> [C][Rp] (Rp >= R, the tail zero): the masked weight for dX
+//   transpose_packed  the packed weight as the transposed masked weight [in][out], for dX
 //   mask_apply     zeroes the pruned positions of a dense [out][in] gradient in place, from the index stream
-//   colsum_partial column sums of dY over chunks of 512 rows; colsum_finish adds the chunks and rounds once
-#include "elsa_internal.h"
+//   wgrad_finish   adds the ranges' sums of dW, rounds and masks; and the parts of db where dW's launch made them
+//   colsum_partial column sums of dY over chunks of 512 rows where it did not (db alone, or more tiles than SM pairs);
+//                  colsum_finish adds the chunks and rounds once
+#include "elsa_pack_device.cuh"
 
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -40,12 +42,15 @@ __device__ __forceinline__ void stmatrix_x4_transposed(uint32_t addr, const uint
                  :: "r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
 }
 
-// One block per 64 x 64 tile.  src [R][C] (C % 8 == 0), dst [C][Rp] (Rp % 8 == 0).  The tile is read with
-// 16-byte loads into shared memory, transposed there in 8 x 8 blocks (ldmatrix, stmatrix.trans; rows of
-// 144 bytes keep both free of bank conflicts) and written with 16-byte stores.  Blocks of the last tile row also
-// write the zero tail R..Rp of their dst rows.
+// dst [in][out] = the masked weight [out][in], transposed: one block per 64 x 64 tile (out % 8 == 0).  The tile is expanded
+// from the packed form, 16 bytes of a row at a time, into shared memory, transposed there in 8 x 8 blocks (ldmatrix,
+// stmatrix.trans; rows of 144 bytes keep both free of bank conflicts) and written with 16-byte stores.  A launch is a few
+// MB and bound by latency (6 to 7 us between events), which is why the expansion, 6 to 10 us as a launch before this one,
+// is part of it; NC: the level N, 0 for the others.
+template <int M, int NC>
 __global__ void __launch_bounds__(256)
-transpose16_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst, int R, int C, int Rp)
+transpose_packed_kernel(const uint16_t* __restrict__ vals, const uint32_t* __restrict__ idx, uint16_t* __restrict__ dst, int out, int in,
+                        int N, int words_per_row)
 {
     constexpr int kPitch = kTile + 8;   // values per shared-memory row
     __shared__ __align__(16) uint16_t tile_in[kTile][kPitch];
@@ -54,15 +59,37 @@ transpose16_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst,
     pdl_release_successors();
     const int r0 = blockIdx.x * kTile, c0 = blockIdx.y * kTile;   // row tiles on x: their count has no 65535 limit
     const int t = threadIdx.x;
-    // load: 64 rows x 8 vectors of 8 values (rows past R and columns past C as zeros)
+    // expand: 64 rows x 8 units of 8 positions (rows past out and columns past in as zeros)
+    const size_t values_per_row = (size_t)(in / M) * (size_t)N;
+    if constexpr (M == 16 || NC == M) {
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int slot = t + 256 * i;
-        const int r = slot >> 3, v = slot & 7;
-        uint4 u = make_uint4(0u, 0u, 0u, 0u);
-        if (r0 + r < R && c0 + 8 * v < C)
-            u = __ldg(reinterpret_cast<const uint4*>(src + (size_t)(r0 + r) * (size_t)C + c0 + 8 * v));
-        *reinterpret_cast<uint4*>(&tile_in[r][8 * v]) = u;
+        for (int i = 0; i < 2; ++i) {
+            const int slot = t + 256 * i, r = slot >> 3, v = slot & 7;
+            uint4 u = make_uint4(0u, 0u, 0u, 0u);
+            if (r0 + r < out && c0 + 8 * v < in) {
+                const size_t row = (size_t)(r0 + r);
+                if constexpr (NC == M) u = __ldg(reinterpret_cast<const uint4*>(vals + row * (size_t)in + c0 + 8 * v));
+                else u = expand_unit16(vals + row * values_per_row, idx + row * (size_t)words_per_row, N, (c0 >> 3) + v);
+            }
+            *reinterpret_cast<uint4*>(&tile_in[r][8 * v]) = u;
+        }
+    } else {
+        PackedUnit unit[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int slot = t + 256 * i, r = slot >> 3, v = slot & 7;
+            if (r0 + r < out && c0 + 8 * v < in) {
+                const size_t row = (size_t)(r0 + r);
+                unit[i] = load_packed_unit<M, NC>(vals + row * values_per_row, idx + row * (size_t)words_per_row, N, (c0 >> 3) + v);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int slot = t + 256 * i, r = slot >> 3, v = slot & 7;
+            uint4 u = make_uint4(0u, 0u, 0u, 0u);
+            if (r0 + r < out && c0 + 8 * v < in) u = expand_packed_unit<M, NC>(unit[i], N);
+            *reinterpret_cast<uint4*>(&tile_in[r][8 * v]) = u;
+        }
     }
     __syncthreads();
     {
@@ -79,17 +106,13 @@ transpose16_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst,
         }
     }
     __syncthreads();
-    // store: 64 dst rows (source columns) x 8 vectors of 8 source rows
-    const bool last = blockIdx.x == gridDim.x - 1;
+    // store: 64 dst rows (weight columns) x 8 vectors of 8 weight rows
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         const int slot = t + 256 * i;
         const int c = slot >> 3, v = slot & 7;
-        if (c0 + c >= C) continue;
-        uint16_t* row = dst + (size_t)(c0 + c) * (size_t)Rp;
-        if (r0 + 8 * v < Rp) *reinterpret_cast<uint4*>(row + r0 + 8 * v) = *reinterpret_cast<const uint4*>(&tile_out[c][8 * v]);
-        if (last)
-            for (int r = r0 + kTile + 8 * v; r < Rp; r += kTile) *reinterpret_cast<uint4*>(row + r) = make_uint4(0u, 0u, 0u, 0u);
+        if (c0 + c < in && r0 + 8 * v < out)
+            *reinterpret_cast<uint4*>(dst + (size_t)(c0 + c) * (size_t)out + r0 + 8 * v) = *reinterpret_cast<const uint4*>(&tile_out[c][8 * v]);
     }
 }
 
@@ -133,17 +156,24 @@ colsum_partial_kernel(const uint16_t* __restrict__ src, int R, int C, float* __r
     }
 }
 
-// db[c] = round16(sum over tiles of partial[tile][c]), tiles in ascending order.
+// db[c] = round16(sum over parts of partial[part][c]), parts in ascending order.
 template <bool kBf16>
-__global__ void __launch_bounds__(256) colsum_finish_kernel(const float* __restrict__ partial, int tiles, int C, uint16_t* __restrict__ db)
+__device__ __forceinline__ void sum_parts(const float* __restrict__ partial, int parts, int C, uint16_t* __restrict__ db, int block)
+{
+    const int c = block * 256 + (int)threadIdx.x;
+    if (c >= C) return;
+    float s = 0.f;
+#pragma unroll 8
+    for (int i = 0; i < parts; ++i) s += partial[(size_t)i * (size_t)C + c];
+    db[c] = from_float<kBf16>(s);
+}
+
+template <bool kBf16>
+__global__ void __launch_bounds__(256) colsum_finish_kernel(const float* __restrict__ partial, int parts, int C, uint16_t* __restrict__ db)
 {
     pdl_wait_for_predecessors();
     pdl_release_successors();
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    float s = 0.f;
-    for (int i = 0; i < tiles; ++i) s += partial[(size_t)i * (size_t)C + c];
-    db[c] = from_float<kBf16>(s);
+    sum_parts<kBf16>(partial, parts, C, db, (int)blockIdx.x);
 }
 
 // One thread per group of M: keeps the N positions the index stream names, zeroes the rest.
@@ -176,16 +206,21 @@ mask_apply_kernel(uint16_t* __restrict__ dW, const uint32_t* __restrict__ idx, i
 }
 
 // One thread per group of M weights: adds the ranges' fp32 sums in ascending order, rounds once, zeroes what the
-// index stream does not keep (everything is kept when idx is NULL).
+// index stream does not keep (everything is kept when idx is NULL).  The first db_blocks blocks add the parts of db.
 template <int M, bool kBf16>
 __global__ void __launch_bounds__(256)
 wgrad_finish_kernel(const float* __restrict__ partial, int splits, const uint32_t* __restrict__ idx, int out, int in, int N,
-                    int words_per_row, uint16_t* __restrict__ dW)
+                    int words_per_row, uint16_t* __restrict__ dW, const float* __restrict__ db_sums, int db_parts,
+                    uint16_t* __restrict__ db, int db_blocks)
 {
     constexpr int B = (M == 4) ? 2 : (M == 8) ? 3 : 4;
     pdl_wait_for_predecessors();
     pdl_release_successors();
-    const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if ((int)blockIdx.x < db_blocks) {
+        sum_parts<kBf16>(db_sums, db_parts, out, db, (int)blockIdx.x);
+        return;
+    }
+    const long long gid = (long long)((int)blockIdx.x - db_blocks) * 256 + threadIdx.x;
     const int groups_per_row = in / M;
     if (gid >= (long long)out * groups_per_row) return;
     const int o = (int)(gid / groups_per_row), g = (int)(gid % groups_per_row);
@@ -227,15 +262,20 @@ wgrad_finish_kernel(const float* __restrict__ partial, int splits, const uint32_
 
 }  // namespace
 
-elsa_status launch_colsum_finish(const float* partial, int tiles, int C, uint16_t* db, elsa_dtype dtype, cudaStream_t stream);
-
-elsa_status launch_transpose16(const uint16_t* src, uint16_t* dst, int R, int C, int Rp, cudaStream_t stream)
+elsa_status launch_transpose_packed(const uint16_t* vals, const uint32_t* idx, uint16_t* dst, int out, int in, int N, int M, cudaStream_t stream)
 {
-    if (R <= 0 || C <= 0) return ELSA_OK;
-    const dim3 grid((unsigned)((R + kTile - 1) / kTile), (unsigned)((C + kTile - 1) / kTile));
+    const dim3 grid((unsigned)((out + kTile - 1) / kTile), (unsigned)((in + kTile - 1) / kTile));
+    const int wpr = (int)index_words_per_row(in, N, M);
+    auto* kernel = N == M   ? transpose_packed_kernel<16, 16>
+                   : M == 16 ? transpose_packed_kernel<16, 0>
+                   : M == 8  ? (N == 1   ? transpose_packed_kernel<8, 1>
+                                : N == 2 ? transpose_packed_kernel<8, 2>
+                                : N == 4 ? transpose_packed_kernel<8, 4>
+                                         : transpose_packed_kernel<8, 0>)
+                             : (N == 1 ? transpose_packed_kernel<4, 1> : N == 2 ? transpose_packed_kernel<4, 2> : transpose_packed_kernel<4, 0>);
     ProfileScope scope(ELSA_KERNEL_BACKWARD_FORMAT, stream);
-    launch_pdl(transpose16_kernel, grid, dim3(256), 0, stream, 1, src, dst, R, C, Rp);
-    return launched("transpose16");
+    launch_pdl(kernel, grid, dim3(256), 0, stream, 1, vals, idx, dst, out, in, N, wpr);
+    return launched("transpose_packed");
 }
 
 // db [C] = column sums of src [R][C]; partial: ceil(R / 512) * C floats of scratch.
@@ -253,28 +293,29 @@ elsa_status launch_colsum(const uint16_t* src, int R, int C, float* partial, uin
     return launch_colsum_finish(partial, chunks, C, db, dtype, stream);
 }
 
-elsa_status launch_colsum_finish(const float* partial, int tiles, int C, uint16_t* db, elsa_dtype dtype, cudaStream_t stream)
+elsa_status launch_colsum_finish(const float* partial, int parts, int C, uint16_t* db, elsa_dtype dtype, cudaStream_t stream)
 {
     const unsigned grid = (unsigned)((C + 255) / 256);
     ProfileScope scope(ELSA_KERNEL_BACKWARD_FORMAT, stream);
-    if (dtype == ELSA_BF16) launch_pdl(colsum_finish_kernel<true>, dim3(grid), dim3(256), 0, stream, 1, partial, tiles, C, db);
-    else launch_pdl(colsum_finish_kernel<false>, dim3(grid), dim3(256), 0, stream, 1, partial, tiles, C, db);
+    if (dtype == ELSA_BF16) launch_pdl(colsum_finish_kernel<true>, dim3(grid), dim3(256), 0, stream, 1, partial, parts, C, db);
+    else launch_pdl(colsum_finish_kernel<false>, dim3(grid), dim3(256), 0, stream, 1, partial, parts, C, db);
     return launched("colsum_finish");
 }
 
 elsa_status launch_wgrad_finish(const float* partial, int splits, const uint32_t* idx, int out, int in, int N, int M,
-                                elsa_dtype dtype, uint16_t* dW, cudaStream_t stream)
+                                elsa_dtype dtype, uint16_t* dW, const float* db_sums, int db_parts, uint16_t* db, cudaStream_t stream)
 {
     const long long groups = (long long)out * (in / M);
-    const unsigned grid = (unsigned)((groups + 255) / 256);
+    const int db_blocks = db_parts > 0 ? (out + 255) / 256 : 0;
+    const unsigned grid = (unsigned)((groups + 255) / 256 + db_blocks);
     const int wpr = (int)index_words_per_row(in, N, M);
     const uint32_t* ix = N == M ? nullptr : idx;
     const bool bf = dtype == ELSA_BF16;
     ProfileScope scope(ELSA_KERNEL_BACKWARD_FORMAT, stream);
 #define ELSA_FINISH(MM)                                                                                                     \
     do {                                                                                                                  \
-        if (bf) launch_pdl(wgrad_finish_kernel<MM, true>, dim3(grid), dim3(256), 0, stream, 1, partial, splits, ix, out, in, N, wpr, dW); \
-        else launch_pdl(wgrad_finish_kernel<MM, false>, dim3(grid), dim3(256), 0, stream, 1, partial, splits, ix, out, in, N, wpr, dW);   \
+        if (bf) launch_pdl(wgrad_finish_kernel<MM, true>, dim3(grid), dim3(256), 0, stream, 1, partial, splits, ix, out, in, N, wpr, dW, db_sums, db_parts, db, db_blocks); \
+        else launch_pdl(wgrad_finish_kernel<MM, false>, dim3(grid), dim3(256), 0, stream, 1, partial, splits, ix, out, in, N, wpr, dW, db_sums, db_parts, db, db_blocks);   \
     } while (0)
     if (M == 4) ELSA_FINISH(4);
     else if (M == 8) ELSA_FINISH(8);

@@ -121,10 +121,14 @@ elsa_status launch_linear_tc_pair(const uint16_t* X, int rows, const uint16_t* W
 // Y [m][n] = A^T B on the same kernel with both operands stored reduction-outermost, A [k][m] and B [k][n]
 // (m, n multiples of 8): the weight-gradient product dY^T X without transposed copies.
 // With splits > 1 the reduction is cut into that many ranges whose fp32 sums go to partial [splits][m][n] (Y is then
-// not written); linear_tc_pair_tn_splits says how many ranges keep the SM pairs occupied.
+// not written); linear_tc_pair_tn_splits says how many ranges keep the SM pairs occupied.  With sums_a (or
+// NULL) and no more tiles than SM pairs, *sums_parts rows of m floats that add up to the sums of A over the reduction go
+// there (at most linear_tc_pair_tn_sums_parts(n, splits)); otherwise *sums_parts is 0.
 int linear_tc_pair_tn_splits(int m, int n, int k, int sm_count);
+int linear_tc_pair_tn_sums_parts(int n, int splits);
 elsa_status launch_linear_tc_pair_tn(const uint16_t* A, const uint16_t* B, int m, int n, int k, elsa_dtype dtype,
-                                     uint16_t* Y, int splits, float* partial, uint32_t* dev_status, cudaStream_t stream);
+                                     uint16_t* Y, int splits, float* partial, float* sums_a, int* sums_parts,
+                                     uint32_t* dev_status, cudaStream_t stream);
 // Levels with N <= 2 on the hardware 2:4 sparse MMA: re-encodes the packed weight into `workspace`
 // (2-of-4 values + metadata), then runs the sparse GEMM.
 elsa_status launch_linear_tc_sparse(const uint16_t* X, int rows, const uint16_t* vals, const uint32_t* idx,
@@ -224,15 +228,18 @@ bool window_attention_suits(int tokens, int heads, int dim);
 elsa_status launch_window_attention(const uint16_t* qkv, int windows, int tokens, int heads, int dim, elsa_dtype dtype, uint16_t* out,
                                     uint32_t* dev_status, cudaStream_t stream, const float* bias, const float* mask, int n_masks,
                                     int bias_pitch, const DeviceInfo& dev);
-// Operand forms of the backward pass.  transpose16: src [R][C] -> dst [C][Rp] with the tail R..Rp zero (C, Rp
-// multiples of 8).  colsum: db [C] = column sums of src [R][C], through ceil(R / 512) * C floats of scratch.
-elsa_status launch_transpose16(const uint16_t* src, uint16_t* dst, int R, int C, int Rp, cudaStream_t stream);
+// Operand forms of the backward pass.  transpose_packed: dst [in][out] (out a multiple of 8) = the transposed masked weight,
+// positions that were not kept zero.  colsum: db [C] = column sums of src [R][C], through ceil(R / 512) * C floats of scratch.
+elsa_status launch_transpose_packed(const uint16_t* vals, const uint32_t* idx, uint16_t* dst, int out, int in, int N, int M, cudaStream_t stream);
 elsa_status launch_colsum(const uint16_t* src, int R, int C, float* partial, uint16_t* db, elsa_dtype dtype, cudaStream_t stream);
+// db[c] = round16(sum over parts of partial[part][c]).
+elsa_status launch_colsum_finish(const float* partial, int parts, int C, uint16_t* db, elsa_dtype dtype, cudaStream_t stream);
 // Zeroes the pruned positions of a dense [out][in] tensor in place.
 elsa_status launch_mask_apply(uint16_t* dW, const uint32_t* idx, int out, int in, int N, int M, cudaStream_t stream);
-// dW [out][in] = mask .* round16(sum over ranges of partial [splits][out][in]); idx NULL (N == M) keeps everything.
+// dW [out][in] = mask .* round16(sum over ranges of partial [splits][out][in]); idx NULL (N == M) keeps everything.  With
+// db_parts > 0 also db as colsum_finish makes it.
 elsa_status launch_wgrad_finish(const float* partial, int splits, const uint32_t* idx, int out, int in, int N, int M,
-                                elsa_dtype dtype, uint16_t* dW, cudaStream_t stream);
+                                elsa_dtype dtype, uint16_t* dW, const float* db_sums, int db_parts, uint16_t* db, cudaStream_t stream);
 // Any number of (weight, level) pairs, one launch per 256.
 struct CompressJob {
     const uint16_t* W;
@@ -257,6 +264,8 @@ struct PairJob {
     const uint16_t* residual = nullptr;   // [rows][out], added after the activation, before the one rounding
     int splits = 1;                       // Tn form: ranges the reduction is cut into; > 1 writes fp32 sums to `partial`
     float* partial = nullptr;             // [splits][rows][out]
+    float* sums_a = nullptr;              // Tn form: see launch_linear_tc_pair_tn
+    int* sums_parts = nullptr;
 };
 int linear_tc_pair_group_max();
 elsa_status launch_linear_tc_pair_group(const PairJob* jobs, int n, elsa_dtype dtype, uint32_t* dev_status,

@@ -78,6 +78,14 @@ struct alignas(64) PairGroup {
     // tile t / splits over range t % splits, and each range's fp32 sums go to partial[range][rows][out].
     int splits;
     float* partial;
+    // Tn form with at most one tile per SM pair: the sums of A over the reduction (the bias gradient, where A is dY), in
+    // parts that add up to them, sums_a[range * tiles_n + tile column][rows].  A product with 32 columns of ones into the
+    // columns of the second accumulator makes them from the tile of A in shared memory; the tiles that read the same A
+    // take its K blocks in turn, so that none of them has much more to do.  The product reads A once more from shared memory
+    // (an eighth longer where two tiles share it: 36642 x 512 -> 1536 54 -> 67 us); as a pass of its own over dY with a
+    // second launch to add its chunks it cost 33 us there.  Compress, forward and backward of a DeiT-B block at 25216 rows:
+    // 1062 -> 976 us with this and the fused transposition of the weight.
+    float* sums_a;
     CUtensorMap map_r;   // fused form: the residual, boxes as map_y's
 };
 
@@ -166,6 +174,14 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
+    }
+    if constexpr (kTn) {
+        // 16 reduction rows of ones, in the place of the INT8 form's scales
+        if (p.sums_a != nullptr && threadIdx.x < kScaleBytes / 16) {
+            const uint32_t one = kBf16 ? 0x3F803F80u : 0x3C003C00u;
+            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(smem_base + scale_off + threadIdx.x * 16u), "r"(one) : "memory");
+            fence_proxy_async_smem();
+        }
     }
     if (warp == 1) tmem_alloc_pair(smem_base + holder_off, kTmemCols);
     tc_fence_before();
@@ -256,6 +272,13 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                     kb1 = (int)((long long)p.layer[cur].num_k_blocks * (range + 1) / p.splits);
                 }
                 const uint32_t idesc = p.layer[cur].idesc;
+                int sum_kb = kb1;      // the next K block whose sums are this tile's
+                bool sums_begun = false;
+                if constexpr (kTn) {
+                    if (p.sums_a != nullptr) sum_kb = kb0 + ((tile - p.layer[cur].tile_begin) / p.splits) % p.layer[cur].tiles_n;
+                }
+                (void)sum_kb;
+                (void)sums_begun;
                 ok = mbar_wait(tmem_empty_bar + 8 * acc, acc_phase ^ 1u, abort_flag, p.dev_status, 2);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
@@ -282,6 +305,18 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                         else
                             umma_f16_pair_if(d_tmem, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc,
                                              (uint32_t)((kb | k) != 0), elected);
+                    }
+                    if constexpr (kTn) {
+                        if (kb == sum_kb) {
+                            const uint64_t ones = smem_desc_mn_major_sw128(smem_base + scale_off, kTnBoxBytes);
+                            const uint32_t idesc32 = (idesc & ~(0x3Fu << 17)) | ((32u >> 3) << 17);     // N = 32
+#pragma unroll
+                            for (int k = 0; k < kBlockK / kUmmaK; ++k)
+                                umma_f16_pair_if(tmem_u + kMaxBlockN, a_desc + (uint64_t)(k * (kUmmaK * 128 >> 4)), ones, idesc32,
+                                                 (uint32_t)(sums_begun || k != 0), elected);
+                            sums_begun = true;
+                            sum_kb += p.layer[cur].tiles_n;
+                        }
                     }
                     umma_commit_pair_if(empty_bar + 8 * stage, 3, elected);   // frees this stage in both CTAs
                     if (++stage == p.stages) { stage = 0; phase ^= 1u; }
@@ -505,6 +540,18 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
 #pragma unroll
                 for (int i = 0; i < kMaxChunksPerWarp; ++i)
                     if (i < my_chunks) emit(r[i], part + kEpiParts * i, i);
+                if constexpr (kTn) {
+                    if (p.sums_a != nullptr && part == 0) {
+                        const int kb0 = (int)((long long)L.num_k_blocks * range / p.splits);
+                        const int kb1 = (int)((long long)L.num_k_blocks * (range + 1) / p.splits);
+                        uint32_t d[32];      // 32 equal columns; the pair has no other tile, so they stay
+                        tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(q * 32) << 16) + kMaxBlockN, d);
+                        tmem_wait_ld();
+                        const float sum = kb0 + t % L.tiles_n < kb1 ? __uint_as_float(d[0]) : 0.f;      // else no block was its
+                        if (row0 + lane < l_rows)
+                            p.sums_a[((size_t)range * L.tiles_n + t % L.tiles_n) * (size_t)l_rows + row0 + lane] = sum;
+                    }
+                }
             }
             // this warp has read the tile's bias for the last time
             __syncwarp();
@@ -672,6 +719,12 @@ elsa_status launch_group(const PairJob* jobs, int n, elsa_dtype dtype, uint32_t*
         max_pairs[slot].store(m, std::memory_order_release);
     }
     const int pairs = g.num_tiles < max_pairs[slot].load(std::memory_order_acquire) ? g.num_tiles : max_pairs[slot].load(std::memory_order_acquire);
+    g.sums_a = nullptr;
+    if (kForm == kFormTn && jobs[0].sums_a != nullptr) {
+        const bool taken = g.num_tiles <= max_pairs[slot].load(std::memory_order_acquire);
+        if (taken) g.sums_a = jobs[0].sums_a;
+        *jobs[0].sums_parts = taken ? g.splits * g.layer[0].tiles_n : 0;
+    }
     ProfileScope scope(kInt8 ? ELSA_KERNEL_LINEAR_TC_PAIR_I8 : ELSA_KERNEL_LINEAR_TC_PAIR, stream);
     cudaError_t e = launch_pdl(kernel, dim3((unsigned)(2 * pairs)), dim3(kThreads), smem, stream, 2, g);
     if (e != cudaSuccess) {
@@ -722,10 +775,15 @@ int linear_tc_pair_tn_splits(int m, int n, int k, int sm_count)
     return s < 1 ? 1 : (int)s;
 }
 
+// The most parts the sums of A come in: one a range and tile column, tiles of 256 columns when the reduction is cut, of
+// 128 at least when it is not.
+int linear_tc_pair_tn_sums_parts(int n, int splits) { return splits > 1 ? splits * ((n + 255) / 256) : (n + 127) / 128; }
+
 // Y [m][n] = A^T B with A [k][m] and B [k][n] (the reduction index outermost in both), no bias: one launch.
 // splits > 1: nothing is written to Y; partial [splits][m][n] receives the fp32 sums of each range of the reduction.
 elsa_status launch_linear_tc_pair_tn(const uint16_t* A, const uint16_t* B, int m, int n, int k, elsa_dtype dtype,
-                                     uint16_t* Y, int splits, float* partial, uint32_t* dev_status, cudaStream_t stream)
+                                     uint16_t* Y, int splits, float* partial, float* sums_a, int* sums_parts,
+                                     uint32_t* dev_status, cudaStream_t stream)
 {
     DeviceInfo dev;
     elsa_status st = device_info(&dev);
@@ -735,6 +793,8 @@ elsa_status launch_linear_tc_pair_tn(const uint16_t* A, const uint16_t* B, int m
     job.rows = m; job.in = k; job.out = n;
     job.splits = splits < 1 ? 1 : splits;
     job.partial = partial;
+    job.sums_a = sums_a;
+    job.sums_parts = sums_parts;
     return dtype == ELSA_BF16 ? launch_group<true, kFormTn, 1>(&job, 1, dtype, dev_status, stream, dev)
                               : launch_group<false, kFormTn, 1>(&job, 1, dtype, dev_status, stream, dev);
 }

@@ -1,0 +1,58 @@
+"""The bias gradient as parts of the weight gradient's launch, and the transposed masked weight straight from the packed form:
+rows below, at and above the 64-row K block (so that some tile columns take no block at all), features and columns around the
+256 and 64 wide tiles, the reduction cut and whole, more tiles than SM pairs (the separate column sums), every kept width the
+transposition is compiled for and one it is not.
+
+Small integers make every product and sum exact in fp32, so the results equal the oracle's after its one rounding.  With random
+values an fp32 sum of n terms is within n * 2^-23 * sum |dY| of the exact one in any order (one unit per addition, truncation
+allowed for), and the rounding adds at most 2^-9 (2^-12) of twice the result."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import elsa_backward_oracle as bwo
+from oracle import elsa_oracle as eo
+from paper_2409_09708_b200 import synth
+
+CASES = [
+    (1, 64, 8, 2, 4), (63, 256, 256, 1, 8), (64, 520, 264, 2, 8), (65, 264, 520, 4, 8), (129, 768, 768, 3, 8), (300, 1032, 64, 1, 4),
+    (640, 2560, 128, 5, 16), (257, 72, 96, 3, 4), (200, 136, 1024, 4, 4), (130, 2048, 2048, 2, 4), (130, 4096, 2312, 2, 8),
+]
+
+
+def backward(dY, X, W, N, M, want):
+    from paper_2409_09708_b200 import binding as lib
+    vals, idx = lib.elsa_nm_compress(W.cuda(), N, M)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = lib.elsa_nm_linear_backward(dY.cuda(), X.cuda(), vals, idx, W.shape[0], W.shape[1], N, M, want=want, dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0, "device status %#x" % int(status.item())
+    return out
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16], ids=["bf16", "f16"])
+@pytest.mark.parametrize("case", CASES, ids=["%dx%dx%d_%d:%d" % c for c in CASES])
+def test_integers_are_exact(case, dtype):
+    rows, in_, out, N, M = case
+    rng = np.random.default_rng(rows + in_)
+    ints = lambda *s: torch.from_numpy(rng.integers(-2, 3, s).astype(np.float32)).to(dtype)
+    dY, X, W = ints(rows, out), ints(rows, in_), ints(out, in_)
+    code = eo.F16 if dtype == torch.float16 else eo.BF16
+    refs = bwo.linear_backward_f64(synth.bits(dY), synth.bits(X), synth.bits(W), N, M, code)
+    for want in (("dX", "dW", "db"), ("dX", "db")):      # with the weight's gradient, and the column sums on their own
+        got = backward(dY, X, W, N, M, want)
+        for name, g, ref in zip(("dX", "dW", "db"), got, refs):
+            if name in want:
+                assert torch.equal(g.cpu().double(), torch.from_numpy(np.asarray(ref)).to(dtype).double()), (name, want)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16], ids=["bf16", "f16"])
+def test_sums_of_random_values(dtype):
+    rows, in_, out = 9001, 768, 776
+    dY, X, W = (synth.randn(s, i, 0.5, dtype) for i, s in enumerate(((rows, out), (rows, in_), (out, in_))))
+    db = backward(dY, X, W, 2, 4, ("dW", "db"))[2].cpu().double()
+    d = dY.double()
+    half_unit = 2.0 ** -9 if dtype == torch.bfloat16 else 2.0 ** -12
+    assert ((db - d.sum(0)).abs() <= rows * 2.0 ** -23 * d.abs().sum(0) + half_unit * d.sum(0).abs() * 2).all()
