@@ -11,12 +11,12 @@
 //   1. TMA brings the Q tile, all K rows and all V rows of the head into shared memory (128-byte swizzle; a 3-D
 //      tensor map [image][token][column] zero-fills the rows past the image's last token).
 //   2. S = Q K^T: four MMAs (K = 16 each) into Tk = tokens rounded up to 16 fp32 columns of tensor memory.
-//   3. Four warps, one query row per lane: row maximum over the real keys, p = 2^((s - max) * log2(e) / 8), row
-//      sum in fp32, p rounded to the 16-bit type and written back into tensor memory as the A operand of the
-//      second product, two keys per column, over the low half of the columns S occupied.
+//   3. Four warps, one query row per lane: p = 2^(s * log2(e) / 8 - ref) with ref at or just below the row's maximum
+//      (see `rise`), row sum in fp32, p rounded to the 16-bit type and written back into tensor memory as the A
+//      operand of the second product, two keys per column, over the low half of the columns S occupied.
 //   4. O = P V: Tk / 16 MMAs with A from tensor memory and V as it lies in memory (keys outermost: MN-major
 //      descriptor) into 64 columns of the part of S that is dead by then.
-//   5. The same four warps read O, divide by the row sum, round once and store each row's 128 bytes.
+//   5. The same four warps read O, divide by the row sum, round once and store it, whole rows at a time.
 // Persistent: one CTA per SM walks the items with the stride of the grid, with several items in flight: two for up
 // to 256 keys, four for up to 128 (Swin's windows), each with its own shared-memory stage (Q, K, V), its own share
 // of tensor memory (256 or 128 columns) and its own group of four softmax warps: item n uses stage, share and group
@@ -24,8 +24,15 @@
 // previous item, V after that item's second product); the MMA warp issues S of item n, then P V of the
 // oldest item whose probabilities are due, so one group's softmax runs under the others' products and epilogues.
 // Every wait is bounded as in the GEMM kernels.
+// What bounds it is an item's chain on its four warps (256 images x 12 heads of 197 tokens, cycles of the 6700 an item takes
+// with another in flight): exponentials 4200 (11 a score for a warp alone, where the special-function unit asks for 8),
+// second product 900 to 1300, output 900, the rest barriers.  113 -> 78 us against a maximum pass of its own (1400), tests
+// for padded keys on every score, a row of the output per lane (1300 to 2200) and the item's divisions on the chain.
+// Two warps to a quarter, half the keys each, with or without the two items exponentiating by turns: 89 and 107 us; units
+// of 64 scores: 103.
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
 #include "elsa_tc_common.cuh"
 
@@ -41,14 +48,17 @@ constexpr int kQBytes = kQRows * kMaxHeadDim * 2;          // the shared-memory 
 
 // kBufs items in flight per CTA: 2 for up to 256 keys (256 tensor-memory columns each), 4 for up to 128 keys (the
 // windows of Swin), where an item's on-chip chain is short and only more of them in flight fill the SM.
-template <int kBufs>
+template <int kBufs, bool kBias>
 struct Shape {
     static constexpr int kBufCols = kTmemCols / kBufs;
     static constexpr int kThreads = (2 + kBufs * kGroupWarps) * 32;
     static constexpr int kKvBytes = (kBufs == 2 ? 256 : 128) * kMaxHeadDim * 2;
     static constexpr int kStageBytes = kQBytes + 2 * kKvBytes;
-    static constexpr int kSmemBytes = kBufs * kStageBytes + 1024 /* alignment */ + 512 /* barriers */;
-    static constexpr int kUnit = kBufs == 2 ? 32 : 16;      // score columns a softmax warp handles at a time (registers)
+    static constexpr int kOutCols = kBufs == 2 ? kMaxHeadDim : 32;     // output columns a softmax warp stages at a time
+    static constexpr int kOutBytes = 32 * kOutCols * 2;
+    static constexpr int kSmemBytes = kBufs * (kStageBytes + kGroupWarps * kOutBytes) + 1024 /* alignment */ + 512 /* barriers */;
+    static constexpr int kBiasUnit = kBufs == 2 ? 32 : 16;  // score columns a softmax warp handles at a time (registers):
+    static constexpr int kUnit = 32;                        // adding the tables, exponentiating
 };
 
 struct AttnParams {
@@ -109,19 +119,27 @@ __device__ __forceinline__ void tmem_st_32x32b_x8(uint32_t taddr, const uint32_t
                  : "memory");
 }
 
+__device__ __forceinline__ void tmem_ld_32x32b_x8(uint32_t taddr, uint32_t (&r)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
 template <bool kBf16, int kD, bool kBias, int kBufs>
-__global__ void __launch_bounds__(Shape<kBufs>::kThreads, 1) attention_kernel(const __grid_constant__ AttnParams p)
+__global__ void __launch_bounds__(Shape<kBufs, kBias>::kThreads, 1) attention_kernel(const __grid_constant__ AttnParams p)
 {
     static_assert(kD == 64 || kD == 32, "head dimension");
     static_assert(kBufs == 2 || kBufs == 4, "items in flight");
-    constexpr int kBufCols = Shape<kBufs>::kBufCols, kStageBytes = Shape<kBufs>::kStageBytes, kKvBytesMax = Shape<kBufs>::kKvBytes;
-    constexpr int U = Shape<kBufs>::kUnit;
+    constexpr int kBufCols = Shape<kBufs, kBias>::kBufCols, kStageBytes = Shape<kBufs, kBias>::kStageBytes, kKvBytesMax = Shape<kBufs, kBias>::kKvBytes;
+    constexpr int U = Shape<kBufs, kBias>::kUnit, B = Shape<kBufs, kBias>::kBiasUnit;
     constexpr int kLag = kBufs - 1;                   // P V of item n - kLag is issued after S of item n
     constexpr int kHeadDim = kD;
     constexpr int kItemQBytes = kQRows * kD * 2;      // bytes TMA delivers for the Q tile; K and V: tk * kD * 2
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t bars = smem_base + kBufs * kStageBytes;
+    const uint32_t out_base = smem_base + kBufs * kStageBytes;
+    const uint32_t bars = out_base + kBufs * kGroupWarps * Shape<kBufs, kBias>::kOutBytes;
     // per buffer b: +0 qk_full, +8 v_full, +16 qk_empty, +24 s_full, +32 p_full, +40 o_full, +48 tmem_empty, +56 v_empty
     auto bar = [&](int which, int b) { return bars + (uint32_t)(64 * b + 8 * which); };
     enum { kQkFull = 0, kVFull, kQkEmpty, kSFull, kPFull, kOFull, kTmemEmpty, kVEmpty };
@@ -253,14 +271,34 @@ __global__ void __launch_bounds__(Shape<kBufs>::kThreads, 1) attention_kernel(co
         // ------------------------------------------------ softmax and output: group g takes the items n = g, g + 2, ...
         const int g = (warp - 2) / kGroupWarps;
         const int quarter = warp & 3;                                  // the TMEM lanes this warp may touch
+        const uint32_t stage_out = out_base + (uint32_t)((warp - 2) * Shape<kBufs, kBias>::kOutBytes);
+        constexpr float kFar = 32768.f;     // no probability above it: inside the 16-bit types and far inside fp32
         const float scale = (kD == 64 ? 0.125f : 0.17677669529663687f) * 1.4426950408889634f;   // log2(e) / sqrt(kD)
         bool ok = true;
+        int mt, head, img, next_mt = 0, next_head = 0, next_img = 0;
+        auto decode = [&](int n) {
+            const int item = first + n * stride;
+            next_mt = item % p.m_tiles; next_head = (item / p.m_tiles) % p.heads; next_img = item / (p.m_tiles * p.heads);
+        };
+        decode(g);
         for (int n = g; ok && n < n_items; n += kBufs) {
             const uint32_t ph = (uint32_t)((n / kBufs) & 1);
-            const int item = first + n * stride;
-            const int mt = item % p.m_tiles, head = (item / p.m_tiles) % p.heads, img = item / (p.m_tiles * p.heads);
+            mt = next_mt; head = next_head; img = next_img;
             const int row = mt * kQRows + quarter * 32 + lane;         // token index inside the image
             const uint32_t t_lane = tmem_base + (uint32_t)(g * kBufCols) + ((uint32_t)(quarter * 32) << 16);
+            if (mt * kQRows + quarter * 32 >= p.tokens) {
+                // none of its rows exists: the warp only keeps its place in the barriers
+                ok = mbar_wait(bar(kSFull, g), ph, abort_flag, p.dev_status, 25);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok) break;
+                if (lane == 0) mbar_arrive(bar(kPFull, g));
+                if (n + kBufs < n_items) decode(n + kBufs);
+                ok = mbar_wait(bar(kOFull, g), ph, abort_flag, p.dev_status, 26);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok) break;
+                if (lane == 0) mbar_arrive(bar(kTmemEmpty, g));
+                continue;
+            }
             float sum = 0.f;
             // biased form: what is exponentiated is s * scale + (bias + mask) * log2(e); the tables' rows of this lane
             const float* brow = nullptr;
@@ -293,7 +331,7 @@ __global__ void __launch_bounds__(Shape<kBufs>::kThreads, 1) attention_kernel(co
             // until the values are used): the first unit is asked for before the scores are waited for, every other
             // one while the unit before it is worked on, which takes most of the L2 latency out of the item's chain.
             // The mask (shifted windows only) is read where it is used: a second array across the wait would spill.
-            constexpr int kReq = kBias ? Shape<kBufs>::kUnit : 1;
+            constexpr int kReq = kBias ? Shape<kBufs, kBias>::kBiasUnit : 1;
             float bq[kReq];
             auto request = [&](int col0) {
 #pragma unroll
@@ -309,181 +347,238 @@ __global__ void __launch_bounds__(Shape<kBufs>::kThreads, 1) attention_kernel(co
             if (!ok) break;
             tc_fence_after();
             {
-                // Tensor-memory reads are waited for all at once, so the loads of a pass are issued in batches: the
-                // row maximum from two units per round trip, the second pass with the next unit in flight while
-                // the current one is exponentiated.  A unit is U = 32 score columns (16 with four items in flight).
-                auto ld_unit = [&](uint32_t taddr, uint32_t (&r)[U]) {
-                    if constexpr (U == 32) tmem_ld_32x32b_x32(taddr, r);
-                    else tmem_ld_32x32b_x16(taddr, r);
-                };
-                const int units = p.tk / U;                      // whole units
-                const bool tail = U == 32 && (p.tk & 31) != 0;   // plus one chunk of 16
                 float m = -INFINITY;
                 if constexpr (kBias) {
+                    auto ld_unit = [&](uint32_t taddr, uint32_t (&r)[B]) {
+                        if constexpr (B == 32) tmem_ld_32x32b_x32(taddr, r);
+                        else tmem_ld_32x32b_x16(taddr, r);
+                    };
+                    const int units = p.tk / B;                      // whole units
+                    const bool tail = B == 32 && (p.tk & 31) != 0;   // plus one chunk of 16
                     // first pass of the biased form: t = s * scale + (bias + mask) * log2(e) replaces s in tensor memory,
                     // so the tables are read once
                     for (int u = 0; u < units; ++u) {
-                        uint32_t r[U];
-                        float bb[U];
-                        ld_unit(t_lane + (uint32_t)(U * u), r);
+                        uint32_t r[B];
+                        float bb[B];
+                        ld_unit(t_lane + (uint32_t)(B * u), r);
 #pragma unroll
-                        for (int v = 0; v < U / 4; ++v) {
+                        for (int v = 0; v < B / 4; ++v) {
                             float4 m4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                            if (mrow != nullptr && U * u + 4 * v < p.bias_pitch) m4 = __ldg(reinterpret_cast<const float4*>(mrow + U * u) + v);
+                            if (mrow != nullptr && B * u + 4 * v < p.bias_pitch) m4 = __ldg(reinterpret_cast<const float4*>(mrow + B * u) + v);
                             bb[4 * v] = (bq[4 * v] + m4.x) * 1.4426950408889634f;
                             bb[4 * v + 1] = (bq[4 * v + 1] + m4.y) * 1.4426950408889634f;
                             bb[4 * v + 2] = (bq[4 * v + 2] + m4.z) * 1.4426950408889634f;
                             bb[4 * v + 3] = (bq[4 * v + 3] + m4.w) * 1.4426950408889634f;
                         }
-                        if (u + 1 < units) request(U * (u + 1));
+                        if (u + 1 < units) request(B * (u + 1));
                         tmem_wait_ld();
 #pragma unroll
-                        for (int j = 0; j < U; ++j) {
+                        for (int j = 0; j < B; ++j) {
                             const float t = fmaf(__uint_as_float(r[j]), scale, bb[j]);
                             r[j] = __float_as_uint(t);
-                            if (U * u + j < p.tokens) m = fmaxf(m, t);
+                            if (B * u + j < p.tokens) m = fmaxf(m, t);
                         }
 #pragma unroll
-                        for (int h = 0; h < U / 16; ++h) {
+                        for (int h = 0; h < B / 16; ++h) {
                             uint32_t part[16];
 #pragma unroll
                             for (int j = 0; j < 16; ++j) part[j] = r[16 * h + j];
-                            tmem_st_32x32b_x16(t_lane + (uint32_t)(U * u + 16 * h), part);
+                            tmem_st_32x32b_x16(t_lane + (uint32_t)(B * u + 16 * h), part);
                         }
                     }
                     if (tail) {
                         uint32_t r[16];
                         float bb[16];
-                        tmem_ld_32x32b_x16(t_lane + (uint32_t)(U * units), r);
-                        load_bias(bb, U * units, 16);
+                        tmem_ld_32x32b_x16(t_lane + (uint32_t)(B * units), r);
+                        load_bias(bb, B * units, 16);
                         tmem_wait_ld();
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
                             const float t = fmaf(__uint_as_float(r[j]), scale, bb[j]);
                             r[j] = __float_as_uint(t);
-                            if (U * units + j < p.tokens) m = fmaxf(m, t);
+                            if (B * units + j < p.tokens) m = fmaxf(m, t);
                         }
-                        tmem_st_32x32b_x16(t_lane + (uint32_t)(U * units), r);
+                        tmem_st_32x32b_x16(t_lane + (uint32_t)(B * units), r);
                     }
                     tmem_wait_st();
-                } else {
-                    for (int u0 = 0; u0 < units; u0 += 2) {
-                        uint32_t r[2][U];
-#pragma unroll
-                        for (int i = 0; i < 2; ++i)
-                            if (u0 + i < units) ld_unit(t_lane + (uint32_t)(U * (u0 + i)), r[i]);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int i = 0; i < 2; ++i)
-                            if (u0 + i < units) {
-                                if (U * (u0 + i) + U <= p.tokens) {       // a unit of real keys only: no per-column test
-                                    float m0 = m, m1 = -INFINITY;
-#pragma unroll
-                                    for (int j = 0; j < U; j += 2) {
-                                        m0 = fmaxf(m0, __uint_as_float(r[i][j]));
-                                        m1 = fmaxf(m1, __uint_as_float(r[i][j + 1]));
-                                    }
-                                    m = fmaxf(m0, m1);
-                                } else {
-#pragma unroll
-                                    for (int j = 0; j < U; ++j)
-                                        if (U * (u0 + i) + j < p.tokens) m = fmaxf(m, __uint_as_float(r[i][j]));
-                                }
-                            }
-                    }
-                    if (tail) {
-                        uint32_t r[16];
-                        tmem_ld_32x32b_x16(t_lane + (uint32_t)(U * units), r);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (U * units + j < p.tokens) m = fmaxf(m, __uint_as_float(r[j]));
-                    }
                 }
-                // p = 2^(s * scale - m * scale) for 16 columns starting at col0: eight packed pairs
-                const float m_scaled = kBias ? m : m * scale;      // the biased maximum is in the exponent's domain already
-                float sum1 = 0.f;
-                auto exp16 = [&](const uint32_t* r, int col0, uint32_t (&w)[8]) {
-                    const bool all_real = col0 + 16 <= p.tokens;
+                // p = 2^(s * scale - ref) for 16 columns from col0, two scores an instruction where there is such an
+                // instruction; eight packed pairs.  Only a unit with padded keys tests every column (at half rate).
+                float ref = m;                                     // biased form: the row's maximum, in the exponent's domain already
+                const uint64_t scale2 = f32x2(scale, scale);
+                uint64_t sum2 = f32x2(0.f, 0.f);
+                auto exp16 = [&](auto masked, const uint32_t* r, int col0, uint64_t& part2, uint32_t (&w)[8]) {
+                    const uint64_t minus_ref = f32x2(-ref, -ref);
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
+                        const uint64_t s2 = f32x2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+                        const float2 a = f32x2_split(kBias ? f32x2_add(s2, minus_ref) : f32x2_fma(s2, scale2, minus_ref));
                         float e0, e1;
-                        const float a0 = kBias ? __uint_as_float(r[2 * j]) - m_scaled : fmaf(__uint_as_float(r[2 * j]), scale, -m_scaled);
-                        const float a1 = kBias ? __uint_as_float(r[2 * j + 1]) - m_scaled
-                                               : fmaf(__uint_as_float(r[2 * j + 1]), scale, -m_scaled);
-                        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(a0));
-                        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(a1));
-                        if (!all_real) {                                  // padded keys take no part
+                        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(a.x));
+                        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(a.y));
+                        if constexpr (decltype(masked)::value) {          // padded keys take no part
                             if (col0 + 2 * j >= p.tokens) e0 = 0.f;
                             if (col0 + 2 * j + 1 >= p.tokens) e1 = 0.f;
                         }
-                        sum += e0;
-                        sum1 += e1;
+                        part2 = f32x2_add(part2, f32x2(e0, e1));
                         w[j] = pack2<kBf16>(e0, e1);
                     }
                 };
-                // P's columns of a unit lie over S columns of units that have been read already
-                auto unit = [&](const uint32_t (&r)[U], int u) {
+                // Unbiased form: the reference is a whole number, the largest of the row's first unit rounded down.  Where the
+                // probabilities of a later unit sum to more than kFar, it becomes that unit's largest, the sum and the
+                // P columns written so far are multiplied by the power of two between the two (exact but for values
+                // below the 16-bit type's normal range) and the unit is done again.  So no probability leaves the
+                // 16-bit types' range, none is smaller than with the maximum of the row as the reference, and the
+                // scores are read once: a pass for the maximum ahead of this one took a sixth of an item's time, a
+                // maximum of each unit ahead of its exponentials as much (half-rate instructions in a serial chain).
+                auto top_of = [&](auto masked, const uint32_t* r, int col0) {
+                    float t0 = -INFINITY, t1 = -INFINITY;
 #pragma unroll
-                    for (int h = 0; h < U / 16; ++h) {
+                    for (int j = 0; j < U; j += 2) {
+                        if (!decltype(masked)::value || col0 + j < p.tokens) t0 = fmaxf(t0, __uint_as_float(r[j]));
+                        if (!decltype(masked)::value || col0 + j + 1 < p.tokens) t1 = fmaxf(t1, __uint_as_float(r[j + 1]));
+                    }
+                    return fmaxf(floorf(fmaxf(t0, t1) * scale), -3.0e38f);      // finite for scores of minus infinity
+                };
+                auto rise = [&](float to, int written) {
+                    const float up = fminf(to - ref, 127.f);
+                    const float factor = __uint_as_float((uint32_t)(127 - (int)up) << 23);         // 2^-up, 0 from 127 on
+                    ref = to;
+                    sum2 = f32x2_mul(sum2, f32x2(factor, factor));
+                    tmem_wait_st();
+                    for (int c = 0; c < written; c += 8) {
                         uint32_t w[8];
-                        exp16(&r[16 * h], U * u + 16 * h, w);
-                        tmem_st_32x32b_x8(t_lane + (uint32_t)(U / 2 * u + 8 * h), w);
+                        tmem_ld_32x32b_x8(t_lane + (uint32_t)c, w);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const float2 v = raw2_to_float2<kBf16>(w[j]);
+                            w[j] = pack2<kBf16>(v.x * factor, v.y * factor);
+                        }
+                        tmem_st_32x32b_x8(t_lane + (uint32_t)c, w);
                     }
                 };
-                uint32_t ra[U], rb[U];
-                if (units > 0) ld_unit(t_lane, ra);
-                for (int u = 0; u < units; u += 2) {
-                    tmem_wait_ld();
-                    if (u + 1 < units) ld_unit(t_lane + (uint32_t)(U * (u + 1)), rb);
-                    unit(ra, u);
-                    if (u + 1 < units) {
+                // unit u, the first 16 columns of it where that is all there is (`halved`); P's columns lie over S columns of
+                // units that have been read already.  A whole unit is one straight run of code: a warp has little else to
+                // overlap its latencies with.
+                auto columns = [&](auto masked, const uint32_t* r, int u, bool halved) {
+                    uint64_t part2;
+                    auto once = [&]() {
+                        part2 = f32x2(0.f, 0.f);
+#pragma unroll
+                        for (int h = 0; h < U / 16; ++h) {
+                            if (decltype(masked)::value && h == 1 && halved) break;
+                            uint32_t w[8];
+                            exp16(masked, r + 16 * h, U * u + 16 * h, part2, w);
+                            tmem_st_32x32b_x8(t_lane + (uint32_t)(U / 2 * u + 8 * h), w);
+                        }
+                    };
+                    once();
+                    if constexpr (!kBias) {
+                        const float2 part = f32x2_split(part2);
+                        const bool far = part.x + part.y > kFar;
+                        if (__any_sync(0xFFFFFFFFu, far)) {
+                            const float top = top_of(masked, r, U * u);
+                            rise(far && top > ref ? top : ref, U / 2 * u);
+                            once();
+                        }
+                    }
+                    sum2 = f32x2_add(sum2, part2);
+                };
+                auto unit = [&](const uint32_t* r, int u) {
+                    if (U * u + U <= p.tokens) columns(std::false_type{}, r, u, false);
+                    else columns(std::true_type{}, r, u, U * u + U > p.tk);
+                };
+                auto first_top = [&](const uint32_t* r) {
+                    return U <= p.tokens ? top_of(std::false_type{}, r, 0) : top_of(std::true_type{}, r, 0);
+                };
+                // the last unit's load may reach past tk, inside the item's share of columns
+                const int units = (p.tk + U - 1) / U;
+                if constexpr (kBufs == 2) {
+                    // the next unit's scores are on their way while one is exponentiated
+                    uint32_t ra[U], rb[U];
+                    tmem_ld_32x32b_x32(t_lane, ra);
+                    if constexpr (!kBias) {
                         tmem_wait_ld();
-                        if (u + 2 < units) ld_unit(t_lane + (uint32_t)(U * (u + 2)), ra);
-                        unit(rb, u + 1);
+                        ref = first_top(ra);
+                    }
+                    for (int u = 0; u < units; u += 2) {
+                        tmem_wait_ld();
+                        if (u + 1 < units) tmem_ld_32x32b_x32(t_lane + (uint32_t)(U * (u + 1)), rb);
+                        unit(ra, u);
+                        if (u + 1 < units) {
+                            tmem_wait_ld();
+                            if (u + 2 < units) tmem_ld_32x32b_x32(t_lane + (uint32_t)(U * (u + 2)), ra);
+                            unit(rb, u + 1);
+                        }
+                    }
+                } else {
+                    // four groups of warps have each other's work to run under a load
+                    for (int u = 0; u < units; ++u) {
+                        uint32_t r[U];
+                        tmem_ld_32x32b_x32(t_lane + (uint32_t)(U * u), r);
+                        tmem_wait_ld();
+                        if (!kBias && u == 0) ref = first_top(r);
+                        unit(r, u);
                     }
                 }
-                if (tail) {
-                    uint32_t r[16], w[8];
-                    tmem_ld_32x32b_x16(t_lane + (uint32_t)(U * units), r);
-                    tmem_wait_ld();
-                    exp16(r, U * units, w);
-                    tmem_st_32x32b_x8(t_lane + (uint32_t)(U / 2 * units), w);
-                }
-                sum += sum1;
+                const float2 both = f32x2_split(sum2);
+                sum = both.x + both.y;
             }
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kPFull, g));
+            if (n + kBufs < n_items) decode(n + kBufs);                // its divisions run under the second product
             ok = mbar_wait(bar(kOFull, g), ph, abort_flag, p.dev_status, 26);
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             tc_fence_after();
             const float inv = 1.0f / sum;
-            uint32_t w[kD / 16][8];                                    // the row's kD outputs, packed
+            // A lane has a row of the output; the rows leave through shared memory (16-byte vectors, swizzled), so that a
+            // store instruction covers whole 64- or 128-byte rows instead of 16 bytes of 32 lines.
+            constexpr int kCols = Shape<kBufs, kBias>::kOutCols < kD ? Shape<kBufs, kBias>::kOutCols : kD;
+            constexpr int kVecs = kCols / 8, kRowsPerStore = 32 / kVecs;
 #pragma unroll
-            for (int half = 0; half < kD / 32; ++half) {
-                uint32_t o[2][16];
-                tmem_ld_32x32b_x16(t_lane + (uint32_t)(p.o_col + 32 * half), o[0]);
-                tmem_ld_32x32b_x16(t_lane + (uint32_t)(p.o_col + 32 * half + 16), o[1]);
+            for (int c = 0; c < kD / kCols; ++c) {
+                uint32_t o[kCols / 16][16];
+#pragma unroll
+                for (int q = 0; q < kCols / 16; ++q) tmem_ld_32x32b_x16(t_lane + (uint32_t)(p.o_col + kCols * c + 16 * q), o[q]);
                 tmem_wait_ld();
-#pragma unroll
-                for (int q = 0; q < 2; ++q)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        w[2 * half + q][j] = pack2<kBf16>(__uint_as_float(o[q][2 * j]) * inv, __uint_as_float(o[q][2 * j + 1]) * inv);
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kTmemEmpty, g));            // the half may take the S of item n + 2
-            if (row < p.tokens) {
-                uint4* dst = reinterpret_cast<uint4*>(p.out + ((size_t)img * p.tokens + row) * (size_t)p.dim + head * kHeadDim);
-#pragma unroll
-                for (int q = 0; q < kD / 16; ++q) {
-                    dst[2 * q] = make_uint4(w[q][0], w[q][1], w[q][2], w[q][3]);
-                    dst[2 * q + 1] = make_uint4(w[q][4], w[q][5], w[q][6], w[q][7]);
+                if (c == kD / kCols - 1) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kTmemEmpty, g));    // the share may take the S of item n + kBufs
                 }
+                const int sw = (kVecs == 8 ? lane : lane >> 1) & (kVecs - 1);
+#pragma unroll
+                for (int v = 0; v < kVecs; ++v) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        w[e] = pack2<kBf16>(__uint_as_float(o[v >> 1][8 * (v & 1) + 2 * e]) * inv, __uint_as_float(o[v >> 1][8 * (v & 1) + 2 * e + 1]) * inv);
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(stage_out + (uint32_t)((lane * kVecs + (v ^ sw)) * 16)),
+                                 "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                                 : "memory");
+                }
+                __syncwarp();
+                const int row0 = mt * kQRows + quarter * 32;
+                uint16_t* dst = p.out + ((size_t)img * p.tokens + row0) * (size_t)p.dim + head * kHeadDim + kCols * c;
+                uint4 w[kVecs];
+#pragma unroll
+                for (int i = 0; i < kVecs; ++i) {
+                    const int r = i * kRowsPerStore + lane / kVecs, v = lane & (kVecs - 1);
+                    const int rsw = (kVecs == 8 ? r : r >> 1) & (kVecs - 1);
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[i].x), "=r"(w[i].y), "=r"(w[i].z), "=r"(w[i].w)
+                                 : "r"(stage_out + (uint32_t)((r * kVecs + (v ^ rsw)) * 16)) : "memory");
+                }
+                uint16_t* at = dst + (size_t)(lane / kVecs) * (size_t)p.dim + 8 * (lane & (kVecs - 1));
+#pragma unroll
+                for (int i = 0; i < kVecs; ++i) {
+                    if (row0 + i * kRowsPerStore + lane / kVecs < p.tokens) *reinterpret_cast<uint4*>(at) = w[i];
+                    at += kRowsPerStore * p.dim;
+                }
+                __syncwarp();                                          // the staging rows have been read
             }
         }
     }
@@ -514,7 +609,7 @@ elsa_status make_map_qkv(CUtensorMap* map, const void* qkv, int images, int toke
 template <bool kBf16, int kD, bool kBias, int kBufs>
 elsa_status launch(const AttnParams& p, int images, int heads, cudaStream_t stream, const DeviceInfo& dev)
 {
-    constexpr int kSmemBytes = Shape<kBufs>::kSmemBytes, kThreads = Shape<kBufs>::kThreads;
+    constexpr int kSmemBytes = Shape<kBufs, kBias>::kSmemBytes, kThreads = Shape<kBufs, kBias>::kThreads;
     auto kernel = attention_kernel<kBf16, kD, kBias, kBufs>;
     static std::atomic<bool> attr_set[64];
     const int slot = dev.device & 63;
