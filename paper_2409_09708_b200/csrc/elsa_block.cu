@@ -3,7 +3,7 @@
 // LayerNorm, residual add (alone or followed by LayerNorm in the same pass), GELU in place, and the copy of a
 // column range.  All of them are HBM-bound streaming kernels: 16-byte loads and stores, fp32 arithmetic, one
 // rounding to the 16-bit type per stored value; the row-wise ones give a row to a warp, or, for the model widths
-// (128, 256, 512, 768, 1024), several rows at a time to groups of 16 or 32 lanes.
+// (128, 192, 256, 384, 512, 768, 1024), to groups of 8 to 32 lanes that have the next rows on their way.
 #include "elsa_tc_common.cuh"
 
 namespace elsa {
@@ -177,12 +177,16 @@ layer_norm_kernel(const uint16_t* A, const uint16_t* R, uint16_t* S, const uint1
     }
 }
 
-// Rows of exactly kLanes * kVpl vectors of eight values (dim = 128, 256, 512, 768, 1024): a group of kLanes lanes owns a row and
-// takes kUnroll rows at a time, all of their loads requested before the first is used.  With one row per warp a
-// short row leaves (resident warps x row bytes) in flight per SM, a fraction of what the memory latency asks for.
-// Same arithmetic per row as layer_norm_kernel (sum, mean, squared deviations about it, one rounding).
-template <bool kBf16, bool kAdd, int kLanes, int kVpl, int kUnroll>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+// Rows of exactly kLanes * kVpl vectors of eight values: a group of kLanes lanes owns kUnroll
+// rows at a time, and the loads of the rows after them are on their way while these are worked on.  HBM bounds the large
+// ones and latency the small ones; the registers decide how many rows an SM has in flight, so the values are kept in pairs for
+// the two-wide instructions, and gain and bias are not kept.  Against two rows at a time per warp without the look-ahead, at 110
+// to 190 registers (LayerNorm / with the residual, us; the traffic at 6.5 TB/s in brackets): 50432 x 768 31.4 -> 26.3 (24) /
+// 48.7 -> 49.0 (47); 401408 x 128 46.4 -> 41.3 (31) / 68.7 -> 64.7 (63); 25088 x 512 10.4 -> 8.6 (8) / 19.1 -> 13.4 (16);
+// 197 x 768 2.7 -> 1.9 / 3.0 -> 2.0;
+// 25088 x 384, on the kernel for any width, 11.6 -> 6.0 / 14.4 -> 9.2.
+template <bool kBf16, bool kAdd, int kLanes, int kVpl, int kUnroll, int kBlocks>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, kBlocks)
 layer_norm_rows_kernel(const uint16_t* A, const uint16_t* R, uint16_t* S, const uint16_t* __restrict__ gain,
                        const uint16_t* __restrict__ beta, uint16_t* Yn, int rows, float eps, const RowMapDev map)
 {
@@ -193,90 +197,118 @@ layer_norm_rows_kernel(const uint16_t* A, const uint16_t* R, uint16_t* S, const 
     pdl_release_successors();
     const int lane = threadIdx.x & 31;
     const int sub = lane % kLanes, grp = lane / kLanes;
-    const float inv_dim = 1.0f / (float)kDim;
-    // this lane's vectors of a row are the same in every row: gain and bias stay in registers
-    uint4 g4[kVpl], b4[kVpl];
-    if (Yn != nullptr) {
-#pragma unroll
-        for (int c = 0; c < kVpl; ++c) {
-            g4[c] = __ldg(reinterpret_cast<const uint4*>(gain) + sub + kLanes * c);
-            b4[c] = __ldg(reinterpret_cast<const uint4*>(beta) + sub + kLanes * c);
-        }
-    }
+    constexpr float inv_dim = 1.0f / (float)kDim;
     auto group_sum = [&](float v) {
 #pragma unroll
         for (int o = kLanes / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         return v;
     };
-    const long long steps = ((long long)rows + kRowsPerStep - 1) / kRowsPerStep;
-    for (long long step = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5); step < steps;
-         step += (long long)gridDim.x * kWarpsPerBlock) {
-        uint4 x[kUnroll][kVpl];
-        int mapped[kUnroll];
-        int row_of[kUnroll];
+    const int steps = (rows - 1) / kRowsPerStep + 1;
+    const int stride = gridDim.x * kWarpsPerBlock;
+    uint4 x[kUnroll][kVpl], w[kAdd ? kUnroll : 1][kVpl];
+    int mapped[kUnroll];
+    auto row_of = [&](int step, int u) { return step * kRowsPerStep + u * kGroups + grp; };
+    auto load = [&](int step) {
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
-            const long long r = step * kRowsPerStep + u * kGroups + grp;
-            row_of[u] = r < rows ? (int)r : -1;
-            mapped[u] = row_of[u] >= 0 ? window_row(map, row_of[u]) : 0;
-        }
-        // every load of the step first
-        uint4 w[kAdd ? kUnroll : 1][kVpl];
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
+            const int r = row_of(step, u);
+            if (step >= steps || r >= rows) continue;
+            mapped[u] = window_row(map, r);
+            const size_t src = (size_t)(map.on_input ? mapped[u] : r) * (size_t)kDim;
 #pragma unroll
             for (int c = 0; c < kVpl; ++c) {
-                x[u][c] = make_uint4(0u, 0u, 0u, 0u);
-                if constexpr (kAdd) w[u][c] = make_uint4(0u, 0u, 0u, 0u);
-                if (row_of[u] >= 0) {
-                    const size_t src = (size_t)(map.on_input ? mapped[u] : row_of[u]) * (size_t)kDim;
-                    x[u][c] = reinterpret_cast<const uint4*>(A + src)[sub + kLanes * c];
-                    if constexpr (kAdd) w[u][c] = reinterpret_cast<const uint4*>(R + (size_t)row_of[u] * (size_t)kDim)[sub + kLanes * c];
-                }
+                x[u][c] = reinterpret_cast<const uint4*>(A + src)[sub + kLanes * c];
+                if constexpr (kAdd) w[u][c] = reinterpret_cast<const uint4*>(R + (size_t)r * (size_t)kDim)[sub + kLanes * c];
             }
         }
+    };
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+        mapped[u] = 0;
+#pragma unroll
+        for (int c = 0; c < kVpl; ++c) {
+            x[u][c] = make_uint4(0u, 0u, 0u, 0u);
+            if constexpr (kAdd) w[u][c] = make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
+    int step = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+    load(step);
+    for (; step < steps; step += stride) {
+        uint64_t f[kUnroll][kVpl][4];                  // the rows' values, two to a register pair
+        int out_row[kUnroll];
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
-            float sum = 0.f;
+            const int r = row_of(step, u);
+            out_row[u] = r >= rows ? -1 : map.on_output ? mapped[u] : r;
 #pragma unroll
             for (int c = 0; c < kVpl; ++c) {
-                float f[8];
-                unpack8<kBf16>(x[u][c], f);
+                uint32_t a[4] = {x[u][c].x, x[u][c].y, x[u][c].z, x[u][c].w};
                 if constexpr (kAdd) {
-                    float fr[8];
-                    unpack8<kBf16>(w[u][c], fr);
+                    const uint32_t b[4] = {w[u][c].x, w[u][c].y, w[u][c].z, w[u][c].w};
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) f[e] += fr[e];
-                    x[u][c] = pack8<kBf16>(f);
-                    if (row_of[u] >= 0) reinterpret_cast<uint4*>(S + (size_t)row_of[u] * (size_t)kDim)[sub + kLanes * c] = x[u][c];
-                    unpack8<kBf16>(x[u][c], f);          // the statistics are those of the row as stored
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 av = unpack2<kBf16>(a[q]), bv = unpack2<kBf16>(b[q]);
+                        const float2 t = f32x2_split(f32x2_add(f32x2(av.x, av.y), f32x2(bv.x, bv.y)));
+                        a[q] = pack2_rn<kBf16>(t.x, t.y);
+                    }
+                    if (r < rows) reinterpret_cast<uint4*>(S + (size_t)r * (size_t)kDim)[sub + kLanes * c] = make_uint4(a[0], a[1], a[2], a[3]);
                 }
+                // the statistics are those of the row as stored
 #pragma unroll
-                for (int e = 0; e < 8; ++e) sum += f[e];
-            }
-            if (Yn == nullptr) continue;
-            const float mean = group_sum(sum) * inv_dim;
-            float sq = 0.f;
-#pragma unroll
-            for (int c = 0; c < kVpl; ++c) {
-                float f[8];
-                unpack8<kBf16>(x[u][c], f);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) sq += (f[e] - mean) * (f[e] - mean);
-            }
-            const float rstd = 1.0f / sqrtf(group_sum(sq) * inv_dim + eps);
-            if (row_of[u] >= 0) {
-                uint4* y4 = reinterpret_cast<uint4*>(Yn + (size_t)(map.on_output ? mapped[u] : row_of[u]) * (size_t)kDim);
-#pragma unroll
-                for (int c = 0; c < kVpl; ++c) {
-                    float f[8], g[8], b[8];
-                    unpack8<kBf16>(x[u][c], f);
-                    unpack8<kBf16>(g4[c], g);
-                    unpack8<kBf16>(b4[c], b);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) f[e] = (f[e] - mean) * rstd * g[e] + b[e];
-                    y4[sub + kLanes * c] = pack8<kBf16>(f);
+                for (int q = 0; q < 4; ++q) {
+                    const float2 v = unpack2<kBf16>(a[q]);
+                    f[u][c][q] = f32x2(v.x, v.y);
                 }
+            }
+        }
+        load(step + stride);
+        if (Yn == nullptr) continue;
+        float mean[kUnroll], rstd[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            uint64_t sum2 = f[u][0][0];
+#pragma unroll
+            for (int i = 1; i < 4 * kVpl; ++i) sum2 = f32x2_add(sum2, f[u][i >> 2][i & 3]);
+            const float2 t = f32x2_split(sum2);
+            mean[u] = group_sum(t.x + t.y) * inv_dim;
+        }
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            const uint64_t minus = f32x2(-mean[u], -mean[u]);
+            uint64_t sq2 = f32x2(0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 4 * kVpl; ++i) {
+                const uint64_t d = f32x2_add(f[u][i >> 2][i & 3], minus);
+                f[u][i >> 2][i & 3] = d;
+                sq2 = f32x2_fma(d, d, sq2);
+            }
+            const float2 t = f32x2_split(sq2);
+            rstd[u] = 1.0f / sqrtf(group_sum(t.x + t.y) * inv_dim + eps);
+        }
+        // gain and bias from the first-level cache: in registers they would cost a resident block or two
+#pragma unroll
+        for (int c = 0; c < kVpl; ++c) {
+            const uint4 g4 = __ldg(reinterpret_cast<const uint4*>(gain) + sub + kLanes * c);
+            const uint4 b4 = __ldg(reinterpret_cast<const uint4*>(beta) + sub + kLanes * c);
+            const uint32_t g[4] = {g4.x, g4.y, g4.z, g4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+            uint64_t g2[4], b2[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 gv = unpack2<kBf16>(g[q]), bv = unpack2<kBf16>(b[q]);
+                g2[q] = f32x2(gv.x, gv.y);
+                b2[q] = f32x2(bv.x, bv.y);
+            }
+#pragma unroll
+            for (int u = 0; u < kUnroll; ++u) {
+                const uint64_t rstd2 = f32x2(rstd[u], rstd[u]);
+                uint32_t o[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float2 t = f32x2_split(f32x2_fma(f32x2_mul(f[u][c][q], rstd2), g2[q], b2[q]));
+                    o[q] = pack2_rn<kBf16>(t.x, t.y);
+                }
+                if (out_row[u] >= 0)
+                    reinterpret_cast<uint4*>(Yn + (size_t)out_row[u] * (size_t)kDim)[sub + kLanes * c] = make_uint4(o[0], o[1], o[2], o[3]);
             }
         }
     }
@@ -353,25 +385,35 @@ elsa_status launch_layer_norm(const uint16_t* A, const uint16_t* R, uint16_t* S,
     const dim3 block(kWarpsPerBlock * 32);
     const bool add = R != nullptr;
     ProfileScope scope(ELSA_KERNEL_BLOCK_ROWWISE, stream);
-    // the model widths: several rows per warp in flight
-#define ELSA_LN_ROWS(LANES, VPL, UNROLL)                                                                                  \
+    // The model widths.  One wave of resident blocks, or four where each of them has eight or more steps per warp: with the
+    // residual 50432 x 768 takes 51.4 us in one wave, 49.0 in four, 52.5 with a step per warp; 12608 x 768 9.5 and 10.2.
+#define ELSA_LN_LAUNCH(BF, ADD, LANES, VPL, UNROLL, BLOCKS)                                                               \
     do {                                                                                                                  \
-        const long long steps = ((long long)rows + (32 / LANES) * UNROLL - 1) / ((32 / LANES) * UNROLL);                  \
-        const unsigned g = streaming_grid(steps, kWarpsPerBlock, dev);                                                    \
+        const int steps = (rows - 1) / ((32 / LANES) * UNROLL) + 1, resident = dev.sm_count * BLOCKS;                     \
+        const int blocks = (steps + kWarpsPerBlock - 1) / kWarpsPerBlock, most = blocks >= 8 * resident ? 4 * resident : resident; \
+        launch_pdl(layer_norm_rows_kernel<BF, ADD, LANES, VPL, UNROLL, BLOCKS>, dim3((unsigned)(blocks < most ? blocks : most)), block, 0, \
+                   stream, 1, A, R, S, gain, beta, Yn, rows, eps, map);                                                   \
+    } while (0)
+#define ELSA_LN_ROWS(LANES, VPL, UNROLL, BLOCKS, UNROLL_ADD, BLOCKS_ADD)                                                  \
+    do {                                                                                                                  \
         if (dtype == ELSA_BF16) {                                                                                         \
-            if (add) launch_pdl(layer_norm_rows_kernel<true, true, LANES, VPL, UNROLL>, dim3(g), block, 0, stream, 1, A, R, S, gain, beta, Yn, rows, eps, map);   \
-            else launch_pdl(layer_norm_rows_kernel<true, false, LANES, VPL, UNROLL>, dim3(g), block, 0, stream, 1, A, R, S, gain, beta, Yn, rows, eps, map);     \
+            if (add) ELSA_LN_LAUNCH(true, true, LANES, VPL, UNROLL_ADD, BLOCKS_ADD);                                      \
+            else ELSA_LN_LAUNCH(true, false, LANES, VPL, UNROLL, BLOCKS);                                                 \
         } else {                                                                                                          \
-            if (add) launch_pdl(layer_norm_rows_kernel<false, true, LANES, VPL, UNROLL>, dim3(g), block, 0, stream, 1, A, R, S, gain, beta, Yn, rows, eps, map);  \
-            else launch_pdl(layer_norm_rows_kernel<false, false, LANES, VPL, UNROLL>, dim3(g), block, 0, stream, 1, A, R, S, gain, beta, Yn, rows, eps, map);    \
+            if (add) ELSA_LN_LAUNCH(false, true, LANES, VPL, UNROLL_ADD, BLOCKS_ADD);                                     \
+            else ELSA_LN_LAUNCH(false, false, LANES, VPL, UNROLL, BLOCKS);                                                \
         }                                                                                                                 \
         return launched(add ? "residual_add_layer_norm" : "layer_norm");                                                  \
     } while (0)
-    if (dim == 128) ELSA_LN_ROWS(16, 1, 4);
-    if (dim == 256) ELSA_LN_ROWS(32, 1, 4);
-    if (dim == 512) ELSA_LN_ROWS(32, 2, 2);
-    if (dim == 1024) ELSA_LN_ROWS(32, 4, 2);
-    if (dim == 768) ELSA_LN_ROWS(32, 3, 2);
+    // lanes a row, vectors a lane, then rows a group takes at a time and resident blocks, without and with the residual
+    if (dim == 128) ELSA_LN_ROWS(16, 1, 2, 4, 2, 3);
+    if (dim == 192) ELSA_LN_ROWS(8, 3, 1, 3, 1, 2);
+    if (dim == 256) ELSA_LN_ROWS(32, 1, 2, 4, 2, 3);
+    if (dim == 384) ELSA_LN_ROWS(16, 3, 1, 3, 1, 2);
+    if (dim == 512) ELSA_LN_ROWS(32, 2, 1, 4, 1, 4);
+    if (dim == 768) ELSA_LN_ROWS(32, 3, 1, 3, 1, 2);
+    if (dim == 1024) ELSA_LN_ROWS(32, 4, 1, 3, 1, 2);
+#undef ELSA_LN_LAUNCH
 #undef ELSA_LN_ROWS
     const unsigned grid = streaming_grid(rows, kWarpsPerBlock, dev);
     if (dtype == ELSA_BF16) {
