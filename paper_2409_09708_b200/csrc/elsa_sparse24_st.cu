@@ -13,7 +13,7 @@
 // activations only (three stages of 256 of K).  While one slot is multiplied the next ones are being
 // written and fetched: a load from L2 takes 1.5-2.5 us under this traffic, several chunk times.
 //
-// A CTA pair owns a tile of 256 features x 224 token rows (one accumulator of 224 columns beside the
+// A CTA pair owns a tile of 256 features x up to 224 token rows (one accumulator of 224 columns beside the
 // four slots of 72); tiles of all layers of a launch form one sequence walked with the stride of the
 // pairs, feature blocks fastest, so that the pairs that share activation rows read them at the same
 // time (once from HBM, then from L2).  With a reduction this long the epilogue's share is small.
@@ -37,13 +37,13 @@ namespace {
 
 constexpr int kFeatPerCta = 128;   // weight rows per CTA = TMEM lanes
 constexpr int kPairFeat = 256;     // MMA M over the pair
-constexpr int kRowTile = 224;      // token rows per pair tile = MMA N
-constexpr int kRowsPerCta = kRowTile / 2;
+constexpr int kMaxRowTile = 224;   // token rows per pair tile = MMA N, at most and at least (see pick_row_tile)
+constexpr int kMinRowTile = 128;
 constexpr int kChunkK = 256;       // logical K per weight slot = per activation stage
 constexpr int kSpUmmaK = 32;
 constexpr int kSlots = 4;
 constexpr int kSlotCols = kChunkK / 4 + kChunkK / 32;   // 64 columns of values + 8 of metadata
-constexpr int kSlotCol0 = kRowTile;                     // slots follow the accumulator
+constexpr int kSlotCol0 = kMaxRowTile;                  // slots follow the accumulator
 constexpr int kTmemCols = 512;
 constexpr int kStages = 3;
 constexpr int kEpiParts = 2;       // epilogue warps per TMEM lane quarter
@@ -53,16 +53,17 @@ constexpr int kLoaderParts = 2;   // loader warps per lane quarter, taking every
 constexpr int kLoaderWarps = 4 * kLoaderParts;
 constexpr int kThreads = (kLoaderWarp0 + kLoaderWarps) * 32;
 constexpr int kStepCols = 16;      // token rows per tcgen05.ld / pair of stmatrix
-constexpr int kStepsPerWarp = kRowTile / kStepCols / kEpiParts;   // 7
+constexpr int kStepsPerWarp = kMaxRowTile / kStepCols / kEpiParts;   // 7 at most
 constexpr int kRoundSteps = 4;     // steps an epilogue warp holds in registers at a time
 constexpr int kRounds = (kStepsPerWarp + kRoundSteps - 1) / kRoundSteps;
-constexpr int kStageBytes = (kChunkK / 64) * kRowsPerCta * 128;   // 64 KB: four quarters of 128 rows x 128 bytes
+constexpr int kStageBytes = (kChunkK / 64) * (kMaxRowTile / 2) * 128;   // 56 KB: four quarters of 112 rows x 128 bytes
 constexpr int kStagingBytes = 2 * kStepCols * 64;                 // per epilogue warp: two buffers of 16 rows x 32 features
 constexpr int kStagingTotal = kEpiWarps * kStagingBytes;
 constexpr int kBarrierBytes = 512;
 
-static_assert(kRowTile + kSlots * kSlotCols <= kTmemCols, "accumulator and weight slots fit tensor memory");
-static_assert(kStepsPerWarp * kEpiParts * kStepCols == kRowTile, "the epilogue warps cover the tile exactly");
+static_assert(kMaxRowTile + kSlots * kSlotCols <= kTmemCols, "accumulator and weight slots fit tensor memory");
+static_assert(kStepsPerWarp * kEpiParts * kStepCols == kMaxRowTile, "the epilogue warps cover the tile exactly");
+static_assert(kMinRowTile / kStepCols / kEpiParts >= kRoundSteps && kRounds == 2, "a warp has a whole first round");
 static_assert(kLoaderWarp0 % 4 == 2, "warp & 3 must walk the lane quarters for epilogue and loader warps alike");
 
 // One layer of a launch; lives in kernel-parameter space.
@@ -86,6 +87,7 @@ struct StGroup {
     StLayer layer[kMaxLayers];
     int n_layers;
     int num_tiles;
+    int nt;            // token rows per tile, a multiple of 16
     uint32_t idesc;
     uint32_t* dev_status;
 };
@@ -158,7 +160,7 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
             while (cur + 1 < p.n_layers && tile >= p.layer[cur + 1].tile_begin) ++cur;
             const StLayer& L = p.layer[cur];
             const int t = tile - L.tile_begin;
-            const int r0 = (t / L.tiles_f) * kRowTile + (int)cta_rank * kRowsPerCta;
+            const int r0 = (t / L.tiles_f) * p.nt + (int)cta_rank * (p.nt >> 1);
             for (int c = 0; c < L.num_chunks; ++c) {
                 ok = mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.dev_status, 1);
                 ok = __all_sync(0xFFFFFFFFu, ok);
@@ -166,7 +168,7 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
                 const uint32_t dst = smem_base + (uint32_t)(stage * kStageBytes);
                 const uint32_t bar = mapa_shared(full_bar + 8 * stage, 0);
                 if (elected) {
-                    if (cta_rank == 0) mbar_arrive_expect_tx(full_bar + 8 * stage, (uint32_t)(2 * kStageBytes));
+                    if (cta_rank == 0) mbar_arrive_expect_tx(full_bar + 8 * stage, (uint32_t)(2 * (kChunkK / 64) * (p.nt >> 1) * 128));
                     tma_load_3d_pair(dst, &L.map_x, bar, 0, r0, (kChunkK / 64) * c);
                 }
                 __syncwarp();
@@ -182,7 +184,7 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
             const uint32_t elected = elect_one() ? 1u : 0u;
             const uint32_t tmem_u = __reduce_or_sync(0xFFFFFFFFu, tmem_base);
             const uint32_t idesc = p.idesc;
-            constexpr uint32_t quarter = (uint32_t)(kRowsPerCta * 128) >> 4;   // descriptor units between K quarters
+            const uint32_t quarter = (uint32_t)((p.nt >> 1) * 128) >> 4;   // descriptor units between K quarters
             int stage = 0, slot = 0;
             uint32_t phase = 0, a_phase = 0, acc_phase = 0;
             bool ok = true;
@@ -326,8 +328,10 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
         // lane t holds feature 8 * (t % 4) + t / 4 of the quarter's 32 (see elsa_sparse24_ws.cu)
         const int feat_in_quarter = 8 * (lane & 3) + (lane >> 2);
         const uint32_t st_off = (uint32_t)((2 * (lane >> 3) + (lane & 1)) * 64 + ((lane & 7) >> 1) * 16);
-        // this warp's run of token columns: kStepsPerWarp steps of 16 from first_step
-        const int first_step = part * kStepsPerWarp;
+        // this warp's run of token columns: my_steps steps of 16 from first_step.  It reads and converts kStepsPerWarp of
+        // them whatever the tile (tests around them cost registers: 60 us for 36 at 25088 x 512 -> 2048) and stores its own.
+        const int steps = p.nt / kStepCols;
+        const int first_step = part == 0 ? 0 : (steps + 1) >> 1, my_steps = part == 0 ? (steps + 1) >> 1 : steps >> 1;
         uint32_t store_count = 0;
 
         int cur = 0;
@@ -336,7 +340,7 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
             const StLayer& L = p.layer[cur];
             const int t = tile - L.tile_begin;
             const int f0 = ((t % L.tiles_f) * 2 + (int)cta_rank) * kFeatPerCta + q * 32;
-            const int row0 = (t / L.tiles_f) * kRowTile + first_step * kStepCols;
+            const int row0 = (t / L.tiles_f) * p.nt + first_step * kStepCols;
             const int f = f0 + feat_in_quarter;
             const int l_rows = L.rows, l_out = L.out;
             const float bias_f = (L.bias != nullptr && f < l_out) ? bias_to_float<kBf16>(__ldg(L.bias + f)) : 0.f;
@@ -361,14 +365,14 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    if (f0 < l_out && row0 + s * kStepCols < l_rows) tma_store_2d(&L.map_y, buf, f0, row0 + s * kStepCols);
+                    if (f0 < l_out && s < my_steps && row0 + s * kStepCols < l_rows) tma_store_2d(&L.map_y, buf, f0, row0 + s * kStepCols);
                     bulk_commit_group();
                 }
                 ++store_count;
             };
 #pragma unroll
             for (int i = 0; i < kRoundSteps; ++i)
-                if (i < kStepsPerWarp) tmem_ld_32x32b_x16(t_col + (uint32_t)(i * kStepCols), rr[i]);
+                tmem_ld_32x32b_x16(t_col + (uint32_t)(i * kStepCols), rr[i]);
             tmem_wait_ld();
 #pragma unroll
             for (int rd = 0; rd < kRounds; ++rd) {
@@ -416,6 +420,23 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
     }
 }
 
+// Token rows per tile.  A tile's time goes with what it reads: nt rows of activations and 256 features of weight values and
+// metadata, together as much as 144 rows; the launch takes as many of these as its busiest pair has tiles.  With 224 rows
+// and with the choice, us: 3152 x 3072 -> 768 13.6, 12.2 (144); 6272 x 4096 -> 1024 26.3, 25.1 (176); 12608 x 3072 -> 768
+// 32.8, 32.3 (176): large launches wait for L2 as a whole, and a pair without a tile leaves its share to the others.
+int pick_row_tile(const SparseJob* jobs, int n, int pairs)
+{
+    int best = kMaxRowTile;
+    long long best_cost = -1;
+    for (int nt = kMaxRowTile; nt >= kMinRowTile; nt -= kStepCols) {
+        long long tiles = 0;
+        for (int i = 0; i < n; ++i) tiles += (long long)((jobs[i].out + kPairFeat - 1) / kPairFeat) * ((jobs[i].rows + nt - 1) / nt);
+        const long long cost = (tiles + pairs - 1) / pairs * (nt + 144);
+        if (best_cost < 0 || cost < best_cost) { best = nt; best_cost = cost; }
+    }
+    return best;
+}
+
 template <bool kBf16, int kMaxLayers, bool kAct>
 elsa_status launch_st_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint32_t* dev_status, cudaStream_t stream,
                             const DeviceInfo& dev)
@@ -454,6 +475,7 @@ elsa_status launch_st_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
     static StGroup<kMaxLayers> g;   // host staging of the kernel parameters
     static std::mutex g_mutex;
     std::lock_guard<std::mutex> lock(g_mutex);
+    const int nt = pick_row_tile(jobs, n, max_pairs[slot].load(std::memory_order_acquire));
     int tile_begin = 0;
     for (int i = 0; i < n; ++i) {
         const SparseJob& j = jobs[i];
@@ -462,7 +484,7 @@ elsa_status launch_st_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
         L.rows = j.rows; L.out = j.out; L.in = j.in;
         L.tiles_f = (j.out + kPairFeat - 1) / kPairFeat;
         L.tile_begin = tile_begin;
-        tile_begin += L.tiles_f * ((j.rows + kRowTile - 1) / kRowTile);
+        tile_begin += L.tiles_f * ((j.rows + nt - 1) / nt);
         L.num_chunks = (j.in + kChunkK - 1) / kChunkK;
         L.num_k_blocks = j.in / 128;
         L.bias = j.bias;
@@ -470,17 +492,18 @@ elsa_status launch_st_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
         L.a_img = (const uint8_t*)j.workspace;
         L.meta = (const uint8_t*)j.workspace + sp24_meta_offset(j.out, j.in);
         elsa_status st;
-        if ((st = make_map_x_quarters(&L.map_x, j.X, (uint64_t)j.in, (uint64_t)j.rows, kRowsPerCta, kChunkK / 64)) != ELSA_OK) return st;
+        if ((st = make_map_x_quarters(&L.map_x, j.X, (uint64_t)j.in, (uint64_t)j.rows, (uint32_t)(nt / 2), kChunkK / 64)) != ELSA_OK) return st;
         if ((st = make_map_2d(&L.map_y, j.Y, (uint64_t)j.out, (uint64_t)j.rows, 32, kStepCols, CU_TENSOR_MAP_SWIZZLE_NONE,
                               "Y")) != ELSA_OK)
             return st;
     }
     g.n_layers = n;
     g.num_tiles = tile_begin;
+    g.nt = nt;
     g.dev_status = dev_status;
     const uint32_t fmt = dtype == ELSA_BF16 ? 1u : 0u;
     // sparse flag, fp32 accumulate, A and B of type fmt, K-major, N = 256, M = 256 over the pair
-    g.idesc = (1u << 2) | (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(kRowTile >> 3) << 17) |
+    g.idesc = (1u << 2) | (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(nt >> 3) << 17) |
               ((uint32_t)(kPairFeat >> 4) << 24);
 
     const int pairs = g.num_tiles < max_pairs[slot].load(std::memory_order_acquire) ? g.num_tiles : max_pairs[slot].load(std::memory_order_acquire);
