@@ -115,7 +115,7 @@ nm_compress_i8_kernel(const int8_t* __restrict__ W, int out, int in, int N, int8
     }
 }
 
-// One thread rebuilds one group: N bytes scattered to their positions, zero elsewhere.
+// Any level: one thread rebuilds one group: N bytes scattered to their positions, zero elsewhere.
 template <int M>
 __global__ void __launch_bounds__(256)
 nm_unpack_i8_kernel(const int8_t* __restrict__ vals, const uint32_t* __restrict__ idx, int out, int in, int N,
@@ -160,6 +160,56 @@ nm_unpack_i8_kernel(const int8_t* __restrict__ vals, const uint32_t* __restrict_
                                               ((uint32_t)w[4 * q + 3] << 24);
 }
 
+// The common levels (N <= 4, the M values of a thread's groups in one or two words): 16 consecutive positions per thread.  The
+// index fields of a group become the selectors of byte permutes that place its N kept bytes among zeros.  A launch is
+// a megabyte or two, so instructions and latency bound it: 12608 x 768 -> 3072 at 4:8 with the image a group per thread,
+// built byte by byte, 36.9 us, 34.2 with this; the four linears of a DeiT-B block 116 -> 106.
+template <int M, int N>
+__global__ void __launch_bounds__(256)
+nm_unpack16_i8_kernel(const int8_t* __restrict__ vals, const uint32_t* __restrict__ idx, int8_t* __restrict__ Wm, uint32_t units,
+                      uint32_t units_per_row, uint32_t magic, int words_per_row)
+{
+    constexpr int B = M == 4 ? 2 : 3, kGroups = 16 / M, kCount = kGroups * N;      // values and fields of a thread
+    static_assert((M == 4 && N <= 2) || (M == 8 && (N == 1 || N == 2 || N == 4)), "at most eight values");
+    pdl_wait_for_predecessors();
+    pdl_release_successors();
+    const uint32_t unit = blockIdx.x * 256u + threadIdx.x;
+    if (unit >= units) return;
+    uint32_t o = __umulhi(unit, magic), u = unit - o * units_per_row;      // magic = floor(2^32 / units_per_row): one short at most
+    if (u >= units_per_row) { ++o; u -= units_per_row; }
+    uint32_t v[2] = {0u, 0u};
+    const int8_t* at = vals + (size_t)unit * kCount;                       // rows hold units_per_row * kCount values
+    if constexpr (kCount == 8) {
+        const uint2 t = __ldg(reinterpret_cast<const uint2*>(at));
+        v[0] = t.x; v[1] = t.y;
+    } else if constexpr (kCount == 4) {
+        v[0] = __ldg(reinterpret_cast<const uint32_t*>(at));
+    } else {
+        v[0] = __ldg(reinterpret_cast<const uint16_t*>(at));
+    }
+    const uint32_t* row = idx + (size_t)o * (size_t)words_per_row;
+    const uint32_t bit0 = u * (uint32_t)(kCount * B), w0 = bit0 >> 5, sh = bit0 & 31u;
+    const uint32_t lo = __ldg(row + w0), hi = sh + (uint32_t)(kCount * B) > 32u ? __ldg(row + w0 + 1) : 0u;
+    const uint32_t fields = __funnelshift_r(lo, hi, sh);
+    uint32_t w[4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {                                          // eight positions: their kept bytes are in one word
+        constexpr int kHere = kCount / 2;                                  // 1, 2 or 4
+        const uint32_t bytes = kCount == 8 ? v[h] : v[0] >> (8 * kHere * h);
+        uint32_t sel = 0x44444444u;                                        // a zero everywhere
+#pragma unroll
+        for (int t = 0; t < kHere; ++t) {
+            const int f = h * kHere + t;
+            uint32_t pos = (fields >> (f * B)) & (uint32_t)(M - 1);
+            if (M == 4 && t >= N) pos += 4u;
+            sel ^= (uint32_t)(4 ^ t) << (4u * pos);
+        }
+        w[2 * h] = prmt(bytes, 0u, sel & 0xFFFFu);
+        w[2 * h + 1] = prmt(bytes, 0u, sel >> 16);
+    }
+    reinterpret_cast<uint4*>(Wm)[unit] = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 elsa_status check_level_i8(int out, int in, int N, int M)
@@ -196,6 +246,15 @@ elsa_status launch_unpack_i8(const int8_t* vals, const uint32_t* idx, int out, i
     const unsigned grid = (unsigned)((total + 255) / 256);
     const int wpr = (int)index_words_per_row(in, N, M);
     ProfileScope scope(ELSA_KERNEL_INT8_FORMAT, stream);
+    const long long units = (long long)out * (in / 16);
+    if (units < (1ll << 32) && ((M == 4 && N <= 2) || (M == 8 && (N <= 2 || N == 4)))) {
+        auto* kernel = M == 4 ? (N == 1 ? nm_unpack16_i8_kernel<4, 1> : nm_unpack16_i8_kernel<4, 2>)
+                       : N == 1 ? nm_unpack16_i8_kernel<8, 1> : N == 2 ? nm_unpack16_i8_kernel<8, 2> : nm_unpack16_i8_kernel<8, 4>;
+        const uint32_t upr = (uint32_t)in / 16;
+        const uint32_t magic = upr == 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / upr);
+        launch_pdl(kernel, dim3((unsigned)((units + 255) / 256)), dim3(256), 0, stream, 1, vals, idx, Wm, (uint32_t)units, upr, magic, wpr);
+        return launched("nm_unpack_i8");
+    }
     if (M == 4) launch_pdl(nm_unpack_i8_kernel<4>, dim3(grid), dim3(256), 0, stream, 1, vals, idx, out, in, N, Wm, wpr);
     else if (M == 8) launch_pdl(nm_unpack_i8_kernel<8>, dim3(grid), dim3(256), 0, stream, 1, vals, idx, out, in, N, Wm, wpr);
     else launch_pdl(nm_unpack_i8_kernel<16>, dim3(grid), dim3(256), 0, stream, 1, vals, idx, out, in, N, Wm, wpr);
