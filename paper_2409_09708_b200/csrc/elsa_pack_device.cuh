@@ -256,8 +256,8 @@ struct PackedUnit {
 // NC: the level's N as a compile-time constant (0 = take `N_runtime`).  N < M.  Reads go past L1, which is not known to be
 // clean of older contents while a predecessor kernel still runs (see `early` in elsa_linear_small.cu).
 template <int M, int NC>
-__device__ __forceinline__ PackedUnit load_packed_unit(const uint16_t* __restrict__ vals_row, const uint32_t* __restrict__ idx_row,
-                                                       int N_runtime, int unit)
+__device__ __forceinline__ PackedUnit load_packed_values(const uint16_t* __restrict__ v, const uint32_t* __restrict__ idx_row,
+                                                         int N_runtime, int unit)
 {
     static_assert(M == 4 || M == 8, "groups of 16 hold two units: expand_unit16");
     constexpr int B = M == 4 ? 2 : 3;
@@ -265,7 +265,6 @@ __device__ __forceinline__ PackedUnit load_packed_unit(const uint16_t* __restric
     const int count = (8 / M) * N;              // values of the unit
     PackedUnit p;
     p.v[0] = p.v[1] = p.v[2] = p.v[3] = 0u;
-    const uint16_t* v = vals_row + (size_t)unit * count;
     if ((count & 3) == 0) {                     // 4 values at most (8 would be the dense level)
         const uint2 t = __ldcg(reinterpret_cast<const uint2*>(v));
         p.v[0] = t.x; p.v[1] = t.y;
@@ -283,6 +282,14 @@ __device__ __forceinline__ PackedUnit load_packed_unit(const uint16_t* __restric
     const uint32_t hi = (sh + count * B > 32) ? __ldcg(idx_row + w0 + 1) : 0u;
     p.fields = __funnelshift_r(lo, hi, sh);
     return p;
+}
+
+// The same from the start of the row's values.
+template <int M, int NC>
+__device__ __forceinline__ PackedUnit load_packed_unit(const uint16_t* __restrict__ vals_row, const uint32_t* __restrict__ idx_row,
+                                                       int N_runtime, int unit)
+{
+    return load_packed_values<M, NC>(vals_row + (size_t)unit * (size_t)((8 / M) * (NC ? NC : N_runtime)), idx_row, N_runtime, unit);
 }
 
 // shl that gives 0 for shifts of 32 and more (negative ones included)
@@ -362,13 +369,28 @@ __device__ __forceinline__ uint4 expand_unit16(const uint16_t* __restrict__ vals
     if (sh + 4 * N > 32) fields |= (unsigned long long)__ldcg(idx_row + w0 + 1) << 32;
     fields >>= sh;
     if (sh + 4 * N > 64) fields |= (unsigned long long)__ldcg(idx_row + w0 + 2) << (64 - sh);
+    // every value is asked for before the first is placed (one at a time each waited for the one before)
     const uint16_t* v = vals_row + (size_t)g * N;
+    uint32_t w[8];
+    if ((N & 1) == 0) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) w[q] = 2 * q < N ? __ldcg(reinterpret_cast<const uint32_t*>(v) + q) : 0u;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            w[q] = 2 * q < N ? (uint32_t)__ldcg(v + 2 * q) : 0u;
+            if (2 * q + 1 < N) w[q] |= (uint32_t)__ldcg(v + 2 * q + 1) << 16;
+        }
+    }
     unsigned long long lo = 0, hi = 0;
-    for (int t = 0; t < N; ++t) {
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+        if (t >= N) break;
         const uint32_t pos = (uint32_t)(fields >> (4 * t)) & 15u;
-        if ((int)(pos >> 3) != (unit & 1)) continue;
-        const unsigned long long x = (unsigned long long)__ldcg(v + t) << (16u * (pos & 3u));
-        if (pos & 4u) hi |= x; else lo |= x;
+        const unsigned long long x = (unsigned long long)((w[t >> 1] >> (16 * (t & 1))) & 0xFFFFu) << (16u * (pos & 3u));
+        if ((int)(pos >> 3) == (unit & 1)) {
+            if (pos & 4u) hi |= x; else lo |= x;
+        }
     }
     return make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
 }

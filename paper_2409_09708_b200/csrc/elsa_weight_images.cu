@@ -8,7 +8,9 @@
 // images are a few MB, so what bounds a launch is latency, and what bounds a large table is the traffic through L2.
 // Against one thread per 8 or 16 positions with a loop over the kept values: image and GEMM of 3152 x 768 -> 3072 at 2:4
 // 20.6 -> 17.1 us back to back (the 2-of-4 image about 6 -> 2.5), of 197 x 768 -> 2304 on the dense image 8.2 -> 7.5; the
-// four images of a DeiT-B block in one launch 22 -> 12.6 us between events.
+// four images of a DeiT-B block in one launch 22 -> 12.6 us between events.  A thread has four dense units, or one where
+// those would be fewer than two blocks for an SM: 256 x 256 2.1 -> 1.5 us, 768 x 768 2.3 -> 1.7, 512 x 2048 at 8:16
+// 4.6 -> 3.1; from there up both take the same.
 
 #include "elsa_pack_device.cuh"
 
@@ -16,7 +18,7 @@ namespace elsa {
 namespace {
 
 constexpr int kImageThreads = 256;
-constexpr int kUnitsPerThread = 4;        // dense images: units of 8 positions
+constexpr int kMostUnits = 4;             // dense images: units of 8 positions per thread, or one (see launch_images)
 
 struct ImageItem {
     const uint16_t* src;
@@ -25,6 +27,7 @@ struct ImageItem {
     uint16_t* meta;
     int first_block;
     int out, in, N, M, words_per_row, kind, layout;
+    uint32_t magic;                       // floor(2^32 / d) of the division that finds a thread's row, see split_by
     int k_blocks, steps;                  // 2-of-4 forms: metadata blocks along K, K steps of 32 per block (2 or 4)
 };
 
@@ -34,35 +37,47 @@ struct ImageTable {
     int n;
 };
 
+// n / d and n % d for any 32-bit n: the product's high half is one short at most.
+__device__ __forceinline__ uint32_t split_by(uint32_t n, uint32_t d, uint32_t magic, uint32_t& rest)
+{
+    uint32_t q = __umulhi(n, magic);
+    rest = n - q * d;
+    if (rest >= d) { ++q; rest -= d; }
+    return q;
+}
+
 // ---------------------------------------------------------------- dense images
 
-template <typename Raw, typename Load, typename Finish>
+// load(unit, row, unit of the row)
+template <typename Raw, int kUnits, typename Load, typename Finish>
 __device__ __forceinline__ void dense_image_block(const ImageItem& it, int block, Load load, Finish finish)
 {
     const uint32_t units_per_row = (uint32_t)it.in >> 3, units = (uint32_t)it.out * units_per_row;
-    const uint32_t base = (uint32_t)block * (kImageThreads * kUnitsPerThread) + threadIdx.x;
-    Raw raw[kUnitsPerThread];
-    uint32_t row[kUnitsPerThread], u[kUnitsPerThread];
+    const uint32_t base = (uint32_t)block * (kImageThreads * kUnits) + threadIdx.x;
+    Raw raw[kUnits];
+    int half[kUnits];
 #pragma unroll
-    for (int i = 0; i < kUnitsPerThread; ++i) {
+    for (int i = 0; i < kUnits; ++i) {
         const uint32_t unit = base + (uint32_t)(i * kImageThreads);
-        row[i] = unit / units_per_row;
-        u[i] = unit - row[i] * units_per_row;
-        if (unit < units) raw[i] = load((int)row[i], (int)u[i]);
+        uint32_t u;
+        const uint32_t row = split_by(unit, units_per_row, it.magic, u);
+        half[i] = (int)(u & 1u);
+        if (unit < units) raw[i] = load((size_t)unit, row, (int)u);
     }
 #pragma unroll
-    for (int i = 0; i < kUnitsPerThread; ++i) {
-        if (base + (uint32_t)(i * kImageThreads) >= units) break;
-        reinterpret_cast<uint4*>(it.dst)[(size_t)row[i] * units_per_row + u[i]] = finish(raw[i], (int)u[i]);
+    for (int i = 0; i < kUnits; ++i) {
+        const uint32_t unit = base + (uint32_t)(i * kImageThreads);
+        if (unit >= units) break;
+        reinterpret_cast<uint4*>(it.dst)[unit] = finish(raw[i], half[i]);
     }
 }
 
-template <int M, int NC>
+template <int M, int NC, int kUnits>
 __device__ __forceinline__ void unpack_block(const ImageItem& it, int block)
 {
-    const int N = it.N, vpr = it.in / M * N, wpr = it.words_per_row;
-    dense_image_block<PackedUnit>(
-        it, block, [&](int row, int u) { return load_packed_unit<M, NC>(it.src + (size_t)row * vpr, it.idx + (size_t)row * wpr, N, u); },
+    const int N = it.N, wpr = it.words_per_row, count = (8 / M) * (NC ? NC : N);
+    dense_image_block<PackedUnit, kUnits>(
+        it, block, [&](size_t unit, uint32_t row, int u) { return load_packed_values<M, NC>(it.src + unit * count, it.idx + (size_t)row * wpr, N, u); },
         [&](const PackedUnit& p, int) { return expand_packed_unit<M, NC>(p, N); });
 }
 
@@ -157,6 +172,40 @@ __device__ __forceinline__ Segment pick_segment(const uint4& x, const uint4& y)
     return s;
 }
 
+// Groups of 8: how the kept values (one or two in a word) make the two words of a group, as selectors of byte permutes against
+// zero, and the two metadata nibbles.  Indexed by the group's fields, two values first, then at 64 one.
+// (Compares and selects for every chunk: 3072 x 768 at 2:8 3.1 us, with the table 2.7.)
+struct alignas(8) Sp24Entry { uint32_t select, nibbles; };
+struct Sp24Table {
+    Sp24Entry e[64 + 8];
+};
+constexpr Sp24Table make_sp24_table()
+{
+    Sp24Table t{};
+    for (int i = 0; i < 72; ++i) {
+        const int n = i < 64 ? 2 : 1, p[2] = {i & 7, (i >> 3) & 7};
+        uint32_t select = 0, nibbles = 0;
+        for (int c = 0; c < 2; ++c) {
+            uint32_t sel = 0x4444u, nib = 4u;                              // an empty chunk: zeros, positions 0 and 1
+            const bool first = p[0] >> 2 == c, second = n == 2 && p[1] >> 2 == c;
+            if (first && second) {
+                sel = 0x3210u;
+                nib = (uint32_t)(p[0] & 3) | (uint32_t)(p[1] & 3) << 2;
+            } else if (first || second) {
+                const uint32_t value = first ? 0x10u : 0x32u, l = (uint32_t)(first ? p[0] : p[1]) & 3u;
+                sel = l == 3u ? value << 8 | 0x44u : 0x4400u | value;      // position 3 comes second, behind a zero at 0
+                nib = l == 3u ? 0xCu : l | 0xCu;
+            }
+            select |= sel << (16 * c);
+            nibbles |= nib << (4 * c);
+        }
+        t.e[i].select = select;
+        t.e[i].nibbles = nibbles;
+    }
+    return t;
+}
+__device__ const Sp24Table kSp24Table = make_sp24_table();
+
 // The 2-of-4 form of a segment: per aligned chunk of 4 two values with ascending positions i0 < i1 and the metadata
 // nibble i0 | i1 << 2.  A chunk with one kept value takes position 3 as the second (0 as the first where the value itself
 // is at 3), one with none takes 0 and 1; the values borrowed there are zero.
@@ -172,17 +221,26 @@ __device__ __forceinline__ uint4 sp24_words(const Segment& s, uint32_t& nibbles)
     if constexpr (M == 4 && N == 2) {
         w[0] = s.v[0]; w[1] = s.v[1]; w[2] = s.v[2]; w[3] = s.v[3];
         nib = s.fields & 0xFFFFu;
+    } else if constexpr (M == 8) {
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+            const uint32_t f = (s.fields >> (g * N * 3)) & (N == 2 ? 63u : 7u), v = N == 2 ? s.v[g] : s.v[0] >> (16 * g);
+            const uint2 e = __ldg(reinterpret_cast<const uint2*>(&kSp24Table.e[(N == 2 ? 0u : 64u) + f]));
+            w[2 * g] = prmt(v, 0u, e.x & 0xFFFFu);
+            w[2 * g + 1] = prmt(v, 0u, e.x >> 16);
+            nib |= e.y << (8 * g);
+        }
     } else if constexpr (M == 4) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) single(true, (s.v[c >> 1] >> (16 * (c & 1))) & 0xFFFFu, (s.fields >> (2 * c)) & 3u, c);
     } else {
-        constexpr int B = M == 8 ? 3 : 4, kChunks = M / 4;
+        constexpr int B = 4, kChunks = 4;       // one group of 16
 #pragma unroll
-        for (int g = 0; g < 16 / M; ++g) {
+        for (int g = 0; g < 1; ++g) {
             const uint32_t f = s.fields >> (g * N * B);
             const uint32_t p0 = f & (uint32_t)(M - 1);
             if constexpr (N == 1) {
-                const uint32_t v = M == 8 ? (s.v[0] >> (16 * g)) & 0xFFFFu : s.v[0];
+                const uint32_t v = s.v[0];
 #pragma unroll
                 for (int c = 0; c < kChunks; ++c) single((p0 >> 2) == (uint32_t)c, v, p0 & 3u, g * kChunks + c);
             } else {
@@ -215,10 +273,11 @@ __device__ __forceinline__ void sp24_block(const ImageItem& it, int block)
     const int segs = k_blocks * steps * 2;                         // per row, padding included
     const int seg_groups = segs >> 2;
     const int slot = block * (kImageThreads / 32) + (int)(threadIdx.x >> 5);      // (16 rows, 4 segments) of this warp
-    const int rows16 = slot / seg_groups;
+    uint32_t group;
+    const int rows16 = (int)split_by((uint32_t)slot, (uint32_t)seg_groups, it.magic, group);
     if (rows16 >= (out + 127) / 128 * 8) return;
     const int lane = threadIdx.x & 31;
-    const int seg = (slot - rows16 * seg_groups) * 4 + (lane >> 3);
+    const int seg = (int)group * 4 + (lane >> 3);
     const int o0 = rows16 * 16 + (lane & 7);
     const int k0 = seg * 16;
     int src_row[2];
@@ -261,18 +320,18 @@ __device__ __forceinline__ void sp24_block(const ImageItem& it, int block)
 }
 
 // Blocks of a weight.
-int image_blocks(const ImageJob& j)
+int image_blocks(const ImageJob& j, int units_per_thread)
 {
     if (j.kind == IMAGE_UNPACK || j.kind == IMAGE_MASK) {
         const long long units = (long long)j.out * (j.in / 8);
-        return (int)((units + kImageThreads * kUnitsPerThread - 1) / (kImageThreads * kUnitsPerThread));
+        return (int)((units + kImageThreads * units_per_thread - 1) / (kImageThreads * units_per_thread));
     }
     const long long segs = (long long)((j.in + j.block_k - 1) / j.block_k) * (j.block_k / 32) * 2;
     const long long warps = (long long)((j.out + 127) / 128 * 8) * (segs / 4);
     return (int)((warps + kImageThreads / 32 - 1) / (kImageThreads / 32));
 }
 
-template <int kMax>
+template <int kMax, int kUnits>
 __global__ void __launch_bounds__(kImageThreads, 4) weight_image_kernel(const __grid_constant__ ImageTable<kMax> t)
 {
     pdl_wait_for_predecessors();
@@ -298,38 +357,40 @@ __global__ void __launch_bounds__(kImageThreads, 4) weight_image_kernel(const __
         else { if (N == 2) sp24_block<16, 2, true>(it, block); else sp24_block<16, 1, true>(it, block); }
     } else if (it.kind == IMAGE_UNPACK) {
         if (N == M) {
-            dense_image_block<uint4>(it, block, [&](int row, int u) { return __ldg(reinterpret_cast<const uint4*>(it.src + (size_t)row * it.in) + u); },
-                                     [](const uint4& v, int) { return v; });
+            dense_image_block<uint4, kUnits>(it, block, [&](size_t unit, uint32_t, int) { return __ldg(reinterpret_cast<const uint4*>(it.src) + unit); },
+                                             [](const uint4& v, int) { return v; });
         } else if (M == 8) {
-            if (N == 1) unpack_block<8, 1>(it, block);
-            else if (N == 2) unpack_block<8, 2>(it, block);
-            else if (N == 4) unpack_block<8, 4>(it, block);
-            else unpack_block<8, 0>(it, block);
+            if (N == 1) unpack_block<8, 1, kUnits>(it, block);
+            else if (N == 2) unpack_block<8, 2, kUnits>(it, block);
+            else if (N == 4) unpack_block<8, 4, kUnits>(it, block);
+            else unpack_block<8, 0, kUnits>(it, block);
         } else if (M == 4) {
-            if (N == 1) unpack_block<4, 1>(it, block);
-            else if (N == 2) unpack_block<4, 2>(it, block);
-            else unpack_block<4, 0>(it, block);
+            if (N == 1) unpack_block<4, 1, kUnits>(it, block);
+            else if (N == 2) unpack_block<4, 2, kUnits>(it, block);
+            else unpack_block<4, 0, kUnits>(it, block);
         } else {
             const int vpr = it.in / 16 * N, wpr = it.words_per_row;
-            dense_image_block<int>(it, block, [](int row, int) { return row; },
-                                   [&](int row, int u) { return expand_unit16(it.src + (size_t)row * vpr, it.idx + (size_t)row * wpr, N, u); });
+            dense_image_block<uint2, kUnits>(
+                it, block, [](size_t, uint32_t row, int u) { return make_uint2(row, (uint32_t)u); },
+                [&](const uint2& at, int) { return expand_unit16(it.src + (size_t)at.x * vpr, it.idx + (size_t)at.x * wpr, N, (int)at.y); });
         }
     } else {
         if (M == 16) {
-            dense_image_block<DenseGroup16>(it, block,
-                                            [&](int row, int u) {
-                                                const uint4* g = reinterpret_cast<const uint4*>(it.src + (size_t)row * it.in) + (u & ~1);
-                                                return DenseGroup16{__ldg(g), __ldg(g + 1)};
-                                            },
-                                            [&](const DenseGroup16& g, int u) { return mask_unit<16>(g.a, g.b, u & 1, N); });
+            dense_image_block<DenseGroup16, kUnits>(
+                it, block,
+                [&](size_t unit, uint32_t, int) {      // rows hold whole groups of 16
+                    const uint4* g = reinterpret_cast<const uint4*>(it.src) + (unit & ~(size_t)1);
+                    return DenseGroup16{__ldg(g), __ldg(g + 1)};
+                },
+                [&](const DenseGroup16& g, int half) { return mask_unit<16>(g.a, g.b, half, N); });
         } else {
-            dense_image_block<uint4>(it, block, [&](int row, int u) { return __ldg(reinterpret_cast<const uint4*>(it.src + (size_t)row * it.in) + u); },
-                                     [&](const uint4& v, int) { return M == 8 ? mask_unit<8>(v, v, 0, N) : mask_unit<4>(v, v, 0, N); });
+            dense_image_block<uint4, kUnits>(it, block, [&](size_t unit, uint32_t, int) { return __ldg(reinterpret_cast<const uint4*>(it.src) + unit); },
+                                             [&](const uint4& v, int) { return M == 8 ? mask_unit<8>(v, v, 0, N) : mask_unit<4>(v, v, 0, N); });
         }
     }
 }
 
-template <int kMax>
+template <int kMax, int kUnits>
 elsa_status launch_table(const ImageJob* jobs, int n, cudaStream_t stream)
 {
     ImageTable<kMax> t;      // on the stack: several threads may launch at once
@@ -343,12 +404,15 @@ elsa_status launch_table(const ImageJob* jobs, int n, cudaStream_t stream)
         it.words_per_row = (int)index_words_per_row(j.in, j.N, j.M);
         it.k_blocks = (j.in + j.block_k - 1) / j.block_k;
         it.steps = j.block_k / 32;
-        blocks += image_blocks(j);
+        const bool dense = j.kind == IMAGE_UNPACK || j.kind == IMAGE_MASK;
+        const uint32_t d = dense ? (uint32_t)j.in / 8 : (uint32_t)(it.k_blocks * it.steps * 2) >> 2;
+        it.magic = d == 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d);
+        blocks += image_blocks(j, kUnits);
     }
     t.n = n;
     const int k = n > 1 || jobs[0].kind == IMAGE_MASK ? ELSA_KERNEL_WEIGHT_IMAGES : jobs[0].kind == IMAGE_UNPACK ? ELSA_KERNEL_UNPACK : ELSA_KERNEL_NM_TO_SP24;
     ProfileScope scope(k, stream);
-    cudaError_t e = launch_pdl(weight_image_kernel<kMax>, dim3((unsigned)blocks), dim3(kImageThreads), 0, stream, 1, t);
+    cudaError_t e = launch_pdl(weight_image_kernel<kMax, kUnits>, dim3((unsigned)blocks), dim3(kImageThreads), 0, stream, 1, t);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(ELSA_ERR_CUDA, "launch of the weight images failed: %s", cudaGetErrorString(e));
@@ -360,12 +424,18 @@ elsa_status launch_table(const ImageJob* jobs, int n, cudaStream_t stream)
 
 elsa_status launch_images(const ImageJob* jobs, int n, cudaStream_t stream)
 {
+    DeviceInfo dev;
+    const elsa_status dev_st = device_info(&dev);
+    if (dev_st != ELSA_OK) return dev_st;
     constexpr int kMost = 256;       // items per launch (kernel parameters are limited to 32 KB)
     for (int at = 0; at < n; at += kMost) {
         const int count = n - at < kMost ? n - at : kMost;
-        const elsa_status st = count == 1   ? launch_table<1>(jobs + at, count, stream)
-                               : count <= 8 ? launch_table<8>(jobs + at, count, stream)
-                                            : launch_table<kMost>(jobs + at, count, stream);
+        int blocks = 0;
+        for (int i = 0; i < count; ++i) blocks += image_blocks(jobs[at + i], kMostUnits);
+        const bool spread = blocks < 2 * dev.sm_count;
+        const elsa_status st = count == 1   ? (spread ? launch_table<1, 1>(jobs + at, count, stream) : launch_table<1, kMostUnits>(jobs + at, count, stream))
+                               : count <= 8 ? (spread ? launch_table<8, 1>(jobs + at, count, stream) : launch_table<8, kMostUnits>(jobs + at, count, stream))
+                                            : launch_table<kMost, kMostUnits>(jobs + at, count, stream);
         if (st != ELSA_OK) return st;
     }
     return ELSA_OK;
