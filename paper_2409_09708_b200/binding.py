@@ -1,4 +1,5 @@
-"""Thin ctypes binding of ``libelsa.so`` (the C ABI declared in ``include/elsa.h``).
+"""Thin binding of ``libelsa.so`` (the C ABI declared in ``include/elsa.h``): ctypes, and for the calls that are made
+once a layer the extension module ``_elsa_host`` (``csrc/elsa_host.cpp``).
 
 Argument marshalling only: every step of the path runs in the library's CUDA
 kernels.  torch supplies device memory and streams.  There is no fallback: if
@@ -22,6 +23,8 @@ if not os.path.exists(LIB_PATH):
     raise ImportError(
         "libelsa.so is missing: build it with `python -m paper_2409_09708_b200.build` "
         "(there is no CPU or PyTorch fallback for the sparse-linear path)")
+
+from . import _elsa_host  # noqa: E402  (built together with libelsa.so)
 
 _lib = ctypes.CDLL(LIB_PATH)
 
@@ -118,6 +121,9 @@ class ElsaBlockWeights(ctypes.Structure):
 
 _backward_ws = _sig("elsa_backward_workspace_bytes", _sz, [_i, _i, _i, _i, _i, _i])
 _backward = _sig("elsa_nm_linear_backward", _i, [_vp, _vp, _i, _vp, _vp, _i, _i, _i, _i, _i, _vp, _vp, _vp, _vp, _sz, _vp, _vp])
+_elsa_host.bind({fn.__name__: ctypes.cast(fn, _vp).value
+                 for fn in (_linear, _linear_masked, _linear_i8, _backward, _compress, _compress_levels, _values_bytes, _index_bytes,
+                            _workspace_bytes, _workspace_bytes_i8, _backward_ws)})
 BLOCK_REGIONS = ("x1", "qkv", "a", "x2", "x3", "h", "t", "workspace")
 _bw = ctypes.POINTER(ElsaBlockWeights)
 _block_scratch = _sig("elsa_vit_block_scratch_bytes", _sz, [_i, _i, _i, _bw, _i, ctypes.POINTER(_sz)])
@@ -161,6 +167,13 @@ def _check(status: int):
         raise ElsaError(status)
 
 
+def _result(r):
+    """What a call of _elsa_host gave: its result, or a status that is not OK."""
+    if type(r) is int:
+        raise ElsaError(r)
+    return r
+
+
 def elsa_last_error() -> str:
     return (_last_error() or b"").decode()
 
@@ -187,13 +200,8 @@ def elsa_nm_linear_i8(X: torch.Tensor, x_scale: float, vals: torch.Tensor, idx, 
                       in_: int, N: int, M: int, out_dtype: torch.dtype, dev_status=None, stream=None):
     """Y [rows, out] (out_dtype) from int8 activations, the packed int8 weight and the scales."""
     assert X.dtype == torch.int8 and w_scale.dtype == torch.float32
-    rows = X.shape[0]
-    Y = X.new_empty((rows, out), dtype=out_dtype)
-    need = int(_workspace_bytes_i8(out, in_, N, M))
-    ws = alloc_workspace(need) if need else None
-    _check(_linear_i8(_ptr(X), rows, float(x_scale), _ptr(vals), _ptr(idx), _ptr(w_scale), _ptr(bias), out, in_, N, M,
-                      dtype_code(out_dtype), _ptr(Y), _ptr(ws), need, _ptr(dev_status), _stream(stream)))
-    return Y
+    return _result(_elsa_host.linear_i8(X, x_scale, vals, idx, w_scale, bias, out, in_, N, M, dtype_code(out_dtype), dev_status,
+                                        _stream(stream)))
 
 
 # ---- search-side host code (lists of numbers in, lists out; argument marshalling only)
@@ -335,26 +343,11 @@ def alloc_packed(out, in_, N, M, dtype: torch.dtype, device="cuda"):
     return vals, idx
 
 
-def _packed_like(W: torch.Tensor, N, M):
-    """alloc_packed for W [out, in] at a level that is known to be valid (fewer lookups per call)."""
-    out, in_ = W.shape
-    per_row = in_ // M * N
-    vals = W.new_empty((out, per_row))
-    if N == M:
-        return vals, None
-    return vals, W.new_empty((out, (per_row * _INDEX_BITS[M] + 31) >> 5), dtype=torch.int32)
-
-
-_INDEX_BITS = {4: 2, 8: 3, 16: 4}
-
-
 def elsa_nm_compress(W: torch.Tensor, N: int, M: int, vals=None, idx=None, stream=None):
     """Packed (vals, idx) of W [out, in] at level N:M."""
-    out, in_ = W.shape
     if vals is None:
-        if _values_bytes(out, in_, N, M, dtype_code(W.dtype)) == 0:
-            _check(_compress(_ptr(W), out, in_, N, M, dtype_code(W.dtype), None, None, _stream(stream)))
-        vals, idx = _packed_like(W, N, M)
+        return _result(_elsa_host.compress(W, N, M, dtype_code(W.dtype), _stream(stream)))
+    out, in_ = W.shape
     _check(_compress(_ptr(W), out, in_, N, M, dtype_code(W.dtype), _ptr(vals), _ptr(idx), _stream(stream)))
     return vals, idx
 
@@ -363,18 +356,9 @@ def elsa_nm_compress_levels(W: torch.Tensor, N_list, M: int, stream=None):
     """Packed (vals, idx) of W at every level N:M of N_list, from one read of W."""
     out, in_ = W.shape
     n = len(N_list)
-    if M in _INDEX_BITS and in_ % M == 0 and all(1 <= N <= M for N in N_list):
-        # all values in one allocation and all index words in another (an allocation costs the host 2 us, a view 1)
-        per_row = [in_ // M * N for N in N_list]
-        words = [0 if N == M else (v * _INDEX_BITS[M] + 31) >> 5 for N, v in zip(N_list, per_row)]
-        values, index = W.new_empty(out * sum(per_row)), W.new_empty(out * sum(words), dtype=torch.int32)
-        packed, vat, iat = [], 0, 0
-        for v, k in zip(per_row, words):
-            packed.append((values.as_strided((out, v), (v, 1), vat), index.as_strided((out, k), (k, 1), iat) if k else None))
-            vat += out * v
-            iat += out * k
-    else:
-        packed = [alloc_packed(out, in_, N, M, W.dtype, W.device) for N in N_list]
+    if M in (4, 8, 16) and in_ % M == 0 and n <= 16 and all(1 <= N <= M for N in N_list):
+        return _result(_elsa_host.compress_levels(W, list(N_list), M, dtype_code(W.dtype), _stream(stream)))
+    packed = [alloc_packed(out, in_, N, M, W.dtype, W.device) for N in N_list]
     Ns = (_i * n)(*N_list)
     vals = (_vp * n)(*[v.data_ptr() for v, _ in packed])
     idx = (_vp * n)(*[None if i is None else i.data_ptr() for _, i in packed])
@@ -385,16 +369,8 @@ def elsa_nm_compress_levels(W: torch.Tensor, N_list, M: int, stream=None):
 def elsa_nm_linear_masked(X: torch.Tensor, W_sup: torch.Tensor, bias, N: int, M: int, Y=None, workspace=None,
                           dev_status=None, stream=None):
     """Y = X . (W_sup projected onto N:M)^T + bias straight from the dense shared weight."""
-    rows, in_ = X.shape
-    out = W_sup.shape[0]
-    code = dtype_code(X.dtype)
-    if Y is None:
-        Y = X.new_empty((rows, out))
-    if workspace is None:
-        workspace = alloc_workspace(elsa_workspace_bytes(rows, in_, out, N, M, code), X.device)
-    _check(_linear_masked(_ptr(X), rows, _ptr(W_sup), _ptr(bias), out, in_, N, M, code, _ptr(Y), _ptr(workspace),
-                          workspace.numel(), _ptr(dev_status), _stream(stream)))
-    return Y
+    r = _result(_elsa_host.linear_masked(X, W_sup, bias, N, M, dtype_code(X.dtype), Y, workspace, dev_status, _stream(stream)))
+    return r if Y is None else Y
 
 
 def elsa_nm_unpack(vals: torch.Tensor, idx, out: int, in_: int, N: int, M: int, W_masked=None, stream=None):
@@ -411,15 +387,10 @@ def alloc_workspace(nbytes: int, device="cuda"):
 def elsa_nm_linear(X: torch.Tensor, vals: torch.Tensor, idx, bias, out: int, in_: int, N: int, M: int,
                    Y=None, workspace=None, dev_status=None, stream=None):
     """Y [rows, out] = X [rows, in] . W_masked^T + bias from the packed weight."""
-    rows = X.shape[0]
-    code = dtype_code(X.dtype)
-    if Y is None:
-        Y = X.new_empty((rows, out))
-    if workspace is None:
-        workspace = alloc_workspace(elsa_workspace_bytes(rows, in_, out, N, M, code), X.device)
-    _check(_linear(_ptr(X), rows, _ptr(vals), _ptr(idx), _ptr(bias), out, in_, N, M, code, _ptr(Y),
-                   _ptr(workspace), workspace.numel(), _ptr(dev_status), _stream(stream)))
-    return Y
+    r = _elsa_host.linear(X, vals, idx, bias, out, in_, N, M, dtype_code(X.dtype), Y, workspace, dev_status, _stream(stream))
+    if type(r) is int:
+        raise ElsaError(r)
+    return r if Y is None else Y
 
 
 def elsa_backward_workspace_bytes(rows, in_, out, N, M, dtype=F16) -> int:
@@ -430,16 +401,8 @@ def elsa_nm_linear_backward(dY, X, vals, idx, out, in_, N, M, want=("dX", "dW", 
                             dev_status=None, stream=None):
     """Backward of Y = X Wm^T + b: returns (dX, dW, db), None for the ones not in `want`.  dW is dense [out, in]
     with zeros at the pruned positions."""
-    rows = dY.shape[0]
-    code = dtype_code(dY.dtype)
-    dX = dY.new_empty((rows, in_)) if "dX" in want else None
-    dW = dY.new_empty((out, in_)) if "dW" in want else None
-    db = dY.new_empty((out,)) if "db" in want else None
-    if workspace is None:
-        workspace = alloc_workspace(elsa_backward_workspace_bytes(rows, in_, out, N, M, code), dY.device)
-    _check(_backward(_ptr(dY), _ptr(X), rows, _ptr(vals), _ptr(idx), out, in_, N, M, code, _ptr(dX), _ptr(dW), _ptr(db),
-                     _ptr(workspace), workspace.numel(), _ptr(dev_status), _stream(stream)))
-    return dX, dW, db
+    return _result(_elsa_host.linear_backward(dY, X, vals, idx, out, in_, N, M, dtype_code(dY.dtype), "dX" in want, "dW" in want,
+                                              "db" in want, workspace, dev_status, _stream(stream)))
 
 
 def make_block_weights(ln1_gain, ln1_bias, ln2_gain, ln2_bias, linears, eps=1e-6):

@@ -1,15 +1,19 @@
-"""Builds ``libelsa.so`` in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds ``libelsa.so`` (nvcc for sm_100a; cross-compiles without a GPU) and the native half of the binding in-tree."""
 from __future__ import annotations
 
+import importlib.util
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libelsa.so")
+HOST_SOURCE = os.path.join(CSRC, "elsa_host.cpp")
+HOST_LIB = os.path.join(HERE, "_elsa_host.so")
 SOURCES = ["elsa_api.cu", "elsa_attention.cu", "elsa_attention_window.cu", "elsa_backward.cu", "elsa_block.cu", "elsa_compress.cu", "elsa_int8.cu", "elsa_linear_simt.cu", "elsa_linear_small.cu", "elsa_linear_tc.cu", "elsa_linear_tc2.cu",
            "elsa_no_alloc.cu", "elsa_search.cu", "elsa_selftest.cu", "elsa_sparse24.cu", "elsa_sparse24_pair.cu", "elsa_sparse24_st.cu", "elsa_sparse24_ws.cu", "elsa_weight_images.cu"]
 
@@ -26,14 +30,32 @@ def sources() -> list[str]:
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "elsa.h")]
-    return any(os.path.getmtime(d) > t for d in deps)
+    header = os.path.join(ROOT, "include", "elsa.h")
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
+    return _older(LIB, [d for d in deps if d != HOST_SOURCE] + [header])
+
+
+def _older(built: str, deps: list[str]) -> bool:
+    return not os.path.exists(built) or any(os.path.getmtime(d) > os.path.getmtime(built) for d in deps)
+
+
+def build_host(force: bool = False) -> str:
+    """The extension module behind binding.py: C++ against torch's headers, the entry points handed to it by address."""
+    if not force and not _older(HOST_LIB, [HOST_SOURCE, os.path.join(ROOT, "include", "elsa.h")]):
+        return HOST_LIB
+    torch = importlib.util.find_spec("torch").submodule_search_locations[0]
+    include = os.path.join(torch, "include")
+    cmd = [os.environ.get("CXX") or "g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"),
+           "-isystem", include, "-isystem", os.path.join(include, "torch", "csrc", "api", "include"),
+           "-isystem", sysconfig.get_paths()["include"], HOST_SOURCE,
+           "-L", os.path.join(torch, "lib"), "-lc10", "-ltorch_cpu", "-ltorch_python", "-o", HOST_LIB + ".tmp"]
+    subprocess.run(cmd, check=True)
+    os.replace(HOST_LIB + ".tmp", HOST_LIB)
+    return HOST_LIB
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_host(force)
     if not force and not is_stale():
         return LIB
     cmd = [nvcc_path(), "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
