@@ -27,6 +27,7 @@ struct ImageItem {
     uint16_t* meta;
     int first_block;
     int out, in, N, M, words_per_row, kind, layout;
+    int rounds;                           // a block works on this many runs of its threads' units, one after the other
     uint32_t magic;                       // floor(2^32 / d) of the division that finds a thread's row, see split_by
     int k_blocks, steps;                  // 2-of-4 forms: metadata blocks along K, K steps of 32 per block (2 or 4)
 };
@@ -53,22 +54,26 @@ template <typename Raw, int kUnits, typename Load, typename Finish>
 __device__ __forceinline__ void dense_image_block(const ImageItem& it, int block, Load load, Finish finish)
 {
     const uint32_t units_per_row = (uint32_t)it.in >> 3, units = (uint32_t)it.out * units_per_row;
-    const uint32_t base = (uint32_t)block * (kImageThreads * kUnits) + threadIdx.x;
-    Raw raw[kUnits];
-    int half[kUnits];
+#pragma unroll 1
+    for (int round = 0; round < it.rounds; ++round) {
+        const uint32_t base = (uint32_t)(block * it.rounds + round) * (kImageThreads * kUnits) + threadIdx.x;
+        Raw raw[kUnits];
+        int half[kUnits];
 #pragma unroll
-    for (int i = 0; i < kUnits; ++i) {
-        const uint32_t unit = base + (uint32_t)(i * kImageThreads);
-        uint32_t u;
-        const uint32_t row = split_by(unit, units_per_row, it.magic, u);
-        half[i] = (int)(u & 1u);
-        if (unit < units) raw[i] = load((size_t)unit, row, (int)u);
-    }
+        for (int i = 0; i < kUnits; ++i) {
+            // a unit past the end reads the last one: no branch stands between the loads
+            const uint32_t unit = min(base + (uint32_t)(i * kImageThreads), units - 1u);
+            uint32_t u;
+            const uint32_t row = split_by(unit, units_per_row, it.magic, u);
+            half[i] = (int)(u & 1u);
+            raw[i] = load((size_t)unit, row, (int)u);
+        }
 #pragma unroll
-    for (int i = 0; i < kUnits; ++i) {
-        const uint32_t unit = base + (uint32_t)(i * kImageThreads);
-        if (unit >= units) break;
-        reinterpret_cast<uint4*>(it.dst)[unit] = finish(raw[i], half[i]);
+        for (int i = 0; i < kUnits; ++i) {
+            const uint32_t unit = base + (uint32_t)(i * kImageThreads);
+            if (unit >= units) break;
+            reinterpret_cast<uint4*>(it.dst)[unit] = finish(raw[i], half[i]);
+        }
     }
 }
 
@@ -272,63 +277,68 @@ __device__ __forceinline__ void sp24_block(const ImageItem& it, int block)
     const int out = it.out, in = it.in, steps = it.steps, k_blocks = it.k_blocks;
     const int segs = k_blocks * steps * 2;                         // per row, padding included
     const int seg_groups = segs >> 2;
-    const int slot = block * (kImageThreads / 32) + (int)(threadIdx.x >> 5);      // (16 rows, 4 segments) of this warp
-    uint32_t group;
-    const int rows16 = (int)split_by((uint32_t)slot, (uint32_t)seg_groups, it.magic, group);
-    if (rows16 >= (out + 127) / 128 * 8) return;
-    const int lane = threadIdx.x & 31;
-    const int seg = (int)group * 4 + (lane >> 3);
-    const int o0 = rows16 * 16 + (lane & 7);
-    const int k0 = seg * 16;
-    int src_row[2];
-    Segment s[2];
+#pragma unroll 1
+    for (int round = 0; round < it.rounds; ++round) {
+        const int slot = (block * it.rounds + round) * (kImageThreads / 32) + (int)(threadIdx.x >> 5);      // (16 rows, 4 segments) of this warp
+        uint32_t group;
+        const int rows16 = (int)split_by((uint32_t)slot, (uint32_t)seg_groups, it.magic, group);
+        if (rows16 >= (out + 127) / 128 * 8) return;
+        const int lane = threadIdx.x & 31;
+        const int seg = (int)group * 4 + (lane >> 3);
+        const int o0 = rows16 * 16 + (lane & 7);
+        const int k0 = seg * 16;
+        int src_row[2];
+        Segment s[2];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int o = o0 + 8 * i, r = o & 31;
-        src_row[i] = it.layout != SP24_ROWS ? (o & ~31) | (8 * (r & 3) + (r >> 2)) : o;
-        if (src_row[i] < out && k0 < in) {
-            if constexpr (kMask) {
-                const uint4* g = reinterpret_cast<const uint4*>(it.src + (size_t)src_row[i] * in + k0);
-                s[i] = pick_segment<M, N>(__ldg(g), __ldg(g + 1));
-            } else {
-                s[i] = load_segment<M, N>(it.src + (size_t)src_row[i] * (in / M * N), it.idx + (size_t)src_row[i] * it.words_per_row, seg);
+        for (int i = 0; i < 2; ++i) {
+            const int o = o0 + 8 * i, r = o & 31;
+            src_row[i] = it.layout != SP24_ROWS ? (o & ~31) | (8 * (r & 3) + (r >> 2)) : o;
+            if (src_row[i] < out && k0 < in) {
+                if constexpr (kMask) {
+                    const uint4* g = reinterpret_cast<const uint4*>(it.src + (size_t)src_row[i] * in + k0);
+                    s[i] = pick_segment<M, N>(__ldg(g), __ldg(g + 1));
+                } else {
+                    s[i] = load_segment<M, N>(it.src + (size_t)src_row[i] * (in / M * N), it.idx + (size_t)src_row[i] * it.words_per_row, seg);
+                }
             }
         }
-    }
-    uint32_t word = 0;
+        uint32_t word = 0;
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        uint32_t nib = 0x4444u;                                    // four empty chunks
-        if (src_row[i] < out && k0 < in) v = sp24_words<M, N>(s[i], nib);
-        word |= nib << (16 * i);
-        if (k0 < in && src_row[i] < ((out + 31) & ~31)) {
-            const int o = o0 + 8 * i;
-            size_t at = (size_t)o * (size_t)in + (size_t)k0;       // byte offset of (row o, k0) in the row-major forms
-            if (it.layout == SP24_TILED)
-                at = (size_t)(o >> 5) * 32 * (size_t)in + (size_t)(k0 >> 8) * 8192 + (size_t)((((k0 & 255) >> 4) * 32 + (o & 31)) * 16);
-            *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(it.dst) + at) = v;
+        for (int i = 0; i < 2; ++i) {
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            uint32_t nib = 0x4444u;                                    // four empty chunks
+            if (src_row[i] < out && k0 < in) v = sp24_words<M, N>(s[i], nib);
+            word |= nib << (16 * i);
+            if (k0 < in && src_row[i] < ((out + 31) & ~31)) {
+                const int o = o0 + 8 * i;
+                size_t at = (size_t)o * (size_t)in + (size_t)k0;       // byte offset of (row o, k0) in the row-major forms
+                if (it.layout == SP24_TILED)
+                    at = (size_t)(o >> 5) * 32 * (size_t)in + (size_t)(k0 >> 8) * 8192 + (size_t)((((k0 & 255) >> 4) * 32 + (o & 31)) * 16);
+                *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(it.dst) + at) = v;
+            }
         }
+        // metadata: block (128 features, k block) -> tensor-memory lane -> 4 words, one per K step of 32; a block of 64 k
+        // leaves the last two zero
+        const int kb = seg / (2 * steps), step = (seg >> 1) % steps, k1 = seg & 1;
+        const int tm_lane = (lane & 7) + 8 * k1 + 16 * (rows16 & 7);
+        uint32_t* meta = reinterpret_cast<uint32_t*>(it.meta) + (((size_t)(rows16 >> 3) * k_blocks + kb) * 128 + tm_lane) * 4 + step;
+        meta[0] = word;
+        if (steps == 2) meta[2] = 0u;
     }
-    // metadata: block (128 features, k block) -> tensor-memory lane -> 4 words, one per K step of 32; a block of 64 k
-    // leaves the last two zero
-    const int kb = seg / (2 * steps), step = (seg >> 1) % steps, k1 = seg & 1;
-    const int tm_lane = (lane & 7) + 8 * k1 + 16 * (rows16 & 7);
-    uint32_t* meta = reinterpret_cast<uint32_t*>(it.meta) + (((size_t)(rows16 >> 3) * k_blocks + kb) * 128 + tm_lane) * 4 + step;
-    meta[0] = word;
-    if (steps == 2) meta[2] = 0u;
 }
 
 // Blocks of a weight.
-int image_blocks(const ImageJob& j, int units_per_thread)
+int image_blocks(const ImageJob& j, int units_per_thread, int rounds)
 {
     if (j.kind == IMAGE_UNPACK || j.kind == IMAGE_MASK) {
         const long long units = (long long)j.out * (j.in / 8);
-        return (int)((units + kImageThreads * units_per_thread - 1) / (kImageThreads * units_per_thread));
+        const long long per_block = (long long)kImageThreads * units_per_thread * rounds;
+        return (int)((units + per_block - 1) / per_block);
     }
     const long long segs = (long long)((j.in + j.block_k - 1) / j.block_k) * (j.block_k / 32) * 2;
     const long long warps = (long long)((j.out + 127) / 128 * 8) * (segs / 4);
-    return (int)((warps + kImageThreads / 32 - 1) / (kImageThreads / 32));
+    const long long per_block = (long long)(kImageThreads / 32) * rounds;
+    return (int)((warps + per_block - 1) / per_block);
 }
 
 template <int kMax, int kUnits>
@@ -391,7 +401,7 @@ __global__ void __launch_bounds__(kImageThreads, 4) weight_image_kernel(const __
 }
 
 template <int kMax, int kUnits>
-elsa_status launch_table(const ImageJob* jobs, int n, cudaStream_t stream)
+elsa_status launch_table(const ImageJob* jobs, int n, int rounds, cudaStream_t stream)
 {
     ImageTable<kMax> t;      // on the stack: several threads may launch at once
     int blocks = 0;
@@ -407,7 +417,8 @@ elsa_status launch_table(const ImageJob* jobs, int n, cudaStream_t stream)
         const bool dense = j.kind == IMAGE_UNPACK || j.kind == IMAGE_MASK;
         const uint32_t d = dense ? (uint32_t)j.in / 8 : (uint32_t)(it.k_blocks * it.steps * 2) >> 2;
         it.magic = d == 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d);
-        blocks += image_blocks(j, kUnits);
+        it.rounds = rounds;
+        blocks += image_blocks(j, kUnits, rounds);
     }
     t.n = n;
     const int k = n > 1 || jobs[0].kind == IMAGE_MASK ? ELSA_KERNEL_WEIGHT_IMAGES : jobs[0].kind == IMAGE_UNPACK ? ELSA_KERNEL_UNPACK : ELSA_KERNEL_NM_TO_SP24;
@@ -431,11 +442,16 @@ elsa_status launch_images(const ImageJob* jobs, int n, cudaStream_t stream)
     for (int at = 0; at < n; at += kMost) {
         const int count = n - at < kMost ? n - at : kMost;
         int blocks = 0;
-        for (int i = 0; i < count; ++i) blocks += image_blocks(jobs[at + i], kMostUnits);
+        for (int i = 0; i < count; ++i) blocks += image_blocks(jobs[at + i], kMostUnits, 1);
         const bool spread = blocks < 2 * dev.sm_count;
-        const elsa_status st = count == 1   ? (spread ? launch_table<1, 1>(jobs + at, count, stream) : launch_table<1, kMostUnits>(jobs + at, count, stream))
-                               : count <= 8 ? (spread ? launch_table<8, 1>(jobs + at, count, stream) : launch_table<8, kMostUnits>(jobs + at, count, stream))
-                                            : launch_table<kMost, kMostUnits>(jobs + at, count, stream);
+        // A block costs a few thousand cycles before its first load, so where there are many waves of them they take three
+        // runs each: 48 DeiT-B weights at 2:8 to dense images 51 -> 46 us, to 2-of-4 ones 60 -> 55; one block's four
+        // weights 4.4 to 4.9 with two runs, 5.0 with four.
+        const int rounds = blocks >= 32 * dev.sm_count ? 3 : 1;
+        const elsa_status st =
+            count == 1   ? (spread ? launch_table<1, 1>(jobs + at, count, 1, stream) : launch_table<1, kMostUnits>(jobs + at, count, rounds, stream))
+            : count <= 8 ? (spread ? launch_table<8, 1>(jobs + at, count, 1, stream) : launch_table<8, kMostUnits>(jobs + at, count, rounds, stream))
+                         : launch_table<kMost, kMostUnits>(jobs + at, count, rounds, stream);
         if (st != ELSA_OK) return st;
     }
     return ELSA_OK;
