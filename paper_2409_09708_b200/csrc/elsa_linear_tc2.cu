@@ -57,6 +57,7 @@ struct alignas(64) PairLayer {
     int rows, out;
     int bn;            // features per pair tile (MMA N)
     int tiles_n;
+    int row_base;      // first token row of the layer's tiles: 0, or where the narrow tiles of a layer's last rows begin
     int tile_begin;    // index of this layer's first tile in the launch's sequence
     int num_k_blocks;
     uint32_t idesc;
@@ -216,7 +217,7 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                     kb1 = (int)((long long)L.num_k_blocks * (range + 1) / p.splits);
                 }
                 const int half_bn = L.bn >> 1;
-                const int m0 = (t / L.tiles_n) * kPairRows + (int)cta_rank * kRowsPerCta;
+                const int m0 = L.row_base + (t / L.tiles_n) * kPairRows + (int)cta_rank * kRowsPerCta;
                 const int n0 = (t % L.tiles_n) * L.bn + (int)cta_rank * half_bn;
                 const uint32_t tx_bytes = (uint32_t)(2 * (kATileBytes + half_bn * kBlockK * 2));
                 for (int kb = kb0; kb < kb1; ++kb) {
@@ -383,7 +384,7 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
             (void)range;
             const int chunks = L.bn / kEpiCols;
             const int my_chunks = (chunks - part + kEpiParts - 1) / kEpiParts;
-            const int m0 = (t / L.tiles_n) * kPairRows + (int)cta_rank * kRowsPerCta;
+            const int m0 = L.row_base + (t / L.tiles_n) * kPairRows + (int)cta_rank * kRowsPerCta;
             const int n0 = (t % L.tiles_n) * L.bn;
             const int l_rows = L.rows, l_out = L.out;
             const uint32_t bias_b = it & 1u;
@@ -600,6 +601,36 @@ int pick_pair_block_n(int out, int rows, int sm_count, bool whole_boxes = false)
     return best;
 }
 
+// A layer on its own whose tiles overflow the SM pairs' last full wave by a few: the rows of the overflow get narrow tiles,
+// which a wave takes in part of the time.  main: feature width of the tiles of the first `row_tiles` tiles of 256 rows,
+// tail: width for the others (row_tiles covers all rows where that is no gain).  In the units of pick_pair_block_n.
+// Us without and with: 12608 x 768 -> 3072 46.3, 43.4 (600 tiles of 256 on 74 pairs); 25216 x 768 -> 768 25.2, 23.2 (297);
+// 25216 x 3072 -> 768 86.2, 83.8; INT8 45.5, 42.8; where the waves come out even nothing changes.
+struct PairWidths {
+    int main, tail;
+    long long row_tiles;
+};
+
+PairWidths pick_pair_widths(int out, int rows, int sm_count)
+{
+    const long long pairs = sm_count / 2 > 0 ? sm_count / 2 : 1;
+    const long long all = (rows + kPairRows - 1) / kPairRows;
+    auto tiles = [&](long long r, int bn) { return r * ((out + bn - 1) / bn); };
+    PairWidths best = {pick_pair_block_n(out, rows, sm_count), 0, all};
+    long long best_cost = (tiles(all, best.main) + pairs - 1) / pairs * (best.main + 32);
+    for (int bn = 256; bn >= 128; bn -= 64) {
+        const long long waves = tiles(all, bn) / pairs, per_row = (out + bn - 1) / bn;
+        const long long r = waves * pairs / per_row;
+        if (waves < 1 || r < 1 || r >= all) continue;
+        for (int tail = bn / 2; tail >= 64; tail -= 64) {
+            const long long left = tiles(all - r, tail) - (waves * pairs - r * per_row);
+            const long long cost = waves * (bn + 32) + (left > 0 ? (left + pairs - 1) / pairs * (tail + 32) : 0);
+            if (cost < best_cost) { best = {bn, tail, r}; best_cost = cost; }
+        }
+    }
+    return best;
+}
+
 }  // namespace
 
 bool linear_tc_pair_suits(int rows, int out, int sm_count)
@@ -622,15 +653,27 @@ elsa_status launch_group(const PairJob* jobs, int n, elsa_dtype dtype, uint32_t*
     static std::mutex g_mutex;
     std::lock_guard<std::mutex> lock(g_mutex);
     const uint32_t fmt = dtype == ELSA_BF16 ? 1u : 0u;
+    // a layer on its own may be two entries: its rows but the last in wide tiles, the last ones in narrow ones
+    PairWidths widths = {0, 0, 0};
+    if (kForm != kFormTn && n == 1 && kMaxLayers > 1) widths = pick_pair_widths(jobs[0].out, jobs[0].rows, dev.sm_count);
+    const int entries = widths.tail != 0 ? 2 : n;
     int tile_begin = 0;
-    for (int i = 0; i < n; ++i) {
-        const PairJob& j = jobs[i];
+    for (int i = 0; i < entries; ++i) {
+        const PairJob& j = jobs[widths.tail != 0 ? 0 : i];
         PairLayer& L = g.layer[i];
         L.rows = j.rows; L.out = j.out;
-        L.bn = (kForm == kFormTn && j.splits > 1) ? 256 : pick_pair_block_n(j.out, j.rows, dev.sm_count, kForm == kFormTn);
+        L.row_base = 0;
+        int row_tiles = (j.rows + kPairRows - 1) / kPairRows;
+        if (widths.tail != 0) {
+            L.bn = i == 0 ? widths.main : widths.tail;
+            if (i == 1) L.row_base = (int)widths.row_tiles * kPairRows;
+            row_tiles = i == 0 ? (int)widths.row_tiles : row_tiles - (int)widths.row_tiles;
+        } else {
+            L.bn = (kForm == kFormTn && j.splits > 1) ? 256 : pick_pair_block_n(j.out, j.rows, dev.sm_count, kForm == kFormTn);
+        }
         L.tiles_n = (j.out + L.bn - 1) / L.bn;
         L.tile_begin = tile_begin;
-        tile_begin += ((j.rows + kPairRows - 1) / kPairRows) * L.tiles_n * (kForm == kFormTn ? j.splits : 1);
+        tile_begin += row_tiles * L.tiles_n * (kForm == kFormTn ? j.splits : 1);
         L.bias = j.bias;
         L.w_scale = j.w_scale;
         L.x_scale = j.x_scale;
@@ -677,7 +720,7 @@ elsa_status launch_group(const PairJob* jobs, int n, elsa_dtype dtype, uint32_t*
                                            CU_TENSOR_MAP_SWIZZLE_64B, "the residual");
         if (st != ELSA_OK) return st;
     }
-    g.n_layers = n;
+    g.n_layers = entries;
     g.splits = kForm == kFormTn ? jobs[0].splits : 1;
     g.partial = kForm == kFormTn && jobs[0].splits > 1 ? jobs[0].partial : nullptr;
     g.num_tiles = tile_begin;
@@ -749,15 +792,15 @@ elsa_status launch_linear_tc_pair_group(const PairJob* jobs, int n, elsa_dtype d
     for (int i = 0; i < n; ++i) fused = fused || jobs[i].act != 0 || jobs[i].residual != nullptr;
     if (fused) {
         for (int i = 0; i < n; ++i) {
-            st = dtype == ELSA_BF16 ? launch_group<true, kFormFused, 1>(jobs + i, 1, dtype, dev_status, stream, dev)
-                                    : launch_group<false, kFormFused, 1>(jobs + i, 1, dtype, dev_status, stream, dev);
+            st = dtype == ELSA_BF16 ? launch_group<true, kFormFused, 2>(jobs + i, 1, dtype, dev_status, stream, dev)
+                                    : launch_group<false, kFormFused, 2>(jobs + i, 1, dtype, dev_status, stream, dev);
             if (st != ELSA_OK) return st;
         }
         return ELSA_OK;
     }
     if (n == 1)
-        return dtype == ELSA_BF16 ? launch_group<true, kFormPlain, 1>(jobs, 1, dtype, dev_status, stream, dev)
-                                  : launch_group<false, kFormPlain, 1>(jobs, 1, dtype, dev_status, stream, dev);
+        return dtype == ELSA_BF16 ? launch_group<true, kFormPlain, 2>(jobs, 1, dtype, dev_status, stream, dev)
+                                  : launch_group<false, kFormPlain, 2>(jobs, 1, dtype, dev_status, stream, dev);
     return dtype == ELSA_BF16 ? launch_group<true, kFormPlain, kGroupMax>(jobs, n, dtype, dev_status, stream, dev)
                               : launch_group<false, kFormPlain, kGroupMax>(jobs, n, dtype, dev_status, stream, dev);
 }
@@ -811,8 +854,8 @@ elsa_status launch_linear_tc_pair_i8(const int8_t* X, int rows, const int8_t* Wd
     job.X = (const uint16_t*)X; job.Wd = (const uint16_t*)Wd; job.bias = bias; job.Y = Y;
     job.rows = rows; job.in = in; job.out = out;
     job.w_scale = w_scale; job.x_scale = x_scale;
-    return dtype == ELSA_BF16 ? launch_group<true, kFormInt8, 1>(&job, 1, dtype, dev_status, stream, dev)
-                              : launch_group<false, kFormInt8, 1>(&job, 1, dtype, dev_status, stream, dev);
+    return dtype == ELSA_BF16 ? launch_group<true, kFormInt8, 2>(&job, 1, dtype, dev_status, stream, dev)
+                              : launch_group<false, kFormInt8, 2>(&job, 1, dtype, dev_status, stream, dev);
 }
 
 elsa_status launch_linear_tc_pair(const uint16_t* X, int rows, const uint16_t* Wd, const uint16_t* bias, int out,
