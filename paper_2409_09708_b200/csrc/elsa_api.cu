@@ -277,7 +277,11 @@ elsa_status pick_kind(LinearUse use, int rows, int out, int in, int N, int M, in
             const bool ws = ws_large || (ws_ok && in <= 896 && rows >= 256 * pairs / tiles_f);
             *kind = ws ? KIND_SPARSE_WS : in > 768 && st_ok ? KIND_SPARSE_ST : KIND_SPARSE_PAIR;
         } else {
-            *kind = pair_full ? KIND_DENSE_PAIR : KIND_SMALL_IMAGE;
+            // At the dense rate the pair kernel's tiles of a table's layers fill its launch together: from a wave of small
+            // tiles up a layer goes there (24 linears of dim 256, 13987 rows: 242 us with its layers on the few-rows kernel
+            // because 55 row tiles do not fill 74 pairs, 180 like this; 96 of a Swin at batch 4, 319 and 258), below it
+            // where the table's small layers add up (see elsa_vit_linears).
+            *kind = pair_full || tiles_small >= sm_count ? KIND_DENSE_PAIR : KIND_SMALL_IMAGE;
         }
         return ELSA_OK;
     }
@@ -607,9 +611,19 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
                          workspace_bytes >= elsa_vit_workspace_bytes(cfg, n_layers, dtype);
     std::vector<LinearKind> kind(n_layers);
     std::vector<SmallJob> small;
+    long long small_tiles = 0;
     for (int l = 0; l < n_layers; ++l) {
         const elsa_layer& c = cfg[l];
         if ((st = pick_kind(USE_TABLE, c.rows, c.out, c.in, c.N, c.M, dev.sm_count, &kind[l])) != ELSA_OK) return layer_fail(st, l);
+        if (kind[l] == KIND_SMALL_IMAGE) small_tiles += (long long)((c.rows + 127) / 128) * ((c.out + 63) / 64);
+    }
+    // Layers too small for the pair kernel by themselves go to it together from 4.5 waves of small tiles up, us on the
+    // few-rows kernel and there: 48 layers of dim 192 at batch 1 (2.5 waves) 28, 30, at batch 4 59, 45; 16 layers of dim 256 at
+    // batch 2 (3.4) 25, 28; 48 of dim 384 at batch 1 (5) 68, 62; 48 of dim 768 at batch 1 193, 183.
+    const bool together = 2 * small_tiles >= 9LL * dev.sm_count;
+    for (int l = 0; l < n_layers; ++l) {
+        const elsa_layer& c = cfg[l];
+        if (together && kind[l] == KIND_SMALL_IMAGE) kind[l] = KIND_DENSE_PAIR;
         if (kind[l] == KIND_SMALL_IMAGE || kind[l] == KIND_SMALL)
             small.push_back(small_dense_job(c.X, c.rows, c.vals, c.bias, c.out, c.in, c.Y));
     }
