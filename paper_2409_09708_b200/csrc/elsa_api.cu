@@ -301,9 +301,12 @@ elsa_status pick_kind(LinearUse use, int rows, int out, int in, int N, int M, in
         else *kind = ranges >= 2 && k_blocks >= 16 ? KIND_SMALL_IMAGE : KIND_DENSE_ONE;
         return ELSA_OK;
     }
-    // More than a wave of small tiles.  Below K = 512 the sparse kernels do not beat the pair kernel until the
-    // weight-stationary one does (384 -> 384, 6304 rows: 8.2 against 8.8); from there up the sparse pair kernel leads,
-    // and from about 5M outputs the streaming one (3072 -> 768: 6304 rows 24.5 against 25.0, 12608 rows 38.7 against 36.6).
+    // More than a wave of small tiles.  Up to K = 512 the sparse kernels do not beat the pair kernel until the
+    // weight-stationary one does, from about 1200 rows per SM pair (pair, best sparse: 512 -> 1536, 6304 rows 13.0, 14.4, 12608
+    // rows 19.6, 19.8, 18912 rows 25.0, 24.5; 512 -> 2048, 3136 rows 10.7, 11.7, 12544 rows 23.4, 22.6; 512 -> 512, 6304 rows
+    // 9.3, 8.6, 12608 rows 10.7, 11.7; 256 -> 1024, 18912 rows 15.0, 15.8, 25088 rows 19.3, 18.5); above, the sparse pair
+    // kernel leads, and from about 5M outputs the streaming one (3072 -> 768: 6304 rows 24.5 against 25.0, 12608 rows 38.7
+    // against 36.6).
     // With GELU the epilogue weighs more: the weight-stationary kernel leads where an SM pair's rows times K pass 390000
     // (768 -> 3072, 3152 rows 16.8 against 17.0 on the pair kernel, 4925 rows 20.9 against 24.3; 384 -> 1536, 12608 rows
     // 19.9 against 21.7), the pair kernel below; the streaming one is slower than either up to K = 1024.
@@ -312,9 +315,10 @@ elsa_status pick_kind(LinearUse use, int rows, int out, int in, int N, int M, in
         *kind = ws ? KIND_SPARSE_WS : in > 1024 && st_ok && (long long)rows * out >= 5000000LL ? KIND_SPARSE_ST : KIND_DENSE_PAIR;
         return ELSA_OK;
     }
-    if (ws_large) *kind = KIND_SPARSE_WS;
-    else if (sparse_ok && in >= 512 && st_ok && (long long)rows * out >= 5000000LL) *kind = KIND_SPARSE_ST;
-    else if (sparse_ok && in >= 512) *kind = KIND_SPARSE_PAIR;
+    if (in <= 512) *kind = ws_ok && (long long)rows * tiles_f >= 1200 * pairs ? KIND_SPARSE_WS : KIND_DENSE_PAIR;
+    else if (ws_large) *kind = KIND_SPARSE_WS;
+    else if (sparse_ok && st_ok && (long long)rows * out >= 5000000LL) *kind = KIND_SPARSE_ST;
+    else if (sparse_ok) *kind = KIND_SPARSE_PAIR;
     else *kind = KIND_DENSE_PAIR;
     return ELSA_OK;
 }
