@@ -1,0 +1,37 @@
+"""The native half of the binding: what it refuses and how, without a device (the checks come before any launch)."""
+import pytest
+import torch
+
+from paper_2409_09708_b200 import _elsa_host, binding as lib
+
+
+def arguments(**changed):
+    a = dict(X=torch.zeros(4, 64, dtype=torch.float16), vals=torch.zeros(8, 32, dtype=torch.float16), idx=torch.zeros(8, 3, dtype=torch.int32),
+             bias=None, out=8, in_=64, N=4, M=8, code=0, Y=None, workspace=None, status=None, stream=0)
+    a.update(changed)
+    return list(a.values())
+
+
+def test_arguments_of_the_wrong_kind():
+    with pytest.raises(ValueError, match="contiguous"):
+        _elsa_host.linear(*arguments(vals=torch.zeros(8, 64, dtype=torch.float16)[:, ::2]))
+    with pytest.raises(TypeError, match="tensor expected"):
+        _elsa_host.linear(*arguments(X=[1.0]))
+    with pytest.raises(TypeError):
+        _elsa_host.linear(*arguments(out="8"))
+    with pytest.raises(TypeError, match="13 arguments"):
+        _elsa_host.linear(*arguments()[:-1])
+    with pytest.raises(IndexError):
+        _elsa_host.compress(torch.zeros(64, dtype=torch.float16), 4, 8, 0, 0)
+    with pytest.raises(ValueError, match="levels"):
+        _elsa_host.compress_levels(torch.zeros(8, 64, dtype=torch.float16), (1, 2), 8, 0, 0)
+    with pytest.raises(RuntimeError):
+        _elsa_host.linear(*arguments(out=-8))
+
+
+def test_a_status_of_the_entry_point_comes_back_as_a_number():
+    assert _elsa_host.linear(*arguments(N=9)) == 3                     # ELSA_ERR_NM
+    assert _elsa_host.compress(torch.zeros(8, 64, dtype=torch.float16), 9, 8, 0, 0) in (1, 3)
+    with pytest.raises(lib.ElsaError) as e:
+        lib._result(_elsa_host.linear(*arguments(M=5)))
+    assert e.value.status == 3
