@@ -441,8 +441,8 @@ elsa_status elsa_attention(const void* qkv, int images, int tokens, int heads, i
 /* The same over windows of `tokens` consecutive rows with additive tables on the scores (Swin's window attention once
  * the rows are in window order): a = softmax(q k^T / sqrt d + bias[head] + mask[window % n_masks]) v.  bias: fp32
  * [heads][tokens][bias_pitch] (the relative-position bias as a dense table), mask: fp32 [n_masks][tokens][bias_pitch] or
- * NULL (the seam mask of shifted windows, one table per window position of an image); rows of bias_pitch >= tokens floats,
- * bias_pitch a multiple of 4, tables 16-byte aligned.  Head dimension 32 or 64 (dim = heads * 32 or heads * 64), tokens <= 256. */
+ * NULL (the seam mask of shifted windows, one table per window position of an image); rows of bias_pitch >= tokens floats
+ * (what lies behind the first `tokens` of a row takes no part), bias_pitch a multiple of 4, tables 16-byte aligned.  Head dimension 32 or 64 (dim = heads * 32 or heads * 64), tokens <= 256. */
 elsa_status elsa_window_attention(const void* qkv, int windows, int tokens, int heads, int dim, const float* bias,
                                   int bias_pitch, const float* mask, int n_masks, elsa_dtype dtype, void* a,
                                   uint32_t* dev_status, void* stream);

@@ -70,3 +70,29 @@ def test_window_in_a_warp_matches_oracle(lib, case, tables, dtype):
     err, tol = np.abs(got - bo._round16(ref, dtype)), tolerance(ref, q64[:, 2 * dim:], T, heads, dtype)
     worst = (err - tol).argmax()
     assert (err <= tol).all(), "error %g at tolerance %g" % (err.flat[worst], tol.flat[worst])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("filler", [float("nan"), float("inf")], ids=["nan", "inf"])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16], ids=["bf16", "f16"])
+@pytest.mark.parametrize("T", [1, 9, 15, 36, 47, 48, 49, 56, 57, 63, 65])
+def test_what_lies_behind_the_tables_rows_takes_no_part(lib, T, dtype, filler):
+    """A table's rows have bias_pitch floats; those from the window's last token on are the caller's to leave as they are."""
+    windows, heads = 5, 2
+    rng = np.random.default_rng(T)
+    qkv = synth.randn((windows * T, 3 * 32 * heads), 43, 1.5, dtype, "cuda")
+    bias = torch.from_numpy(rng.standard_normal((heads, T, T)).astype(np.float32))
+    mask = torch.from_numpy(np.where(rng.random((3, T, T)) < 0.3, -100.0, 0.0).astype(np.float32))
+
+    def padded(table, pitch, value):
+        out = torch.full((table.shape[0], T, pitch), value)
+        out[:, :, :T] = table
+        return out.cuda()
+
+    for pitch in ((T + 3) // 4 * 4, (T + 3) // 4 * 4 + 12):
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        got = [lib.elsa_window_attention(qkv, T, heads, padded(bias, pitch, v), padded(mask, pitch, v), dev_status=status)
+               for v in (0.0, filler)]
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        assert torch.isfinite(got[0]).all() and torch.equal(got[0], got[1])
