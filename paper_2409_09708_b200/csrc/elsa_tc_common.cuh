@@ -257,6 +257,13 @@ __device__ __forceinline__ uint64_t f32x2_add(uint64_t a, uint64_t b)
 // the polynomial and of the last product: 6.5 instructions and one special-function operation a value, 11 for one value
 // at a time, which made the epilogue the slowest part of a GELU layer on every GEMM kernel (50432 x 768 -> 3072, pair
 // kernel 304 -> 223 us, weight-stationary one 167 -> 137).
+// A NaN stays one: the clamp drops it from n, the maximum with 0 keeps it.  +inf gives +inf, -inf the limit, 0 within the error.
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 __device__ __forceinline__ float2 gelu_pair(float x, float y)
 {
     const float nx = fmaxf(-fabsf(x), -5.9375f), ny = fmaxf(-fabsf(y), -5.9375f);
@@ -271,7 +278,7 @@ __device__ __forceinline__ float2 gelu_pair(float x, float y)
     float ex, ey;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(p.x));
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ey) : "f"(p.y));
-    return f32x2_split(f32x2_fma(n, f32x2(ex, ey), f32x2(fmaxf(x, 0.0f), fmaxf(y, 0.0f))));
+    return f32x2_split(f32x2_fma(n, f32x2(ex, ey), f32x2(max_nan(x, 0.0f), max_nan(y, 0.0f))));
 }
 
 // What a GEMM's epilogue stores for two accumulators: + bias, GELU where the layer has it, rounded once.
