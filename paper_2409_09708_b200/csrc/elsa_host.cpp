@@ -75,6 +75,17 @@ int64_t size_at(const at::Tensor& t, int64_t dim)
     return t.size(dim);
 }
 
+// A tensor read as a matrix: a third dimension would be dropped without a word.
+const at::Tensor& matrix(PyObject* o)
+{
+    const at::Tensor& t = tensor(o);
+    if (t.dim() != 2) {
+        PyErr_Format(t.dim() < 2 ? PyExc_IndexError : PyExc_ValueError, "tensor of two dimensions expected, got %d", (int)t.dim());
+        throw Raised();
+    }
+    return t;
+}
+
 // The given tensor, or a new one of this shape beside `like`.
 at::Tensor given_or_new(PyObject* o, const at::Tensor& like, at::IntArrayRef shape, at::ScalarType type)
 {
@@ -143,7 +154,7 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n)
 PyObject* linear_masked(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     return guarded(n, 10, [&] {
-        const at::Tensor &X = tensor(a[0]), &W = tensor(a[1]);
+        const at::Tensor &X = matrix(a[0]), &W = matrix(a[1]);
         const int rows = (int)size_at(X, 0), in = (int)size_at(X, 1), out = (int)size_at(W, 0), N = integer(a[3]), M = integer(a[4]);
         const elsa_dtype code = (elsa_dtype)integer(a[5]);
         const at::Tensor Y = given_or_new(a[6], X, {rows, out}, X.scalar_type());
@@ -228,7 +239,7 @@ PyObject* packed_pair(const at::Tensor& vals, const at::Tensor& idx)
 PyObject* compress(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     return guarded(n, 5, [&]() -> PyObject* {
-        const at::Tensor& W = tensor(a[0]);
+        const at::Tensor& W = matrix(a[0]);
         const int out = (int)size_at(W, 0), in = (int)size_at(W, 1), N = integer(a[1]), M = integer(a[2]);
         const elsa_dtype code = (elsa_dtype)integer(a[3]);
         void *w = pointer(W), *stream = handle(a[4]);
@@ -250,7 +261,7 @@ PyObject* compress_levels(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     return guarded(n, 5, [&]() -> PyObject* {
         constexpr int kMost = 16;
-        const at::Tensor& W = tensor(a[0]);
+        const at::Tensor& W = matrix(a[0]);
         const int64_t out = size_at(W, 0), in = size_at(W, 1);
         const int M = integer(a[2]);
         const elsa_dtype code = (elsa_dtype)integer(a[3]);

@@ -35,3 +35,25 @@ def test_a_status_of_the_entry_point_comes_back_as_a_number():
     with pytest.raises(lib.ElsaError) as e:
         lib._result(_elsa_host.linear(*arguments(M=5)))
     assert e.value.status == 3
+
+
+class NullStream:
+    cuda_stream = 0
+
+
+def test_tensors_of_the_wrong_rank_are_refused():
+    """A weight is [out, in] and a masked linear's activations [rows, in]; other ranks would be read as if the first two sizes were all."""
+    f16 = lambda *shape: torch.zeros(shape, dtype=torch.float16)
+    wrong = pytest.raises((ValueError, IndexError))
+    for W in (f16(8, 4, 16), f16(1, 8, 64), f16(64)):
+        with wrong:
+            lib.elsa_nm_compress(W, 4, 8, stream=NullStream)
+        with wrong:
+            lib.elsa_nm_compress_levels(W, [1, 4], 8, stream=NullStream)
+        with wrong:
+            _elsa_host.compress_levels(W, [1, 4], 8, 0, 0)
+        with wrong:
+            lib.elsa_nm_linear_masked(f16(4, 64), W, None, 4, 8, stream=NullStream)
+    for X in (f16(4, 2, 64), f16(64)):
+        with wrong:
+            lib.elsa_nm_linear_masked(X, f16(8, 64), None, 4, 8, stream=NullStream)
