@@ -24,7 +24,14 @@ if not os.path.exists(LIB_PATH):
         "libelsa.so is missing: build it with `python -m paper_2409_09708_b200.build` "
         "(there is no CPU or PyTorch fallback for the sparse-linear path)")
 
-from . import _elsa_host  # noqa: E402  (built together with libelsa.so)
+_REBUILD = ("build the binding's native half for this Python and torch %s with `python -m paper_2409_09708_b200.build`"
+            % torch.__version__)
+try:
+    from . import _elsa_host  # noqa: E402  (built together with libelsa.so)
+except ImportError as e:
+    raise ImportError("%s: %s" % (e, _REBUILD)) from e
+if _elsa_host.torch_version != str(torch.__version__):
+    raise ImportError("_elsa_host was built with torch %s: %s" % (_elsa_host.torch_version or "of unknown version", _REBUILD))
 
 _lib = ctypes.CDLL(LIB_PATH)
 

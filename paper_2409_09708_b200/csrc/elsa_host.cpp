@@ -321,4 +321,17 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_elsa_host", nullptr, -1, g_meth
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__elsa_host() { return PyModule_Create(&g_module); }
+#ifndef ELSA_TORCH_VERSION
+#define ELSA_TORCH_VERSION ""
+#endif
+
+// torch_version: the torch whose headers this was compiled against; binding.py refuses another.
+PyMODINIT_FUNC PyInit__elsa_host()
+{
+    PyObject* m = PyModule_Create(&g_module);
+    if (m != nullptr && PyModule_AddStringConstant(m, "torch_version", ELSA_TORCH_VERSION) != 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

@@ -1,4 +1,9 @@
 """The native half of the binding: what it refuses and how, without a device (the checks come before any launch)."""
+import os
+import subprocess
+import sys
+import sysconfig
+
 import pytest
 import torch
 
@@ -57,3 +62,26 @@ def test_tensors_of_the_wrong_rank_are_refused():
     for X in (f16(4, 2, 64), f16(64)):
         with wrong:
             lib.elsa_nm_linear_masked(X, f16(8, 64), None, 4, 8, stream=NullStream)
+
+
+def test_the_module_is_of_this_python_and_torch(monkeypatch, tmp_path):
+    from paper_2409_09708_b200 import build
+    assert os.path.basename(_elsa_host.__file__) == "_elsa_host" + sysconfig.get_config_var("EXT_SUFFIX")
+    assert _elsa_host.torch_version == torch.__version__
+    stamp = tmp_path / "stamp"
+    monkeypatch.setattr(build, "_older", lambda built, deps: False)     # what the sources' times say is another matter
+    monkeypatch.setattr(build, "HOST_STAMP", str(stamp))
+    assert build.host_is_stale()                                       # no record of a torch
+    stamp.write_text("1.0")
+    assert build.host_is_stale()
+    stamp.write_text(torch.__version__)
+    assert not build.host_is_stale()
+
+
+@pytest.mark.parametrize("module", ["None", "type(sys)('paper_2409_09708_b200._elsa_host')"], ids=["missing", "other_torch"])
+def test_a_module_that_does_not_fit_says_what_to_run(module):
+    code = ("import sys, torch\nimport paper_2409_09708_b200 as p\nm = %s\nif m is not None: m.torch_version = '1.0'; p._elsa_host = m\n"
+            "sys.modules['paper_2409_09708_b200._elsa_host'] = m\nimport paper_2409_09708_b200.binding" % module)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    run = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True)
+    assert run.returncode != 0 and "ImportError" in run.stderr and "python -m paper_2409_09708_b200.build" in run.stderr, run.stderr
