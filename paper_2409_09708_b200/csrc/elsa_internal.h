@@ -121,9 +121,9 @@ elsa_status launch_linear_tc_pair(const uint16_t* X, int rows, const uint16_t* W
 // Y [m][n] = A^T B on the same kernel with both operands stored reduction-outermost, A [k][m] and B [k][n]
 // (m, n multiples of 8): the weight-gradient product dY^T X without transposed copies.
 // With splits > 1 the reduction is cut into that many ranges whose fp32 sums go to partial [splits][m][n] (Y is then
-// not written); linear_tc_pair_tn_splits says how many ranges keep the SM pairs occupied.  With sums_a (or
-// NULL) and no more tiles than SM pairs, *sums_parts rows of m floats that add up to the sums of A over the reduction go
-// there (at most linear_tc_pair_tn_sums_parts(n, splits)); otherwise *sums_parts is 0.
+// not written); linear_tc_pair_tn_splits says how many ranges keep the SM pairs occupied.  Where sums_a is not NULL, there
+// are no more tiles than SM pairs and no part has too many rows for the running sums, *sums_parts rows of m floats that add
+// up to the sums of A over the reduction go there (at most linear_tc_pair_tn_sums_parts(n, splits)); else *sums_parts is 0.
 int linear_tc_pair_tn_splits(int m, int n, int k, int sm_count);
 int linear_tc_pair_tn_sums_parts(int n, int splits);
 elsa_status launch_linear_tc_pair_tn(const uint16_t* A, const uint16_t* B, int m, int n, int k, elsa_dtype dtype,

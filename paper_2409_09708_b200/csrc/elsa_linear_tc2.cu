@@ -86,6 +86,10 @@ struct alignas(64) PairGroup {
     // (an eighth longer where two tiles share it: 36642 x 512 -> 1536 54 -> 67 us); as a pass of its own over dY with a
     // second launch to add its chunks it cost 33 us there.  Compress, forward and backward of a DeiT-B block at 25216 rows:
     // 1062 -> 976 us with this and the fused transposition of the weight.
+    // A tile's K blocks go to kSumSlots running sums by turns, so that none has more than kSumBlocksMost (above that the
+    // sums are a pass of their own): the tensor cores round a running sum worse than fp32 additions do, and with one of
+    // 50176 rows (401408 rows of one sign on one tile column) the largest error, 3.98e-4 of the sum by fp16's rounding
+    // alone, was 5.0e-4.
     float* sums_a;
     CUtensorMap map_r;   // fused form: the residual, boxes as map_y's
 };
@@ -114,6 +118,9 @@ struct PairShape {
     static constexpr int kStagingBufs = kForm == kFormFused ? kMaxChunksPerWarp : 1;
     static constexpr int kStagingTotal = kEpiWarps * kStagingBufs * kStagingBytes;
 };
+constexpr int kSumSlots = 8;               // running sums of A: 32 columns each of the second accumulator
+constexpr int kSumBlocksMost = 100;        // K blocks of one: 400 accumulations
+static_assert(kSumSlots * 32 <= kMaxBlockN, "the running sums fit the second accumulator");
 constexpr int kTnBoxBytes = 64 * 64 * 2;   // one box of the Tn form: 64 reduction rows of 128 bytes
 constexpr int kGroupMax = 72;   // layers per grouped launch (kernel parameters are limited to 32 KB)
 
@@ -273,13 +280,12 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                     kb1 = (int)((long long)p.layer[cur].num_k_blocks * (range + 1) / p.splits);
                 }
                 const uint32_t idesc = p.layer[cur].idesc;
-                int sum_kb = kb1;      // the next K block whose sums are this tile's
-                bool sums_begun = false;
+                int sum_kb = kb1, sum_count = 0;      // the next K block whose sums are this tile's, those before it
                 if constexpr (kTn) {
                     if (p.sums_a != nullptr) sum_kb = kb0 + ((tile - p.layer[cur].tile_begin) / p.splits) % p.layer[cur].tiles_n;
                 }
                 (void)sum_kb;
-                (void)sums_begun;
+                (void)sum_count;
                 ok = mbar_wait(tmem_empty_bar + 8 * acc, acc_phase ^ 1u, abort_flag, p.dev_status, 2);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
@@ -313,9 +319,10 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                             const uint32_t idesc32 = (idesc & ~(0x3Fu << 17)) | ((32u >> 3) << 17);     // N = 32
 #pragma unroll
                             for (int k = 0; k < kBlockK / kUmmaK; ++k)
-                                umma_f16_pair_if(tmem_u + kMaxBlockN, a_desc + (uint64_t)(k * (kUmmaK * 128 >> 4)), ones, idesc32,
-                                                 (uint32_t)(sums_begun || k != 0), elected);
-                            sums_begun = true;
+                                umma_f16_pair_if(tmem_u + (uint32_t)(kMaxBlockN + 32 * (sum_count % kSumSlots)),
+                                                 a_desc + (uint64_t)(k * (kUmmaK * 128 >> 4)), ones, idesc32,
+                                                 (uint32_t)(sum_count >= kSumSlots || k != 0), elected);
+                            ++sum_count;
                             sum_kb += p.layer[cur].tiles_n;
                         }
                     }
@@ -545,10 +552,16 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
                     if (p.sums_a != nullptr && part == 0) {
                         const int kb0 = (int)((long long)L.num_k_blocks * range / p.splits);
                         const int kb1 = (int)((long long)L.num_k_blocks * (range + 1) / p.splits);
-                        uint32_t d[32];      // 32 equal columns; the pair has no other tile, so they stay
-                        tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(q * 32) << 16) + kMaxBlockN, d);
+                        const int blocks = (kb1 - kb0 - t % L.tiles_n + L.tiles_n - 1) / L.tiles_n;      // this tile's
+                        uint32_t d[kSumSlots];      // of 32 equal columns one; the pair has no other tile, so they stay
+#pragma unroll
+                        for (int s = 0; s < kSumSlots; ++s)
+                            tmem_ld_32x32b_x1(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(kMaxBlockN + 32 * s), d[s]);
                         tmem_wait_ld();
-                        const float sum = kb0 + t % L.tiles_n < kb1 ? __uint_as_float(d[0]) : 0.f;      // else no block was its
+                        float sum = 0.f;
+#pragma unroll
+                        for (int s = 0; s < kSumSlots; ++s)
+                            if (s < blocks) sum += __uint_as_float(d[s]);      // the others were never written
                         if (row0 + lane < l_rows)
                             p.sums_a[((size_t)range * L.tiles_n + t % L.tiles_n) * (size_t)l_rows + row0 + lane] = sum;
                     }
@@ -764,7 +777,9 @@ elsa_status launch_group(const PairJob* jobs, int n, elsa_dtype dtype, uint32_t*
     const int pairs = g.num_tiles < max_pairs[slot].load(std::memory_order_acquire) ? g.num_tiles : max_pairs[slot].load(std::memory_order_acquire);
     g.sums_a = nullptr;
     if (kForm == kFormTn && jobs[0].sums_a != nullptr) {
-        const bool taken = g.num_tiles <= max_pairs[slot].load(std::memory_order_acquire);
+        const int blocks = (g.layer[0].num_k_blocks + g.splits - 1) / g.splits;
+        const bool taken = g.num_tiles <= max_pairs[slot].load(std::memory_order_acquire) &&
+                           (blocks + g.layer[0].tiles_n - 1) / g.layer[0].tiles_n <= kSumSlots * kSumBlocksMost;
         if (taken) g.sums_a = jobs[0].sums_a;
         *jobs[0].sums_parts = taken ? g.splits * g.layer[0].tiles_n : 0;
     }

@@ -56,3 +56,44 @@ def test_sums_of_random_values(dtype):
     d = dY.double()
     half_unit = 2.0 ** -9 if dtype == torch.bfloat16 else 2.0 ** -12
     assert ((db - d.sum(0)).abs() <= rows * 2.0 ** -23 * d.abs().sum(0) + half_unit * d.sum(0).abs() * 2).all()
+
+
+# Rows in the thousands, where a part of the sums has many K blocks: (rows, in, out) with 1, 2, 3 and 4 tile columns that take the K
+# blocks in turn, the reduction cut into 8, 4, 2 ranges and whole, remainders of the 64-row block, parts of unequal length,
+# and the row count above which the sums are a pass of their own.
+LONG = [(9001, 64, 256), (25216, 256, 256), (25217, 512, 1024), (9023, 1024, 520), (12608, 768, 2304), (39400, 768, 768), (4159, 1024, 4096),
+        (65536, 64, 256), (65600, 256, 264), (409600, 64, 72), (409601, 64, 72)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16], ids=["bf16", "f16"])
+@pytest.mark.parametrize("case", LONG, ids=["%dx%dx%d" % c for c in LONG])
+def test_long_sums_of_integers_are_exact(case, dtype):
+    """Integers up to 3, so that losing or repeating one row shows: |sums| < 2^24 in any order, one rounding at the end."""
+    rows, in_, out = case
+    rng = np.random.default_rng(rows)
+    ints = lambda *s: torch.from_numpy(rng.integers(-3, 4, s).astype(np.float32)).to(dtype)
+    dY, X, W = ints(rows, out), ints(rows, in_), ints(out, in_)
+    db = backward(dY, X, W, 2, 4, ("dW", "db"))[2].cpu()
+    assert torch.equal(db.double(), dY.double().sum(0).to(dtype).double())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16], ids=["bf16", "f16"])
+@pytest.mark.parametrize("case", [(25216, 64, 256), (65536, 64, 256), (401408, 64, 128), (420000, 64, 128)], ids=lambda c: "%dx%dx%d" % c)
+def test_long_sums_of_one_sign_lose_nothing_to_their_length(case, dtype):
+    """Values of one sign are where a running fp32 sum loses most.  At most 400 accumulations follow one another in a running sum and
+    8 such sums and 8 ranges are added after, each losing at most a unit (2^-23, truncation allowed for); as a pass of its own 64
+    additions of a thread, 8 of threads and one for every 512 rows, each rounded to nearest (2^-24).  The rounding at the end adds
+    half a unit of the type."""
+    rows, in_, out = case
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(rows)
+    dY = (torch.rand((rows, out), device="cuda", generator=gen) * 0.1 + 0.05).to(dtype)
+    X = torch.zeros((rows, in_), dtype=dtype, device="cuda")
+    W = synth.randn((out, in_), 3, 0.05, dtype)
+    db = backward(dY, X, W, 2, 4, ("dW", "db"))[2].double()
+    exact = dY.double().sum(0)
+    half_unit = 2.0 ** torch.floor(torch.log2(exact)) * (2.0 ** -8 if dtype == torch.bfloat16 else 2.0 ** -11)
+    chain = max(416 * 2.0 ** -23, (72 + rows / 512) * 2.0 ** -24)
+    assert ((db - exact).abs() <= half_unit + chain * exact).all(), float(((db - exact).abs() / half_unit).max())
