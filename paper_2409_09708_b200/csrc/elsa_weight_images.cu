@@ -12,6 +12,8 @@
 // those would be fewer than two blocks for an SM: 256 x 256 2.1 -> 1.5 us, 768 x 768 2.3 -> 1.7, 512 x 2048 at 8:16
 // 4.6 -> 3.1; from there up both take the same.
 
+#include <vector>
+
 #include "elsa_pack_device.cuh"
 
 namespace elsa {
@@ -19,6 +21,7 @@ namespace {
 
 constexpr int kImageThreads = 256;
 constexpr int kMostUnits = 4;             // dense images: units of 8 positions per thread, or one (see launch_images)
+constexpr long long kUnitsMost = 1ll << 31;   // of one image in a launch: a block's first unit and its last fit 32 bits
 
 struct ImageItem {
     const uint16_t* src;
@@ -435,6 +438,25 @@ elsa_status launch_table(const ImageJob* jobs, int n, int rounds, cudaStream_t s
 
 elsa_status launch_images(const ImageJob* jobs, int n, cudaStream_t stream)
 {
+    // A dense image's units are counted in 32 bits: a weight of more goes in runs of rows, each with its part of the packed form.
+    for (int i = 0; i < n; ++i) {
+        const ImageJob& j = jobs[i];
+        const long long rows = kUnitsMost / (j.in / 8);
+        if ((j.kind != IMAGE_UNPACK && j.kind != IMAGE_MASK) || j.out <= rows) continue;
+        const bool packed = j.kind == IMAGE_UNPACK;
+        const size_t src_row = packed ? values_per_row(j.in, j.N, j.M) : (size_t)j.in, idx_row = index_words_per_row(j.in, j.N, j.M);
+        std::vector<ImageJob> cut(jobs, jobs + i);
+        for (long long r = 0; r < j.out; r += rows) {
+            ImageJob part = j;
+            part.src = j.src + (size_t)r * src_row;
+            part.idx = j.idx != nullptr ? j.idx + (size_t)r * idx_row : nullptr;
+            part.dst = j.dst + (size_t)r * (size_t)j.in;
+            part.out = (int)(j.out - r < rows ? j.out - r : rows);
+            cut.push_back(part);
+        }
+        cut.insert(cut.end(), jobs + i + 1, jobs + n);
+        return launch_images(cut.data(), (int)cut.size(), stream);
+    }
     DeviceInfo dev;
     const elsa_status dev_st = device_info(&dev);
     if (dev_st != ELSA_OK) return dev_st;

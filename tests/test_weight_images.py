@@ -75,3 +75,27 @@ def test_ties_of_many_kinds_compress_as_the_oracle(lib, dtype):
                 assert (synth.bits(vals) == ovals).all(), (out, in_, N, M)
                 if N < M:
                     assert (idx.cpu().numpy().view(np.uint32) == oidx).all(), (out, in_, N, M)
+
+
+@pytest.mark.gpu
+def test_an_image_of_more_units_than_32_bits_count():
+    """2^32 units of eight positions and a few rows more (a 64 GB image, from 5 GB of packed values and words drawn at random: at 1:16
+    every field is a position): rows from the start, the middle and the end."""
+    from paper_2409_09708_b200 import binding as lib
+    in_, out = 1 << 15, (1 << 20) + 8
+    free, _ = torch.cuda.mem_get_info()
+    if free < 90 << 30:
+        pytest.skip("needs 90 GB of free device memory")
+    vals = torch.randint(1, 1 << 14, (out, in_ // 16), dtype=torch.int16, device="cuda").view(torch.float16)
+    idx = torch.randint(-(1 << 31), 1 << 31, (out, in_ // 128), dtype=torch.int64, device="cuda").to(torch.int32)
+    Wm = torch.empty((out, in_), dtype=torch.float16, device="cuda")
+    for r in (0, 1, out // 2 - 1, out // 2, out - 9, out - 8, out - 1):
+        Wm[r].fill_(7.0)
+    lib.elsa_nm_unpack(vals, idx, out, in_, 1, 16, W_masked=Wm)
+    torch.cuda.synchronize()
+    for r in (0, 1, out // 2 - 1, out // 2, out - 9, out - 8, out - 1):
+        words = idx[r].cpu().numpy().view(np.uint32)
+        pos = (words[:, None] >> (4 * np.arange(8, dtype=np.uint32))[None, :]).reshape(-1) & 15
+        want = np.zeros((in_ // 16, 16), np.int16)
+        want[np.arange(in_ // 16), pos] = vals[r].view(torch.int16).cpu().numpy()
+        assert (Wm[r].view(torch.int16).cpu().numpy() == want.reshape(-1)).all(), r
