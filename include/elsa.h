@@ -485,9 +485,11 @@ elsa_status elsa_vit_block_attn(const void* x, int images, int tokens, int heads
  * over the whole encoder), optionally followed by the model's final LayerNorm (final_gain / final_bias: [dim] device,
  * or both NULL).  Same results, bit for bit, as n_blocks calls of elsa_vit_block_attn; where a block's last linear runs
  * on a kernel that cannot add the residual, the next block's first LayerNorm (or the final one) adds it in the same
- * pass instead of a kernel of its own.  scratch: elsa_vit_encoder_scratch_bytes(...) bytes, 256-byte aligned (the
- * largest block's scratch plus two activation buffers); y [images * tokens][dim] may not alias x.  All blocks are
- * validated before the first launch.
+ * pass instead of a kernel of its own.  scratch: elsa_vit_encoder_scratch_bytes(...) bytes, 256-byte aligned: the
+ * largest block's scratch, two activation buffers and the weight images of all blocks, which are then built in one
+ * launch ahead of the chain.  With less, down to the largest block's scratch and two buffers of images * tokens * dim
+ * 16-bit values (each rounded up to 256 bytes), every block's images are built before the block: the same results.
+ * y [images * tokens][dim] may not alias x.  All blocks are validated before the first launch.
  */
 size_t elsa_vit_encoder_scratch_bytes(int images, int tokens, int dim, int mlp_dim, const elsa_block_weights* blocks,
                                       int n_blocks, elsa_dtype dtype);

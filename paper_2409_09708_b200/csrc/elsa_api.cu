@@ -1272,8 +1272,8 @@ elsa_status run_block(const void* x, int rows, int dim, int mlp_dim, const elsa_
 
 struct EncoderPlan {
     size_t block_bytes;   // scratch of the largest block
-    size_t images;        // the weight images of every block
     size_t buf[2];        // byte offsets of the two activation buffers the blocks alternate between
+    size_t images;        // the weight images of every block, behind what the chain cannot do without
     size_t total;
 };
 
@@ -1333,7 +1333,9 @@ elsa_status elsa_vit_encoder(const void* x, int images, int tokens, int heads, i
     if (!encoder_plan(rows, dim, mlp_dim, blocks, n_blocks, dtype, &plan))
         return fail(ELSA_ERR_SHAPE, "dim and mlp_dim must be multiples of 8 and every level valid");
     if (((uintptr_t)scratch & 255u) != 0) return fail(ELSA_ERR_ALIGN, "scratch must be 256-byte aligned");
-    if (scratch_bytes < plan.total) return fail(ELSA_ERR_WORKSPACE, "scratch of %zu bytes needed, %zu given", plan.total, scratch_bytes);
+    // With less than the whole the images of a block go to its own scratch, built before it runs: same results.
+    if (scratch_bytes < plan.images) return fail(ELSA_ERR_WORKSPACE, "scratch of %zu bytes needed, %zu given", plan.images, scratch_bytes);
+    const bool ahead = scratch_bytes >= plan.total;
     DeviceInfo dev;
     elsa_status st = device_info(&dev);
     if (st != ELSA_OK) return st;
@@ -1342,7 +1344,7 @@ elsa_status elsa_vit_encoder(const void* x, int images, int tokens, int heads, i
     // every block is validated before the first launch
     std::vector<PreparedBlock> prepared(n_blocks);
     std::vector<ImageJob> image_jobs;
-    uint8_t* image_at = s8 + plan.images;
+    uint8_t* image_at = ahead ? s8 + plan.images : nullptr;
     for (int b = 0; b < n_blocks; ++b) {
         PreparedBlock& p = prepared[b];
         if ((st = block_check(x, rows, dim, mlp_dim, blocks + b, dtype, buf[0], true, scratch, plan.block_bytes, &p.plan, p.lin, dev,
@@ -1351,6 +1353,7 @@ elsa_status elsa_vit_encoder(const void* x, int images, int tokens, int heads, i
             snprintf(msg, sizeof msg, "%s", elsa_last_error());
             return fail(st, "block %d: %s", b, msg);
         }
+        if (!ahead) continue;
         image_at += p.plan.total - p.plan.off[ELSA_BLOCK_WORKSPACE];
         add_images(p.lin, 4, &image_jobs);
         for (int l = 0; l < 4; ++l) p.lin[l].image_ready = takes_image(p.lin[l]);
@@ -1366,6 +1369,7 @@ elsa_status elsa_vit_encoder(const void* x, int images, int tokens, int heads, i
         const bool last = b + 1 == n_blocks;
         void* out = (last && final_gain == nullptr) ? y : (void*)buf[(b + 1) & 1];
         BlockCarry next;
+        if (!ahead && (st = block_images(prepared[b].lin, 4, (cudaStream_t)stream)) != ELSA_OK) return st;
         st = run_prepared(in, rows, dim, mlp_dim, blocks + b, dtype, out, scratch, prepared[b], dev_status, (cudaStream_t)stream,
                           tokens, heads, &carry, buf[b & 1], last && final_gain == nullptr ? nullptr : &next);
         if (st != ELSA_OK) return st;
