@@ -138,7 +138,8 @@ elsa_status check_linear(const void* X, int rows, const void* vals, const uint32
 
 // A side stream with its fork and join events, for the weight images that are built beside a call's other kernels.  A
 // call takes one from the device's pool and hands it back when all it enqueued is joined into the caller's stream, so
-// calls of several threads never share events; the pool holds as many as calls have ever overlapped.
+// calls of several threads never share events; the pool holds as many as calls have ever overlapped.  A stream that was
+// forked from a capturing one belongs to that capture until it ends: meanwhile only calls of the same capture take it.
 struct SidePipe {
     int device;
     cudaStream_t stream;
@@ -159,11 +160,19 @@ public:
     elsa_status fork(int device, cudaStream_t from)
     {
         if (!have_) {
+            unsigned long long capture = 0;
+            elsa_status st = capture_of(from, &capture);
+            if (st != ELSA_OK) return st;
             std::lock_guard<std::mutex> lock(g_side_mutex);
             std::vector<SidePipe>& pool = g_side[device & 63];
-            if (!pool.empty()) {
-                pipe_ = pool.back();
-                pool.pop_back();
+            size_t at = pool.size();
+            for (size_t i = pool.size(); i-- > 0 && at == pool.size();) {
+                unsigned long long held = 0;
+                if (pool[i].device == device && capture_of(pool[i].stream, &held) == ELSA_OK && (held == 0 || held == capture)) at = i;
+            }
+            if (at < pool.size()) {
+                pipe_ = pool[at];
+                pool.erase(pool.begin() + (long)at);
             } else {
                 pipe_.device = device;
                 const bool ok = cudaStreamCreateWithFlags(&pipe_.stream, cudaStreamNonBlocking) == cudaSuccess &&
@@ -197,6 +206,17 @@ public:
     cudaStream_t stream() const { return pipe_.stream; }
 
 private:
+    // The capture a stream takes part in, 0 if none.  (One that was invalidated stays until its owner ends it.)
+    static elsa_status capture_of(cudaStream_t s, unsigned long long* id)
+    {
+        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamGetCaptureInfo(s, &status, id);
+        if (e != cudaSuccess) { cudaGetLastError(); return fail(ELSA_ERR_CUDA, "asking for a stream's capture: %s", cudaGetErrorString(e)); }
+        if (status == cudaStreamCaptureStatusNone) *id = 0;
+        else if (status == cudaStreamCaptureStatusInvalidated) *id = ~0ull;
+        return ELSA_OK;
+    }
+
     bool have_ = false, forked_ = false;
     SidePipe pipe_;
 };

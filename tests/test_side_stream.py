@@ -69,3 +69,68 @@ def test_encoders_and_tables_of_several_threads_do_not_disturb_each_other():
         t.join()
     assert not errors, errors[0]
     assert not wrong, wrong
+
+
+@pytest.mark.gpu
+def test_a_capture_in_progress_keeps_its_side_stream_to_itself():
+    """A table's images fork to a side stream, which stays part of a capture until the capture ends.  Calls made meanwhile on other
+    streams, captured into another graph or not, succeed, the captures stay valid, and everything computes the same."""
+    from paper_2409_09708_b200 import binding as lib
+    dtype = torch.bfloat16
+    code = lib.dtype_code(dtype)
+
+    def table(seed):
+        layers = []
+        for i, (N, M) in enumerate([(4, 4), (2, 4), (1, 8), (4, 8)]):
+            X, W, bias = synth.layer_tensors(synth.Layer("l", 9000, 512, 512, N, M, 3 * i + seed, 3 * i + 1, 3 * i + 2), dtype, device="cuda")
+            vals, idx = lib.elsa_nm_compress(W, N, M)
+            layers.append(dict(X=X, vals=vals, idx=idx, bias=bias, N=N, M=M, Y=torch.empty((9000, 512), dtype=dtype, device="cuda")))
+        lt = lib.make_layer_table(layers)
+        return dict(lt=lt, Y=[l["Y"] for l in layers], ws=lib.alloc_workspace(lib.elsa_vit_workspace_bytes(lt, code)), keep=layers)
+
+    def run(t):
+        lib.elsa_vit_linears(t["lt"], code, t["ws"])
+
+    tables = [table(s) for s in (0, 100, 200)]
+    for t in tables:
+        run(t)
+    torch.cuda.synchronize()
+    want = [[y.clone() for y in t["Y"]] for t in tables]
+    for t in tables:
+        for y in t["Y"]:
+            y.zero_()
+    torch.cuda.synchronize()
+
+    first, second, plain = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.Stream()
+    g1, g2 = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+    errors = []
+
+    def meanwhile():
+        """What another thread does while the first capture is open: an ordinary call, then a capture of its own."""
+        try:
+            with torch.cuda.stream(plain):
+                run(tables[2])
+            with torch.cuda.stream(second):
+                g2.capture_begin(capture_error_mode="thread_local")
+                run(tables[1])
+                run(tables[1])
+                g2.capture_end()
+        except Exception as e:
+            errors.append(e)
+
+    with torch.cuda.stream(first):
+        g1.capture_begin(capture_error_mode="thread_local")
+        run(tables[0])
+        other = threading.Thread(target=meanwhile)
+        other.start()
+        other.join()
+        run(tables[0])                                               # the capture's own pipe again
+        g1.capture_end()
+    assert not errors, errors[0]
+    g1.replay()
+    g2.replay()
+    run(tables[2])                                                   # pipes of ended captures serve ordinary calls
+    torch.cuda.synchronize()
+    for t, ys in zip(tables, want):
+        for y, w in zip(t["Y"], ys):
+            assert torch.equal(y, w)
