@@ -42,10 +42,10 @@ def family_bytes(csv_path):
         if not m:
             continue
         args = [a.strip() for a in m.group(2).split(",")]
-        # the layer-table launches are the instantiations whose layer capacity is above one: <bf16, capacity, ...> for
-        # the sparse kernels, <bf16, form, capacity> for the dense pair kernel
+        # the layer-table launches are the instantiations for more layers than a launch of one layer has entries (two on the
+        # dense pair kernel, which may cut its rows): <bf16, capacity, ...> for the sparse kernels, <bf16, form, capacity> there
         capacity = int(args[2]) if m.group(1) == "linear_tc_pair" else int(args[1])
-        if capacity <= 1:
+        if capacity <= 2:
             continue
         f = fam.setdefault(m.group(1), {"bytes": 0.0, "launches": 0})
         f["bytes"] += d["bytes"]

@@ -128,3 +128,17 @@ def test_kernel_source_hash_follows_the_sources():
     import bench
     h = bench.kernel_source_hash()
     assert len(h) == 64 and h == bench.kernel_source_hash()
+
+
+def test_traffic_counts_the_launches_that_carry_a_table(tmp_path):
+    import bench_traffic
+    kernels = [("linear_tc_pair_kernel<1, 0, 72>", 5), ("linear_tc_pair_kernel<1, 0, 2>", 100), ("linear_tc_pair_kernel<1, 3, 1>", 200),
+               ("linear_tc_sp24_ws_kernel<1, 68, 0>", 7), ("linear_tc_sp24_ws_kernel<1, 1, 0>", 300)]
+    lines = ['"ID","Kernel Name","Metric Name","Metric Value"']
+    for i, (name, value) in enumerate(kernels):
+        for metric in ("dram__bytes_read.sum", "dram__bytes_write.sum"):
+            lines.append('"%d","void elsa::<unnamed>::%s(elsa::P)","%s","%d"' % (i, name, metric, value))
+    path = tmp_path / "dram.csv"
+    path.write_text("\n".join(lines))
+    fam = bench_traffic.family_bytes(str(path))
+    assert {k: (v["bytes"], v["launches"]) for k, v in fam.items()} == {"linear_tc_pair": (10.0, 1), "linear_tc_sp24_ws": (14.0, 1)}
