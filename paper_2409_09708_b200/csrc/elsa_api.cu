@@ -1100,7 +1100,8 @@ elsa_status block_linear(BlockLinear& L, const uint16_t* X, int rows, elsa_dtype
         job.act = act; job.residual = residual;
         DeviceInfo dev;
         if ((st = device_info(&dev)) != ELSA_OK) return st;
-        // after another kernel of the same call the weights are older than that kernel's start
+        // after another kernel of the same call the weights are older than that kernel's start (KIND_SMALL: only where the
+        // variant is forced, a chain picks KIND_SMALL_IMAGE)
         const bool early = !L.first && (L.kind == KIND_SMALL || w.N == w.M || ready);
         return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, dev.sm_count), early, dtype, dev_status, stream);
     }

@@ -4,17 +4,18 @@
 // A layer of one or a few images has too few 256-row tiles to occupy the SM pairs of the persistent kernels, and what
 // it pays for is latency: the launch of the kernel that rebuilds the weight image, a persistent kernel's set-up, one
 // long reduction per tile.  Here
-//   * the weight tile is expanded on the way to shared memory by eight warps that read the packed values and index
-//     words (or project the dense shared weight, for the masked form), so that there is no image and no second
-//     launch; the dense level's tile comes by TMA;
+//   * a call of one layer has the weight tile expanded on the way to shared memory by eight warps that read the packed
+//     values and index words (or project the dense shared weight, for the masked form), so that there is no image and
+//     no second launch; the dense level's tile comes by TMA, and so do the images that the layers of a table and of a
+//     chained block bring along (one launch builds those of a whole call);
 //   * a CTA computes one tile of 128 rows x 64 features and leaves; two CTAs fit an SM, so that one's set-up and
 //     epilogue run under the other's tile, or the next kernel's set-up under this one's;
 //   * where the tiles alone leave SMs idle, the reduction is cut into 2, 4 or 8 ranges, one CTA of a cluster each:
 //     every CTA sends the rows of its fp32 sums to the CTA that owns them through distributed shared memory, one
 //     cluster barrier, and each owner adds its rows in rank order (deterministic), applies bias, activation and
 //     residual, and rounds once;
-//   * a call that knows the weights to be older than its own first kernel (the chained block) lets the expansion
-//     start before the predecessor kernel has ended (`early`): only X and the outputs wait for it.
+//   * a call that knows the weights to be older than its own first kernel (the chained block) has their first tiles
+//     fetched before the predecessor kernel has ended (`early`): only X and the outputs wait for it.
 // Measured back to back on 197 rows (us, weight image + one-CTA-per-tile GEMM before, this kernel after): 768 -> 768 at
 // 2:4 6.9 -> 6.4, 768 -> 2304 at 2:4 8.2 -> 7.7, 3072 -> 768 at 2:4 15.4 -> 10.6, at 4:4 11.6 -> 6.9.  The expansion
 // is repeated for every 128 rows and bound by its loads' latency and its instructions: at 788 rows and 2:4 the image
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
     const int tile = tile_all - L.tile_begin;
     const int m0 = (tile / L.tiles_n) * kTileM, n0 = (tile % L.tiles_n) * kTileN;
     const int kb0 = L.k_blocks * rank / splits, kb1 = L.k_blocks * (rank + 1) / splits;
-    const bool expand = L.source != SRC_DENSE;
+    const bool expand = kMax == 1 && L.source != SRC_DENSE;      // a group's weights are all dense or images
 
     const int sums_off = split ? p.stages * kStageBytes : 0;
     const int bar_off = split ? sums_off + kSumBytes : p.stages * kStageBytes;
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
         // ------------------------------------------------ expansion, then epilogue
         if (!p.early) pdl_wait_for_predecessors();
         bool ok = true;
-        if (expand) {
+        if constexpr (kMax == 1) if (expand) {
             const uint16_t* w = L.w;
             const uint32_t* idx = L.idx;
             const int N = L.N, in = L.in, wpr = L.words_per_row;
@@ -450,6 +451,8 @@ elsa_status launch_linear_small_group(const SmallJob* jobs, int n, int splits, b
     elsa_status st = device_info(&dev);
     if (st != ELSA_OK) return st;
     if (n < 1 || n > kSmallGroupMax) return fail(ELSA_ERR_SHAPE, "a grouped launch carries 1 to %d layers, got %d", kSmallGroupMax, n);
+    for (int i = 0; n > 1 && i < n; ++i)
+        if (jobs[i].N != jobs[i].M) return fail(ELSA_ERR_NM, "layer %d of a grouped launch is packed (%d:%d)", i, jobs[i].N, jobs[i].M);
     if (dtype == ELSA_BF16)
         return n == 1 ? launch_small<true, 1>(jobs, n, splits, early, dev_status, stream, dev)
                       : launch_small<true, kSmallGroupMax>(jobs, n, splits, early, dev_status, stream, dev);

@@ -1,7 +1,6 @@
-// Device code of the weight-format kernels, shared by the per-weight launches and the batched ones:
-// N:M projection + packing (Sec. 3.1 / Eq. 1 and the compressed form of Sec. 1 / Sec. 2 of the ELSA
-// paper), its inverse, and the re-encoding of a packed weight as 2-of-4 values + tensor-memory
-// metadata for the sparse MMA.  Each function handles one unit of work given its global index.
+// Device code shared by the kernels that read or write the packed weight: the choice of the kept positions of a group
+// (Sec. 3.1 / Eq. 1 of the ELSA paper), the general form of packing (the levels in use have their own in elsa_compress.cu),
+// and the expansion of eight consecutive positions from the packed form (Sec. 1 / Sec. 2) or from a dense weight.
 #pragma once
 
 #include "elsa_internal.h"
@@ -30,9 +29,6 @@ __device__ __forceinline__ void load_group(const uint16_t* p, uint16_t (&w)[M])
     }
 }
 
-// One warp compresses 32 consecutive groups of one row, one group per lane.  The 32 groups own
-// exactly N*b whole index words of the row's bitstream, so each warp assembles its words in shared
-// memory and writes them with one coalesced store.
 // Ranks of the M magnitudes of one group, 4 bits each: rank_i = #{j : |w_j| > |w_i|} + #{j < i : |w_j| == |w_i|}
 // (larger magnitude first, lower position first among equals).  Magnitudes are compared as the 15 low
 // bits of the pattern.  The level N keeps exactly the elements with rank < N, for every N at once.
