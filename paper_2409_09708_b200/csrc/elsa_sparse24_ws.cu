@@ -57,7 +57,7 @@ constexpr int kStagingTotal = kEpiWarps * kStagingBytes;
 constexpr int kBarrierBytes = 512;
 
 struct alignas(64) WsLayer {
-    CUtensorMap map_x, map_y, map_y16;   // map_y: a warp's whole run of token rows, map_y16: one step of it
+    CUtensorMap map_x, map_y;   // map_y: one step of 16 token rows
     const uint16_t* a_img;   // 2-of-4 values [out rounded up to 32][in / 2], rows in the permuted order
     const uint8_t* meta;     // metadata blocks of 2 KB per (128 features, 128 k)
     const uint16_t* bias;
@@ -71,7 +71,7 @@ struct alignas(64) WsLayer {
     int act;           // epilogue activation (0 none, 1 GELU) on acc + bias
 };
 
-constexpr int kGroupMax = 68;   // layers per launch (kernel parameters are limited to 32 KB)
+constexpr int kGroupMax = 92;   // layers per launch (kernel parameters are limited to 32 KB)
 
 template <int kMaxLayers>
 struct WsGroup {
@@ -80,6 +80,7 @@ struct WsGroup {
     int stages;
     int stage_bytes;   // one pipeline stage: kStageK / 64 quarters of (largest nt / 2) rows of 128 bytes
     uint32_t* dev_status;
+    CUtensorMap map_run;   // kAct: Y in boxes of a warp's whole run of token rows
 };
 
 // kAct: the instantiation whose epilogue applies the layer's activation (single-layer launches).
@@ -367,13 +368,16 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
                 __syncwarp();
                 if (lane == 0) {
                     if (f0 < l_out) {
-                        if (my_steps == L.steps_per_warp) {
-                            if (row0 < l_rows) tma_store_2d(&L.map_y, buf, f0, row0);
+                        // With GELU the warps are short of issue slots and a run leaves as one store (50432 x 768 -> 3072 138
+                        // -> 131 us); without it as one a step, which start while the rest is on its way: 65536 x
+                        // 768 -> 3072 alone 136 us, 144 by runs, back to back 141.2 and 142.2.
+                        if (kAct && my_steps == L.steps_per_warp) {
+                            if (row0 < l_rows) tma_store_2d(&p.map_run, buf, f0, row0);
                         } else {
 #pragma unroll
                             for (int s = 0; s < kMaxSteps; ++s)
                                 if (s < my_steps && row0 + s * kStepCols < l_rows)
-                                    tma_store_2d(&L.map_y16, buf + (uint32_t)(s * kStepCols * 64), f0, row0 + s * kStepCols);
+                                    tma_store_2d(&L.map_y, buf + (uint32_t)(s * kStepCols * 64), f0, row0 + s * kStepCols);
                         }
                     }
                     bulk_commit_group();
@@ -483,11 +487,11 @@ elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
                   ((uint32_t)(kPairFeat >> 4) << 24);
         elsa_status st;
         if ((st = make_map_x_quarters(&L.map_x, j.X, (uint64_t)j.in, (uint64_t)j.rows, (uint32_t)(L.nt / 2), kStageK / 64)) != ELSA_OK) return st;
-        if ((st = make_map_2d(&L.map_y, j.Y, (uint64_t)j.out, (uint64_t)j.rows, 32, (uint32_t)(kStepCols * L.steps_per_warp),
-                              CU_TENSOR_MAP_SWIZZLE_NONE, "Y")) != ELSA_OK)
-            return st;
-        if ((st = make_map_2d(&L.map_y16, j.Y, (uint64_t)j.out, (uint64_t)j.rows, 32, kStepCols, CU_TENSOR_MAP_SWIZZLE_NONE,
+        if ((st = make_map_2d(&L.map_y, j.Y, (uint64_t)j.out, (uint64_t)j.rows, 32, kStepCols, CU_TENSOR_MAP_SWIZZLE_NONE,
                               "Y")) != ELSA_OK)
+            return st;
+        if (kAct && (st = make_map_2d(&g.map_run, j.Y, (uint64_t)j.out, (uint64_t)j.rows, 32, (uint32_t)(kStepCols * L.steps_per_warp),
+                                      CU_TENSOR_MAP_SWIZZLE_NONE, "Y")) != ELSA_OK)
             return st;
     }
     g.n_layers = n;
