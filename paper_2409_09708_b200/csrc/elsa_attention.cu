@@ -48,7 +48,7 @@ constexpr int kQBytes = kQRows * kMaxHeadDim * 2;          // the shared-memory 
 
 // kBufs items in flight per CTA: 2 for up to 256 keys (256 tensor-memory columns each), 4 for up to 128 keys (the
 // windows of Swin), where an item's on-chip chain is short and only more of them in flight fill the SM.
-template <int kBufs, bool kBias>
+template <int kD, int kBufs, bool kBias>
 struct Shape {
     static constexpr int kBufCols = kTmemCols / kBufs;
     static constexpr int kThreads = (2 + kBufs * kGroupWarps) * 32;
@@ -58,7 +58,7 @@ struct Shape {
     static constexpr int kOutBytes = 32 * kOutCols * 2;
     static constexpr int kSmemBytes = kBufs * (kStageBytes + kGroupWarps * kOutBytes) + 1024 /* alignment */ + 512 /* barriers */;
     static constexpr int kBiasUnit = kBufs == 2 ? 32 : 16;  // score columns a softmax warp handles at a time (registers):
-    static constexpr int kUnit = 32;                        // adding the tables, exponentiating
+    static constexpr int kUnit = kBufs == 4 && kD == 32 && !kBias ? 16 : 32;   // adding the tables; exponentiating
 };
 
 struct AttnParams {
@@ -127,19 +127,19 @@ __device__ __forceinline__ void tmem_ld_32x32b_x8(uint32_t taddr, uint32_t (&r)[
 }
 
 template <bool kBf16, int kD, bool kBias, int kBufs>
-__global__ void __launch_bounds__(Shape<kBufs, kBias>::kThreads, 1) attention_kernel(const __grid_constant__ AttnParams p)
+__global__ void __launch_bounds__(Shape<kD, kBufs, kBias>::kThreads, 1) attention_kernel(const __grid_constant__ AttnParams p)
 {
     static_assert(kD == 64 || kD == 32, "head dimension");
     static_assert(kBufs == 2 || kBufs == 4, "items in flight");
-    constexpr int kBufCols = Shape<kBufs, kBias>::kBufCols, kStageBytes = Shape<kBufs, kBias>::kStageBytes, kKvBytesMax = Shape<kBufs, kBias>::kKvBytes;
-    constexpr int U = Shape<kBufs, kBias>::kUnit, B = Shape<kBufs, kBias>::kBiasUnit;
+    constexpr int kBufCols = Shape<kD, kBufs, kBias>::kBufCols, kStageBytes = Shape<kD, kBufs, kBias>::kStageBytes, kKvBytesMax = Shape<kD, kBufs, kBias>::kKvBytes;
+    constexpr int U = Shape<kD, kBufs, kBias>::kUnit, B = Shape<kD, kBufs, kBias>::kBiasUnit;
     constexpr int kLag = kBufs - 1;                   // P V of item n - kLag is issued after S of item n
     constexpr int kHeadDim = kD;
     constexpr int kItemQBytes = kQRows * kD * 2;      // bytes TMA delivers for the Q tile; K and V: tk * kD * 2
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t out_base = smem_base + kBufs * kStageBytes;
-    const uint32_t bars = out_base + kBufs * kGroupWarps * Shape<kBufs, kBias>::kOutBytes;
+    const uint32_t bars = out_base + kBufs * kGroupWarps * Shape<kD, kBufs, kBias>::kOutBytes;
     // per buffer b: +0 qk_full, +8 v_full, +16 qk_empty, +24 s_full, +32 p_full, +40 o_full, +48 tmem_empty, +56 v_empty
     auto bar = [&](int which, int b) { return bars + (uint32_t)(64 * b + 8 * which); };
     enum { kQkFull = 0, kVFull, kQkEmpty, kSFull, kPFull, kOFull, kTmemEmpty, kVEmpty };
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(Shape<kBufs, kBias>::kThreads, 1) attention_ke
         // ------------------------------------------------ softmax and output: group g takes the items n = g, g + 2, ...
         const int g = (warp - 2) / kGroupWarps;
         const int quarter = warp & 3;                                  // the TMEM lanes this warp may touch
-        const uint32_t stage_out = out_base + (uint32_t)((warp - 2) * Shape<kBufs, kBias>::kOutBytes);
+        const uint32_t stage_out = out_base + (uint32_t)((warp - 2) * Shape<kD, kBufs, kBias>::kOutBytes);
         constexpr float kFar = 32768.f;     // no probability above it: inside the 16-bit types and far inside fp32
         const float scale = (kD == 64 ? 0.125f : 0.17677669529663687f) * 1.4426950408889634f;   // log2(e) / sqrt(kD)
         bool ok = true;
@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(Shape<kBufs, kBias>::kThreads, 1) attention_ke
             // until the values are used): the first unit is asked for before the scores are waited for, every other
             // one while the unit before it is worked on, which takes most of the L2 latency out of the item's chain.
             // The mask (shifted windows only) is read where it is used: a second array across the wait would spill.
-            constexpr int kReq = kBias ? Shape<kBufs, kBias>::kBiasUnit : 1;
+            constexpr int kReq = kBias ? Shape<kD, kBufs, kBias>::kBiasUnit : 1;
             float bq[kReq];
             auto request = [&](int col0) {
 #pragma unroll
@@ -516,7 +516,8 @@ __global__ void __launch_bounds__(Shape<kBufs, kBias>::kThreads, 1) attention_ke
                     // four groups of warps have each other's work to run under a load
                     for (int u = 0; u < units; ++u) {
                         uint32_t r[U];
-                        tmem_ld_32x32b_x32(t_lane + (uint32_t)(U * u), r);
+                        if constexpr (U == 32) tmem_ld_32x32b_x32(t_lane + (uint32_t)(U * u), r);
+                        else tmem_ld_32x32b_x16(t_lane + (uint32_t)(U * u), r);
                         tmem_wait_ld();
                         if (!kBias && u == 0) ref = first_top(r);
                         unit(r, u);
@@ -537,7 +538,7 @@ __global__ void __launch_bounds__(Shape<kBufs, kBias>::kThreads, 1) attention_ke
             const float inv = 1.0f / sum;
             // A lane has a row of the output; the rows leave through shared memory (16-byte vectors, swizzled), so that a
             // store instruction covers whole 64- or 128-byte rows instead of 16 bytes of 32 lines.
-            constexpr int kCols = Shape<kBufs, kBias>::kOutCols < kD ? Shape<kBufs, kBias>::kOutCols : kD;
+            constexpr int kCols = Shape<kD, kBufs, kBias>::kOutCols < kD ? Shape<kD, kBufs, kBias>::kOutCols : kD;
             constexpr int kVecs = kCols / 8, kRowsPerStore = 32 / kVecs;
 #pragma unroll
             for (int c = 0; c < kD / kCols; ++c) {
@@ -609,7 +610,7 @@ elsa_status make_map_qkv(CUtensorMap* map, const void* qkv, int images, int toke
 template <bool kBf16, int kD, bool kBias, int kBufs>
 elsa_status launch(const AttnParams& p, int images, int heads, cudaStream_t stream, const DeviceInfo& dev)
 {
-    constexpr int kSmemBytes = Shape<kBufs, kBias>::kSmemBytes, kThreads = Shape<kBufs, kBias>::kThreads;
+    constexpr int kSmemBytes = Shape<kD, kBufs, kBias>::kSmemBytes, kThreads = Shape<kD, kBufs, kBias>::kThreads;
     auto kernel = attention_kernel<kBf16, kD, kBias, kBufs>;
     static std::atomic<bool> attr_set[64];
     const int slot = dev.device & 63;

@@ -10,7 +10,8 @@ import torch
 from oracle import elsa_block_oracle as bo
 from paper_2409_09708_b200 import synth
 
-SHAPES = [(3, 17, 1, 64), (2, 64, 2, 64), (2, 65, 2, 64), (1, 128, 1, 32), (2, 129, 2, 64), (2, 197, 3, 64), (1, 256, 2, 64), (1, 200, 2, 32)]
+SHAPES = [(3, 17, 1, 64), (2, 64, 2, 64), (2, 65, 2, 64), (1, 128, 1, 32), (2, 129, 2, 64), (2, 197, 3, 64), (1, 256, 2, 64), (1, 200, 2, 32),
+          (3, 65, 2, 32), (2, 80, 1, 32), (2, 97, 3, 32)]
 
 
 def profile(kind, tokens):
