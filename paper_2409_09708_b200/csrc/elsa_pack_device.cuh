@@ -29,89 +29,6 @@ __device__ __forceinline__ void load_group(const uint16_t* p, uint16_t (&w)[M])
     }
 }
 
-// Ranks of the M magnitudes of one group, 4 bits each: rank_i = #{j : |w_j| > |w_i|} + #{j < i : |w_j| == |w_i|}
-// (larger magnitude first, lower position first among equals).  Magnitudes are compared as the 15 low
-// bits of the pattern.  The level N keeps exactly the elements with rank < N, for every N at once.
-template <int M>
-__device__ __forceinline__ unsigned long long group_ranks(const uint16_t (&w)[M])
-{
-    unsigned long long ranks = 0;
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-        const uint32_t ki = w[i] & 0x7FFFu;
-        int rank = 0;
-#pragma unroll
-        for (int j = 0; j < M; ++j) {
-            const uint32_t kj = w[j] & 0x7FFFu;
-            rank += (kj > ki) || (j < i && kj == ki);
-        }
-        ranks |= (unsigned long long)rank << (4 * i);
-    }
-    return ranks;
-}
-
-template <int M>
-__device__ __forceinline__ uint32_t keep_mask(unsigned long long ranks, int N)
-{
-    uint32_t keep = 0;
-#pragma unroll
-    for (int i = 0; i < M; ++i) keep |= (uint32_t)((int)((ranks >> (4 * i)) & 15ull) < N) << i;
-    return keep;
-}
-
-// One warp compresses 32 consecutive groups of one row, one group per lane, at any level N < M: the form for the levels
-// that have none of their own (elsa_compress.cu).  The 32 groups own exactly N*b whole index words of the row's
-// bitstream, so the warp assembles its words in shared memory and writes them with one coalesced store.
-template <int M>
-__device__ __forceinline__ void compress_segment(const uint16_t* __restrict__ W, int in, int N, uint16_t* __restrict__ vals,
-                                                 uint32_t* __restrict__ idx, int segs_per_row, int words_per_row, long long seg_id,
-                                                 uint32_t (*words)[kMaxIndexWordsPerSegment])
-{
-    constexpr int B = (M == 4) ? 2 : (M == 8) ? 3 : 4;
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-
-    const int o = (int)(seg_id / segs_per_row);
-    const int seg = (int)(seg_id % segs_per_row);
-    const int groups_per_row = in / M;
-    const int g = seg * 32 + lane;
-    const int seg_words = N * B;  // index words this segment owns
-
-    for (int k = lane; k < seg_words; k += 32) words[warp][k] = 0;
-    __syncwarp();
-    if (g < groups_per_row) {
-        uint16_t w[M];
-        load_group<M>(W + (size_t)o * in + (size_t)g * M, w);
-        const uint32_t keep = keep_mask<M>(group_ranks<M>(w), N);
-        uint16_t* v = vals + (size_t)o * ((size_t)groups_per_row * N) + (size_t)g * N;
-        unsigned long long fields = 0;
-        int t = 0;
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            if ((keep >> i) & 1u) {
-                v[t] = w[i];
-                fields |= (unsigned long long)i << (t * B);
-                ++t;
-            }
-        }
-        const int bit0 = lane * seg_words;  // bit offset of this group's fields in the segment
-        const int w0 = bit0 >> 5, sh = bit0 & 31;
-        // up to 60 bits shifted by up to 31: three words at most
-        const uint32_t lo = (uint32_t)(fields << sh);
-        const uint32_t mid = (uint32_t)(fields >> (32 - sh));
-        const uint32_t hi = sh ? (uint32_t)(fields >> (64 - sh)) : 0u;
-        // a zero part may lie past the segment's last word and is skipped
-        if (lo) atomicOr(&words[warp][w0], lo);
-        if (mid) atomicOr(&words[warp][w0 + 1], mid);
-        if (hi) atomicOr(&words[warp][w0 + 2], hi);
-    }
-    __syncwarp();
-    const int first = seg * seg_words;
-    uint32_t* row = idx + (size_t)o * words_per_row;
-    for (int k = lane; k < seg_words && first + k < words_per_row; k += 32) row[first + k] = words[warp][k];
-    __syncwarp();
-}
-
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
 {
     uint32_t r;
@@ -196,15 +113,12 @@ __device__ __forceinline__ uint32_t half_of(const uint32_t (&a)[kWords], uint32_
     return (pos & 1u ? w >> 16 : w) & 0xFFFFu;
 }
 
-// Keep mask of a group of 16 (words of two positions), N <= 8.  The even and the odd positions' magnitudes are sorted side
+// Keep mask of a group of 16 (words of two positions).  The even and the odd positions' magnitudes are sorted side
 // by side, two to an instruction; the N-th largest of the two sorted lists A, B is the largest of the minima of A's i-th
 // and B's (N - i)-th.  What exceeds it is kept, and of what equals it the lowest positions that are still needed.  (768 x
 // 768 at 2:16 1.8 us against 5.8 by ranks; groups of 8 and 4 are 5 to 20 % quicker by keep_mask_sorted.)
-template <int N>
-__device__ __forceinline__ uint32_t keep_mask16(const uint32_t (&a)[8])
+__device__ __forceinline__ void sort_halves16(const uint32_t (&a)[8], uint32_t (&k)[8], uint32_t (&s)[8])
 {
-    static_assert(N >= 1 && N <= 8, "candidates from two lists of eight");
-    uint32_t k[8], s[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) s[q] = k[q] = a[q] & 0x7FFF7FFFu;
     auto sort2 = [&](int x, int y) {
@@ -217,12 +131,25 @@ __device__ __forceinline__ uint32_t keep_mask16(const uint32_t (&a)[8])
     sort2(0, 4); sort2(1, 5); sort2(2, 6); sort2(3, 7);
     sort2(2, 4); sort2(3, 5);
     sort2(1, 2); sort2(3, 4); sort2(5, 6);
+}
+
+// The N-th largest magnitude of the two sorted lists.
+template <int N>
+__device__ __forceinline__ uint32_t threshold16(const uint32_t (&s)[8])
+{
+    static_assert(N >= 1 && N <= 15, "levels below the dense one");
+    constexpr int kFirst = N > 8 ? N - 8 : 0, kLast = N < 8 ? N : 8;      // how many of the N may come from A
     uint32_t thr = 0;
 #pragma unroll
-    for (int i = 0; i <= N; ++i) {       // i of A and N - i of B lie at or above the candidate
+    for (int i = kFirst; i <= kLast; ++i) {       // i of A and N - i of B lie at or above the candidate
         const uint32_t x = i > 0 ? s[i > 0 ? i - 1 : 0] & 0xFFFFu : 0xFFFFu, y = i < N ? s[i < N ? N - i - 1 : 0] >> 16 : 0xFFFFu;
         thr = max(thr, min(x, y));
     }
+    return thr;
+}
+
+__device__ __forceinline__ uint32_t keep_above16(const uint32_t (&k)[8], uint32_t thr, int N)
+{
     const uint32_t thr2 = thr | (thr << 16);
     uint32_t above = 0, least = 0;       // magnitudes > thr, >= thr (15-bit values: a borrow clears the half's top bit)
 #pragma unroll
@@ -240,6 +167,103 @@ __device__ __forceinline__ uint32_t keep_mask16(const uint32_t (&a)[8])
         equal &= equal - 1u;
     }
     return keep;
+}
+
+template <int N>
+__device__ __forceinline__ uint32_t keep_mask16(const uint32_t (&a)[8])
+{
+    uint32_t k[8], s[8];
+    sort_halves16(a, k, s);
+    return keep_above16(k, threshold16<N>(s), N);
+}
+
+// The same for a level known at run time.
+__device__ __forceinline__ uint32_t keep_mask16_any(const uint32_t (&a)[8], int N)
+{
+    uint32_t k[8], s[8], thr;
+    sort_halves16(a, k, s);
+    switch (N) {
+    case 1: thr = threshold16<1>(s); break;
+    case 2: thr = threshold16<2>(s); break;
+    case 3: thr = threshold16<3>(s); break;
+    case 4: thr = threshold16<4>(s); break;
+    case 5: thr = threshold16<5>(s); break;
+    case 6: thr = threshold16<6>(s); break;
+    case 7: thr = threshold16<7>(s); break;
+    case 8: thr = threshold16<8>(s); break;
+    case 9: thr = threshold16<9>(s); break;
+    case 10: thr = threshold16<10>(s); break;
+    case 11: thr = threshold16<11>(s); break;
+    case 12: thr = threshold16<12>(s); break;
+    case 13: thr = threshold16<13>(s); break;
+    case 14: thr = threshold16<14>(s); break;
+    default: thr = threshold16<15>(s); break;
+    }
+    return keep_above16(k, thr, N);
+}
+
+// One warp compresses 32 consecutive groups of one row, one group per lane, at any level N < M: the form for the levels
+// that have none of their own (elsa_compress.cu).  The 32 groups own exactly N*b whole index words of the row's
+// bitstream, so the warp assembles its words in shared memory and writes them with one coalesced store.
+template <int M>
+__device__ __forceinline__ void compress_segment(const uint16_t* __restrict__ W, int in, int N, uint16_t* __restrict__ vals,
+                                                 uint32_t* __restrict__ idx, int segs_per_row, int words_per_row, long long seg_id,
+                                                 uint32_t (*words)[kMaxIndexWordsPerSegment])
+{
+    constexpr int B = (M == 4) ? 2 : (M == 8) ? 3 : 4;
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+
+    const int o = (int)(seg_id / segs_per_row);
+    const int seg = (int)(seg_id % segs_per_row);
+    const int groups_per_row = in / M;
+    const int g = seg * 32 + lane;
+    const int seg_words = N * B;  // index words this segment owns
+
+    for (int k = lane; k < seg_words; k += 32) words[warp][k] = 0;
+    __syncwarp();
+    if (g < groups_per_row) {
+        uint16_t w[M];
+        load_group<M>(W + (size_t)o * in + (size_t)g * M, w);
+        uint32_t keep;
+        if constexpr (M == 16) {
+            uint32_t a[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) a[q] = (uint32_t)w[2 * q] | ((uint32_t)w[2 * q + 1] << 16);
+            keep = keep_mask16_any(a, N);
+        } else {
+            uint32_t h[M];
+#pragma unroll
+            for (int i = 0; i < M; ++i) h[i] = w[i];
+            keep = keep_mask_sorted<M>(h, N);
+        }
+        uint16_t* v = vals + (size_t)o * ((size_t)groups_per_row * N) + (size_t)g * N;
+        unsigned long long fields = 0;
+        int t = 0;
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            if ((keep >> i) & 1u) {
+                v[t] = w[i];
+                fields |= (unsigned long long)i << (t * B);
+                ++t;
+            }
+        }
+        const int bit0 = lane * seg_words;  // bit offset of this group's fields in the segment
+        const int w0 = bit0 >> 5, sh = bit0 & 31;
+        // up to 60 bits shifted by up to 31: three words at most
+        const uint32_t lo = (uint32_t)(fields << sh);
+        const uint32_t mid = (uint32_t)(fields >> (32 - sh));
+        const uint32_t hi = sh ? (uint32_t)(fields >> (64 - sh)) : 0u;
+        // a zero part may lie past the segment's last word and is skipped
+        if (lo) atomicOr(&words[warp][w0], lo);
+        if (mid) atomicOr(&words[warp][w0 + 1], mid);
+        if (hi) atomicOr(&words[warp][w0 + 2], hi);
+    }
+    __syncwarp();
+    const int first = seg * seg_words;
+    uint32_t* row = idx + (size_t)o * words_per_row;
+    for (int k = lane; k < seg_words && first + k < words_per_row; k += 32) row[first + k] = words[warp][k];
+    __syncwarp();
 }
 
 // ---- eight consecutive positions of a packed row as one 16-byte unit (groups of 4: two groups, groups of 8: one),
@@ -357,6 +381,68 @@ __device__ __forceinline__ uint4 expand_packed_unit(const PackedUnit& p, int N_r
     return make_uint4(prmt(pl03, ph03, 0x5140u), prmt(pl03, ph03, 0x7362u), prmt(pl47, ph47, 0x5140u), prmt(pl47, ph47, 0x7362u));
 }
 
+// ---- a whole group of 16 of a packed row, N < 16, in the same two halves
+struct PackedGroup16 {
+    uint32_t w[8];                 // kept values in order, two per word
+    unsigned long long fields;
+};
+
+__device__ __forceinline__ PackedGroup16 load_packed_group16(const uint16_t* __restrict__ vals_row, const uint32_t* __restrict__ idx_row, int N, int g)
+{
+    PackedGroup16 p;
+    const int bit0 = g * N * 4, w0 = bit0 >> 5, sh = bit0 & 31;
+    unsigned long long fields = __ldcg(idx_row + w0);
+    if (sh + 4 * N > 32) fields |= (unsigned long long)__ldcg(idx_row + w0 + 1) << 32;
+    fields >>= sh;
+    if (sh + 4 * N > 64) fields |= (unsigned long long)__ldcg(idx_row + w0 + 2) << (64 - sh);
+    p.fields = fields;
+    const uint16_t* v = vals_row + (size_t)g * N;
+    if ((N & 3) == 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint2 t = 4 * q < N ? __ldcg(reinterpret_cast<const uint2*>(v) + q) : make_uint2(0u, 0u);
+            p.w[2 * q] = t.x; p.w[2 * q + 1] = t.y;
+        }
+    } else if ((N & 1) == 0) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) p.w[q] = 2 * q < N ? __ldcg(reinterpret_cast<const uint32_t*>(v) + q) : 0u;
+    } else {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            p.w[q] = 2 * q < N ? (uint32_t)__ldcg(v + 2 * q) : 0u;
+            if (2 * q + 1 < N) p.w[q] |= (uint32_t)__ldcg(v + 2 * q + 1) << 16;
+        }
+    }
+    return p;
+}
+
+struct Group16 { uint4 a, b; };    // sixteen positions
+
+__device__ __forceinline__ Group16 expand_packed_group16(const PackedGroup16& p, int N)
+{
+    uint32_t d[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int t = 0; t < 15; ++t) {
+        if (t >= N) break;
+        const uint32_t pos = (uint32_t)(p.fields >> (4 * t)) & 15u, x = (p.w[t >> 1] >> (16 * (t & 1))) & 0xFFFFu, s = 16u * (pos & 3u);
+        const uint32_t lo = shl_or_zero(x, s), hi = shl_or_zero(x, s - 32u);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if ((pos >> 2) == (uint32_t)q) { d[2 * q] |= lo; d[2 * q + 1] |= hi; }
+    }
+    return Group16{make_uint4(d[0], d[1], d[2], d[3]), make_uint4(d[4], d[5], d[6], d[7])};
+}
+
+// A dense group of 16 projected onto level N:16.
+__device__ __forceinline__ Group16 mask_group16(const Group16& g, int N)
+{
+    uint32_t a[8] = {g.a.x, g.a.y, g.a.z, g.a.w, g.b.x, g.b.y, g.b.z, g.b.w};
+    const uint32_t keep = keep_mask16_any(a, N);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[q] &= ((keep >> (2 * q)) & 1u ? 0xFFFFu : 0u) | ((keep >> (2 * q + 1)) & 1u ? 0xFFFF0000u : 0u);
+    return Group16{make_uint4(a[0], a[1], a[2], a[3]), make_uint4(a[4], a[5], a[6], a[7])};
+}
+
 // A unit of a packed row with groups of 16: half of group unit / 2.
 __device__ __forceinline__ uint4 expand_unit16(const uint16_t* __restrict__ vals_row, const uint32_t* __restrict__ idx_row, int N, int unit)
 {
@@ -399,10 +485,7 @@ __device__ __forceinline__ uint4 mask_unit(const uint4& w, const uint4& w16, int
     uint32_t keep = 0, a[4] = {w.x, w.y, w.z, w.w};
     if constexpr (M == 16) {
         const uint32_t b[8] = {w.x, w.y, w.z, w.w, w16.x, w16.y, w16.z, w16.w};
-        uint16_t h[16];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) { h[2 * q] = (uint16_t)(b[q] & 0xFFFFu); h[2 * q + 1] = (uint16_t)(b[q] >> 16); }
-        keep = keep_mask<16>(group_ranks<16>(h), N) >> (8 * half);
+        keep = keep_mask16_any(b, N) >> (8 * half);
         if (half) { a[0] = w16.x; a[1] = w16.y; a[2] = w16.z; a[3] = w16.w; }
     } else {
 #pragma unroll

@@ -89,7 +89,34 @@ __device__ __forceinline__ void unpack_block(const ImageItem& it, int block)
         [&](const PackedUnit& p, int) { return expand_packed_unit<M, NC>(p, N); });
 }
 
-struct DenseGroup16 { uint4 a, b; };
+// The same for groups of 16, one a thread: load(group, row, group of the row), finish(raw) -> Group16.  (By halves of a group every
+// thread read and ranked the whole of it: image and GEMM of 3152 x 1024 -> 4096 at 4:16 from the shared weight 53 us, 36 with a
+// thread to a group and ranks, 33 with the sorted halves.  Two groups a thread: 4096 x 1024 at 8:16 9.3 us, one 8.5.)
+template <typename Raw, int kGroups, typename Load, typename Finish>
+__device__ __forceinline__ void group16_image_block(const ImageItem& it, int block, Load load, Finish finish)
+{
+    const uint32_t groups_per_row = (uint32_t)it.in >> 4, groups = (uint32_t)it.out * groups_per_row;
+#pragma unroll 1
+    for (int round = 0; round < it.rounds; ++round) {
+        const uint32_t base = (uint32_t)(block * it.rounds + round) * (kImageThreads * kGroups) + threadIdx.x;
+        Raw raw[kGroups];
+#pragma unroll
+        for (int i = 0; i < kGroups; ++i) {
+            const uint32_t group = min(base + (uint32_t)(i * kImageThreads), groups - 1u);
+            uint32_t g;
+            const uint32_t row = split_by(group, groups_per_row, it.magic, g);
+            raw[i] = load((size_t)group, row, (int)g);
+        }
+#pragma unroll
+        for (int i = 0; i < kGroups; ++i) {
+            const uint32_t group = base + (uint32_t)(i * kImageThreads);
+            if (group >= groups) break;
+            const Group16 d = finish(raw[i]);
+            reinterpret_cast<uint4*>(it.dst)[2 * (size_t)group] = d.a;
+            reinterpret_cast<uint4*>(it.dst)[2 * (size_t)group + 1] = d.b;
+        }
+    }
+}
 
 // ---------------------------------------------------------------- 2-of-4 images
 
@@ -334,8 +361,9 @@ __device__ __forceinline__ void sp24_block(const ImageItem& it, int block)
 int image_blocks(const ImageJob& j, int units_per_thread, int rounds)
 {
     if (j.kind == IMAGE_UNPACK || j.kind == IMAGE_MASK) {
-        const long long units = (long long)j.out * (j.in / 8);
-        const long long per_block = (long long)kImageThreads * units_per_thread * rounds;
+        const bool groups16 = j.M == 16 && (j.kind == IMAGE_MASK || j.N != j.M);      // two units of 8 positions in one
+        const long long units = (long long)j.out * (groups16 ? j.in / 16 : j.in / 8);
+        const long long per_block = (long long)kImageThreads * (groups16 ? 1 : units_per_thread) * rounds;
         return (int)((units + per_block - 1) / per_block);
     }
     const long long segs = (long long)((j.in + j.block_k - 1) / j.block_k) * (j.block_k / 32) * 2;
@@ -383,19 +411,19 @@ __global__ void __launch_bounds__(kImageThreads, 4) weight_image_kernel(const __
             else unpack_block<4, 0, kUnits>(it, block);
         } else {
             const int vpr = it.in / 16 * N, wpr = it.words_per_row;
-            dense_image_block<uint2, kUnits>(
-                it, block, [](size_t, uint32_t row, int u) { return make_uint2(row, (uint32_t)u); },
-                [&](const uint2& at, int) { return expand_unit16(it.src + (size_t)at.x * vpr, it.idx + (size_t)at.x * wpr, N, (int)at.y); });
+            group16_image_block<PackedGroup16, 1>(
+                it, block, [&](size_t, uint32_t row, int g) { return load_packed_group16(it.src + (size_t)row * vpr, it.idx + (size_t)row * wpr, N, g); },
+                [&](const PackedGroup16& p) { return expand_packed_group16(p, N); });
         }
     } else {
         if (M == 16) {
-            dense_image_block<DenseGroup16, kUnits>(
+            group16_image_block<Group16, 1>(
                 it, block,
-                [&](size_t unit, uint32_t, int) {      // rows hold whole groups of 16
-                    const uint4* g = reinterpret_cast<const uint4*>(it.src) + (unit & ~(size_t)1);
-                    return DenseGroup16{__ldg(g), __ldg(g + 1)};
+                [&](size_t group, uint32_t, int) {
+                    const uint4* g = reinterpret_cast<const uint4*>(it.src) + 2 * group;
+                    return Group16{__ldg(g), __ldg(g + 1)};
                 },
-                [&](const DenseGroup16& g, int half) { return mask_unit<16>(g.a, g.b, half, N); });
+                [&](const Group16& g) { return mask_group16(g, N); });
         } else {
             dense_image_block<uint4, kUnits>(it, block, [&](size_t unit, uint32_t, int) { return __ldg(reinterpret_cast<const uint4*>(it.src) + unit); },
                                              [&](const uint4& v, int) { return M == 8 ? mask_unit<8>(v, v, 0, N) : mask_unit<4>(v, v, 0, N); });
@@ -418,7 +446,7 @@ elsa_status launch_table(const ImageJob* jobs, int n, int rounds, cudaStream_t s
         it.k_blocks = (j.in + j.block_k - 1) / j.block_k;
         it.steps = j.block_k / 32;
         const bool dense = j.kind == IMAGE_UNPACK || j.kind == IMAGE_MASK;
-        const uint32_t d = dense ? (uint32_t)j.in / 8 : (uint32_t)(it.k_blocks * it.steps * 2) >> 2;
+        const uint32_t d = dense ? (uint32_t)j.in / (j.M == 16 && (j.kind == IMAGE_MASK || j.N != j.M) ? 16 : 8) : (uint32_t)(it.k_blocks * it.steps * 2) >> 2;
         it.magic = d == 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d);
         it.rounds = rounds;
         blocks += image_blocks(j, kUnits, rounds);

@@ -60,6 +60,29 @@ def test_unpack_around_a_block_of_units(lib, level):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("M", [8, 16])
+def test_every_level_packs_unpacks_and_masks_as_the_oracle(lib, M):
+    """Ties and signs throughout, all N < M one call each: packed bytes, the rebuilt weight, and (X = I) the weight as projected from the
+    shared one; one group a row and a block, ragged counts, and enough for a warp to take four segments."""
+    rng = np.random.default_rng(M)
+    for out, in_ in [(8, 16), (264, 16), (24, 16 * 23), (16, 4096 + 16), (2400, 1024)]:
+        W = torch.from_numpy(rng.integers(-4, 5, (out, in_)).astype(np.float32)).to(torch.float16)
+        Wd, Wb, X = W.cuda(), synth.bits(W), torch.eye(in_, dtype=torch.float16, device="cuda")
+        for N in range(1, M):
+            ovals, oidx, mask = eo.nm_compress(Wb, N, M)
+            vals, idx = lib.elsa_nm_compress(Wd, N, M)
+            assert (synth.bits(vals) == ovals).all() and (idx.cpu().numpy().view(np.uint32) == oidx).all(), (out, in_, N)
+            want = torch.from_numpy(W.numpy() * mask)
+            assert torch.equal(lib.elsa_nm_unpack(vals, idx, out, in_, N, M).cpu(), want), (out, in_, N)
+            lib.elsa_set_linear_variant(lib.VARIANT_TC_PAIR)
+            try:
+                got = lib.elsa_nm_linear_masked(X, Wd, None, N, M).cpu()
+            finally:
+                lib.elsa_set_linear_variant(lib.VARIANT_AUTO)
+            assert torch.equal(got, want.t()), (out, in_, N)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16], ids=["f16", "bf16"])
 def test_ties_of_many_kinds_compress_as_the_oracle(lib, dtype):
     """Few distinct magnitudes, so most groups have ties around the threshold: every level, rows whose index bits do and do
