@@ -164,17 +164,14 @@ __device__ __forceinline__ void copy_block(const CompressItem& it, int block)
         if (base + i * kThreads < units) reinterpret_cast<uint4*>(it.vals)[base + i * kThreads] = v[i];
 }
 
-// Any other level; kept out of line so that its registers do not count against the levels in use.
-template <int M, int kSegsPerWarp>
+// Any other level (of 16), one segment a warp whatever the launch's others take; kept out of line so that its registers do not
+// count against the levels in use.
 __device__ __noinline__ void compress_block_any(const uint16_t* W, uint16_t* vals, uint32_t* idx, int out, int in, int N, int words_per_row,
                                                 int block, uint32_t (*words)[kMaxIndexWordsPerSegment])
 {
-    constexpr int kSegsPerBlock = kWarpsPerBlock * kSegsPerWarp;
-    const int segs_per_row = (in / M + 31) / 32;
-    for (int i = 0; i < kSegsPerWarp; ++i) {
-        const long long seg = (long long)block * kSegsPerBlock + (int)(threadIdx.x >> 5) * kSegsPerWarp + i;
-        if (seg < (long long)out * segs_per_row) compress_segment<M>(W, in, N, vals, idx, segs_per_row, words_per_row, seg, words);
-    }
+    const int segs_per_row = (in / 16 + 31) / 32;
+    const long long seg = (long long)block * kWarpsPerBlock + (int)(threadIdx.x >> 5);
+    if (seg < (long long)out * segs_per_row) compress_segment<16>(W, in, N, vals, idx, segs_per_row, words_per_row, seg, words);
 }
 
 template <int kMax, int kSegs>
@@ -202,18 +199,19 @@ __global__ void __launch_bounds__(kThreads, 4) nm_compress_kernel(const __grid_c
     case 8 * 32 + 2: compress_block<8, 2, kSegs>(it, block); break;
     case 8 * 32 + 3: compress_block<8, 3, kSegs>(it, block); break;
     case 8 * 32 + 4: compress_block<8, 4, kSegs>(it, block); break;
+    case 8 * 32 + 5: compress_block<8, 5, kSegs>(it, block); break;
+    case 8 * 32 + 6: compress_block<8, 6, kSegs>(it, block); break;
+    case 8 * 32 + 7: compress_block<8, 7, kSegs>(it, block); break;
     case 16 * 32 + 1: compress_block<16, 1, kSegs>(it, block); break;
     case 16 * 32 + 2: compress_block<16, 2, kSegs>(it, block); break;
     case 16 * 32 + 4: compress_block<16, 4, kSegs>(it, block); break;
     case 16 * 32 + 8: compress_block<16, 8, kSegs>(it, block); break;
-    default:
-        if (it.M == 8) compress_block_any<8, kSegs>(it.W, it.vals, it.idx, it.out, it.in, it.N, it.words, block, words);
-        else compress_block_any<16, kSegs>(it.W, it.vals, it.idx, it.out, it.in, it.N, it.words, block, words);
+    default: compress_block_any(it.W, it.vals, it.idx, it.out, it.in, it.N, it.words, block, words);      // of 16
     }
 }
 
 // Whether compress_block has the level.
-bool fast_level(int N, int M) { return M == 4 || (M == 8 && N <= 4) || (M == 16 && (N == 1 || N == 2 || N == 4 || N == 8)); }
+bool fast_level(int N, int M) { return M == 4 || M == 8 || (M == 16 && (N == 1 || N == 2 || N == 4 || N == 8)); }
 
 template <int kMax>
 elsa_status launch_table(const CompressJob* jobs, int n, cudaStream_t stream)
@@ -250,7 +248,8 @@ elsa_status launch_table(const CompressJob* jobs, int n, cudaStream_t stream)
     int blocks = 0;
     for (int i = 0; i < n; ++i) {
         t.item[i].first_block = blocks;
-        blocks += (int)((segs[i] + kWarpsPerBlock * per_warp - 1) / (kWarpsPerBlock * per_warp));
+        const int per_block = kWarpsPerBlock * (jobs[i].N == jobs[i].M || fast_level(jobs[i].N, jobs[i].M) ? per_warp : 1);
+        blocks += (int)((segs[i] + per_block - 1) / per_block);
     }
     t.n = n;
     ProfileScope scope(ELSA_KERNEL_COMPRESS, stream);
