@@ -245,7 +245,7 @@ ImageJob image_job(LinearKind kind, const void* vals, const uint32_t* idx, int o
 
 // What a layer is part of: a call of its own, a table whose layers share persistent launches, or a chained block, where
 // the images are built off the critical path and an epilogue that takes GELU or the residual saves a pass.
-enum LinearUse { USE_SINGLE, USE_TABLE, USE_CHAIN };
+enum LinearUse { USE_SINGLE, USE_MASKED, USE_TABLE, USE_CHAIN };      // USE_MASKED: a call of its own on the shared weight
 
 // Which kernel a layer runs on.  AUTO is the product rule; a forced variant is honoured where it applies.
 // gelu: the layer's epilogue applies GELU (USE_CHAIN).
@@ -314,9 +314,13 @@ elsa_status pick_kind(LinearUse use, int rows, int out, int in, int N, int M, in
             j.rows = rows; j.out = out; j.in = in;
             ranges = linear_small_splits(&j, 1, sm_count);
         }
-        // Expanding in the kernel saves a launch on the host and costs ~0.3 us of device time per K block and CTA: taken
-        // up to 6 blocks (197 rows, 768 -> 768: 7.8 against 7.6; 3072 -> 768 would be 13.7 against 10).
-        if (N != M && ranges >= 2 && k_blocks <= 6 * ranges) *kind = KIND_SMALL;
+        // Expanding in the kernel saves a launch, but every row tile repeats it and a CTA's loads wait for one another, from HBM
+        // above all.  Us with the weight in L2 and from HBM, expanded and by an image: packed 1:4 and 2:4, 197 x 768 -> 768
+        // 6.6 and 6.9 against 7.1 and 7.9, 197 x 1024 -> 1024 7.4 and 7.7 against 8.4 and 11.1 (49 x 768 -> 2304 the other way
+        // round, 9.6 and 9.8 against 8.0 and 9.2); 4:8 7.8 and 8.8 against 7.2 and 8.0, 394 rows 10.4 and 11.5 against 7.4
+        // and 8.0; 3:8 9.8 and 12.0 against 7.6 and 8.1; 8:16 12.9 and 15.1 against 9.1 and 9.7; the shared weight at 2:4
+        // 7.3 and 7.3 against 7.2 and 7.5, at 4:8 8.7 and 8.7 against 7.3 and 7.7.
+        if (use == USE_SINGLE && M == 4 && N <= 2 && ranges >= 2 && k_blocks <= 6 * ranges) *kind = KIND_SMALL;
         // A cut reduction pays from 16 K blocks up (4:4, 197 rows: 3072 -> 768 7.4 against 12.2, 768 -> 768 5.3 both).
         else *kind = ranges >= 2 && k_blocks >= 16 ? KIND_SMALL_IMAGE : KIND_DENSE_ONE;
         return ELSA_OK;
@@ -523,7 +527,7 @@ elsa_status elsa_nm_linear_masked(const void* X, int rows, const void* W_sup, co
     if ((st = device_info(&dev)) != ELSA_OK) return st;
     cudaStream_t stream = (cudaStream_t)stream_;
     LinearKind kind;
-    if ((st = pick_kind(USE_SINGLE, rows, out, in, N, M, dev.sm_count, &kind)) != ELSA_OK) return st;
+    if ((st = pick_kind(USE_MASKED, rows, out, in, N, M, dev.sm_count, &kind)) != ELSA_OK) return st;
     if (kind == KIND_SIMT || kind == KIND_SPARSE_ONE)
         return fail(ELSA_ERR_NM, "the forced variant has no mask-on-load form");
     if (kind == KIND_SMALL) {

@@ -4,10 +4,11 @@
 // A layer of one or a few images has too few 256-row tiles to occupy the SM pairs of the persistent kernels, and what
 // it pays for is latency: the launch of the kernel that rebuilds the weight image, a persistent kernel's set-up, one
 // long reduction per tile.  Here
-//   * a call of one layer has the weight tile expanded on the way to shared memory by eight warps that read the packed
-//     values and index words (or project the dense shared weight, for the masked form), so that there is no image and
-//     no second launch; the dense level's tile comes by TMA, and so do the images that the layers of a table and of a
-//     chained block bring along (one launch builds those of a whole call);
+//   * a call of one layer at 1:4 or 2:4 has the weight tile expanded on the way to shared memory by eight warps that read
+//     the packed values and index words, so that there is no image and no second launch (the code takes every level, and
+//     the dense shared weight for the masked form, where the variant is forced; by itself the library brings an image, see
+//     the rule in elsa_api.cu); the dense level's tile comes by TMA, and so do the images that the layers of a table and
+//     of a chained block bring along (one launch builds those of a whole call);
 //   * a CTA computes one tile of 128 rows x 64 features and leaves; two CTAs fit an SM, so that one's set-up and
 //     epilogue run under the other's tile, or the next kernel's set-up under this one's;
 //   * where the tiles alone leave SMs idle, the reduction is cut into 2, 4 or 8 ranges, one CTA of a cluster each:
@@ -19,7 +20,7 @@
 // Measured back to back on 197 rows (us, weight image + one-CTA-per-tile GEMM before, this kernel after): 768 -> 768 at
 // 2:4 6.9 -> 6.4, 768 -> 2304 at 2:4 8.2 -> 7.7, 3072 -> 768 at 2:4 15.4 -> 10.6, at 4:4 11.6 -> 6.9.  The expansion
 // is repeated for every 128 rows and bound by its loads' latency and its instructions: at 788 rows and 2:4 the image
-// kernel and a GEMM that reads it take 10.9 us where this one takes 20, hence the rule in elsa_api.cu.
+// kernel and a GEMM that reads it take 10.9 us where this one takes 20.
 //
 // Warps: 0 TMA producer, 1 MMA issuer (tcgen05, M = 128), 2-9 expansion, then epilogue, 10-11 only barriers.
 

@@ -60,6 +60,27 @@ def test_small_linear_matches_oracle_packed_and_masked(lib, case, dtype):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("level", [(1, 4), (2, 4), (3, 4), (4, 4), (2, 8), (3, 8), (4, 8), (4, 16), (8, 16)], ids=lambda l: "%dof%d" % l)
+def test_few_rows_under_the_automatic_choice(lib, level):
+    """The packed weight and the shared one, whichever kernel a wave of small tiles goes to at this level; 1:4 and 2:4 are one launch."""
+    N, M = level
+    for rows, in_, out in [(1, 128, 64), (49, 768, 2304), (197, 768, 768), (394, 1024, 200), (100, 3072, 768)]:
+        X = synth.randn((rows, in_), rows + in_, synth.X_STD, torch.bfloat16).cuda()
+        W = synth.randn((out, in_), out + in_, synth.W_STD, torch.bfloat16).cuda()
+        bias = synth.randn((out,), out, synth.B_STD, torch.bfloat16).cuda()
+        vals, idx = lib.elsa_nm_compress(W, N, M)
+        Wm = W if N == M else lib.elsa_nm_unpack(vals, idx, out, in_, N, M)
+        ref = (X.double() @ Wm.double().t() + bias.double()).cpu().numpy()
+        before = lib.elsa_launch_count()
+        Y = lib.elsa_nm_linear(X, vals, idx, bias, out, in_, N, M)
+        launches = lib.elsa_launch_count() - before
+        close(Y, ref)
+        close(lib.elsa_nm_linear_masked(X, W, bias, N, M), ref)
+        if (rows, in_, out) == (197, 768, 768):
+            assert launches == (1 if M == 4 and N != 3 else 2)
+
+
+@pytest.mark.gpu
 def test_small_layers_of_a_table_share_a_launch(lib):
     """More layers than one launch carries, of every weight source, against the same table run layer by layer."""
     dtype = torch.bfloat16
