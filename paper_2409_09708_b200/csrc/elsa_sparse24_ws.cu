@@ -57,7 +57,7 @@ constexpr int kStagingTotal = kEpiWarps * kStagingBytes;
 constexpr int kBarrierBytes = 512;
 
 struct alignas(64) WsLayer {
-    CUtensorMap map_x, map_y;   // map_y: one step of 16 token rows
+    CUtensorMap map_x, map_y, map_run;   // map_y: one step of 16 token rows, map_run: a warp's whole run of them
     const uint16_t* a_img;   // 2-of-4 values [out rounded up to 32][in / 2], rows in the permuted order
     const uint8_t* meta;     // metadata blocks of 2 KB per (128 features, 128 k)
     const uint16_t* bias;
@@ -71,7 +71,7 @@ struct alignas(64) WsLayer {
     int act;           // epilogue activation (0 none, 1 GELU) on acc + bias
 };
 
-constexpr int kGroupMax = 92;   // layers per launch (kernel parameters are limited to 32 KB)
+constexpr int kGroupMax = 68;   // layers per launch (kernel parameters are limited to 32 KB)
 
 template <int kMaxLayers>
 struct WsGroup {
@@ -80,7 +80,6 @@ struct WsGroup {
     int stages;
     int stage_bytes;   // one pipeline stage: kStageK / 64 quarters of (largest nt / 2) rows of 128 bytes
     uint32_t* dev_status;
-    CUtensorMap map_run;   // kAct: Y in boxes of a warp's whole run of token rows
 };
 
 // kAct: the instantiation whose epilogue applies the layer's activation (single-layer launches).
@@ -88,6 +87,7 @@ template <bool kBf16, int kMaxLayers, bool kAct>
 __global__ void __launch_bounds__(kThreads, 1)
 linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
 {
+    constexpr bool kRuns = kAct || kMaxLayers > 1;      // how the rows leave, see the epilogue
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -369,10 +369,11 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
                 if (lane == 0) {
                     if (f0 < l_out) {
                         // With GELU the warps are short of issue slots and a run leaves as one store (50432 x 768 -> 3072 138
-                        // -> 131 us); without it as one a step, which start while the rest is on its way: 65536 x
-                        // 768 -> 3072 alone 136 us, 144 by runs, back to back 141.2 and 142.2.
-                        if (kAct && my_steps == L.steps_per_warp) {
-                            if (row0 < l_rows) tma_store_2d(&p.map_run, buf, f0, row0);
+                        // -> 131 us), and so it does in tables, whose layers follow one another without a gap (a DeiT-B block
+                        // of 12608 rows 129.3 us, 130.5 by steps); a layer on its own as one store a step, which start while the
+                        // rest is on its way: 65536 x 768 -> 3072 136 us, 144 by runs, back to back 141.2 and 142.2.
+                        if (kRuns && my_steps == L.steps_per_warp) {
+                            if (row0 < l_rows) tma_store_2d(&L.map_run, buf, f0, row0);
                         } else {
 #pragma unroll
                             for (int s = 0; s < kMaxSteps; ++s)
@@ -416,6 +417,7 @@ template <bool kBf16, int kMaxLayers, bool kAct>
 elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint32_t* dev_status, cudaStream_t stream,
                             const DeviceInfo& dev)
 {
+    constexpr bool kRuns = kAct || kMaxLayers > 1;
     auto kernel = linear_tc_sp24_ws_kernel<kBf16, kMaxLayers, kAct>;
     const int fixed = kStagingTotal + kBarrierBytes + 1024;
     int max_nt = 0;
@@ -490,8 +492,8 @@ elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
         if ((st = make_map_2d(&L.map_y, j.Y, (uint64_t)j.out, (uint64_t)j.rows, 32, kStepCols, CU_TENSOR_MAP_SWIZZLE_NONE,
                               "Y")) != ELSA_OK)
             return st;
-        if (kAct && (st = make_map_2d(&g.map_run, j.Y, (uint64_t)j.out, (uint64_t)j.rows, 32, (uint32_t)(kStepCols * L.steps_per_warp),
-                                      CU_TENSOR_MAP_SWIZZLE_NONE, "Y")) != ELSA_OK)
+        if (kRuns && (st = make_map_2d(&L.map_run, j.Y, (uint64_t)j.out, (uint64_t)j.rows, 32, (uint32_t)(kStepCols * L.steps_per_warp),
+                                       CU_TENSOR_MAP_SWIZZLE_NONE, "Y")) != ELSA_OK)
             return st;
     }
     g.n_layers = n;
