@@ -90,8 +90,8 @@ __device__ __forceinline__ void unpack_block(const ImageItem& it, int block)
 }
 
 // The same for groups of 16, one a thread: load(group, row, group of the row), finish(raw) -> Group16.  (By halves of a group every
-// thread read and ranked the whole of it: image and GEMM of 3152 x 1024 -> 4096 at 4:16 from the shared weight 53 us, 36 with a
-// thread to a group and ranks, 33 with the sorted halves.  Two groups a thread: 4096 x 1024 at 8:16 9.3 us, one 8.5.)
+// thread read and ranked the whole of it: image and GEMM of 3152 x 1024 -> 4096 at 4:16 from the shared weight 53 us, 24.7 like this.
+// From the packed form the halves stay quicker where the launch leaves SMs idle: 2048 x 512 at 8:16 and below about 1 us.)
 template <typename Raw, int kGroups, typename Load, typename Finish>
 __device__ __forceinline__ void group16_image_block(const ImageItem& it, int block, Load load, Finish finish)
 {
@@ -357,11 +357,14 @@ __device__ __forceinline__ void sp24_block(const ImageItem& it, int block)
     }
 }
 
+// Whether a dense image's unit is a whole group of 16, one a thread, instead of 8 positions.
+bool in_groups16(const ImageJob& j, int units_per_thread) { return j.M == 16 && (j.kind == IMAGE_MASK || (j.kind == IMAGE_UNPACK && j.N != 16 && units_per_thread > 1)); }
+
 // Blocks of a weight.
 int image_blocks(const ImageJob& j, int units_per_thread, int rounds)
 {
     if (j.kind == IMAGE_UNPACK || j.kind == IMAGE_MASK) {
-        const bool groups16 = j.M == 16 && (j.kind == IMAGE_MASK || j.N != j.M);      // two units of 8 positions in one
+        const bool groups16 = in_groups16(j, units_per_thread);
         const long long units = (long long)j.out * (groups16 ? j.in / 16 : j.in / 8);
         const long long per_block = (long long)kImageThreads * (groups16 ? 1 : units_per_thread) * rounds;
         return (int)((units + per_block - 1) / per_block);
@@ -403,15 +406,20 @@ __global__ void __launch_bounds__(kImageThreads, 4) weight_image_kernel(const __
         } else if (M == 8) {
             if (N == 1) unpack_block<8, 1, kUnits>(it, block);
             else if (N == 2) unpack_block<8, 2, kUnits>(it, block);
+            else if (N == 3) unpack_block<8, 3, kUnits>(it, block);
             else if (N == 4) unpack_block<8, 4, kUnits>(it, block);
             else unpack_block<8, 0, kUnits>(it, block);
         } else if (M == 4) {
             if (N == 1) unpack_block<4, 1, kUnits>(it, block);
             else if (N == 2) unpack_block<4, 2, kUnits>(it, block);
-            else unpack_block<4, 0, kUnits>(it, block);
+            else unpack_block<4, 3, kUnits>(it, block);
         } else {
             const int vpr = it.in / 16 * N, wpr = it.words_per_row;
-            group16_image_block<PackedGroup16, 1>(
+            if constexpr (kUnits == 1)      // a small launch: threads before instructions
+                dense_image_block<uint2, 1>(
+                    it, block, [](size_t, uint32_t row, int u) { return make_uint2(row, (uint32_t)u); },
+                    [&](const uint2& at, int) { return expand_unit16(it.src + (size_t)at.x * vpr, it.idx + (size_t)at.x * wpr, N, (int)at.y); });
+            else group16_image_block<PackedGroup16, 1>(
                 it, block, [&](size_t, uint32_t row, int g) { return load_packed_group16(it.src + (size_t)row * vpr, it.idx + (size_t)row * wpr, N, g); },
                 [&](const PackedGroup16& p) { return expand_packed_group16(p, N); });
         }
@@ -446,7 +454,7 @@ elsa_status launch_table(const ImageJob* jobs, int n, int rounds, cudaStream_t s
         it.k_blocks = (j.in + j.block_k - 1) / j.block_k;
         it.steps = j.block_k / 32;
         const bool dense = j.kind == IMAGE_UNPACK || j.kind == IMAGE_MASK;
-        const uint32_t d = dense ? (uint32_t)j.in / (j.M == 16 && (j.kind == IMAGE_MASK || j.N != j.M) ? 16 : 8) : (uint32_t)(it.k_blocks * it.steps * 2) >> 2;
+        const uint32_t d = dense ? (uint32_t)j.in / (in_groups16(j, kUnits) ? 16 : 8) : (uint32_t)(it.k_blocks * it.steps * 2) >> 2;
         it.magic = d == 1 ? 0xFFFFFFFFu : (uint32_t)((1ull << 32) / d);
         it.rounds = rounds;
         blocks += image_blocks(j, kUnits, rounds);
@@ -492,7 +500,10 @@ elsa_status launch_images(const ImageJob* jobs, int n, cudaStream_t stream)
     for (int at = 0; at < n; at += kMost) {
         const int count = n - at < kMost ? n - at : kMost;
         int blocks = 0;
-        for (int i = 0; i < count; ++i) blocks += image_blocks(jobs[at + i], kMostUnits, 1);
+        for (int i = 0; i < count; ++i) {      // groups of 16 count as what their positions are elsewhere
+            const int b = image_blocks(jobs[at + i], kMostUnits, 1);
+            blocks += in_groups16(jobs[at + i], kMostUnits) ? (b + 1) / 2 : b;
+        }
         const bool spread = blocks < 2 * dev.sm_count;
         // A block costs a few thousand cycles before its first load, so where there are many waves of them they take three
         // runs each: 48 DeiT-B weights at 2:8 to dense images 51 -> 46 us, to 2-of-4 ones 60 -> 55; one block's four
