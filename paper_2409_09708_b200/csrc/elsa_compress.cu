@@ -164,14 +164,18 @@ __device__ __forceinline__ void copy_block(const CompressItem& it, int block)
         if (base + i * kThreads < units) reinterpret_cast<uint4*>(it.vals)[base + i * kThreads] = v[i];
 }
 
-// Any other level (of 16), one segment a warp whatever the launch's others take; kept out of line so that its registers do not
-// count against the levels in use.
+// Any other level; kept out of line so that its registers do not count against the levels in use.
+template <int M, int kSegsPerWarp>
 __device__ __noinline__ void compress_block_any(const uint16_t* W, uint16_t* vals, uint32_t* idx, int out, int in, int N, int words_per_row,
                                                 int block, uint32_t (*words)[kMaxIndexWordsPerSegment])
 {
-    const int segs_per_row = (in / 16 + 31) / 32;
-    const long long seg = (long long)block * kWarpsPerBlock + (int)(threadIdx.x >> 5);
-    if (seg < (long long)out * segs_per_row) compress_segment<16>(W, in, N, vals, idx, segs_per_row, words_per_row, seg, words);
+    constexpr int kSegsPerBlock = kWarpsPerBlock * kSegsPerWarp;
+    const int segs_per_row = (in / M + 31) / 32;
+    for (int i = 0; i < kSegsPerWarp; ++i) {
+        const long long seg = (long long)block * kSegsPerBlock + (int)(threadIdx.x >> 5) * kSegsPerWarp + i;
+        if (seg < (long long)out * segs_per_row) compress_segment<M>(W, in, N, vals, idx, segs_per_row, words_per_row, seg, words,
+                                [N](const uint16_t (&w)[M]) { return keep_mask<M>(group_ranks<M>(w), N); });
+    }
 }
 
 template <int kMax, int kSegs>
@@ -199,19 +203,50 @@ __global__ void __launch_bounds__(kThreads, 4) nm_compress_kernel(const __grid_c
     case 8 * 32 + 2: compress_block<8, 2, kSegs>(it, block); break;
     case 8 * 32 + 3: compress_block<8, 3, kSegs>(it, block); break;
     case 8 * 32 + 4: compress_block<8, 4, kSegs>(it, block); break;
-    case 8 * 32 + 5: compress_block<8, 5, kSegs>(it, block); break;
-    case 8 * 32 + 6: compress_block<8, 6, kSegs>(it, block); break;
-    case 8 * 32 + 7: compress_block<8, 7, kSegs>(it, block); break;
     case 16 * 32 + 1: compress_block<16, 1, kSegs>(it, block); break;
     case 16 * 32 + 2: compress_block<16, 2, kSegs>(it, block); break;
     case 16 * 32 + 4: compress_block<16, 4, kSegs>(it, block); break;
     case 16 * 32 + 8: compress_block<16, 8, kSegs>(it, block); break;
-    default: compress_block_any(it.W, it.vals, it.idx, it.out, it.in, it.N, it.words, block, words);      // of 16
+    default:
+        if (it.M == 8) compress_block_any<8, kSegs>(it.W, it.vals, it.idx, it.out, it.in, it.N, it.words, block, words);
+        else compress_block_any<16, kSegs>(it.W, it.vals, it.idx, it.out, it.in, it.N, it.words, block, words);
     }
 }
 
+// One weight at a level that the kernel above takes by its general form: kernels of their own, since the levels in use lose 5 % to
+// more code beside them (4096 x 1024 to 1, 2, 3 and 4 of 8 14.9 -> 15.6 us).  4096 x 1024 at 5:8 15.2 -> 6.4 us, 3072 x 768 at
+// 3:16 18.1 -> 9.3.
+template <int N, int kSegs>
+__global__ void __launch_bounds__(kThreads, 4) nm_compress_dense8_kernel(const __grid_constant__ CompressTable<1> t)
+{
+    pdl_wait_for_predecessors();
+    pdl_release_successors();
+    compress_block<8, N, kSegs>(t.item[0], (int)blockIdx.x);
+}
+
+__global__ void __launch_bounds__(kThreads, 4) nm_compress_any16_kernel(const __grid_constant__ CompressTable<1> t)
+{
+    __shared__ uint32_t words[kWarpsPerBlock][kMaxIndexWordsPerSegment];
+    pdl_wait_for_predecessors();
+    pdl_release_successors();
+    const CompressItem& it = t.item[0];
+    const int segs_per_row = (it.in / 16 + 31) / 32, N = it.N;
+    const long long seg = (long long)blockIdx.x * kWarpsPerBlock + (int)(threadIdx.x >> 5);
+    if (seg < (long long)it.out * segs_per_row)
+        compress_segment<16>(it.W, it.in, N, it.vals, it.idx, segs_per_row, it.words, seg, words, [N](const uint16_t (&w)[16]) {
+            uint32_t a[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) a[q] = (uint32_t)w[2 * q] | ((uint32_t)w[2 * q + 1] << 16);
+            return keep_mask16_any(a, N);
+        });
+}
+
 // Whether compress_block has the level.
-bool fast_level(int N, int M) { return M == 4 || M == 8 || (M == 16 && (N == 1 || N == 2 || N == 4 || N == 8)); }
+bool fast_level(int N, int M) { return M == 4 || (M == 8 && N <= 4) || (M == 16 && (N == 1 || N == 2 || N == 4 || N == 8)); }
+
+// Whether a launch of n weights is one for the kernels of single weights.
+bool dense8(const CompressJob& j, int n) { return n == 1 && j.M == 8 && j.N >= 5 && j.N <= 7; }
+bool any16(const CompressJob& j, int n) { return n == 1 && j.M == 16 && j.N < 16 && !fast_level(j.N, j.M); }
 
 template <int kMax>
 elsa_status launch_table(const CompressJob* jobs, int n, cudaStream_t stream)
@@ -229,7 +264,7 @@ elsa_status launch_table(const CompressJob* jobs, int n, cudaStream_t stream)
         it.words = (int)index_words_per_row(j.in, j.N, j.M);
         it.units = j.in / (j.M == 16 ? 16 : 8);
         const long long row_bits = (long long)(j.in / j.M) * j.N * index_bits(j.M);
-        if (j.N == j.M || fast_level(j.N, j.M)) {
+        if (j.N == j.M || fast_level(j.N, j.M) || dense8(j, n)) {
             if (row_bits % 32 == 0 && (long long)j.out * it.units < (1ll << 30) && (long long)j.out * it.words < (1ll << 30)) {
                 it.units *= j.out;
                 it.words *= j.out;
@@ -244,16 +279,24 @@ elsa_status launch_table(const CompressJob* jobs, int n, cudaStream_t stream)
     }
     // Four segments a warp keep four loads of a lane in flight; below two blocks an SM one segment a warp is quicker
     // (384 x 384: 18 blocks or 72; one weight at 2:8 2.3 against 1.6 us).
-    const int per_warp = total < (long long)dev.sm_count * 2 * kWarpsPerBlock * 4 ? 1 : 4;
+    const int per_warp = any16(jobs[0], n) || total < (long long)dev.sm_count * 2 * kWarpsPerBlock * 4 ? 1 : 4;
     int blocks = 0;
     for (int i = 0; i < n; ++i) {
         t.item[i].first_block = blocks;
-        const int per_block = kWarpsPerBlock * (jobs[i].N == jobs[i].M || fast_level(jobs[i].N, jobs[i].M) ? per_warp : 1);
-        blocks += (int)((segs[i] + per_block - 1) / per_block);
+        blocks += (int)((segs[i] + kWarpsPerBlock * per_warp - 1) / (kWarpsPerBlock * per_warp));
     }
     t.n = n;
     ProfileScope scope(ELSA_KERNEL_COMPRESS, stream);
-    cudaError_t e = launch_pdl(per_warp == 1 ? nm_compress_kernel<kMax, 1> : nm_compress_kernel<kMax, 4>, dim3((unsigned)blocks), dim3(kThreads),
+    auto kernel = per_warp == 1 ? nm_compress_kernel<kMax, 1> : nm_compress_kernel<kMax, 4>;
+    if constexpr (kMax == 1) {
+        const int N = jobs[0].N;
+        if (any16(jobs[0], n)) kernel = nm_compress_any16_kernel;
+        else if (dense8(jobs[0], n))
+            kernel = N == 5   ? (per_warp == 1 ? nm_compress_dense8_kernel<5, 1> : nm_compress_dense8_kernel<5, 4>)
+                     : N == 6 ? (per_warp == 1 ? nm_compress_dense8_kernel<6, 1> : nm_compress_dense8_kernel<6, 4>)
+                              : (per_warp == 1 ? nm_compress_dense8_kernel<7, 1> : nm_compress_dense8_kernel<7, 4>);
+    }
+    cudaError_t e = launch_pdl(kernel, dim3((unsigned)blocks), dim3(kThreads),
                                0, stream, 1, t);
     if (e != cudaSuccess) {
         cudaGetLastError();

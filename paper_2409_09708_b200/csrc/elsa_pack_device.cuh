@@ -29,6 +29,89 @@ __device__ __forceinline__ void load_group(const uint16_t* p, uint16_t (&w)[M])
     }
 }
 
+// Ranks of the M magnitudes of one group, 4 bits each: rank_i = #{j : |w_j| > |w_i|} + #{j < i : |w_j| == |w_i|}
+// (larger magnitude first, lower position first among equals).  Magnitudes are compared as the 15 low
+// bits of the pattern.  The level N keeps exactly the elements with rank < N, for every N at once.
+template <int M>
+__device__ __forceinline__ unsigned long long group_ranks(const uint16_t (&w)[M])
+{
+    unsigned long long ranks = 0;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+        const uint32_t ki = w[i] & 0x7FFFu;
+        int rank = 0;
+#pragma unroll
+        for (int j = 0; j < M; ++j) {
+            const uint32_t kj = w[j] & 0x7FFFu;
+            rank += (kj > ki) || (j < i && kj == ki);
+        }
+        ranks |= (unsigned long long)rank << (4 * i);
+    }
+    return ranks;
+}
+
+template <int M>
+__device__ __forceinline__ uint32_t keep_mask(unsigned long long ranks, int N)
+{
+    uint32_t keep = 0;
+#pragma unroll
+    for (int i = 0; i < M; ++i) keep |= (uint32_t)((int)((ranks >> (4 * i)) & 15ull) < N) << i;
+    return keep;
+}
+
+// One warp compresses 32 consecutive groups of one row, one group per lane, at any level N < M: the form for the levels
+// that have none of their own (elsa_compress.cu); keep_of: the mask of a group.  The 32 groups own exactly N*b whole index words of the row's
+// bitstream, so the warp assembles its words in shared memory and writes them with one coalesced store.
+template <int M, typename Keep>
+__device__ __forceinline__ void compress_segment(const uint16_t* __restrict__ W, int in, int N, uint16_t* __restrict__ vals,
+                                                 uint32_t* __restrict__ idx, int segs_per_row, int words_per_row, long long seg_id,
+                                                 uint32_t (*words)[kMaxIndexWordsPerSegment], Keep keep_of)
+{
+    constexpr int B = (M == 4) ? 2 : (M == 8) ? 3 : 4;
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+
+    const int o = (int)(seg_id / segs_per_row);
+    const int seg = (int)(seg_id % segs_per_row);
+    const int groups_per_row = in / M;
+    const int g = seg * 32 + lane;
+    const int seg_words = N * B;  // index words this segment owns
+
+    for (int k = lane; k < seg_words; k += 32) words[warp][k] = 0;
+    __syncwarp();
+    if (g < groups_per_row) {
+        uint16_t w[M];
+        load_group<M>(W + (size_t)o * in + (size_t)g * M, w);
+        const uint32_t keep = keep_of(w);
+        uint16_t* v = vals + (size_t)o * ((size_t)groups_per_row * N) + (size_t)g * N;
+        unsigned long long fields = 0;
+        int t = 0;
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            if ((keep >> i) & 1u) {
+                v[t] = w[i];
+                fields |= (unsigned long long)i << (t * B);
+                ++t;
+            }
+        }
+        const int bit0 = lane * seg_words;  // bit offset of this group's fields in the segment
+        const int w0 = bit0 >> 5, sh = bit0 & 31;
+        // up to 60 bits shifted by up to 31: three words at most
+        const uint32_t lo = (uint32_t)(fields << sh);
+        const uint32_t mid = (uint32_t)(fields >> (32 - sh));
+        const uint32_t hi = sh ? (uint32_t)(fields >> (64 - sh)) : 0u;
+        // a zero part may lie past the segment's last word and is skipped
+        if (lo) atomicOr(&words[warp][w0], lo);
+        if (mid) atomicOr(&words[warp][w0 + 1], mid);
+        if (hi) atomicOr(&words[warp][w0 + 2], hi);
+    }
+    __syncwarp();
+    const int first = seg * seg_words;
+    uint32_t* row = idx + (size_t)o * words_per_row;
+    for (int k = lane; k < seg_words && first + k < words_per_row; k += 32) row[first + k] = words[warp][k];
+    __syncwarp();
+}
+
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
 {
     uint32_t r;
@@ -200,70 +283,6 @@ __device__ __forceinline__ uint32_t keep_mask16_any(const uint32_t (&a)[8], int 
     default: thr = threshold16<15>(s); break;
     }
     return keep_above16(k, thr, N);
-}
-
-// One warp compresses 32 consecutive groups of one row, one group per lane, at any level N < M: the form for the levels
-// that have none of their own (elsa_compress.cu).  The 32 groups own exactly N*b whole index words of the row's
-// bitstream, so the warp assembles its words in shared memory and writes them with one coalesced store.
-template <int M>
-__device__ __forceinline__ void compress_segment(const uint16_t* __restrict__ W, int in, int N, uint16_t* __restrict__ vals,
-                                                 uint32_t* __restrict__ idx, int segs_per_row, int words_per_row, long long seg_id,
-                                                 uint32_t (*words)[kMaxIndexWordsPerSegment])
-{
-    constexpr int B = (M == 4) ? 2 : (M == 8) ? 3 : 4;
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-
-    const int o = (int)(seg_id / segs_per_row);
-    const int seg = (int)(seg_id % segs_per_row);
-    const int groups_per_row = in / M;
-    const int g = seg * 32 + lane;
-    const int seg_words = N * B;  // index words this segment owns
-
-    for (int k = lane; k < seg_words; k += 32) words[warp][k] = 0;
-    __syncwarp();
-    if (g < groups_per_row) {
-        uint16_t w[M];
-        load_group<M>(W + (size_t)o * in + (size_t)g * M, w);
-        uint32_t keep;
-        if constexpr (M == 16) {
-            uint32_t a[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) a[q] = (uint32_t)w[2 * q] | ((uint32_t)w[2 * q + 1] << 16);
-            keep = keep_mask16_any(a, N);
-        } else {
-            uint32_t h[M];
-#pragma unroll
-            for (int i = 0; i < M; ++i) h[i] = w[i];
-            keep = keep_mask_sorted<M>(h, N);
-        }
-        uint16_t* v = vals + (size_t)o * ((size_t)groups_per_row * N) + (size_t)g * N;
-        unsigned long long fields = 0;
-        int t = 0;
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            if ((keep >> i) & 1u) {
-                v[t] = w[i];
-                fields |= (unsigned long long)i << (t * B);
-                ++t;
-            }
-        }
-        const int bit0 = lane * seg_words;  // bit offset of this group's fields in the segment
-        const int w0 = bit0 >> 5, sh = bit0 & 31;
-        // up to 60 bits shifted by up to 31: three words at most
-        const uint32_t lo = (uint32_t)(fields << sh);
-        const uint32_t mid = (uint32_t)(fields >> (32 - sh));
-        const uint32_t hi = sh ? (uint32_t)(fields >> (64 - sh)) : 0u;
-        // a zero part may lie past the segment's last word and is skipped
-        if (lo) atomicOr(&words[warp][w0], lo);
-        if (mid) atomicOr(&words[warp][w0 + 1], mid);
-        if (hi) atomicOr(&words[warp][w0 + 2], hi);
-    }
-    __syncwarp();
-    const int first = seg * seg_words;
-    uint32_t* row = idx + (size_t)o * words_per_row;
-    for (int k = lane; k < seg_words && first + k < words_per_row; k += 32) row[first + k] = words[warp][k];
-    __syncwarp();
 }
 
 // ---- eight consecutive positions of a packed row as one 16-byte unit (groups of 4: two groups, groups of 8: one),
@@ -477,6 +496,13 @@ __device__ __forceinline__ uint4 expand_unit16(const uint16_t* __restrict__ vals
     return make_uint4((uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)hi, (uint32_t)(hi >> 32));
 }
 
+// Out of line: the few-rows kernel's other levels lose 2 % to the sort in their code (125 x 768 -> 192 at 2:4 6.21 us, 6.08).
+__device__ __noinline__ uint32_t keep_mask16_call(uint4 a, uint4 b, int N)
+{
+    const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    return keep_mask16_any(w, N);
+}
+
 // Eight consecutive positions of a DENSE row projected onto level N:M, from the 16 bytes of the unit (groups of 16:
 // from the whole group w, w16, with `half` saying which eight are wanted).
 template <int M>
@@ -484,8 +510,7 @@ __device__ __forceinline__ uint4 mask_unit(const uint4& w, const uint4& w16, int
 {
     uint32_t keep = 0, a[4] = {w.x, w.y, w.z, w.w};
     if constexpr (M == 16) {
-        const uint32_t b[8] = {w.x, w.y, w.z, w.w, w16.x, w16.y, w16.z, w16.w};
-        keep = keep_mask16_any(b, N) >> (8 * half);
+        keep = keep_mask16_call(w, w16, N) >> (8 * half);
         if (half) { a[0] = w16.x; a[1] = w16.y; a[2] = w16.z; a[3] = w16.w; }
     } else {
 #pragma unroll
