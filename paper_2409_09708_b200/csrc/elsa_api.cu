@@ -243,6 +243,20 @@ ImageJob image_job(LinearKind kind, const void* vals, const uint32_t* idx, int o
     return j;
 }
 
+// Whether a packed weight (N < M) goes through an image: the few-rows kernel and the weight-stationary one expand it themselves.
+bool reads_image(LinearKind kind) { return kind != KIND_SIMT && kind != KIND_SMALL && kind != KIND_SPARSE_WS; }
+
+// A layer of the sparse kernels: on the packed weight (weight-stationary kernel) or on its image.
+SparseJob sparse_job(LinearKind kind, const void* X, int rows, const void* vals, const uint32_t* idx, const void* bias, int out, int in, int N,
+                     int M, void* Y, const void* image)
+{
+    SparseJob j;
+    j.X = (const uint16_t*)X; j.bias = (const uint16_t*)bias; j.Y = (uint16_t*)Y; j.workspace = image;
+    j.rows = rows; j.in = in; j.out = out;
+    if (kind == KIND_SPARSE_WS) { j.w = (const uint16_t*)vals; j.idx = idx; j.N = N; j.M = M; }
+    return j;
+}
+
 // What a layer is part of: a call of its own, a table whose layers share persistent launches, or a chained block, where
 // the images are built off the critical path and an epilogue that takes GELU or the residual saves a pass.
 enum LinearUse { USE_SINGLE, USE_MASKED, USE_TABLE, USE_CHAIN };      // USE_MASKED: a call of its own on the shared weight
@@ -339,7 +353,16 @@ elsa_status pick_kind(LinearUse use, int rows, int out, int in, int N, int M, in
         *kind = ws ? KIND_SPARSE_WS : in > 1024 && st_ok && (long long)rows * out >= 5000000LL ? KIND_SPARSE_ST : KIND_DENSE_PAIR;
         return ELSA_OK;
     }
-    if (in <= 512) *kind = ws_ok && (long long)rows * tiles_f >= 1200 * pairs ? KIND_SPARSE_WS : KIND_DENSE_PAIR;
+    // A call of its own has no image to wait for on the weight-stationary kernel, which leads from 240 rows per SM pair, 128 up to
+    // K = 256 (a block is small), 640 above K = 768 (accumulators get narrow).  Us there and on the best other kernel, image
+    // included, at 2:4: 768 -> 3072, 1576 rows (255 per pair) 11.8, 12.7, 4925 rows 17.1, 20.0; 768 -> 768, 3152 rows (128) 11.2,
+    // 10.2, 6304 rows 12.1, 12.6; 768 -> 2304, 1576 rows (192) 13.2, 12.6, 3152 rows 13.6, 14.4; 512 -> 1536, 6304 rows 12.1,
+    // 13.4; 384 -> 1152 at 2:16, 2000 rows (135) 9.5, 8.4; 384 -> 1536, 3152 rows 9.3, 9.9, 12608 rows 14.6, 18.1; 256 -> 1024, 3152
+    // rows (170) 7.2, 8.4; 896 -> 896, 6304 rows (341) 15.1, 13.6, 12608 rows 19.0, 19.7; 1024 -> 4096, 1576 rows (341) 16.9, 14.3,
+    // 6304 rows 30.5, 34.7.
+    const int ws_rows = in <= 256 ? 128 : in <= 768 ? 240 : 640;
+    if (use == USE_SINGLE && ws_ok && (long long)rows * tiles_f >= ws_rows * pairs) *kind = KIND_SPARSE_WS;
+    else if (in <= 512) *kind = ws_ok && (long long)rows * tiles_f >= 1200 * pairs ? KIND_SPARSE_WS : KIND_DENSE_PAIR;
     else if (ws_large) *kind = KIND_SPARSE_WS;
     else if (sparse_ok && st_ok && (long long)rows * out >= 5000000LL) *kind = KIND_SPARSE_ST;
     else if (sparse_ok) *kind = KIND_SPARSE_PAIR;
@@ -384,9 +407,10 @@ elsa_status run_linear(LinearKind kind, const void* X, int rows, const void* val
     if (kind == KIND_SPARSE_PAIR)
         return launch_linear_tc_sparse_pair((const uint16_t*)X, rows, (const uint16_t*)vals, idx, (const uint16_t*)bias,
                                             out, in, N, M, dtype, (uint16_t*)Y, workspace, dev_status, stream);
-    if (kind == KIND_SPARSE_WS)
-        return launch_linear_tc_sparse_ws((const uint16_t*)X, rows, (const uint16_t*)vals, idx, (const uint16_t*)bias,
-                                          out, in, N, M, dtype, (uint16_t*)Y, workspace, dev_status, stream);
+    if (kind == KIND_SPARSE_WS) {
+        const SparseJob job = sparse_job(kind, X, rows, vals, idx, bias, out, in, N, M, Y, nullptr);
+        return launch_linear_tc_sparse_ws_group(&job, 1, dtype, dev_status, stream);
+    }
     if (kind == KIND_SPARSE_ST)
         return launch_linear_tc_sparse_st((const uint16_t*)X, rows, (const uint16_t*)vals, idx, (const uint16_t*)bias,
                                           out, in, N, M, dtype, (uint16_t*)Y, workspace, dev_status, stream);
@@ -712,7 +736,7 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
         std::vector<ImageJob> jobs;
         for (int l = 0; l < n_layers; ++l) {
             const elsa_layer& c = cfg[l];
-            if (c.N != c.M)
+            if (c.N != c.M && reads_image(kind[l]))
                 jobs.push_back(image_job(kind[l], c.vals, c.idx, c.out, c.in, c.N, c.M, region[l]));
         }
         if (!jobs.empty()) st = launch_images(jobs.data(), (int)jobs.size(), image_stream);
@@ -728,10 +752,7 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
         for (int l = 0; l <= n_layers; ++l) {
             if (l < n_layers && kind[l] == KIND_SPARSE_PAIR) {
                 const elsa_layer& c = cfg[l];
-                SparseJob j;
-                j.X = (const uint16_t*)c.X; j.bias = (const uint16_t*)c.bias; j.Y = (uint16_t*)c.Y;
-                j.workspace = region[l]; j.rows = c.rows; j.in = c.in; j.out = c.out;
-                jobs.push_back(j);
+                jobs.push_back(sparse_job(kind[l], c.X, c.rows, c.vals, c.idx, c.bias, c.out, c.in, c.N, c.M, c.Y, region[l]));
             }
             if (!jobs.empty() && (l == n_layers || (int)jobs.size() == linear_tc_sparse_pair_group_max())) {
                 if ((st = launch_linear_tc_sparse_pair_group(jobs.data(), (int)jobs.size(), dtype, dev_status, stream)) != ELSA_OK)
@@ -746,10 +767,7 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
         for (int l = 0; l <= n_layers; ++l) {
             if (l < n_layers && kind[l] == KIND_SPARSE_ST) {
                 const elsa_layer& c = cfg[l];
-                SparseJob j;
-                j.X = (const uint16_t*)c.X; j.bias = (const uint16_t*)c.bias; j.Y = (uint16_t*)c.Y;
-                j.workspace = region[l]; j.rows = c.rows; j.in = c.in; j.out = c.out;
-                jobs.push_back(j);
+                jobs.push_back(sparse_job(kind[l], c.X, c.rows, c.vals, c.idx, c.bias, c.out, c.in, c.N, c.M, c.Y, region[l]));
             }
             if (!jobs.empty() && (l == n_layers || (int)jobs.size() == linear_tc_sparse_st_group_max())) {
                 if ((st = launch_linear_tc_sparse_st_group(jobs.data(), (int)jobs.size(), dtype, dev_status, stream)) != ELSA_OK)
@@ -764,10 +782,7 @@ elsa_status elsa_vit_linears(const elsa_layer* cfg, int n_layers, elsa_dtype dty
         for (int l = 0; l <= n_layers; ++l) {
             if (l < n_layers && kind[l] == KIND_SPARSE_WS) {
                 const elsa_layer& c = cfg[l];
-                SparseJob j;
-                j.X = (const uint16_t*)c.X; j.bias = (const uint16_t*)c.bias; j.Y = (uint16_t*)c.Y;
-                j.workspace = region[l]; j.rows = c.rows; j.in = c.in; j.out = c.out;
-                jobs.push_back(j);
+                jobs.push_back(sparse_job(kind[l], c.X, c.rows, c.vals, c.idx, c.bias, c.out, c.in, c.N, c.M, c.Y, region[l]));
             }
             if (!jobs.empty() && (l == n_layers || (int)jobs.size() == linear_tc_sparse_ws_group_max())) {
                 if ((st = launch_linear_tc_sparse_ws_group(jobs.data(), (int)jobs.size(), dtype, dev_status, stream)) != ELSA_OK)
@@ -1055,7 +1070,7 @@ elsa_status block_check(const void* x, int rows, int dim, int mlp_dim, const els
 // Whether a linear's kernel takes a ready-made weight image (the others build theirs when they run, or need none).
 bool takes_image(const BlockLinear& L)
 {
-    return L.w->N != L.w->M && (L.kind == KIND_DENSE_PAIR || L.kind == KIND_SMALL_IMAGE || L.kind == KIND_SPARSE_PAIR || L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST);
+    return L.w->N != L.w->M && (L.kind == KIND_DENSE_PAIR || L.kind == KIND_SMALL_IMAGE || L.kind == KIND_SPARSE_PAIR || L.kind == KIND_SPARSE_ST);
 }
 
 // Adds the images that n linears take to `jobs`.
@@ -1113,9 +1128,8 @@ elsa_status block_linear(BlockLinear& L, const uint16_t* X, int rows, elsa_dtype
     uint16_t* dst = residual ? tmp : Y;
     if (L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST || (L.kind == KIND_SPARSE_PAIR && act == 0)) {
         if ((st = block_images(&L, 1, stream)) != ELSA_OK) return st;
-        SparseJob job;
-        job.X = X; job.bias = (const uint16_t*)w.bias; job.Y = dst; job.workspace = L.ws;
-        job.rows = rows; job.in = L.in; job.out = L.out; job.act = act;
+        SparseJob job = sparse_job(L.kind, X, rows, w.vals, w.idx, w.bias, L.out, L.in, w.N, w.M, dst, L.ws);
+        job.act = act;
         return L.kind == KIND_SPARSE_WS   ? launch_linear_tc_sparse_ws_group(&job, 1, dtype, dev_status, stream)
                : L.kind == KIND_SPARSE_ST ? launch_linear_tc_sparse_st_group(&job, 1, dtype, dev_status, stream)
                                           : launch_linear_tc_sparse_pair_group(&job, 1, dtype, dev_status, stream);

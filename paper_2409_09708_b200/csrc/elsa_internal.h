@@ -173,6 +173,11 @@ struct SparseJob {
     const void* workspace;
     int rows, in, out;
     int act = 0;      // epilogue activation: 0 none, 1 GELU (weight-stationary and streaming kernels only)
+    // weight-stationary kernel: the packed weight (kept values, index words, level), from which it makes its weight block
+    // itself; without it the block comes from the image in `workspace`
+    const uint16_t* w = nullptr;
+    const uint32_t* idx = nullptr;
+    int N = 0, M = 0;
 };
 int linear_tc_sparse_pair_group_max();
 elsa_status launch_linear_tc_sparse_pair_prepare(const uint16_t* vals, const uint32_t* idx, int out, int in, int N, int M,
@@ -181,14 +186,11 @@ elsa_status launch_linear_tc_sparse_pair_group(const SparseJob* jobs, int n, els
                                                cudaStream_t stream);
 bool linear_tc_sparse_suits(int in, int N);
 // The same product with the 256-feature weight block of each CTA pair resident in tensor memory for a
-// whole layer (in % 128 == 0, in <= 1024); jobs as for the pair kernel, same re-encoded weight.
+// whole layer (in % 128 == 0, in <= 1024); the weight as it is packed, or re-encoded as for the pair kernel (SP24_PERMUTED).
 int linear_tc_sparse_ws_group_max();
 bool linear_tc_sparse_ws_suits(int in, int out, int N, int sm_count);
 elsa_status launch_linear_tc_sparse_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint32_t* dev_status,
                                              cudaStream_t stream);
-elsa_status launch_linear_tc_sparse_ws(const uint16_t* X, int rows, const uint16_t* vals, const uint32_t* idx,
-                                       const uint16_t* bias, int out, int in, int N, int M, elsa_dtype dtype, uint16_t* Y,
-                                       void* workspace, uint32_t* dev_status, cudaStream_t stream);
 size_t linear_tc_sparse_workspace(int out, int in);
 // The same product with the weight block streaming through tensor memory in K chunks of 256 (in % 128 == 0,
 // any length); jobs as for the pair kernel, weight image in the SP24_TILED form.

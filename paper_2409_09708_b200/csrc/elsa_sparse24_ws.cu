@@ -25,13 +25,20 @@
 // start of a layer and run the epilogue.  The accumulator is transposed (lanes are features, columns
 // are token rows) and Y is row-major, so the epilogue has to turn a lane's column pair into a row's
 // feature run.  stmatrix with .trans does that in one instruction per 8 x 32 outputs if lane t of a
-// quarter holds feature 8 * (t % 4) + t / 4 of its 32; the weight image is therefore built with its
-// rows in that order (SP24_PERMUTED form of nm_to_sp24), and only the bias index and the store address
-// here know about it.  Waits are bounded as in the other kernels.
+// quarter holds feature 8 * (t % 4) + t / 4 of its 32, so lane t writes that feature's row into tensor memory.
+//
+// The weight block is made from the packed weight itself: a lane expands its feature's row to two values per chunk of 4 and
+// metadata on the way to tensor memory, 128 k at a time.  As an image the weight cost a launch of 2 to 3 us ahead of the layer
+// and a trip through L2 for work that is a few hundred instructions a lane here, once a layer: 4925 x 768 -> 3072 at 2:4 20.4
+// (on the streaming kernel, image included) -> 17.1 us, 3152 rows 16.0 -> 14.1; the linears of a DeiT-B block at 12608
+// rows in a table 145 -> 143.  Only the masked form, whose dense shared weight would be ranked again by every row group, brings an image
+// (SP24_PERMUTED form of launch_images: rows in the lanes' order).  Waits are bounded as in the other kernels.
 
 #include <atomic>
 #include <mutex>
+#include <type_traits>
 
+#include "elsa_sp24_device.cuh"
 #include "elsa_tc_common.cuh"
 
 namespace elsa {
@@ -56,19 +63,26 @@ constexpr int kStagingBytes = kMaxSteps * kStepCols * 64;        // per epilogue
 constexpr int kStagingTotal = kEpiWarps * kStagingBytes;
 constexpr int kBarrierBytes = 512;
 
+// What a layer's weight block is made from.
+enum WsLevel : uint8_t { LEVEL_IMAGE, LEVEL_1_4, LEVEL_2_4, LEVEL_1_8, LEVEL_2_8, LEVEL_1_16, LEVEL_2_16 };
+
 struct alignas(64) WsLayer {
     CUtensorMap map_x, map_y, map_run;   // map_y: one step of 16 token rows, map_run: a warp's whole run of them
-    const uint16_t* a_img;   // 2-of-4 values [out rounded up to 32][in / 2], rows in the permuted order
-    const uint8_t* meta;     // metadata blocks of 2 KB per (128 features, 128 k)
+    // LEVEL_IMAGE: 2-of-4 values [out rounded up to 32][in / 2], rows in the permuted order, and metadata blocks of 2 KB per
+    // (128 features, 128 k).  Otherwise the packed weight: kept values and index words.
+    const void* w;
+    const void* meta;
     const uint16_t* bias;
     int rows, out, in;
     int nt;            // token rows per pair tile
-    int steps_per_warp;   // 16-column steps each epilogue warp of a quarter takes
+    uint8_t level;     // WsLevel
+    uint8_t steps_per_warp;   // 16-column steps each epilogue warp of a quarter takes
+    uint8_t act;       // epilogue activation (0 none, 1 GELU) on acc + bias
+    int words_per_row; // of the index words
     int tiles_f;       // F
     int groups;        // G
     int row_tiles;     // ceil(rows / nt)
     uint32_t idesc;
-    int act;           // epilogue activation (0 none, 1 GELU) on acc + bias
 };
 
 constexpr int kGroupMax = 68;   // layers per launch (kernel parameters are limited to 32 KB)
@@ -81,6 +95,80 @@ struct WsGroup {
     int stage_bytes;   // one pipeline stage: kStageK / 64 quarters of (largest nt / 2) rows of 128 bytes
     uint32_t* dev_status;
 };
+
+// 128 k of a row of the packed weight: whole words of values and, but for half a word at 1:8, of index fields.
+template <int M, int N>
+struct PackedBlock {
+    static constexpr int kCount = 16 / M * N, kBits = kCount * (M == 4 ? 2 : M == 8 ? 3 : 4);      // of a segment of 16 k
+    static constexpr int kIdxBits = 8 * kBits, kIdxWords = kIdxBits % 32 ? 2 : kIdxBits / 32;
+    uint4 v[kCount];
+    uint32_t f[kIdxWords];
+
+    __device__ __forceinline__ void load(const uint16_t* vals_row, const uint32_t* idx_row, int kb)
+    {
+        const uint4* src = reinterpret_cast<const uint4*>(vals_row) + kb * kCount;
+#pragma unroll
+        for (int i = 0; i < kCount; ++i) v[i] = __ldg(src + i);
+        const int bit0 = kb * kIdxBits;
+#pragma unroll
+        for (int i = 0; i < kIdxWords; ++i) f[i] = __ldg(idx_row + (bit0 >> 5) + i);
+        if constexpr (kIdxBits % 32 != 0) {      // 48 bits from bit 0 or 16 on
+            f[0] = __funnelshift_r(f[0], f[1], bit0 & 31);
+            f[1] >>= bit0 & 31;
+        }
+    }
+    __device__ __forceinline__ uint32_t word(int i) const
+    {
+        const uint4& u = v[i >> 2];
+        return (i & 3) == 0 ? u.x : (i & 3) == 1 ? u.y : (i & 3) == 2 ? u.z : u.w;
+    }
+    __device__ __forceinline__ Segment segment(int i) const
+    {
+        Segment s;
+        s.v[0] = s.v[1] = s.v[2] = s.v[3] = 0u;
+        if constexpr (kCount == 1) s.v[0] = word(i >> 1) >> (16 * (i & 1)) & 0xFFFFu;
+#pragma unroll
+        for (int j = 0; j < kCount / 2; ++j) s.v[j] = word(i * (kCount / 2) + j);
+        const int bit = i * kBits, w0 = bit >> 5;
+        s.fields = (bit & 31) + kBits > 32 ? __funnelshift_r(f[w0], f[w0 + 1 < kIdxWords ? w0 + 1 : w0], bit & 31) : f[w0] >> (bit & 31);
+        return s;
+    }
+};
+
+// A warp's blocks of 128 k, straight from the packed weight into tensor memory: 32 columns of values and 4 of metadata each.
+// A lane expands its own feature's row; a metadata word holds 16 k of two rows eight apart (lane l: rows l % 8 and l % 8 + 8
+// of its 16, the half of the 32 k that bit 3 of l says), so the nibbles change lanes by two shuffles a word.  All of a
+// block's loads are in flight together (the next block's under them spill).
+template <int M, int N>
+__device__ __forceinline__ void write_packed(const uint16_t* vals_row, const uint32_t* idx_row, bool row_ok, int first, int blocks, int step,
+                                             uint32_t a_col0, uint32_t e_col0)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int kb = first; kb < blocks; kb += step) {
+        PackedBlock<M, N> cur;
+        cur.load(vals_row, idx_row, kb);
+        uint32_t e[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {          // 32 k
+            uint32_t v[8], nib[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                uint4 t = sp24_words<M, N>(cur.segment(2 * h + i), nib[i]);
+                if (!row_ok) {                 // a feature past the last one: zeros, four empty chunks of 4
+                    t = make_uint4(0u, 0u, 0u, 0u);
+                    nib[i] = 0x4444u;
+                }
+                v[4 * i] = t.x; v[4 * i + 1] = t.y; v[4 * i + 2] = t.z; v[4 * i + 3] = t.w;
+            }
+            tmem_st_32x32b_x8(a_col0 + (uint32_t)(32 * kb + 8 * h), v);
+            const uint32_t mine = nib[0] | nib[1] << 16;
+            const uint32_t lo = __shfl_sync(0xFFFFFFFFu, mine, lane & 23), hi = __shfl_sync(0xFFFFFFFFu, mine, (lane & 23) | 8);
+            e[h] = prmt(lo, hi, lane & 8 ? 0x7632u : 0x5410u);
+        }
+        tmem_st_32x32b_x4(e_col0 + (uint32_t)(4 * kb), e);
+    }
+}
 
 // kAct: the instantiation whose epilogue applies the layer's activation (single-layer launches).
 template <bool kBf16, int kMaxLayers, bool kAct>
@@ -295,27 +383,46 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
             {
                 const uint32_t a_col0 = lane_base + (uint32_t)(kNumAccum * nt);
                 const uint32_t e_col0 = a_col0 + (uint32_t)(L.in >> 2);
-                const uint4* a_row = reinterpret_cast<const uint4*>(L.a_img + (size_t)(ft128 * kFeatPerCta + q * 32 + lane) * (size_t)(L.in >> 1));
-                const bool blk_ok = ft128 * kFeatPerCta < l_out;     // rows of a started block of 32 exist (zero beyond out)
-                const bool row_ok = f0 < l_out;
-                const int a_chunks = L.in >> 6;          // 16 columns (64 bytes) each
-                for (int c = part; c < a_chunks; c += kEpiParts) {
-                    uint32_t v[16];
+                if (L.level == LEVEL_IMAGE) {
+                    const int a_chunks = L.in >> 6;          // 16 columns (64 bytes) each
+                    const uint4* a_row = static_cast<const uint4*>(L.w) + (size_t)(ft128 * kFeatPerCta + q * 32 + lane) * (size_t)(L.in >> 4);
+                    const bool blk_ok = ft128 * kFeatPerCta < l_out;     // rows of a started block of 32 exist (zero beyond out)
+                    const bool row_ok = f0 < l_out;
+                    for (int c = part; c < a_chunks; c += kEpiParts) {
+                        uint32_t v[16];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        uint4 t = make_uint4(0u, 0u, 0u, 0u);
-                        if (row_ok) t = __ldg(a_row + 4 * c + i);
-                        v[4 * i] = t.x; v[4 * i + 1] = t.y; v[4 * i + 2] = t.z; v[4 * i + 3] = t.w;
+                        for (int i = 0; i < 4; ++i) {
+                            uint4 t = make_uint4(0u, 0u, 0u, 0u);
+                            if (row_ok) t = __ldg(a_row + 4 * c + i);
+                            v[4 * i] = t.x; v[4 * i + 1] = t.y; v[4 * i + 2] = t.z; v[4 * i + 3] = t.w;
+                        }
+                        tmem_st_32x32b_x16(a_col0 + (uint32_t)(16 * c), v);
                     }
-                    tmem_st_32x32b_x16(a_col0 + (uint32_t)(16 * c), v);
-                }
-                const uint4* e_blk = reinterpret_cast<const uint4*>(L.meta) +
-                                     (size_t)(blk_ok ? ft128 : 0) * (size_t)(L.in / kBlockK) * 128 + (size_t)(q * 32 + lane);
-                for (int kb = part; kb < L.in / kBlockK; kb += kEpiParts) {
-                    uint4 t = make_uint4(0u, 0u, 0u, 0u);
-                    if (blk_ok) t = __ldg(e_blk + (size_t)kb * 128);
-                    uint32_t v[4] = {t.x, t.y, t.z, t.w};
-                    tmem_st_32x32b_x4(e_col0 + (uint32_t)(4 * kb), v);
+                    const uint4* e_blk = static_cast<const uint4*>(L.meta) +
+                                         (size_t)(blk_ok ? ft128 : 0) * (size_t)(L.in / kBlockK) * 128 + (size_t)(q * 32 + lane);
+                    for (int kb = part; kb < L.in / kBlockK; kb += kEpiParts) {
+                        uint4 t = make_uint4(0u, 0u, 0u, 0u);
+                        if (blk_ok) t = __ldg(e_blk + (size_t)kb * 128);
+                        uint32_t v[4] = {t.x, t.y, t.z, t.w};
+                        tmem_st_32x32b_x4(e_col0 + (uint32_t)(4 * kb), v);
+                    }
+                } else {
+                    const int row = f_ok ? f : l_out - 1;      // always one that can be read
+                    const uint16_t* vals = static_cast<const uint16_t*>(L.w);
+                    const uint32_t* idx_row = static_cast<const uint32_t*>(L.meta) + (size_t)row * (size_t)L.words_per_row;
+                    auto block = [&](auto m, auto n) {
+                        constexpr int M = decltype(m)::value, N = decltype(n)::value;
+                        write_packed<M, N>(vals + (size_t)row * (size_t)(L.in / M * N), idx_row, f_ok, part, L.in / kBlockK, kEpiParts, a_col0, e_col0);
+                    };
+                    using std::integral_constant;
+                    switch (L.level) {
+                    case LEVEL_1_4: block(integral_constant<int, 4>{}, integral_constant<int, 1>{}); break;
+                    case LEVEL_2_4: block(integral_constant<int, 4>{}, integral_constant<int, 2>{}); break;
+                    case LEVEL_1_8: block(integral_constant<int, 8>{}, integral_constant<int, 1>{}); break;
+                    case LEVEL_2_8: block(integral_constant<int, 8>{}, integral_constant<int, 2>{}); break;
+                    case LEVEL_1_16: block(integral_constant<int, 16>{}, integral_constant<int, 1>{}); break;
+                    default: block(integral_constant<int, 16>{}, integral_constant<int, 2>{}); break;
+                    }
                 }
                 tmem_wait_st();
                 tc_fence_before();
@@ -475,15 +582,24 @@ elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
         if (L.nt == 0 || j.in % kBlockK != 0 || L.tiles_f > pairs)
             return fail(ELSA_ERR_SHAPE, "in=%d out=%d does not fit the weight-stationary sparse kernel", j.in, j.out);
         L.rows = j.rows; L.out = j.out; L.in = j.in;
-        L.steps_per_warp = (L.nt / kStepCols + kEpiParts - 1) / kEpiParts;
+        L.steps_per_warp = (uint8_t)((L.nt / kStepCols + kEpiParts - 1) / kEpiParts);
         L.row_tiles = (j.rows + L.nt - 1) / L.nt;
         L.groups = pairs / L.tiles_f;
         if (L.groups > L.row_tiles) L.groups = L.row_tiles;
         if (L.groups * L.tiles_f > used_pairs) used_pairs = L.groups * L.tiles_f;
         L.bias = j.bias;
-        L.act = j.act;
-        L.a_img = (const uint16_t*)j.workspace;
-        L.meta = (const uint8_t*)j.workspace + sp24_meta_offset(j.out, j.in);
+        L.act = (uint8_t)j.act;
+        if (j.w != nullptr) {
+            L.w = j.w;
+            L.meta = j.idx;
+            L.level = j.M == 4 ? (j.N == 1 ? LEVEL_1_4 : LEVEL_2_4) : j.M == 8 ? (j.N == 1 ? LEVEL_1_8 : LEVEL_2_8) : j.N == 1 ? LEVEL_1_16 : LEVEL_2_16;
+            L.words_per_row = (int)index_words_per_row(j.in, j.N, j.M);
+        } else {
+            L.w = j.workspace;
+            L.meta = (const uint8_t*)j.workspace + sp24_meta_offset(j.out, j.in);
+            L.level = LEVEL_IMAGE;
+            L.words_per_row = 0;
+        }
         // sparse flag, fp32 accumulate, A and B of type fmt, K-major, N = nt, M = 256 over the pair
         L.idesc = (1u << 2) | (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(L.nt >> 3) << 17) |
                   ((uint32_t)(kPairFeat >> 4) << 24);
@@ -543,18 +659,6 @@ elsa_status launch_linear_tc_sparse_ws_group(const SparseJob* jobs, int n, elsa_
                                   : launch_ws_group<false, 1, false>(jobs, 1, dtype, dev_status, stream, dev);
     return dtype == ELSA_BF16 ? launch_ws_group<true, kGroupMax, false>(jobs, n, dtype, dev_status, stream, dev)
                               : launch_ws_group<false, kGroupMax, false>(jobs, n, dtype, dev_status, stream, dev);
-}
-
-elsa_status launch_linear_tc_sparse_ws(const uint16_t* X, int rows, const uint16_t* vals, const uint32_t* idx,
-                                       const uint16_t* bias, int out, int in, int N, int M, elsa_dtype dtype, uint16_t* Y,
-                                       void* workspace, uint32_t* dev_status, cudaStream_t stream)
-{
-    elsa_status st = launch_linear_tc_sparse_pair_prepare(vals, idx, out, in, N, M, SP24_PERMUTED, workspace, stream);
-    if (st != ELSA_OK) return st;
-    SparseJob job;
-    job.X = X; job.bias = bias; job.Y = Y; job.workspace = workspace;
-    job.rows = rows; job.in = in; job.out = out;
-    return launch_linear_tc_sparse_ws_group(&job, 1, dtype, dev_status, stream);
 }
 
 }  // namespace elsa
