@@ -17,7 +17,7 @@ HOST_SOURCE = os.path.join(CSRC, "elsa_host.cpp")
 # The module holds for one Python and one torch: its name has the one's tag, the file beside it the other's version.
 HOST_LIB = os.path.join(HERE, "_elsa_host" + sysconfig.get_config_var("EXT_SUFFIX"))
 HOST_STAMP = os.path.join(HERE, "_build", "elsa_host_torch_version")
-SOURCES = ["elsa_api.cu", "elsa_attention.cu", "elsa_attention_window.cu", "elsa_backward.cu", "elsa_block.cu", "elsa_compress.cu", "elsa_int8.cu", "elsa_linear_simt.cu", "elsa_linear_small.cu", "elsa_linear_tc.cu", "elsa_linear_tc2.cu",
+SOURCES = ["elsa_api.cu", "elsa_attention.cu", "elsa_attention_rows.cu", "elsa_attention_window.cu", "elsa_backward.cu", "elsa_block.cu", "elsa_compress.cu", "elsa_int8.cu", "elsa_linear_simt.cu", "elsa_linear_small.cu", "elsa_linear_tc.cu", "elsa_linear_tc2.cu",
            "elsa_no_alloc.cu", "elsa_search.cu", "elsa_selftest.cu", "elsa_sparse24.cu", "elsa_sparse24_pair.cu", "elsa_sparse24_st.cu", "elsa_sparse24_ws.cu", "elsa_weight_images.cu"]
 
 

@@ -34,7 +34,7 @@
 #include <mutex>
 #include <type_traits>
 
-#include "elsa_tc_common.cuh"
+#include "elsa_attention_common.cuh"
 
 namespace elsa {
 namespace {
@@ -87,14 +87,6 @@ __device__ __forceinline__ uint64_t smem_desc_mn_major_sw64(uint32_t addr, uint3
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)4 << 61;
     return d;
-}
-
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
-        : "memory");
 }
 
 // D[tmem] (+)= A[tmem] * B[smem]: A's 16-bit values two per column, lane = row.  Predicated as the other forms.
@@ -584,22 +576,6 @@ __global__ void __launch_bounds__(Shape<kD, kBufs, kBias>::kThreads, 1) attentio
     }
 }
 
-elsa_status make_map_qkv(CUtensorMap* map, const void* qkv, int images, int tokens, int dim, int head_dim, uint32_t box_rows,
-                         const char* what)
-{
-    EncodeTiledFn fn = encode_tiled_fn();
-    if (!fn) return fail(ELSA_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
-    cuuint64_t dims[3] = {(cuuint64_t)(3 * dim), (cuuint64_t)tokens, (cuuint64_t)images};
-    cuuint64_t strides[2] = {(cuuint64_t)(3 * dim) * 2, (cuuint64_t)tokens * (cuuint64_t)(3 * dim) * 2};
-    cuuint32_t box[3] = {(cuuint32_t)head_dim, box_rows, 1};
-    cuuint32_t elem[3] = {1, 1, 1};
-    CUresult rc = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<void*>(qkv), dims, strides, box, elem,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, head_dim == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
-                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (rc != CUDA_SUCCESS) return fail(ELSA_ERR_CUDA, "tensor map for %s rejected (CUresult %d)", what, (int)rc);
-    return ELSA_OK;
-}
-
 template <bool kBf16, int kD, bool kBias, int kBufs>
 elsa_status launch(const AttnParams& p, int images, int heads, cudaStream_t stream, const DeviceInfo& dev)
 {
@@ -652,6 +628,9 @@ elsa_status launch_attention(const uint16_t* qkv, int images, int tokens, int he
     // windows that fit a warp's registers: 286 us here against 89 us there for 32768 windows x heads of 49 tokens
     if (window_attention_suits(tokens, heads, dim))
         return launch_window_attention(qkv, images, tokens, heads, dim, dtype, out, dev_status, stream, bias, mask, n_masks, bias_pitch, dev);
+    // A call whose items leave SMs idle is bound by the chain of one: sixteen query rows a CTA instead of 128.
+    if (bias == nullptr && attention_rows_suits(images, tokens, heads, dev.sm_count))
+        return launch_attention_rows(qkv, images, tokens, heads, dim, dtype, out, dev_status, stream, dev);
     AttnParams p;
     p.out = out;
     p.tokens = tokens;
