@@ -988,6 +988,7 @@ struct BlockLinear {
     void* ws;          // this linear's part of region WORKSPACE
     bool image_ready;  // its weight image has been enqueued already
     bool first;        // no kernel of the same call runs before it
+    const BlockLinear* next;   // the linear that runs after it in the same call, or NULL
 };
 
 struct BlockPlan {
@@ -1061,6 +1062,7 @@ elsa_status block_check(const void* x, int rows, int dim, int mlp_dim, const els
         lin[l].ws = images ? images + (plan->ws_off[l] - plan->off[ELSA_BLOCK_WORKSPACE]) : (uint8_t*)scratch + plan->ws_off[l];
         lin[l].image_ready = false;
         lin[l].first = false;
+        lin[l].next = l < 3 ? &lin[l + 1] : nullptr;
         elsa_status st = pick_kind(USE_CHAIN, rows, outs[l], ins[l], src[l]->N, src[l]->M, dev.sm_count, &lin[l].kind, l == 2);
         if (st != ELSA_OK) return st;
     }
@@ -1117,6 +1119,11 @@ elsa_status block_linear(BlockLinear& L, const uint16_t* X, int rows, elsa_dtype
         SmallJob job = L.kind == KIND_SMALL ? small_job(X, rows, w.vals, w.N == w.M ? nullptr : w.idx, w.bias, L.out, L.in, w.N, w.M, Y)
                                             : small_dense_job(X, rows, w.N == w.M ? w.vals : L.ws, w.bias, L.out, L.in, Y);
         job.act = act; job.residual = residual;
+        if (L.next != nullptr && L.next->kind == KIND_SMALL_IMAGE) {
+            const elsa_block_linear& n = *L.next->w;
+            job.ahead = n.N == n.M ? n.vals : L.next->ws;
+            job.ahead_bytes = (size_t)L.next->out * L.next->in * 2;
+        }
         DeviceInfo dev;
         if ((st = device_info(&dev)) != ELSA_OK) return st;
         // after another kernel of the same call the weights are older than that kernel's start (KIND_SMALL: only where the
@@ -1404,6 +1411,7 @@ elsa_status elsa_vit_encoder(const void* x, int images, int tokens, int heads, i
     // block's last residual is still to be added, the next block's first LayerNorm does it while it normalises.
     BlockCarry carry;
     const void* in = x;
+    for (int b = 0; b + 1 < n_blocks; ++b) prepared[b].lin[3].next = &prepared[b + 1].lin[0];
     for (int b = 0; b < n_blocks; ++b) {
         const bool last = b + 1 == n_blocks;
         void* out = (last && final_gain == nullptr) ? y : (void*)buf[(b + 1) & 1];

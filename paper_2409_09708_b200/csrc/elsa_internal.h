@@ -107,6 +107,8 @@ struct SmallJob {
     bool masked = false;
     int act = 0;                          // 0 none, 1 GELU
     const uint16_t* residual = nullptr;   // [rows][out], added after the activation, before the one rounding
+    const void* ahead = nullptr;          // launches of one job: the next linear's weight, brought into L2 meanwhile (16-byte
+    size_t ahead_bytes = 0;               // aligned; nothing reads it here, so it may still be written)
 };
 int linear_small_group_max();
 // Ranges the reductions of these jobs are cut into when they run together.  A result depends on it in its last bits.

@@ -12,11 +12,14 @@
 //   * a CTA computes one tile of 128 rows x 64 features and leaves; two CTAs fit an SM, so that one's set-up and
 //     epilogue run under the other's tile, or the next kernel's set-up under this one's;
 //   * where the tiles alone leave SMs idle, the reduction is cut into 2, 4 or 8 ranges, one CTA of a cluster each:
-//     every CTA sends the rows of its fp32 sums to the CTA that owns them through distributed shared memory, one
-//     cluster barrier, and each owner adds its rows in rank order (deterministic), applies bias, activation and
-//     residual, and rounds once;
+//     every CTA sends the rows of its fp32 sums to the CTA that owns them as bulk copies between their shared memories,
+//     whose bytes the owner's barrier counts, and each owner adds its rows in rank order (deterministic), applies bias,
+//     activation and residual, which it has asked for by then, and rounds once (stores into the other CTA's memory behind a
+//     cluster barrier, bias and residual loaded last: 3072 x 768 at 4:4, 197 rows, 7.3 -> 7.1 us, one-image encoder 500 -> 492);
 //   * a call that knows the weights to be older than its own first kernel (the chained block) has their first tiles
-//     fetched before the predecessor kernel has ended (`early`): only X and the outputs wait for it.
+//     fetched before the predecessor kernel has ended (`early`): only X and the outputs wait for it;
+//   * in a chain each launch has the next linear's weight brought into L2 (`ahead`): a model's weights do not stay there
+//     from one call to the next (one-image encoder 486 -> 476 us).
 // Measured back to back on 197 rows (us, weight image + one-CTA-per-tile GEMM before, this kernel after): 768 -> 768 at
 // 2:4 6.9 -> 6.4, 768 -> 2304 at 2:4 8.2 -> 7.7, 3072 -> 768 at 2:4 15.4 -> 10.6, at 4:4 11.6 -> 6.9.  The expansion
 // is repeated for every 128 rows and bound by its loads' latency and its instructions: at 788 rows and 2:4 the image
@@ -45,13 +48,15 @@ constexpr int kWBytes = kTileN * kTileK * 2;
 constexpr int kStageBytes = kXBytes + kWBytes;
 constexpr int kStagesMax = 4;
 constexpr int kStagesSplit = 3;
-constexpr int kPitch = kTileN + 4;         // floats of a row of sums: 16-byte accesses of 8 rows fall on 32 banks
-constexpr int kSumBytes = kTileM * kPitch * 4;
+constexpr int kHalfN = kTileN / 2;         // columns of an epilogue warp
+constexpr int kPitch = kHalfN + 4;         // floats of a row of a warp's sums: 16-byte accesses of 8 rows fall on 32 banks
+constexpr int kSumBytes = 2 * kTileM * kPitch * 4;
 constexpr int kSplitsMax = 8;
+constexpr int kAheadUnits = 512;           // of 16 bytes in one request for the next linear's weight
 constexpr int kSmallGroupMax = 72;         // layers per launch (kernel parameters are limited to 32 KB)
 
-// Two CTAs per SM need at most 113 KB each.  With one range the sums take the place of the stages; with several they
-// have their own, since another CTA of the cluster may send its sums while this one's MMAs still read.
+// Two CTAs per SM need at most 113 KB each.  With one range the sums take the place of the stages; with several those
+// that arrive have their own, since another CTA of the cluster may send its sums while this one's MMAs still read.
 constexpr int small_smem(bool split)
 {
     return (split ? kStagesSplit * kStageBytes + kSumBytes : kStagesMax * kStageBytes) + 256 /* barriers */ + 1024 /* alignment */;
@@ -78,15 +83,24 @@ struct SmallGroup {
     int splits;                   // CTAs of a cluster = ranges of the reduction
     int stages;
     int early;
+    int rehearse;                 // 0: the epilogue's first pass is a rehearsal (a value that the compiler does not know)
     uint32_t idesc;
     uint32_t* dev_status;
+    const void* ahead;            // what the call's next linear reads as its weight: brought into L2 meanwhile
+    uint32_t ahead_units;         // of 16 bytes
 };
 
-__device__ __forceinline__ void named_barrier_workers() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers * 32) : "memory"); }
-
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+__device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes)
 {
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
+// Copies shared memory of this CTA into another one of the cluster, the bytes counted on an mbarrier there.
+__device__ __forceinline__ void bulk_send(uint32_t dst_cluster, uint32_t src, uint32_t bytes, uint32_t bar_cluster)
+{
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst_cluster), "r"(src),
+                 "r"(bytes), "r"(bar_cluster)
+                 : "memory");
 }
 
 // The expansion of the K blocks kb0..kb1 by two groups of four warps that take turns, kAhead K blocks at a time: one
@@ -174,7 +188,9 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
     const uint32_t full_bar = smem_base + (uint32_t)bar_off;
     const uint32_t empty_bar = full_bar + 8 * kStagesMax;
     const uint32_t done_bar = empty_bar + 8 * kStagesMax;
-    volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 16 * kStagesMax + 8);
+    const uint32_t sums_bar = done_bar + 8;       // the sums of this CTA's rows: its own warps' arrivals, the others' bytes
+    volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 16 * kStagesMax + 16);
+    const int slice = kTileM / splits;            // rows each CTA of the cluster finishes
     volatile uint32_t* abort_flag = tmem_holder + 1;
 
     if (threadIdx.x == 0) {
@@ -183,16 +199,19 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
             mbar_init(empty_bar + 8 * s, 1);
         }
         mbar_init(done_bar, 1);
+        mbar_init(sums_bar, 1 + kWorkers);
+        mbar_arrive_expect_tx(sums_bar, (uint32_t)((splits - 1) * slice * 2 * kPitch * 4));
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
     }
-    if (warp == 1) tmem_alloc(smem_base + (uint32_t)(bar_off + 16 * kStagesMax + 8), kTileN);
+    if (warp == 1) tmem_alloc(smem_base + (uint32_t)(bar_off + 16 * kStagesMax + 16), kTileN);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
-    // a CTA of the cluster writes into another's shared memory only once that one runs
+    // A CTA of the cluster writes into another's shared memory only once that one runs (first phase of the cluster's
+    // barrier), and leaves only when what it sent has arrived (second phase).
     if (split) cluster_arrive();
 
     if (warp == 0) {
@@ -259,6 +278,14 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
         __syncwarp();
         if (split) { cluster_wait(); cluster_arrive(); cluster_wait(); }
     } else if (warp >= 2 + kWorkers) {
+        if (warp == 2 + kWorkers && p.ahead != nullptr && elect_one()) {
+            // a chained block's weights do not stay in L2 from one call to the next: each CTA asks for its share of the next ones
+            pdl_wait_for_predecessors();
+            const uint32_t share = (p.ahead_units + gridDim.x - 1) / gridDim.x, end = min(p.ahead_units, share * (blockIdx.x + 1));
+            for (uint32_t at = share * blockIdx.x; at < end; at += kAheadUnits)
+                bulk_prefetch_l2(static_cast<const uint4*>(p.ahead) + at, 16u * min((uint32_t)kAheadUnits, end - at));
+        }
+        __syncwarp();
         if (split) { cluster_wait(); cluster_arrive(); cluster_wait(); }
     } else {
         // ------------------------------------------------ expansion, then epilogue
@@ -308,58 +335,101 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
         }
         if (p.early) pdl_wait_for_predecessors();     // before the residual is read or Y written
         const int q = warp & 3, half = (warp - 2) >> 2;
-        const int slice = kTileM / splits;            // rows each CTA of the cluster finishes
-        float* sums = reinterpret_cast<float*>(smem_gen + sums_off);      // [splits][slice][pitch]
-        ok = ok && mbar_wait(done_bar, 0, abort_flag, p.dev_status, 44);
-        ok = __all_sync(0xFFFFFFFFu, ok);
-        if (split) cluster_wait();
-        if (ok) {
-            tc_fence_after();
-            const int row = q * 32 + lane;
-            uint32_t dst = smem_base + (uint32_t)(sums_off + ((rank * slice + row % slice) * kPitch + half * (kTileN / 2)) * 4);
-            if (split) dst = mapa_shared(dst, (uint32_t)(row / slice));
-            uint32_t r[32];
-            tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * (kTileN / 2)), r);
-            tmem_wait_ld();
-#pragma unroll
-            for (int v = 0; v < 8; ++v) st_cluster_v4(dst + (uint32_t)(16 * v), r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
-            tc_fence_before();
+        // What the finished rows need besides the sums is asked for ahead of them.
+        constexpr int kUnits = kTileN / 8, kRowsAStep = kWorkers * 32 / kUnits;
+        const int tid = (int)threadIdx.x - 64;
+        const int col_l = (tid % kUnits) * 8, col = n0 + col_l;      // the same for all of a thread's units
+        uint4 bw = make_uint4(0u, 0u, 0u, 0u), rw = bw;
+        if (L.bias != nullptr && col < L.out) bw = __ldg(reinterpret_cast<const uint4*>(L.bias + col));
+        const uint16_t* residual = L.residual;
+        {
+            const int row = m0 + rank * slice + tid / kUnits;
+            if (residual != nullptr && row < L.rows && col < L.out) rw = *reinterpret_cast<const uint4*>(residual + (size_t)row * L.out + col);
         }
-        __syncwarp();
-        if (split) { cluster_arrive(); cluster_wait(); }
-        else named_barrier_workers();
-        if (ok) {
-            constexpr int kUnits = kTileN / 8;
-            for (int e = (int)threadIdx.x - 64; e < slice * kUnits; e += kWorkers * 32) {
-                const int row_l = e / kUnits, col_l = (e % kUnits) * 8;
-                const int row = m0 + rank * slice + row_l, col = n0 + col_l;
-                if (row >= L.rows || col >= L.out) continue;
-                uint4 bw = make_uint4(0u, 0u, 0u, 0u), rw = make_uint4(0u, 0u, 0u, 0u);
-                if (L.bias != nullptr) bw = __ldg(reinterpret_cast<const uint4*>(L.bias + col));
-                if (L.residual != nullptr) rw = *reinterpret_cast<const uint4*>(L.residual + (size_t)row * L.out + col);
-                float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                for (int s = 0; s < splits; ++s) {
-                    const float4* src = reinterpret_cast<const float4*>(sums + (size_t)(s * slice + row_l) * kPitch + col_l);
-                    const float4 x = src[0], y = src[1];
-                    a[0] += x.x; a[1] += x.y; a[2] += x.z; a[3] += x.w;
-                    a[4] += y.x; a[5] += y.y; a[6] += y.z; a[7] += y.w;
-                }
-                const uint32_t b[4] = {bw.x, bw.y, bw.z, bw.w}, r[4] = {rw.x, rw.y, rw.z, rw.w};
-                uint32_t o[4];
+        // The sums of 32 rows x 32 columns a warp lie [half][row][pitch]; those that come from CTA s of the cluster at
+        // s * slice rows of either half.
+        const uint32_t inbox = smem_base + (uint32_t)sums_off;
+        const float* sums = reinterpret_cast<const float*>(smem_gen + sums_off) + (size_t)(col_l / kHalfN * kTileM) * kPitch + col_l % kHalfN;
+        // The first pass is a rehearsal: while the loads and MMAs are under way it runs the last part's instructions and stores
+        // nothing.  In a chain of kernels their code is in none of the SM's caches, and fetched when it is needed it took
+        // longer than it ran: one-image encoder of DeiT-B 492 -> 486 us; for the same reason the loops here are not unrolled.
+#pragma unroll 1
+        for (int real = p.rehearse; real < 2; ++real) {
+            if (real) {
+                ok = ok && mbar_wait(done_bar, 0, abort_flag, p.dev_status, 44);
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (split) cluster_wait();
+                if (ok) {
+                    tc_fence_after();
+                    const int row = q * 32 + lane, to = row / slice;
+                    uint32_t r[32];
+                    tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * kHalfN), r);
+                    tmem_wait_ld();
+                    tc_fence_before();
+                    // rows of this CTA go where they are added, the others' to the stages (no MMA reads them any more) and from
+                    // there to their CTA as one copy for each
+                    const uint32_t outbox = smem_base + (uint32_t)(half * kTileM * kPitch * 4);
+                    const uint32_t dst = to == rank ? inbox + (uint32_t)((half * kTileM + rank * slice + row % slice) * kPitch * 4)
+                                                    : outbox + (uint32_t)(row * kPitch * 4);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float2 bv = raw2_to_float2<kBf16>(b[i]), rv = raw2_to_float2<kBf16>(r[i]);
-                    float x = a[2 * i] + bv.x, y = a[2 * i + 1] + bv.y;
-                    if (L.act == 1) {
-                        const float2 g = gelu_pair(x, y);
-                        x = g.x;
-                        y = g.y;
+                    for (int v = 0; v < 8; ++v)
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(16 * v)), "r"(r[4 * v]), "r"(r[4 * v + 1]),
+                                     "r"(r[4 * v + 2]), "r"(r[4 * v + 3])
+                                     : "memory");
+                    if (split) fence_proxy_async_smem();
+                    __syncwarp();
+                    if (split) {
+                        const int run = min(slice, 32);      // a warp's rows for one CTA
+                        if (to != rank && lane % run == 0)
+                            bulk_send(mapa_shared(inbox + (uint32_t)((half * kTileM + rank * slice + row % slice) * kPitch * 4), (uint32_t)to),
+                                      outbox + (uint32_t)(row * kPitch * 4), (uint32_t)(run * kPitch * 4), mapa_shared(sums_bar, (uint32_t)to));
                     }
-                    o[i] = pack2<kBf16>(x + rv.x, y + rv.y);
+                    if (lane == 0) mbar_arrive(sums_bar);
+                    ok = mbar_wait(sums_bar, 0, abort_flag, p.dev_status, 45);
+                    ok = __all_sync(0xFFFFFFFFu, ok);
                 }
-                *reinterpret_cast<uint4*>(L.Y + (size_t)row * L.out + col) = make_uint4(o[0], o[1], o[2], o[3]);
+                if (split) cluster_arrive();
+            }
+            if (ok) {
+#pragma unroll 1
+                for (int row_l = real ? tid / kUnits : slice - 1; row_l < slice; row_l += kRowsAStep) {
+                    const int row = m0 + rank * slice + row_l;
+                    if (real && row_l >= kRowsAStep && residual != nullptr && row < L.rows && col < L.out)
+                        rw = *reinterpret_cast<const uint4*>(residual + (size_t)row * L.out + col);
+                    float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+                    for (int s = 0; s < splits; ++s) {
+                        const float4* src = reinterpret_cast<const float4*>(sums + (size_t)(s * slice + row_l) * kPitch);
+                        const float4 x = src[0], y = src[1];
+                        a[0] += x.x; a[1] += x.y; a[2] += x.z; a[3] += x.w;
+                        a[4] += y.x; a[5] += y.y; a[6] += y.z; a[7] += y.w;
+                    }
+                    const uint32_t b[4] = {bw.x, bw.y, bw.z, bw.w}, r[4] = {rw.x, rw.y, rw.z, rw.w};
+                    uint32_t o[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float2 bv = raw2_to_float2<kBf16>(b[j]);
+                        a[2 * j] += bv.x;
+                        a[2 * j + 1] += bv.y;
+                    }
+                    if (L.act == 1) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const float2 g = gelu_pair(a[2 * j], a[2 * j + 1]);
+                            a[2 * j] = g.x;
+                            a[2 * j + 1] = g.y;
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float2 rv = raw2_to_float2<kBf16>(r[j]);
+                        o[j] = pack2<kBf16>(a[2 * j] + rv.x, a[2 * j + 1] + rv.y);
+                    }
+                    if (real && row < L.rows && col < L.out) *reinterpret_cast<uint4*>(L.Y + (size_t)row * L.out + col) = make_uint4(o[0], o[1], o[2], o[3]);
+                }
             }
         }
+        if (split) cluster_wait();
     }
 
     // ------------------------------------------------ teardown
@@ -401,8 +471,11 @@ elsa_status launch_small(const SmallJob* jobs, int n, int splits, bool early, ui
     g.splits = splits;
     g.stages = splits > 1 ? kStagesSplit : kStagesMax;
     g.early = early ? 1 : 0;
+    g.rehearse = 0;
     g.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(kTileN >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
     g.dev_status = dev_status;
+    g.ahead = n == 1 ? jobs[0].ahead : nullptr;
+    g.ahead_units = n == 1 ? (uint32_t)(jobs[0].ahead_bytes / 16) : 0;
 
     auto kernel = linear_small_kernel<kBf16, kMax>;
     constexpr int kSmemMost = small_smem(true) > small_smem(false) ? small_smem(true) : small_smem(false);
