@@ -1548,6 +1548,7 @@ namespace {
 
 struct BackwardPlan {
     size_t wmt, partial, sums, total;   // byte offsets of the regions
+    int parts;                          // rows of `out` floats in `partial`
 };
 
 // Upper bound, from host arithmetic alone, of the ranges the dW product may be cut into: what a device of 256 SMs
@@ -1567,8 +1568,10 @@ BackwardPlan backward_plan(int rows, int in, int out)
     p.wmt = at;     at += round_up((size_t)out * in * 2, 256);                      // transposed masked weight [in][out]
     const int bound = wgrad_splits_bound(in, out);
     int parts = (rows + 511) / 512;                                                 // parts of the column sums of dY:
-    if (parts < linear_tc_pair_tn_sums_parts(in, 1)) parts = linear_tc_pair_tn_sums_parts(in, 1);   // 512 rows each, or
-    if (parts < linear_tc_pair_tn_sums_parts(in, bound)) parts = linear_tc_pair_tn_sums_parts(in, bound);   // from dW's product
+    const int product = bound > 1 ? bound * ((in + 255) / 256) : 0;                 // 512 rows each, or from dW's product
+    if (parts < (in + 127) / 128) parts = (in + 127) / 128;
+    if (parts < product) parts = product;
+    p.parts = parts;
     p.partial = at; at += round_up((size_t)parts * out * 4, 256);
     // fp32 sums of dW per range of rows
     p.sums = at;    at += bound > 1 ? round_up((size_t)bound * out * in * 4, 256) : 0;
@@ -1637,15 +1640,15 @@ elsa_status elsa_nm_linear_backward(const void* dY, const void* X, int rows, con
     if (dW) {
         // dW = dY^T X, reduction over the token rows: both operands are read as they are stored (reduction index
         // outermost), then the mask
-        // when 256 x 256 tiles alone leave SM pairs idle, the rows are cut into ranges summed afterwards
-        int splits = linear_tc_pair_tn_splits(out, in, rows, dev.sm_count);
-        if (splits > wgrad_splits_bound(in, out)) splits = wgrad_splits_bound(in, out);
+        // when tiles alone leave SM pairs idle, the rows are cut into ranges summed afterwards
+        const TnShape shape = linear_tc_pair_tn_shape(out, in, rows, wgrad_splits_bound(in, out), dev.sm_count);
         float* sums = (float*)(ws + plan.sums);
-        if ((st = launch_linear_tc_pair_tn(dy, (const uint16_t*)X, out, in, rows, dtype, (uint16_t*)dW, splits, sums,
-                                           db ? db_sums : nullptr, &db_parts, dev_status, stream)) != ELSA_OK)
+        const bool db_here = db && linear_tc_pair_tn_sums_parts(in, shape) <= plan.parts;
+        if ((st = launch_linear_tc_pair_tn(dy, (const uint16_t*)X, out, in, rows, dtype, (uint16_t*)dW, shape, sums,
+                                           db_here ? db_sums : nullptr, &db_parts, dev_status, stream)) != ELSA_OK)
             return st;
-        if (splits > 1) {
-            st = launch_wgrad_finish(sums, splits, idx, out, in, N, M, dtype, (uint16_t*)dW, db_sums, db_parts, (uint16_t*)db, stream);
+        if (shape.splits > 1) {
+            st = launch_wgrad_finish(sums, shape.splits, idx, out, in, N, M, dtype, (uint16_t*)dW, db_sums, db_parts, (uint16_t*)db, stream);
             if (st != ELSA_OK || db_parts > 0) return st;
         } else if ((st = launch_mask_apply((uint16_t*)dW, idx, out, in, N, M, stream)) != ELSA_OK) {
             return st;

@@ -122,14 +122,17 @@ elsa_status launch_linear_tc_pair(const uint16_t* X, int rows, const uint16_t* W
                                   cudaStream_t stream);
 // Y [m][n] = A^T B on the same kernel with both operands stored reduction-outermost, A [k][m] and B [k][n]
 // (m, n multiples of 8): the weight-gradient product dY^T X without transposed copies.
-// With splits > 1 the reduction is cut into that many ranges whose fp32 sums go to partial [splits][m][n] (Y is then
-// not written); linear_tc_pair_tn_splits says how many ranges keep the SM pairs occupied.  Where sums_a is not NULL, there
-// are no more tiles than SM pairs and no part has too many rows for the running sums, *sums_parts rows of m floats that add
-// up to the sums of A over the reduction go there (at most linear_tc_pair_tn_sums_parts(n, splits)); else *sums_parts is 0.
-int linear_tc_pair_tn_splits(int m, int n, int k, int sm_count);
-int linear_tc_pair_tn_sums_parts(int n, int splits);
+// shape: columns of a tile (256 or 128) and ranges the reduction is cut into, by linear_tc_pair_tn_shape with at most
+// splits_most ranges; with several their fp32 sums go to partial [splits][m][n] (Y is then not written).  Where sums_a is not
+// NULL, there are no more tiles than SM pairs and no part has too many rows for the running sums, *sums_parts rows of m floats
+// that add up to the sums of A over the reduction go there (linear_tc_pair_tn_sums_parts(n, shape) of them); else *sums_parts is 0.
+struct TnShape {
+    int columns, splits;
+};
+TnShape linear_tc_pair_tn_shape(int m, int n, int k, int splits_most, int sm_count);
+int linear_tc_pair_tn_sums_parts(int n, const TnShape& shape);
 elsa_status launch_linear_tc_pair_tn(const uint16_t* A, const uint16_t* B, int m, int n, int k, elsa_dtype dtype,
-                                     uint16_t* Y, int splits, float* partial, float* sums_a, int* sums_parts,
+                                     uint16_t* Y, const TnShape& shape, float* partial, float* sums_a, int* sums_parts,
                                      uint32_t* dev_status, cudaStream_t stream);
 // Levels with N <= 2 on the hardware 2:4 sparse MMA: re-encodes the packed weight into `workspace`
 // (2-of-4 values + metadata), then runs the sparse GEMM.
@@ -272,6 +275,7 @@ struct PairJob {
     int act = 0;                          // epilogue activation: 0 none, 1 GELU (applied to acc + bias)
     const uint16_t* residual = nullptr;   // [rows][out], added after the activation, before the one rounding
     int splits = 1;                       // Tn form: ranges the reduction is cut into; > 1 writes fp32 sums to `partial`
+    int tn_columns = 256;                 // Tn form: columns of a tile
     float* partial = nullptr;             // [splits][rows][out]
     float* sums_a = nullptr;              // Tn form: see launch_linear_tc_pair_tn
     int* sums_parts = nullptr;

@@ -596,7 +596,7 @@ linear_tc_pair_kernel(const __grid_constant__ PairGroup<kMaxLayers> p)
 // its width plus a fixed share (operand staging, pipeline fill), and features past `out` in the last tile are
 // wasted work; among equals the widest wins (fewest re-reads of X).  For the large layers this picks 256 or
 // the width that divides `out`; below a wave of tiles it narrows the tile until the pairs are occupied.
-int pick_pair_block_n(int out, int rows, int sm_count, bool whole_boxes = false)
+int pick_pair_block_n(int out, int rows, int sm_count)
 {
     const int pairs = sm_count / 2 > 0 ? sm_count / 2 : 1;
     const long long row_tiles = (rows + kPairRows - 1) / kPairRows;
@@ -605,7 +605,6 @@ int pick_pair_block_n(int out, int rows, int sm_count, bool whole_boxes = false)
     const int cand[4] = {256, 192, 128, 64};
     for (int i = 0; i < 4; ++i) {
         const int bn = cand[i];
-        if (whole_boxes && bn % 128 != 0) continue;   // the Tn form loads each CTA's half in boxes of 64 features
         const long long tiles = row_tiles * ((out + bn - 1) / bn);
         const long long waves = (tiles + pairs - 1) / pairs;
         const long long cost = waves * (bn + 32);
@@ -682,7 +681,7 @@ elsa_status launch_group(const PairJob* jobs, int n, elsa_dtype dtype, uint32_t*
             if (i == 1) L.row_base = (int)widths.row_tiles * kPairRows;
             row_tiles = i == 0 ? (int)widths.row_tiles : row_tiles - (int)widths.row_tiles;
         } else {
-            L.bn = (kForm == kFormTn && j.splits > 1) ? 256 : pick_pair_block_n(j.out, j.rows, dev.sm_count, kForm == kFormTn);
+            L.bn = kForm == kFormTn ? j.tn_columns : pick_pair_block_n(j.out, j.rows, dev.sm_count);
         }
         L.tiles_n = (j.out + L.bn - 1) / L.bn;
         L.tile_begin = tile_begin;
@@ -820,27 +819,36 @@ elsa_status launch_linear_tc_pair_group(const PairJob* jobs, int n, elsa_dtype d
                               : launch_group<false, kFormPlain, kGroupMax>(jobs, n, dtype, dev_status, stream, dev);
 }
 
-// How many ranges the reduction of an m x n product is cut into: with 256 x 256 tiles, as many as keep one wave of
-// work units on the SM pairs (1 when the tiles alone fill them).
-int linear_tc_pair_tn_splits(int m, int n, int k, int sm_count)
+// Tile width and ranges of an m x n product's reduction: those with the least time for the busiest SM pair, in units of a column of
+// a K block.  A wave of tiles takes the K blocks of a range times what a tile loads for one, 32 KB at 256 columns and 24 at 128 (this
+// form waits for its loads: 192 columns, which load as much as 256, gained nothing in 36 x 2 tiles against 27 x 2 and lost 2 to 10 %
+// of a training block elsewhere); fp32 sums of ranges are written and read again, about 1000 of them in a unit's time.
+// Compress, forward and backward of a block, us, 256 columns in as many ranges as fit the pairs and like this: dim 192 at 25216 rows
+// 260 -> 229, dim 256 at 19700 rows 249 -> 233, dim 384 at 25216 rows 367 -> 356, dim 768 at 3152 rows 290-315 -> 236-258; 768 at 25216
+// rows chooses what it had.
+TnShape linear_tc_pair_tn_shape(int m, int n, int k, int splits_most, int sm_count)
 {
-    const int pairs = sm_count / 2 > 0 ? sm_count / 2 : 1;
-    const long long tiles = (long long)((m + kPairRows - 1) / kPairRows) * ((n + 255) / 256);
-    long long s = pairs / tiles;
-    const int k_blocks = (k + kBlockK - 1) / kBlockK;
-    if (s > 8) s = 8;
-    if (s > k_blocks) s = k_blocks;
-    return s < 1 ? 1 : (int)s;
+    const long long pairs = sm_count / 2 > 0 ? sm_count / 2 : 1;
+    const long long row_tiles = (m + kPairRows - 1) / kPairRows, k_blocks = (k + kBlockK - 1) / kBlockK;
+    TnShape best = {256, 1};
+    long long best_cost = -1;
+    for (int bn = 256; bn >= 128; bn -= 128) {
+        const long long tiles = row_tiles * ((n + bn - 1) / bn);
+        for (int s = 1; s <= splits_most && s <= k_blocks; ++s) {
+            const long long cost = (tiles * s + pairs - 1) / pairs * ((k_blocks + s - 1) / s) * (bn == 256 ? 288 : 216) + (s > 1 ? (long long)s * m * n / 1000 : 0);
+            if (best_cost < 0 || cost < best_cost) { best.columns = bn; best.splits = s; best_cost = cost; }
+        }
+    }
+    return best;
 }
 
-// The most parts the sums of A come in: one a range and tile column, tiles of 256 columns when the reduction is cut, of
-// 128 at least when it is not.
-int linear_tc_pair_tn_sums_parts(int n, int splits) { return splits > 1 ? splits * ((n + 255) / 256) : (n + 127) / 128; }
+// The most parts the sums of A come in: one a range and tile column.
+int linear_tc_pair_tn_sums_parts(int n, const TnShape& shape) { return shape.splits * ((n + shape.columns - 1) / shape.columns); }
 
 // Y [m][n] = A^T B with A [k][m] and B [k][n] (the reduction index outermost in both), no bias: one launch.
-// splits > 1: nothing is written to Y; partial [splits][m][n] receives the fp32 sums of each range of the reduction.
+// shape.splits > 1: nothing is written to Y; partial [splits][m][n] receives the fp32 sums of each range of the reduction.
 elsa_status launch_linear_tc_pair_tn(const uint16_t* A, const uint16_t* B, int m, int n, int k, elsa_dtype dtype,
-                                     uint16_t* Y, int splits, float* partial, float* sums_a, int* sums_parts,
+                                     uint16_t* Y, const TnShape& shape, float* partial, float* sums_a, int* sums_parts,
                                      uint32_t* dev_status, cudaStream_t stream)
 {
     DeviceInfo dev;
@@ -849,7 +857,8 @@ elsa_status launch_linear_tc_pair_tn(const uint16_t* A, const uint16_t* B, int m
     PairJob job;
     job.X = A; job.Wd = B; job.bias = nullptr; job.Y = Y;
     job.rows = m; job.in = k; job.out = n;
-    job.splits = splits < 1 ? 1 : splits;
+    job.splits = shape.splits;
+    job.tn_columns = shape.columns;
     job.partial = partial;
     job.sums_a = sums_a;
     job.sums_parts = sums_parts;
