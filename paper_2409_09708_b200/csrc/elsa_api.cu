@@ -1131,12 +1131,15 @@ elsa_status block_linear(BlockLinear& L, const uint16_t* X, int rows, elsa_dtype
         const bool early = !L.first && (L.kind == KIND_SMALL || w.N == w.M || ready);
         return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, dev.sm_count), early, dtype, dev_status, stream);
     }
-    *residual_left = residual != nullptr;
-    uint16_t* dst = residual ? tmp : Y;
+    // GELU and a residual never come together; where they did, or the kernel has no residual, the next row-wise kernel adds it
+    const bool adds = residual != nullptr && act == 0 && (L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST);
+    *residual_left = residual != nullptr && !adds;
+    uint16_t* dst = *residual_left ? tmp : Y;
     if (L.kind == KIND_SPARSE_WS || L.kind == KIND_SPARSE_ST || (L.kind == KIND_SPARSE_PAIR && act == 0)) {
         if ((st = block_images(&L, 1, stream)) != ELSA_OK) return st;
         SparseJob job = sparse_job(L.kind, X, rows, w.vals, w.idx, w.bias, L.out, L.in, w.N, w.M, dst, L.ws);
         job.act = act;
+        if (adds) job.residual = residual;
         return L.kind == KIND_SPARSE_WS   ? launch_linear_tc_sparse_ws_group(&job, 1, dtype, dev_status, stream)
                : L.kind == KIND_SPARSE_ST ? launch_linear_tc_sparse_st_group(&job, 1, dtype, dev_status, stream)
                                           : launch_linear_tc_sparse_pair_group(&job, 1, dtype, dev_status, stream);

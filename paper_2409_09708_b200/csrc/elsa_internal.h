@@ -183,6 +183,8 @@ struct SparseJob {
     const uint16_t* w = nullptr;
     const uint32_t* idx = nullptr;
     int N = 0, M = 0;
+    // weight-stationary and streaming kernels, without an activation: [rows][out] added before the one rounding
+    const uint16_t* residual = nullptr;
 };
 int linear_tc_sparse_pair_group_max();
 elsa_status launch_linear_tc_sparse_pair_prepare(const uint16_t* vals, const uint32_t* idx, int out, int in, int N, int M,

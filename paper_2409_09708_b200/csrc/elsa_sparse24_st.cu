@@ -57,8 +57,9 @@ constexpr int kStepsPerWarp = kMaxRowTile / kStepCols / kEpiParts;   // 7 at mos
 constexpr int kRoundSteps = 4;     // steps an epilogue warp holds in registers at a time
 constexpr int kRounds = (kStepsPerWarp + kRoundSteps - 1) / kRoundSteps;
 constexpr int kStageBytes = (kChunkK / 64) * (kMaxRowTile / 2) * 128;   // 56 KB: four quarters of 112 rows x 128 bytes
-constexpr int kStagingBytes = 2 * kStepCols * 64;                 // per epilogue warp: two buffers of 16 rows x 32 features
-constexpr int kStagingTotal = kEpiWarps * kStagingBytes;
+// Per epilogue warp: two buffers of 16 rows x 32 features, or with a residual one for every step.
+template <int kEpi>
+constexpr int kStagingOf = (kEpi == kEpiResidual ? kStepsPerWarp : 2) * kStepCols * 64;
 constexpr int kBarrierBytes = 512;
 
 static_assert(kMaxRowTile + kSlots * kSlotCols <= kTmemCols, "accumulator and weight slots fit tensor memory");
@@ -83,22 +84,25 @@ struct alignas(64) StLayer {
 constexpr int kGroupMax = 84;   // layers per launch (kernel parameters are limited to 32 KB)
 
 template <int kMaxLayers>
-struct StGroup {
+struct alignas(64) StGroup {
     StLayer layer[kMaxLayers];
     int n_layers;
     int num_tiles;
     int nt;            // token rows per tile, a multiple of 16
     uint32_t idesc;
     uint32_t* dev_status;
+    CUtensorMap map_r; // kEpiResidual: the residual, boxes as map_y's
 };
 
 // (22 warps are allocated as 24: 80 registers per thread is what the register file allows, and a loader warp
 // holds a whole chunk, 72 of them, between its loads and its tensor-memory stores)
-// kAct: the instantiation whose epilogue applies the layer's activation (single-layer launches).
-template <bool kBf16, int kMaxLayers, bool kAct>
+// kEpi: as in elsa_sparse24_ws.cu; a tile's residual is asked for when the tile before it has been stored.
+template <bool kBf16, int kMaxLayers, int kEpi>
 __global__ void __launch_bounds__(kThreads, 1)
 linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
 {
+    constexpr bool kAct = kEpi == kEpiGelu, kRes = kEpi == kEpiResidual;
+    constexpr int kStagingBytes = kStagingOf<kEpi>, kStagingTotal = kEpiWarps * kStagingBytes;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -118,7 +122,8 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
     const uint32_t a_empty_bar = a_full_bar + 8 * kSlots;        // per CTA: the MMAs that read a slot are done
     const uint32_t tmem_full_bar = a_empty_bar + 8 * kSlots;     // per CTA
     const uint32_t tmem_empty_bar = tmem_full_bar + 8;           // leader only
-    const uint32_t holder_off = bar_off + 16 * kStages + 16 * kSlots + 16;
+    const uint32_t res_bar = tmem_empty_bar + 8;                 // kEpiResidual: one per epilogue warp
+    const uint32_t holder_off = bar_off + 16 * kStages + 16 * kSlots + 16 + 8 * kEpiWarps;
     volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(smem_gen + holder_off);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem_gen + holder_off + 4);
 
@@ -133,6 +138,8 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
         }
         mbar_init(tmem_full_bar, 1);
         mbar_init(tmem_empty_bar, 2 * kEpiWarps);
+        if constexpr (kRes)
+            for (int w = 0; w < kEpiWarps; ++w) mbar_init(res_bar + 8 * w, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
@@ -333,6 +340,9 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
         const int steps = p.nt / kStepCols;
         const int first_step = part == 0 ? 0 : (steps + 1) >> 1, my_steps = part == 0 ? (steps + 1) >> 1 : steps >> 1;
         uint32_t store_count = 0;
+        uint32_t res_phase = 0;
+        (void)store_count;
+        (void)res_phase;
 
         int cur = 0;
         for (int tile = pair; tile < p.num_tiles; tile += num_pairs) {
@@ -347,6 +357,18 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
             const uint64_t bias2 = f32x2(bias_f, bias_f);
             const int l_act = kAct ? L.act : 0;
             (void)l_act;
+            const bool has_res = kRes && f0 < l_out && row0 < l_rows;
+            (void)has_res;
+            if constexpr (kRes) {
+                if (has_res && lane == 0) {
+                    bulk_wait_group_read<0>();          // the stores of the previous tile have drained the buffers
+                    const int last = l_rows - row0 < my_steps * kStepCols ? (l_rows - row0 + kStepCols - 1) / kStepCols : my_steps;
+                    mbar_arrive_expect_tx(res_bar + 8 * (warp - 2), (uint32_t)(last * kStepCols * 64));
+                    for (int s = 0; s < last; ++s)
+                        tma_load_2d(buf0 + (uint32_t)(s * kStepCols * 64), &p.map_r, res_bar + 8 * (warp - 2), f0, row0 + s * kStepCols);
+                }
+                __syncwarp();
+            }
             bool ok = mbar_wait(tmem_full_bar, acc_phase, abort_flag, p.dev_status, 4);
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
@@ -357,9 +379,11 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
             // Staging: rows of 32 features (64 bytes, no swizzle), two buffers of one step per warp.
             uint32_t rr[kRoundSteps][16];
             auto store_step = [&](int s, const uint32_t (&w)[8]) {
-                const uint32_t buf = buf0 + (store_count & 1u) * (uint32_t)(kStepCols * 64);
-                if (lane == 0) bulk_wait_group_read<1>();   // the store two steps ago has drained this buffer
-                __syncwarp();
+                const uint32_t buf = buf0 + (kRes ? (uint32_t)s : store_count & 1u) * (uint32_t)(kStepCols * 64);
+                if constexpr (!kRes) {
+                    if (lane == 0) bulk_wait_group_read<1>();   // the store two steps ago has drained this buffer
+                    __syncwarp();
+                }
                 stmatrix_x4_trans(buf + st_off, w[0], w[1], w[2], w[3]);
                 stmatrix_x4_trans(buf + st_off + 512, w[4], w[5], w[6], w[7]);
                 fence_proxy_async_smem();
@@ -374,14 +398,33 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
             for (int i = 0; i < kRoundSteps; ++i)
                 tmem_ld_32x32b_x16(t_col + (uint32_t)(i * kStepCols), rr[i]);
             tmem_wait_ld();
+            if constexpr (kRes) {
+                if (has_res) {
+                    ok = mbar_wait(res_bar + 8 * (warp - 2), res_phase, abort_flag, p.dev_status, 9);
+                    ok = __all_sync(0xFFFFFFFFu, ok);
+                    if (!ok) break;
+                    res_phase ^= 1u;
+                }
+            }
 #pragma unroll
             for (int rd = 0; rd < kRounds; ++rd) {
                 uint32_t w[kRoundSteps][8];
 #pragma unroll
-                for (int i = 0; i < kRoundSteps; ++i)
+                for (int i = 0; i < kRoundSteps; ++i) {
+                    if constexpr (kRes) {
+                        const int s = rd * kRoundSteps + i;
+                        if (s >= kStepsPerWarp) continue;
+                        const uint32_t at = buf0 + st_off + (uint32_t)(s * kStepCols * 64);
+                        ldmatrix_x4_trans(at, w[i][0], w[i][1], w[i][2], w[i][3]);
+                        ldmatrix_x4_trans(at + 512, w[i][4], w[i][5], w[i][6], w[i][7]);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        w[i][j] = finish_pair<kBf16, kAct>(rr[i][2 * j], rr[i][2 * j + 1], bias2, l_act);
+                        for (int j = 0; j < 8; ++j) w[i][j] = finish_pair_residual<kBf16>(rr[i][2 * j], rr[i][2 * j + 1], bias2, w[i][j]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            w[i][j] = finish_pair<kBf16, kAct>(rr[i][2 * j], rr[i][2 * j + 1], bias2, l_act);
+                    }
+                }
                 if (rd + 1 < kRounds) {
 #pragma unroll
                     for (int i = 0; i < kRoundSteps; ++i)
@@ -437,12 +480,12 @@ int pick_row_tile(const SparseJob* jobs, int n, int pairs)
     return best;
 }
 
-template <bool kBf16, int kMaxLayers, bool kAct>
+template <bool kBf16, int kMaxLayers, int kEpi>
 elsa_status launch_st_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint32_t* dev_status, cudaStream_t stream,
                             const DeviceInfo& dev)
 {
-    auto kernel = linear_tc_sp24_st_kernel<kBf16, kMaxLayers, kAct>;
-    const size_t smem = (size_t)kStages * kStageBytes + kStagingTotal + kBarrierBytes + 1024;
+    auto kernel = linear_tc_sp24_st_kernel<kBf16, kMaxLayers, kEpi>;
+    const size_t smem = (size_t)kStages * kStageBytes + kEpiWarps * kStagingOf<kEpi> + kBarrierBytes + 1024;
     if (smem > dev.smem_optin) return fail(ELSA_ERR_CUDA, "not enough shared memory for the streaming sparse kernel");
 
     static std::atomic<int> max_pairs[64];   // zero-initialised; racing first calls compute the same value
@@ -497,6 +540,11 @@ elsa_status launch_st_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
                               "Y")) != ELSA_OK)
             return st;
     }
+    if (kEpi == kEpiResidual) {
+        const elsa_status st = make_map_2d(&g.map_r, jobs[0].residual, (uint64_t)jobs[0].out, (uint64_t)jobs[0].rows, 32, kStepCols,
+                                           CU_TENSOR_MAP_SWIZZLE_NONE, "the residual");
+        if (st != ELSA_OK) return st;
+    }
     g.n_layers = n;
     g.num_tiles = tile_begin;
     g.nt = nt;
@@ -529,22 +577,27 @@ elsa_status launch_linear_tc_sparse_st_group(const SparseJob* jobs, int n, elsa_
     elsa_status st = device_info(&dev);
     if (st != ELSA_OK) return st;
     if (n < 1 || n > kGroupMax) return fail(ELSA_ERR_SHAPE, "a grouped launch carries 1 to %d layers, got %d", kGroupMax, n);
-    bool act = false;
-    for (int i = 0; i < n; ++i) act = act || jobs[i].act != 0;
-    if (act) {
-        // layers with an activation in the epilogue run one per launch, on the instantiation that has it
+    bool alone = false;
+    for (int i = 0; i < n; ++i) alone = alone || jobs[i].act != 0 || jobs[i].residual != nullptr;
+    if (alone) {
+        // layers with an activation or a residual in the epilogue run one per launch, on the instantiation that has it
         for (int i = 0; i < n; ++i) {
-            st = dtype == ELSA_BF16 ? launch_st_group<true, 1, true>(jobs + i, 1, dtype, dev_status, stream, dev)
-                                    : launch_st_group<false, 1, true>(jobs + i, 1, dtype, dev_status, stream, dev);
+            if (jobs[i].act != 0 && jobs[i].residual != nullptr) return fail(ELSA_ERR_SHAPE, "an activation and a residual in one epilogue of this kernel");
+            if (jobs[i].residual != nullptr)
+                st = dtype == ELSA_BF16 ? launch_st_group<true, 1, kEpiResidual>(jobs + i, 1, dtype, dev_status, stream, dev)
+                                        : launch_st_group<false, 1, kEpiResidual>(jobs + i, 1, dtype, dev_status, stream, dev);
+            else
+                st = dtype == ELSA_BF16 ? launch_st_group<true, 1, kEpiGelu>(jobs + i, 1, dtype, dev_status, stream, dev)
+                                        : launch_st_group<false, 1, kEpiGelu>(jobs + i, 1, dtype, dev_status, stream, dev);
             if (st != ELSA_OK) return st;
         }
         return ELSA_OK;
     }
     if (n == 1)
-        return dtype == ELSA_BF16 ? launch_st_group<true, 1, false>(jobs, 1, dtype, dev_status, stream, dev)
-                                  : launch_st_group<false, 1, false>(jobs, 1, dtype, dev_status, stream, dev);
-    return dtype == ELSA_BF16 ? launch_st_group<true, kGroupMax, false>(jobs, n, dtype, dev_status, stream, dev)
-                              : launch_st_group<false, kGroupMax, false>(jobs, n, dtype, dev_status, stream, dev);
+        return dtype == ELSA_BF16 ? launch_st_group<true, 1, kEpiPlain>(jobs, 1, dtype, dev_status, stream, dev)
+                                  : launch_st_group<false, 1, kEpiPlain>(jobs, 1, dtype, dev_status, stream, dev);
+    return dtype == ELSA_BF16 ? launch_st_group<true, kGroupMax, kEpiPlain>(jobs, n, dtype, dev_status, stream, dev)
+                              : launch_st_group<false, kGroupMax, kEpiPlain>(jobs, n, dtype, dev_status, stream, dev);
 }
 
 elsa_status launch_linear_tc_sparse_st(const uint16_t* X, int rows, const uint16_t* vals, const uint32_t* idx,

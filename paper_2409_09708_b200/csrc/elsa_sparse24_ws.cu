@@ -88,12 +88,13 @@ struct alignas(64) WsLayer {
 constexpr int kGroupMax = 68;   // layers per launch (kernel parameters are limited to 32 KB)
 
 template <int kMaxLayers>
-struct WsGroup {
+struct alignas(64) WsGroup {
     WsLayer layer[kMaxLayers];
     int n_layers;
     int stages;
     int stage_bytes;   // one pipeline stage: kStageK / 64 quarters of (largest nt / 2) rows of 128 bytes
     uint32_t* dev_status;
+    CUtensorMap map_r; // kEpiResidual: the residual, boxes as map_y's
 };
 
 // 128 k of a row of the packed weight: whole words of values and, but for half a word at 1:8, of index fields.
@@ -170,11 +171,15 @@ __device__ __forceinline__ void write_packed(const uint16_t* vals_row, const uin
     }
 }
 
-// kAct: the instantiation whose epilogue applies the layer's activation (single-layer launches).
-template <bool kBf16, int kMaxLayers, bool kAct>
+// kEpi: kEpiGelu, the instantiation whose epilogue applies the layer's activation, and kEpiResidual, which adds a residual, are for
+// single-layer launches.  The residual comes by TMA into the staging buffer, in the rows that the result leaves by, while the tile is
+// multiplied, and ldmatrix brings it to the lanes the way stmatrix takes the result back: as a pass of its own over four
+// tensors it cost a LayerNorm 64 us where the plain one takes 34 (50432 rows of 768).
+template <bool kBf16, int kMaxLayers, int kEpi>
 __global__ void __launch_bounds__(kThreads, 1)
 linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
 {
+    constexpr bool kAct = kEpi == kEpiGelu, kRes = kEpi == kEpiResidual;
     constexpr bool kRuns = kAct || kMaxLayers > 1;      // how the rows leave, see the epilogue
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -194,7 +199,8 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
     const uint32_t tmem_empty_bar = tmem_full_bar + 8 * kNumAccum;    // leader only
     const uint32_t w_ready_bar = tmem_empty_bar + 8 * kNumAccum;      // leader only
     const uint32_t layer_bar = w_ready_bar + 8;                       // per CTA: epilogue warps between layers
-    const uint32_t holder_off = bar_off + 16 * kMaxStages + 16 * kNumAccum + 16;
+    const uint32_t res_bar = layer_bar + 8;                           // kEpiResidual: one per epilogue warp
+    const uint32_t holder_off = bar_off + 16 * kMaxStages + 16 * kNumAccum + 16 + 8 * kEpiWarps;
     volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(smem_gen + holder_off);
     volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(smem_gen + holder_off + 4);
 
@@ -209,6 +215,8 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
         }
         mbar_init(w_ready_bar, 2 * kEpiWarps);
         mbar_init(layer_bar, kEpiWarps);
+        if constexpr (kRes)
+            for (int w = 0; w < kEpiWarps; ++w) mbar_init(res_bar + 8 * w, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
@@ -343,6 +351,8 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
         int acc = 0;
         uint32_t acc_phase = 0;
         uint32_t layer_phase = 0;
+        uint32_t res_phase = 0;
+        (void)res_phase;
         const uint32_t buf = staging_base + (uint32_t)((warp - 2) * kStagingBytes);
         // Lane t holds feature 8 * (t % 4) + t / 4 of the quarter's 32.  The staging buffer is rows of 32
         // features (64 bytes, no swizzle); one stmatrix.x4.trans writes 8 token rows: lane t gives the
@@ -442,6 +452,18 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
 
             for (int r = g; r < L.row_tiles; r += L.groups) {
                 const int row0 = r * nt + first_step * kStepCols;
+                const bool has_res = kRes && f0 < l_out && my_steps > 0 && row0 < l_rows;
+                (void)has_res;
+                if constexpr (kRes) {
+                    if (has_res && lane == 0) {
+                        bulk_wait_group_read<0>();          // the stores of the previous tile have drained the buffer
+                        const int last = l_rows - row0 < my_steps * kStepCols ? (l_rows - row0 + kStepCols - 1) / kStepCols : my_steps;
+                        mbar_arrive_expect_tx(res_bar + 8 * (warp - 2), (uint32_t)(last * kStepCols * 64));
+                        for (int s = 0; s < last; ++s)
+                            tma_load_2d(buf + (uint32_t)(s * kStepCols * 64), &p.map_r, res_bar + 8 * (warp - 2), f0, row0 + s * kStepCols);
+                    }
+                    __syncwarp();
+                }
                 ok = mbar_wait(tmem_full_bar + 8 * acc, acc_phase, abort_flag, p.dev_status, 4);
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
@@ -461,13 +483,29 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
                     bulk_wait_group_read<0>();   // the stores of the previous tile have drained the buffer
                 }
                 __syncwarp();
+                if constexpr (kRes) {
+                    if (has_res) {
+                        ok = mbar_wait(res_bar + 8 * (warp - 2), res_phase, abort_flag, p.dev_status, 9);
+                        ok = __all_sync(0xFFFFFFFFu, ok);
+                        if (!ok) break;
+                        res_phase ^= 1u;
+                    }
+                }
 #pragma unroll
                 for (int s = 0; s < kMaxSteps; ++s) {
                     if (s >= my_steps) continue;
                     uint32_t w[8];
+                    if constexpr (kRes) {
+                        // (of a step past the last row, or features past the last one, what the buffer held; nothing of it is stored)
+                        ldmatrix_x4_trans(st_addr + (uint32_t)(s * kStepCols * 64), w[0], w[1], w[2], w[3]);
+                        ldmatrix_x4_trans(st_addr + (uint32_t)(s * kStepCols * 64 + 512), w[4], w[5], w[6], w[7]);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        w[j] = finish_pair<kBf16, kAct>(rr[s][2 * j], rr[s][2 * j + 1], bias2, l_act);
+                        for (int j = 0; j < 8; ++j) w[j] = finish_pair_residual<kBf16>(rr[s][2 * j], rr[s][2 * j + 1], bias2, w[j]);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            w[j] = finish_pair<kBf16, kAct>(rr[s][2 * j], rr[s][2 * j + 1], bias2, l_act);
+                    }
                     stmatrix_x4_trans(st_addr + (uint32_t)(s * kStepCols * 64), w[0], w[1], w[2], w[3]);
                     stmatrix_x4_trans(st_addr + (uint32_t)(s * kStepCols * 64 + 512), w[4], w[5], w[6], w[7]);
                 }
@@ -520,12 +558,12 @@ int ws_row_tile(int in)
     return nt >= 64 ? nt : 0;
 }
 
-template <bool kBf16, int kMaxLayers, bool kAct>
+template <bool kBf16, int kMaxLayers, int kEpi>
 elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint32_t* dev_status, cudaStream_t stream,
                             const DeviceInfo& dev)
 {
-    constexpr bool kRuns = kAct || kMaxLayers > 1;
-    auto kernel = linear_tc_sp24_ws_kernel<kBf16, kMaxLayers, kAct>;
+    constexpr bool kRuns = kEpi == kEpiGelu || kMaxLayers > 1;
+    auto kernel = linear_tc_sp24_ws_kernel<kBf16, kMaxLayers, kEpi>;
     const int fixed = kStagingTotal + kBarrierBytes + 1024;
     int max_nt = 0;
     for (int i = 0; i < n; ++i) {
@@ -612,6 +650,11 @@ elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
                                        CU_TENSOR_MAP_SWIZZLE_NONE, "Y")) != ELSA_OK)
             return st;
     }
+    if (kEpi == kEpiResidual) {
+        const elsa_status st = make_map_2d(&g.map_r, jobs[0].residual, (uint64_t)jobs[0].out, (uint64_t)jobs[0].rows, 32, kStepCols,
+                                           CU_TENSOR_MAP_SWIZZLE_NONE, "the residual");
+        if (st != ELSA_OK) return st;
+    }
     g.n_layers = n;
     g.stages = stages;
     g.stage_bytes = stage_bytes;
@@ -643,22 +686,27 @@ elsa_status launch_linear_tc_sparse_ws_group(const SparseJob* jobs, int n, elsa_
     elsa_status st = device_info(&dev);
     if (st != ELSA_OK) return st;
     if (n < 1 || n > kGroupMax) return fail(ELSA_ERR_SHAPE, "a grouped launch carries 1 to %d layers, got %d", kGroupMax, n);
-    bool act = false;
-    for (int i = 0; i < n; ++i) act = act || jobs[i].act != 0;
-    if (act) {
-        // layers with an activation in the epilogue run one per launch, on the instantiation that has it
+    bool alone = false;
+    for (int i = 0; i < n; ++i) alone = alone || jobs[i].act != 0 || jobs[i].residual != nullptr;
+    if (alone) {
+        // layers with an activation or a residual in the epilogue run one per launch, on the instantiation that has it
         for (int i = 0; i < n; ++i) {
-            st = dtype == ELSA_BF16 ? launch_ws_group<true, 1, true>(jobs + i, 1, dtype, dev_status, stream, dev)
-                                    : launch_ws_group<false, 1, true>(jobs + i, 1, dtype, dev_status, stream, dev);
+            if (jobs[i].act != 0 && jobs[i].residual != nullptr) return fail(ELSA_ERR_SHAPE, "an activation and a residual in one epilogue of this kernel");
+            if (jobs[i].residual != nullptr)
+                st = dtype == ELSA_BF16 ? launch_ws_group<true, 1, kEpiResidual>(jobs + i, 1, dtype, dev_status, stream, dev)
+                                        : launch_ws_group<false, 1, kEpiResidual>(jobs + i, 1, dtype, dev_status, stream, dev);
+            else
+                st = dtype == ELSA_BF16 ? launch_ws_group<true, 1, kEpiGelu>(jobs + i, 1, dtype, dev_status, stream, dev)
+                                        : launch_ws_group<false, 1, kEpiGelu>(jobs + i, 1, dtype, dev_status, stream, dev);
             if (st != ELSA_OK) return st;
         }
         return ELSA_OK;
     }
     if (n == 1)
-        return dtype == ELSA_BF16 ? launch_ws_group<true, 1, false>(jobs, 1, dtype, dev_status, stream, dev)
-                                  : launch_ws_group<false, 1, false>(jobs, 1, dtype, dev_status, stream, dev);
-    return dtype == ELSA_BF16 ? launch_ws_group<true, kGroupMax, false>(jobs, n, dtype, dev_status, stream, dev)
-                              : launch_ws_group<false, kGroupMax, false>(jobs, n, dtype, dev_status, stream, dev);
+        return dtype == ELSA_BF16 ? launch_ws_group<true, 1, kEpiPlain>(jobs, 1, dtype, dev_status, stream, dev)
+                                  : launch_ws_group<false, 1, kEpiPlain>(jobs, 1, dtype, dev_status, stream, dev);
+    return dtype == ELSA_BF16 ? launch_ws_group<true, kGroupMax, kEpiPlain>(jobs, n, dtype, dev_status, stream, dev)
+                              : launch_ws_group<false, kGroupMax, kEpiPlain>(jobs, n, dtype, dev_status, stream, dev);
 }
 
 }  // namespace elsa

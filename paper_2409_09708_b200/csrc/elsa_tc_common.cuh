@@ -296,6 +296,18 @@ __device__ __forceinline__ uint32_t finish_pair(uint32_t a, uint32_t b, uint64_t
     return pack2<kBf16>(v.x, v.y);
 }
 
+// Epilogues of the transposing kernels: acc + bias, GELU of it, or a residual added to it.
+constexpr int kEpiPlain = 0, kEpiGelu = 1, kEpiResidual = 2;
+
+// Two accumulators + bias + two values of the residual, rounded once.
+template <bool kBf16>
+__device__ __forceinline__ uint32_t finish_pair_residual(uint32_t a, uint32_t b, uint64_t bias2, uint32_t res)
+{
+    const float2 r = raw2_to_float2<kBf16>(res);
+    const float2 v = f32x2_split(f32x2_add(f32x2_add(f32x2(__uint_as_float(a), __uint_as_float(b)), bias2), f32x2(r.x, r.y)));
+    return pack2<kBf16>(v.x, v.y);
+}
+
 template <bool kBf16>
 __device__ __forceinline__ float bias_to_float(uint16_t u)
 {
@@ -526,6 +538,13 @@ __device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t r0, ui
     asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r0), "r"(r1),
                  "r"(r2), "r"(r3)
                  : "memory");
+}
+
+// The way back: what stmatrix_x4_trans wrote from these addresses, in the same registers.
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr) : "memory");
 }
 
 // Lane i of the warp writes 16 / 4 consecutive columns of TMEM lane (lane base + i).
