@@ -558,6 +558,23 @@ int ws_row_tile(int in)
     return nt >= 64 ? nt : 0;
 }
 
+// Row tile of a layer whose rows `groups` row groups share: the busiest group takes its tiles one after the other, each in a time
+// that goes with its rows and a fixed share, so narrower tiles pay where the widest leave a group's last one to few of the groups.
+// Us with the widest and with the choice: 5319 x 512 -> 1536 at 2:8 11.5, 11.1; 3940 x 384 -> 1152 at 1:8 8.4, 8.1; 9000 x 768 -> 768
+// at 1:8 10.5, 10.3; 3152 x 768 -> 2304 and larger launches the same.
+int ws_layer_row_tile(int in, int rows, int groups)
+{
+    const int most = ws_row_tile(in);
+    int best = most;
+    long long best_cost = -1;
+    for (int nt = most; nt >= 64; nt -= kStepCols) {
+        const long long tiles = (rows + nt - 1) / nt;
+        const long long cost = (tiles + groups - 1) / groups * (nt + 32);
+        if (best_cost < 0 || cost < best_cost) { best = nt; best_cost = cost; }
+    }
+    return best;
+}
+
 template <bool kBf16, int kMaxLayers, int kEpi>
 elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint32_t* dev_status, cudaStream_t stream,
                             const DeviceInfo& dev)
@@ -615,10 +632,10 @@ elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
     for (int i = 0; i < n; ++i) {
         const SparseJob& j = jobs[i];
         WsLayer& L = g.layer[i];
-        L.nt = ws_row_tile(j.in);
         L.tiles_f = (j.out + kPairFeat - 1) / kPairFeat;
-        if (L.nt == 0 || j.in % kBlockK != 0 || L.tiles_f > pairs)
+        if (ws_row_tile(j.in) == 0 || j.in % kBlockK != 0 || L.tiles_f > pairs)
             return fail(ELSA_ERR_SHAPE, "in=%d out=%d does not fit the weight-stationary sparse kernel", j.in, j.out);
+        L.nt = ws_layer_row_tile(j.in, j.rows, pairs / L.tiles_f);
         L.rows = j.rows; L.out = j.out; L.in = j.in;
         L.steps_per_warp = (uint8_t)((L.nt / kStepCols + kEpiParts - 1) / kEpiParts);
         L.row_tiles = (j.rows + L.nt - 1) / L.nt;
