@@ -823,10 +823,10 @@ elsa_status launch_linear_tc_pair_group(const PairJob* jobs, int n, elsa_dtype d
 // a K block.  A wave of tiles takes the K blocks of a range times what a tile loads for one, 32 KB at 256 columns and 24 at 128 (this
 // form waits for its loads: 192 columns, which load as much as 256, gained nothing in 36 x 2 tiles against 27 x 2 and lost 2 to 10 %
 // of a training block elsewhere); fp32 sums of ranges are written and read again, about 1000 of them in a unit's time.
-// Compress, forward and backward of a block, us, 256 columns in as many ranges as fit the pairs and like this: dim 192 at 25216 rows
-// 260 -> 229, dim 256 at 19700 rows 249 -> 233, dim 384 at 25216 rows 367 -> 356, dim 768 at 3152 rows 290-315 -> 236-258; 768 at 25216
-// rows chooses what it had.
-TnShape linear_tc_pair_tn_shape(int m, int n, int k, int splits_most, int sm_count)
+// Compress, forward and backward of a block, us, 256 columns in as many ranges as fit the pairs and like this: dim 192, 25216 rows
+// 259 -> 228, 1576 rows 134 -> 124 (138 with sums of A that found no room); dim 256, 19700 rows 249 -> 225; dim 384, 3152 rows
+// 176 -> 156; dim 512, 985 rows 156 -> 132; dim 768, 3152 rows 249 -> 231; 768 at 25216 rows chooses what it had.
+TnShape linear_tc_pair_tn_shape(int m, int n, int k, int splits_most, int parts_most, int sm_count)
 {
     const long long pairs = sm_count / 2 > 0 ? sm_count / 2 : 1;
     const long long row_tiles = (m + kPairRows - 1) / kPairRows, k_blocks = (k + kBlockK - 1) / kBlockK;
@@ -835,6 +835,8 @@ TnShape linear_tc_pair_tn_shape(int m, int n, int k, int splits_most, int sm_cou
     for (int bn = 256; bn >= 128; bn -= 128) {
         const long long tiles = row_tiles * ((n + bn - 1) / bn);
         for (int s = 1; s <= splits_most && s <= k_blocks; ++s) {
+            // more sums of A than there is room for would be a pass of their own, two launches more
+            if (bn < 256 && s * ((n + bn - 1) / bn) > parts_most) break;
             const long long cost = (tiles * s + pairs - 1) / pairs * ((k_blocks + s - 1) / s) * (bn == 256 ? 288 : 216) + (s > 1 ? (long long)s * m * n / 1000 : 0);
             if (best_cost < 0 || cost < best_cost) { best.columns = bn; best.splits = s; best_cost = cost; }
         }
