@@ -360,12 +360,16 @@ linear_tc_sp24_st_kernel(const __grid_constant__ StGroup<kMaxLayers> p)
             const bool has_res = kRes && f0 < l_out && row0 < l_rows;
             (void)has_res;
             if constexpr (kRes) {
-                if (has_res && lane == 0) {
-                    bulk_wait_group_read<0>();          // the stores of the previous tile have drained the buffers
-                    const int last = l_rows - row0 < my_steps * kStepCols ? (l_rows - row0 + kStepCols - 1) / kStepCols : my_steps;
-                    mbar_arrive_expect_tx(res_bar + 8 * (warp - 2), (uint32_t)(last * kStepCols * 64));
-                    for (int s = 0; s < last; ++s)
-                        tma_load_2d(buf0 + (uint32_t)(s * kStepCols * 64), &p.map_r, res_bar + 8 * (warp - 2), f0, row0 + s * kStepCols);
+                // All buffers are written below, those of a warp without rows or features in this tile too (it stores nothing of
+                // them): the stores of the previous tile drain them first.
+                if (lane == 0) {
+                    bulk_wait_group_read<0>();
+                    if (has_res) {
+                        const int last = l_rows - row0 < my_steps * kStepCols ? (l_rows - row0 + kStepCols - 1) / kStepCols : my_steps;
+                        mbar_arrive_expect_tx(res_bar + 8 * (warp - 2), (uint32_t)(last * kStepCols * 64));
+                        for (int s = 0; s < last; ++s)
+                            tma_load_2d(buf0 + (uint32_t)(s * kStepCols * 64), &p.map_r, res_bar + 8 * (warp - 2), f0, row0 + s * kStepCols);
+                    }
                 }
                 __syncwarp();
             }

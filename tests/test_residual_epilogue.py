@@ -41,3 +41,15 @@ def test_exact_block(kernel, dim, mlp, rows, dtype):
     assert torch.equal(lib.block_region(scratch, off, "x2", rows, dim, dtype), x2)
     assert torch.equal(guard[:rows], y)
     assert bool((guard[rows:] == 7.0).all())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16], ids=["bf16", "f16"])
+@pytest.mark.parametrize("kernel", ["WS", "ST"])
+@pytest.mark.parametrize("rows,dim,mlp", [(25000, 256, 512), (5400, 640, 256), (18600, 128, 384)])
+def test_several_tiles_a_pair(rows, dim, mlp, kernel, dtype):
+    """A pair takes a second tile in which some of its warps have no rows (25000: the last of 143 tiles of 176 rows has 8) or no features
+    (640: the third block of 256 has 128), while the stores of the first one still read the staging rows.  Three times over: nothing but
+    an order of reads and writes can go wrong, and that need not show at once."""
+    for _ in range(3):
+        test_exact_block(kernel, dim, mlp, rows, dtype)
