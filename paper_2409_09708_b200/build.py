@@ -28,6 +28,10 @@ def nvcc_path() -> str:
     raise RuntimeError("nvcc not found")
 
 
+def cuda_include() -> str:
+    return os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc_path()))), "include")
+
+
 def sources() -> list[str]:
     return [os.path.join(CSRC, s) for s in SOURCES]
 
@@ -59,8 +63,8 @@ def build_host(force: bool = False) -> str:
     include = os.path.join(torch, "include")
     cmd = [os.environ.get("CXX") or "g++", "-O2", "-std=c++17", "-shared", "-fPIC", '-DELSA_TORCH_VERSION="%s"' % version,
            "-I", os.path.join(ROOT, "include"), "-isystem", include, "-isystem", os.path.join(include, "torch", "csrc", "api", "include"),
-           "-isystem", sysconfig.get_paths()["include"], HOST_SOURCE,
-           "-L", os.path.join(torch, "lib"), "-lc10", "-ltorch_cpu", "-ltorch_python", "-o", HOST_LIB + ".tmp"]
+           "-isystem", sysconfig.get_paths()["include"], "-isystem", cuda_include(), HOST_SOURCE,
+           "-L", os.path.join(torch, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-o", HOST_LIB + ".tmp"]
     subprocess.run(cmd, check=True)
     os.replace(HOST_LIB + ".tmp", HOST_LIB)
     os.makedirs(os.path.dirname(HOST_STAMP), exist_ok=True)
