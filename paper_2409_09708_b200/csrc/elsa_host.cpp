@@ -12,7 +12,7 @@
 #include <ATen/ATen.h>
 #include <ATen/EmptyTensor.h>
 #include <c10/core/impl/DeviceGuardImplInterface.h>
-#include <c10/core/impl/TorchDispatchModeTLS.h>
+#include <c10/core/impl/LocalDispatchKeySet.h>
 #include <c10/cuda/CUDACachingAllocator.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -93,13 +93,14 @@ const at::Tensor& matrix(PyObject* o)
 // A new tensor of this shape beside `like`.  On the current GPU straight from torch's current CUDA allocator (the one that
 // torch.cuda.memory.change_current_allocator puts in place; c10::GetAllocator keeps the built-in one): by way of at::empty's dispatch
 // eight outputs, four levels of a weight, were most of the call (3072 x 768 11.5 us with it, 9.4 without).  What at::empty
-// does besides is left to it: another device, dispatch modes, filled memory.
+// does besides is left to it: another device, filled memory, and whatever takes part in a call on this thread beyond the ordinary
+// (dispatch modes, functional transforms, tracing), which shows as a dispatch key included.
 at::Tensor fresh(const at::Tensor& like, at::IntArrayRef shape, at::ScalarType type)
 {
     const c10::Device device = like.device();
     const at::Context& context = at::globalContext();
     if (device.is_cuda() && c10::impl::getDeviceGuardImpl(c10::DeviceType::CUDA)->getDevice() == device &&
-        !c10::impl::TorchDispatchModeTLS::any_modes_set() && !(context.deterministicAlgorithms() && context.deterministicFillUninitializedMemory()))
+        (c10::impl::tls_local_dispatch_key_set().included_ - c10::default_included_set).empty() && !(context.deterministicAlgorithms() && context.deterministicFillUninitializedMemory()))
         return at::detail::empty_generic(shape, c10::cuda::CUDACachingAllocator::get(), c10::DispatchKeySet(c10::DispatchKey::CUDA), type, std::nullopt);
     return at::empty(shape, like.options().dtype(type));
 }

@@ -65,3 +65,21 @@ def test_outputs_come_from_the_allocator_in_place(tmp_path):
                     "-o", str(built)], check=True)
     run = subprocess.run([sys.executable, "-c", PROGRAM, str(built)], cwd=ROOT, capture_output=True, text=True, timeout=600)
     assert run.returncode == 0 and "ok 11" in run.stdout, run.stdout + run.stderr
+
+
+@pytest.mark.gpu
+def test_transforms_reach_the_outputs():
+    """Inside a transform torch.empty's result belongs to the transform and has no memory to hand to the library: the call is refused,
+    with outputs from the allocator it would leave the transform without a word."""
+    import torch
+    from paper_2409_09708_b200 import binding as lib
+    W = torch.randn(16, 64, device="cuda", dtype=torch.float16)
+
+    def f(s):
+        with pytest.raises(RuntimeError, match="storage"):
+            lib.elsa_nm_compress(W, 2, 8)
+        return 2 * s
+
+    assert float(torch.func.grad(f)(torch.tensor(1.0))) == 2.0
+    lib.elsa_nm_compress(W, 2, 8)
+    torch.cuda.synchronize()
