@@ -571,6 +571,9 @@ __global__ void __launch_bounds__(Shape<kD, kBufs, kBias>::kThreads, 1) attentio
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
+        if (*abort_flag)
+            // a wait gave up: let copies and MMAs that may still be in flight land first
+            for (int i = 0; i < 200; ++i) __nanosleep(10000);
         tc_fence_after();
         tmem_dealloc(tmem_base, kTmemCols);
     }

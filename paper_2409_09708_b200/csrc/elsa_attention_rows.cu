@@ -200,6 +200,9 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(const __grid_c
             make_uint4(pack2<kBf16>(v[0] * inv, v[1] * inv), pack2<kBf16>(v[2] * inv, v[3] * inv), pack2<kBf16>(v[4] * inv, v[5] * inv),
                        pack2<kBf16>(v[6] * inv, v[7] * inv));
     }
+    if (*abort_flag)
+        // a wait gave up: let copies that may still be in flight land before shared memory is released
+        for (int i = 0; i < 200; ++i) __nanosleep(10000);
 }
 
 template <bool kBf16, int kD>
