@@ -161,10 +161,10 @@ __global__ void __launch_bounds__(Shape<kD, kBufs, kBias>::kThreads, 1) attentio
     pdl_wait_for_predecessors();
     pdl_release_successors();
 
+    bool ok = true;
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
         const bool elected = elect_one();
-        bool ok = true;
         // Q and K of a stage are free as soon as the scores of its previous item are complete, V only after that item's
         // second product.  The loop asks for Q and K of item n, then for V of item n - 1: the order in which the MMA
         // warp frees them (S of item n - kBufs, then P V of item n - 1 - kBufs), so the next item's Q and K arrive under
@@ -207,7 +207,6 @@ __global__ void __launch_bounds__(Shape<kD, kBufs, kBias>::kThreads, 1) attentio
         const uint32_t elected = elect_one() ? 1u : 0u;
         const uint32_t tmem_u = __reduce_or_sync(0xFFFFFFFFu, tmem_base);
         const int steps = p.tk / 16;
-        bool ok = true;
         for (int n = 0; ok && n < n_items + kLag; ++n) {
             if (n < n_items) {
                 const int b = n % kBufs;
@@ -259,7 +258,6 @@ __global__ void __launch_bounds__(Shape<kD, kBufs, kBias>::kThreads, 1) attentio
         const uint32_t stage_out = out_base + (uint32_t)((warp - 2) * Shape<kD, kBufs, kBias>::kOutBytes);
         constexpr float kFar = 32768.f;     // no probability above it: inside the 16-bit types and far inside fp32
         const float scale = (kD == 64 ? 0.125f : 0.17677669529663687f) * 1.4426950408889634f;   // log2(e) / sqrt(kD)
-        bool ok = true;
         int mt, head, img, next_mt = 0, next_head = 0, next_img = 0;
         auto decode = [&](int n) {
             const int item = first + n * stride;
@@ -568,12 +566,10 @@ __global__ void __launch_bounds__(Shape<kD, kBufs, kBias>::kThreads, 1) attentio
             }
         }
     }
+    if (!ok) let_copies_land();
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
-        if (*abort_flag)
-            // a wait gave up: let copies and MMAs that may still be in flight land first
-            for (int i = 0; i < 200; ++i) __nanosleep(10000);
         tc_fence_after();
         tmem_dealloc(tmem_base, kTmemCols);
     }

@@ -39,6 +39,14 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// For a thread whose wait gave up, before it meets the others of its CTA at the kernel's end: copies and MMAs may still be in flight and
+// land first.  (Asked of the abort flag at the very end, the pause costs launches that need none 0.1 to 0.2 us.)
+__device__ __forceinline__ void let_copies_land()
+{
+#pragma unroll 1
+    for (int i = 0; i < 200; ++i) __nanosleep(10000);
+}
+
 elsa_status make_map_qkv(CUtensorMap* map, const void* qkv, int images, int tokens, int dim, int head_dim, uint32_t box_rows,
                          const char* what)
 {

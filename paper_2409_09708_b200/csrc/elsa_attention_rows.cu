@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(const __grid_c
     for (int n = 0; n < kD / 8; ++n) o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.f;
 
     bool ok = mbar_wait(qk_bar, 0, abort_flag, p.dev_status, 60);
+    if (!ok) let_copies_land();
     ok = __all_sync(0xFFFFFFFFu, ok);
     if (ok) {
         uint32_t q[kD / 16][4];
@@ -133,6 +134,7 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(const __grid_c
         top0 = fmaxf(top0 * kScale, -3.0e38f);      // finite for scores of minus infinity, and for a warp without keys
         top1 = fmaxf(top1 * kScale, -3.0e38f);
         ok = mbar_wait(v_bar, 0, abort_flag, p.dev_status, 61);
+        if (!ok) let_copies_land();
         ok = __all_sync(0xFFFFFFFFu, ok);
     }
     if (ok) {
@@ -200,9 +202,6 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(const __grid_c
             make_uint4(pack2<kBf16>(v[0] * inv, v[1] * inv), pack2<kBf16>(v[2] * inv, v[3] * inv), pack2<kBf16>(v[4] * inv, v[5] * inv),
                        pack2<kBf16>(v[6] * inv, v[7] * inv));
     }
-    if (*abort_flag)
-        // a wait gave up: let copies that may still be in flight land before shared memory is released
-        for (int i = 0; i < 200; ++i) __nanosleep(10000);
 }
 
 template <bool kBf16, int kD>
