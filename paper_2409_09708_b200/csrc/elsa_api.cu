@@ -426,7 +426,8 @@ elsa_status run_linear(LinearKind kind, const void* X, int rows, const void* val
         return launch_linear_tc_pair((const uint16_t*)X, rows, Wd, (const uint16_t*)bias, out, in, dtype,
                                      (uint16_t*)Y, dev_status, stream);
     if (kind == KIND_SMALL_IMAGE) {
-        const SmallJob job = small_dense_job(X, rows, Wd, bias, out, in, Y);
+        SmallJob job = small_dense_job(X, rows, Wd, bias, out, in, Y);
+        job.after_image = N != M;
         if (small_splits == 0) small_splits = linear_small_splits(&job, 1, dev.sm_count);
         return launch_linear_small_group(&job, 1, small_splits, false, dtype, dev_status, stream);
     }
@@ -582,7 +583,8 @@ elsa_status elsa_nm_linear_masked(const void* X, int rows, const void* W_sup, co
         return launch_linear_tc_pair((const uint16_t*)X, rows, Wd, (const uint16_t*)bias, out, in, dtype, (uint16_t*)Y,
                                      dev_status, stream);
     if (kind == KIND_SMALL_IMAGE) {
-        const SmallJob job = small_dense_job(X, rows, Wd, bias, out, in, Y);
+        SmallJob job = small_dense_job(X, rows, Wd, bias, out, in, Y);
+        job.after_image = N != M;
         return launch_linear_small_group(&job, 1, linear_small_splits(&job, 1, dev.sm_count), false, dtype, dev_status, stream);
     }
     return launch_linear_tc_dense((const uint16_t*)X, rows, Wd, (const uint16_t*)bias, out, in, dtype, (uint16_t*)Y,
@@ -1118,7 +1120,7 @@ elsa_status block_linear(BlockLinear& L, const uint16_t* X, int rows, elsa_dtype
         if ((st = block_images(&L, 1, stream)) != ELSA_OK) return st;
         SmallJob job = L.kind == KIND_SMALL ? small_job(X, rows, w.vals, w.N == w.M ? nullptr : w.idx, w.bias, L.out, L.in, w.N, w.M, Y)
                                             : small_dense_job(X, rows, w.N == w.M ? w.vals : L.ws, w.bias, L.out, L.in, Y);
-        job.act = act; job.residual = residual;
+        job.act = act; job.residual = residual; job.chained = true;
         if (L.next != nullptr && L.next->kind == KIND_SMALL_IMAGE) {
             const elsa_block_linear& n = *L.next->w;
             job.ahead = n.N == n.M ? n.vals : L.next->ws;
@@ -1587,7 +1589,8 @@ elsa_status dense_product(const uint16_t* A, int m, const uint16_t* B, int n, in
                           uint32_t* dev_status, cudaStream_t stream, int sm_count)
 {
     const int variant = g_variant.load(std::memory_order_relaxed);
-    const SmallJob job = small_dense_job(A, m, B, nullptr, n, k, Y);
+    SmallJob job = small_dense_job(A, m, B, nullptr, n, k, Y);
+    job.after_image = true;      // B is what a transpose has just written
     LinearKind kind;       // the dense level's rule
     const elsa_status st = pick_kind(USE_SINGLE, m, n, k, 4, 4, sm_count, &kind);
     if (st != ELSA_OK || variant == ELSA_VARIANT_TC_DENSE || kind == KIND_DENSE_ONE)

@@ -109,6 +109,8 @@ struct SmallJob {
     const uint16_t* residual = nullptr;   // [rows][out], added after the activation, before the one rounding
     const void* ahead = nullptr;          // launches of one job: the next linear's weight, brought into L2 meanwhile (16-byte
     size_t ahead_bytes = 0;               // aligned; nothing reads it here, so it may still be written)
+    bool chained = false;                 // one of a chain of linears with other kernels between them
+    bool after_image = false;             // of a call that has just made this weight with another kernel
 };
 int linear_small_group_max();
 // Ranges the reductions of these jobs are cut into when they run together.  A result depends on it in its last bits.

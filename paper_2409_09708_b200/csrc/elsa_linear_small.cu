@@ -12,10 +12,12 @@
 //   * a CTA computes one tile of 128 rows x 64 features and leaves; two CTAs fit an SM, so that one's set-up and
 //     epilogue run under the other's tile, or the next kernel's set-up under this one's;
 //   * where the tiles alone leave SMs idle, the reduction is cut into 2, 4 or 8 ranges, one CTA of a cluster each:
-//     every CTA sends the rows of its fp32 sums to the CTA that owns them as bulk copies between their shared memories,
-//     whose bytes the owner's barrier counts, and each owner adds its rows in rank order (deterministic), applies bias,
-//     activation and residual, which it has asked for by then, and rounds once (stores into the other CTA's memory behind a
-//     cluster barrier, bias and residual loaded last: 3072 x 768 at 4:4, 197 rows, 7.3 -> 7.1 us, one-image encoder 500 -> 492);
+//     every CTA sends the rows of its fp32 sums to the CTA that owns them, and each owner adds its rows in rank order
+//     (deterministic), applies bias, activation and residual, which it has asked for by then, and rounds once;
+//   * the sums go as bulk copies between the CTAs' shared memories, whose bytes the owner's barrier counts, in a chain and in a call
+//     of its own on a dense weight (1024 -> 1024 at 4:4, 49 rows, 6.9 -> 6.1 us; one-image encoder 500 -> 492), elsewhere as stores into
+//     the other CTA's memory and a cluster barrier: that is less code, and where an image kernel runs between any two of
+//     these no cache holds it (1536 -> 384 at 1:8, 197 rows, image included, bulk copies 7.5, stores 7.0 us);
 //   * a call that knows the weights to be older than its own first kernel (the chained block) has their first tiles
 //     fetched before the predecessor kernel has ended (`early`): only X and the outputs wait for it;
 //   * in a chain each launch has the next linear's weight brought into L2 (`ahead`): a model's weights do not stay there
@@ -83,7 +85,7 @@ struct SmallGroup {
     int splits;                   // CTAs of a cluster = ranges of the reduction
     int stages;
     int early;
-    int rehearse;                 // 0: the epilogue's first pass is a rehearsal (a value that the compiler does not know)
+    int first_pass;               // of the epilogue: 0 the rehearsal, 1 the real one
     uint32_t idesc;
     uint32_t* dev_status;
     const void* ahead;            // what the call's next linear reads as its weight: brought into L2 meanwhile
@@ -94,6 +96,8 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes
 {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
+
+__device__ __forceinline__ void named_barrier_workers() { asm volatile("bar.sync 1, %0;" ::"n"(kWorkers * 32) : "memory"); }
 
 // Copies shared memory of this CTA into another one of the cluster, the bytes counted on an mbarrier there.
 __device__ __forceinline__ void bulk_send(uint32_t dst_cluster, uint32_t src, uint32_t bytes, uint32_t bar_cluster)
@@ -156,7 +160,8 @@ __device__ __forceinline__ bool expand_range(int kb0, int kb1, int stages, uint3
 struct DenseRaw { uint4 a, b; };
 struct NoRaw { int row; };
 
-template <bool kBf16, int kMax>
+// kBulk: how the sums of a cut reduction go to their owners, see above.
+template <bool kBf16, int kMax, bool kBulk>
 __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __grid_constant__ SmallGroup<kMax> p)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -188,7 +193,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
     const uint32_t full_bar = smem_base + (uint32_t)bar_off;
     const uint32_t empty_bar = full_bar + 8 * kStagesMax;
     const uint32_t done_bar = empty_bar + 8 * kStagesMax;
-    const uint32_t sums_bar = done_bar + 8;       // the sums of this CTA's rows: its own warps' arrivals, the others' bytes
+    const uint32_t sums_bar = done_bar + 8;       // kBulk: the sums of this CTA's rows: its own warps' arrivals, the others' bytes
     volatile uint32_t* tmem_holder = reinterpret_cast<volatile uint32_t*>(smem_gen + bar_off + 16 * kStagesMax + 16);
     const int slice = kTileM / splits;            // rows each CTA of the cluster finishes
     volatile uint32_t* abort_flag = tmem_holder + 1;
@@ -199,8 +204,10 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
             mbar_init(empty_bar + 8 * s, 1);
         }
         mbar_init(done_bar, 1);
-        mbar_init(sums_bar, 1 + kWorkers);
-        mbar_arrive_expect_tx(sums_bar, (uint32_t)((splits - 1) * slice * 2 * kPitch * 4));
+        if constexpr (kBulk) {
+            mbar_init(sums_bar, 1 + kWorkers);
+            mbar_arrive_expect_tx(sums_bar, (uint32_t)((splits - 1) * slice * 2 * kPitch * 4));
+        }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async_smem();
@@ -342,19 +349,22 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
         uint4 bw = make_uint4(0u, 0u, 0u, 0u), rw = bw;
         if (L.bias != nullptr && col < L.out) bw = __ldg(reinterpret_cast<const uint4*>(L.bias + col));
         const uint16_t* residual = L.residual;
+        const int rows_here = col < L.out ? min(slice, L.rows - m0 - rank * slice) : 0;      // to finish; none if it is not positive
         {
             const int row = m0 + rank * slice + tid / kUnits;
-            if (residual != nullptr && row < L.rows && col < L.out) rw = *reinterpret_cast<const uint4*>(residual + (size_t)row * L.out + col);
+            if (residual != nullptr && tid / kUnits < rows_here) rw = *reinterpret_cast<const uint4*>(residual + (size_t)row * L.out + col);
         }
         // The sums of 32 rows x 32 columns a warp lie [half][row][pitch]; those that come from CTA s of the cluster at
         // s * slice rows of either half.
         const uint32_t inbox = smem_base + (uint32_t)sums_off;
         const float* sums = reinterpret_cast<const float*>(smem_gen + sums_off) + (size_t)(col_l / kHalfN * kTileM) * kPitch + col_l % kHalfN;
-        // The first pass is a rehearsal: while the loads and MMAs are under way it runs the last part's instructions and stores
-        // nothing.  In a chain of kernels their code is in none of the SM's caches, and fetched when it is needed it took
-        // longer than it ran: one-image encoder of DeiT-B 492 -> 486 us; for the same reason the loops here are not unrolled.
+        // In a chain the first pass is a rehearsal: while the loads and MMAs are under way it runs the last part's instructions and
+        // stores nothing (what it reads of the sums is whatever lies there, stages that TMA is filling included, and goes nowhere).
+        // In a chain of kernels their code is in none of the SM's caches, and fetched when it is needed it took longer than it ran:
+        // one-image encoder of DeiT-B 492 -> 486 us; for the same reason the loops here are not unrolled.  Calls of one's own keep
+        // the code and only pay for the pass: 1536 -> 384 at 4:4, 49 rows, 5.6 us with it, 4.9 without.
 #pragma unroll 1
-        for (int real = p.rehearse; real < 2; ++real) {
+        for (int real = p.first_pass; real < 2; ++real) {
             if (real) {
                 ok = ok && mbar_wait(done_bar, 0, abort_flag, p.dev_status, 44);
                 ok = __all_sync(0xFFFFFFFFu, ok);
@@ -366,35 +376,49 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
                     tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * kHalfN), r);
                     tmem_wait_ld();
                     tc_fence_before();
-                    // rows of this CTA go where they are added, the others' to the stages (no MMA reads them any more) and from
-                    // there to their CTA as one copy for each
-                    const uint32_t outbox = smem_base + (uint32_t)(half * kTileM * kPitch * 4);
-                    const uint32_t dst = to == rank ? inbox + (uint32_t)((half * kTileM + rank * slice + row % slice) * kPitch * 4)
-                                                    : outbox + (uint32_t)(row * kPitch * 4);
+                    const uint32_t in_owner = inbox + (uint32_t)((half * kTileM + rank * slice + row % slice) * kPitch * 4);
+                    if constexpr (kBulk) {
+                        // rows of this CTA go where they are added, the others' to the stages (no MMA reads them any more) and from
+                        // there to their CTA as one copy for each
+                        const uint32_t outbox = smem_base + (uint32_t)(half * kTileM * kPitch * 4);
+                        const uint32_t dst = to == rank ? in_owner : outbox + (uint32_t)(row * kPitch * 4);
 #pragma unroll
-                    for (int v = 0; v < 8; ++v)
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(16 * v)), "r"(r[4 * v]), "r"(r[4 * v + 1]),
-                                     "r"(r[4 * v + 2]), "r"(r[4 * v + 3])
-                                     : "memory");
-                    if (split) fence_proxy_async_smem();
-                    __syncwarp();
-                    if (split) {
-                        const int run = min(slice, 32);      // a warp's rows for one CTA
-                        if (to != rank && lane % run == 0)
-                            bulk_send(mapa_shared(inbox + (uint32_t)((half * kTileM + rank * slice + row % slice) * kPitch * 4), (uint32_t)to),
-                                      outbox + (uint32_t)(row * kPitch * 4), (uint32_t)(run * kPitch * 4), mapa_shared(sums_bar, (uint32_t)to));
+                        for (int v = 0; v < 8; ++v)
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(16 * v)), "r"(r[4 * v]),
+                                         "r"(r[4 * v + 1]), "r"(r[4 * v + 2]), "r"(r[4 * v + 3])
+                                         : "memory");
+                        if (split) fence_proxy_async_smem();
+                        __syncwarp();
+                        if (split) {
+                            const int run = min(slice, 32);      // a warp's rows for one CTA
+                            if (to != rank && lane % run == 0)
+                                bulk_send(mapa_shared(in_owner, (uint32_t)to), outbox + (uint32_t)(row * kPitch * 4),
+                                          (uint32_t)(run * kPitch * 4), mapa_shared(sums_bar, (uint32_t)to));
+                        }
+                        if (lane == 0) mbar_arrive(sums_bar);
+                        ok = mbar_wait(sums_bar, 0, abort_flag, p.dev_status, 45);
+                        ok = __all_sync(0xFFFFFFFFu, ok);
+                    } else {
+                        const uint32_t dst = split ? mapa_shared(in_owner, (uint32_t)to) : in_owner;
+#pragma unroll
+                        for (int v = 0; v < 8; ++v)
+                            asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + (uint32_t)(16 * v)), "r"(r[4 * v]),
+                                         "r"(r[4 * v + 1]), "r"(r[4 * v + 2]), "r"(r[4 * v + 3])
+                                         : "memory");
                     }
-                    if (lane == 0) mbar_arrive(sums_bar);
-                    ok = mbar_wait(sums_bar, 0, abort_flag, p.dev_status, 45);
-                    ok = __all_sync(0xFFFFFFFFu, ok);
                 }
                 if (split) cluster_arrive();
+                if constexpr (!kBulk) {
+                    __syncwarp();
+                    if (split) cluster_wait();
+                    else named_barrier_workers();
+                }
             }
             if (ok) {
 #pragma unroll 1
-                for (int row_l = real ? tid / kUnits : slice - 1; row_l < slice; row_l += kRowsAStep) {
+                for (int row_l = real ? tid / kUnits : slice - 1; row_l < (real ? rows_here : slice); row_l += kRowsAStep) {
                     const int row = m0 + rank * slice + row_l;
-                    if (real && row_l >= kRowsAStep && residual != nullptr && row < L.rows && col < L.out)
+                    if (real && row_l >= kRowsAStep && residual != nullptr)
                         rw = *reinterpret_cast<const uint4*>(residual + (size_t)row * L.out + col);
                     float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
@@ -425,11 +449,11 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
                         const float2 rv = raw2_to_float2<kBf16>(r[j]);
                         o[j] = pack2<kBf16>(a[2 * j] + rv.x, a[2 * j + 1] + rv.y);
                     }
-                    if (real && row < L.rows && col < L.out) *reinterpret_cast<uint4*>(L.Y + (size_t)row * L.out + col) = make_uint4(o[0], o[1], o[2], o[3]);
+                    if (real) *reinterpret_cast<uint4*>(L.Y + (size_t)row * L.out + col) = make_uint4(o[0], o[1], o[2], o[3]);
                 }
             }
         }
-        if (split) cluster_wait();
+        if (kBulk && split) cluster_wait();
     }
 
     // ------------------------------------------------ teardown
@@ -443,7 +467,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) linear_small_kernel(const __
     }
 }
 
-template <bool kBf16, int kMax>
+template <bool kBf16, int kMax, bool kBulk>
 elsa_status launch_small(const SmallJob* jobs, int n, int splits, bool early, uint32_t* dev_status, cudaStream_t stream, const DeviceInfo& dev)
 {
     SmallGroup<kMax> g;      // on the stack: several threads may launch at once
@@ -471,13 +495,13 @@ elsa_status launch_small(const SmallJob* jobs, int n, int splits, bool early, ui
     g.splits = splits;
     g.stages = splits > 1 ? kStagesSplit : kStagesMax;
     g.early = early ? 1 : 0;
-    g.rehearse = 0;
+    g.first_pass = n == 1 && jobs[0].chained ? 0 : 1;
     g.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(kTileN >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
     g.dev_status = dev_status;
     g.ahead = n == 1 ? jobs[0].ahead : nullptr;
     g.ahead_units = n == 1 ? (uint32_t)(jobs[0].ahead_bytes / 16) : 0;
 
-    auto kernel = linear_small_kernel<kBf16, kMax>;
+    auto kernel = linear_small_kernel<kBf16, kMax, kBulk>;
     constexpr int kSmemMost = small_smem(true) > small_smem(false) ? small_smem(true) : small_smem(false);
     static std::atomic<bool> attr_set[64];
     const int slot = dev.device & 63;
@@ -527,11 +551,13 @@ elsa_status launch_linear_small_group(const SmallJob* jobs, int n, int splits, b
     if (n < 1 || n > kSmallGroupMax) return fail(ELSA_ERR_SHAPE, "a grouped launch carries 1 to %d layers, got %d", kSmallGroupMax, n);
     for (int i = 0; n > 1 && i < n; ++i)
         if (jobs[i].N != jobs[i].M) return fail(ELSA_ERR_NM, "layer %d of a grouped launch is packed (%d:%d)", i, jobs[i].N, jobs[i].M);
-    if (dtype == ELSA_BF16)
-        return n == 1 ? launch_small<true, 1>(jobs, n, splits, early, dev_status, stream, dev)
-                      : launch_small<true, kSmallGroupMax>(jobs, n, splits, early, dev_status, stream, dev);
-    return n == 1 ? launch_small<false, 1>(jobs, n, splits, early, dev_status, stream, dev)
-                  : launch_small<false, kSmallGroupMax>(jobs, n, splits, early, dev_status, stream, dev);
+    const bool bulk = n == 1 && (jobs[0].chained || (jobs[0].N == jobs[0].M && !jobs[0].after_image));
+#define ELSA_SMALL(MAX, BULK)                                                                                   \
+    (dtype == ELSA_BF16 ? launch_small<true, MAX, BULK>(jobs, n, splits, early, dev_status, stream, dev)        \
+                        : launch_small<false, MAX, BULK>(jobs, n, splits, early, dev_status, stream, dev))
+    if (n > 1) return ELSA_SMALL(kSmallGroupMax, false);
+    return bulk ? ELSA_SMALL(1, true) : ELSA_SMALL(1, false);
+#undef ELSA_SMALL
 }
 
 }  // namespace elsa

@@ -114,3 +114,25 @@ def test_small_layers_of_a_table_share_a_launch(lib):
         out, in_ = d["W"].shape
         Wm = d["W"] if d["N"] == d["M"] else lib.elsa_nm_unpack(d["vals"], d["idx"], out, in_, d["N"], d["M"])
         close(y, (d["X"].double() @ Wm.double().t() + d["bias"].double()).cpu().numpy())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("rows", [1, 15, 16, 17, 33, 64, 65, 127, 128, 130, 197])
+@pytest.mark.parametrize("k,out", [(1024, 256), (1040, 200), (1024, 1544), (1024, 2376)])       # up to 128 rows cut into 8, 8, 4 and 2 ranges
+def test_both_ways_of_the_sums_give_the_same(rows, k, out):
+    """A call on a dense weight sends its sums as bulk copies, one behind an image as stores: the same operands, order and rounding."""
+    from paper_2409_09708_b200 import binding as lib
+    gen = torch.Generator().manual_seed(rows + k)
+    X = torch.randn(rows, k, generator=gen).to(torch.bfloat16).cuda()
+    W = (0.05 * torch.randn(out, k, generator=gen)).to(torch.bfloat16).cuda()
+    bias = torch.randn(out, generator=gen).to(torch.bfloat16).cuda()
+    vals, idx = lib.elsa_nm_compress(W, 3, 8)
+    dense = lib.elsa_nm_unpack(vals, idx, out, k, 3, 8)
+    guard = torch.full((rows + 130, out), 7.0, dtype=torch.bfloat16, device="cuda")
+    lib.elsa_nm_linear(X, vals, idx, bias, out, k, 3, 8, Y=guard[:rows])
+    assert torch.equal(guard[:rows], lib.elsa_nm_linear(X, dense, None, bias, out, k, 8, 8))
+    assert bool((guard[rows:] == 7.0).all())
+    exact = X.double() @ dense.double().t() + bias.double()
+    # fp32 sums of k terms (error at most k 2^-24 of their absolute sum), one rounding to bf16
+    bound = 2.0 ** -8 * exact.abs() + k * 2.0 ** -24 * (X.double().abs() @ dense.double().abs().t() + bias.double().abs())
+    assert bool(((guard[:rows].double() - exact).abs() <= bound).all())
