@@ -181,7 +181,7 @@ struct SparseJob {
     int rows, in, out;
     int act = 0;      // epilogue activation: 0 none, 1 GELU (weight-stationary and streaming kernels only)
     // weight-stationary kernel: the packed weight (kept values, index words, level), from which it makes its weight block
-    // itself; without it the block comes from the image in `workspace`
+    // itself; without it (one plain layer) the block comes from the image in `workspace`
     const uint16_t* w = nullptr;
     const uint32_t* idx = nullptr;
     int N = 0, M = 0;

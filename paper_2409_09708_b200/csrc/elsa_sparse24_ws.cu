@@ -63,12 +63,12 @@ constexpr int kStagingBytes = kMaxSteps * kStepCols * 64;        // per epilogue
 constexpr int kStagingTotal = kEpiWarps * kStagingBytes;
 constexpr int kBarrierBytes = 512;
 
-// What a layer's weight block is made from.
-enum WsLevel : uint8_t { LEVEL_IMAGE, LEVEL_1_4, LEVEL_2_4, LEVEL_1_8, LEVEL_2_8, LEVEL_1_16, LEVEL_2_16 };
+// The level of a packed weight.
+enum WsLevel : uint8_t { LEVEL_1_4, LEVEL_2_4, LEVEL_1_8, LEVEL_2_8, LEVEL_1_16, LEVEL_2_16 };
 
 struct alignas(64) WsLayer {
     CUtensorMap map_x, map_y, map_run;   // map_y: one step of 16 token rows, map_run: a warp's whole run of them
-    // LEVEL_IMAGE: 2-of-4 values [out rounded up to 32][in / 2], rows in the permuted order, and metadata blocks of 2 KB per
+    // kImage: 2-of-4 values [out rounded up to 32][in / 2], rows in the permuted order, and metadata blocks of 2 KB per
     // (128 features, 128 k).  Otherwise the packed weight: kept values and index words.
     const void* w;
     const void* meta;
@@ -175,7 +175,9 @@ __device__ __forceinline__ void write_packed(const uint16_t* vals_row, const uin
 // single-layer launches.  The residual comes by TMA into the staging buffer, in the rows that the result leaves by, while the tile is
 // multiplied, and ldmatrix brings it to the lanes the way stmatrix takes the result back: as a pass of its own over four
 // tensors it cost a LayerNorm 64 us where the plain one takes 34 (50432 rows of 768).
-template <bool kBf16, int kMaxLayers, int kEpi>
+// kImage: the weight block comes from an image (masked form; with both ways in one instantiation the expansions' registers cost that
+// form 1.3 us, 12608 x 768 -> 3072 at 1:8 37.1 -> 38.4).
+template <bool kBf16, int kMaxLayers, int kEpi, bool kImage>
 __global__ void __launch_bounds__(kThreads, 1)
 linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
 {
@@ -393,7 +395,7 @@ linear_tc_sp24_ws_kernel(const __grid_constant__ WsGroup<kMaxLayers> p)
             {
                 const uint32_t a_col0 = lane_base + (uint32_t)(kNumAccum * nt);
                 const uint32_t e_col0 = a_col0 + (uint32_t)(L.in >> 2);
-                if (L.level == LEVEL_IMAGE) {
+                if constexpr (kImage) {
                     const int a_chunks = L.in >> 6;          // 16 columns (64 bytes) each
                     const uint4* a_row = static_cast<const uint4*>(L.w) + (size_t)(ft128 * kFeatPerCta + q * 32 + lane) * (size_t)(L.in >> 4);
                     const bool blk_ok = ft128 * kFeatPerCta < l_out;     // rows of a started block of 32 exist (zero beyond out)
@@ -575,12 +577,12 @@ int ws_layer_row_tile(int in, int rows, int groups)
     return best;
 }
 
-template <bool kBf16, int kMaxLayers, int kEpi>
+template <bool kBf16, int kMaxLayers, int kEpi, bool kImage = false>
 elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint32_t* dev_status, cudaStream_t stream,
                             const DeviceInfo& dev)
 {
     constexpr bool kRuns = kEpi == kEpiGelu || kMaxLayers > 1;
-    auto kernel = linear_tc_sp24_ws_kernel<kBf16, kMaxLayers, kEpi>;
+    auto kernel = linear_tc_sp24_ws_kernel<kBf16, kMaxLayers, kEpi, kImage>;
     const int fixed = kStagingTotal + kBarrierBytes + 1024;
     int max_nt = 0;
     for (int i = 0; i < n; ++i) {
@@ -644,7 +646,7 @@ elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
         if (L.groups * L.tiles_f > used_pairs) used_pairs = L.groups * L.tiles_f;
         L.bias = j.bias;
         L.act = (uint8_t)j.act;
-        if (j.w != nullptr) {
+        if constexpr (!kImage) {
             L.w = j.w;
             L.meta = j.idx;
             L.level = j.M == 4 ? (j.N == 1 ? LEVEL_1_4 : LEVEL_2_4) : j.M == 8 ? (j.N == 1 ? LEVEL_1_8 : LEVEL_2_8) : j.N == 1 ? LEVEL_1_16 : LEVEL_2_16;
@@ -652,7 +654,7 @@ elsa_status launch_ws_group(const SparseJob* jobs, int n, elsa_dtype dtype, uint
         } else {
             L.w = j.workspace;
             L.meta = (const uint8_t*)j.workspace + sp24_meta_offset(j.out, j.in);
-            L.level = LEVEL_IMAGE;
+            L.level = 0;
             L.words_per_row = 0;
         }
         // sparse flag, fp32 accumulate, A and B of type fmt, K-major, N = nt, M = 256 over the pair
@@ -703,8 +705,16 @@ elsa_status launch_linear_tc_sparse_ws_group(const SparseJob* jobs, int n, elsa_
     elsa_status st = device_info(&dev);
     if (st != ELSA_OK) return st;
     if (n < 1 || n > kGroupMax) return fail(ELSA_ERR_SHAPE, "a grouped launch carries 1 to %d layers, got %d", kGroupMax, n);
-    bool alone = false;
-    for (int i = 0; i < n; ++i) alone = alone || jobs[i].act != 0 || jobs[i].residual != nullptr;
+    bool alone = false, image = false;
+    for (int i = 0; i < n; ++i) {
+        alone = alone || jobs[i].act != 0 || jobs[i].residual != nullptr;
+        image = image || jobs[i].w == nullptr;
+    }
+    if (image) {
+        if (n > 1 || alone) return fail(ELSA_ERR_SHAPE, "an image of the weight in a table or a chain of this kernel");
+        return dtype == ELSA_BF16 ? launch_ws_group<true, 1, kEpiPlain, true>(jobs, 1, dtype, dev_status, stream, dev)
+                                  : launch_ws_group<false, 1, kEpiPlain, true>(jobs, 1, dtype, dev_status, stream, dev);
+    }
     if (alone) {
         // layers with an activation or a residual in the epilogue run one per launch, on the instantiation that has it
         for (int i = 0; i < n; ++i) {
