@@ -156,30 +156,25 @@ __device__ __forceinline__ uint4 sp24_words(const Segment& s, uint32_t& nibbles)
     } else if constexpr (M == 4) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) single(true, (s.v[c >> 1] >> (16 * (c & 1))) & 0xFFFFu, (s.fields >> (2 * c)) & 3u, c);
+    } else if constexpr (N == 1) {              // one group of 16
+        const uint32_t p0 = s.fields & 15u;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) single((p0 >> 2) == (uint32_t)c, s.v[0], p0 & 3u, c);
     } else {
-        constexpr int B = 4, kChunks = 4;       // one group of 16
-#pragma unroll
-        for (int g = 0; g < 1; ++g) {
-            const uint32_t f = s.fields >> (g * N * B);
-            const uint32_t p0 = f & (uint32_t)(M - 1);
-            if constexpr (N == 1) {
-                const uint32_t v = s.v[0];
-#pragma unroll
-                for (int c = 0; c < kChunks; ++c) single((p0 >> 2) == (uint32_t)c, v, p0 & 3u, g * kChunks + c);
-            } else {
-                const uint32_t p1 = (f >> B) & (uint32_t)(M - 1), v = s.v[g];
-#pragma unroll
-                for (int c = 0; c < kChunks; ++c) {
-                    const bool h0 = (p0 >> 2) == (uint32_t)c, h1 = (p1 >> 2) == (uint32_t)c;
-                    if (h0 && h1) {
-                        w[g * kChunks + c] = v;
-                        nib |= ((p0 & 3u) | ((p1 & 3u) << 2)) << (4 * (g * kChunks + c));
-                    } else {
-                        single(h0 || h1, h0 ? v & 0xFFFFu : v >> 16, (h0 ? p0 : p1) & 3u, g * kChunks + c);
-                    }
-                }
-            }
-        }
+        // Selectors of byte permutes as with groups of 8, made by arithmetic: four empty chunks, and what each value changes in
+        // its chunk's selector and nibble.  Two values of one chunk take its halves in order, as 0x3210 says.
+        // (Compares and selects for every chunk, on the weight-stationary kernel: 12608 x 512 -> 512 at 2:16 13.2 us, like this 9.7.)
+        const uint32_t p0 = s.fields & 15u, p1 = (s.fields >> 4) & 15u, l0 = p0 & 3u, l1 = p1 & 3u, at0 = p0 & 12u, at1 = p1 & 12u;
+        const bool same = at0 == at1;
+        const uint64_t select = 0x4444444444444444ull ^ ((uint64_t)(l0 == 3u ? 0x5400u : 0x0054u) << (4u * at0)) ^
+                                ((uint64_t)(l1 == 3u || same ? 0x7600u : 0x0076u) << (4u * at1));
+        const uint32_t lo = (uint32_t)select, hi = (uint32_t)(select >> 32);
+        w[0] = prmt(s.v[0], 0u, lo & 0xFFFFu);
+        w[1] = prmt(s.v[0], 0u, lo >> 16);
+        w[2] = prmt(s.v[0], 0u, hi & 0xFFFFu);
+        w[3] = prmt(s.v[0], 0u, hi >> 16);
+        const uint32_t n0 = same ? (l0 | l1 << 2) ^ 4u : l0 == 3u ? 8u : 8u | l0, n1 = same ? 0u : l1 == 3u ? 8u : 8u | l1;
+        nib = 0x4444u ^ (n0 << at0) ^ (n1 << at1);
     }
     nibbles = nib;
     return make_uint4(w[0], w[1], w[2], w[3]);
