@@ -111,8 +111,18 @@ struct PackedBlock {
 #pragma unroll
         for (int i = 0; i < kCount; ++i) v[i] = __ldg(src + i);
         const int bit0 = kb * kIdxBits;
+        // As wide as the words allow (rows are whole blocks of 128 k): a load of a warp touches 32 rows however little it takes of each
+        // (2:4 word by word: 3152 x 1024 -> 4096 23.1 us, like this 21.2).
+        if constexpr (kIdxWords == 4) {
+            const uint4 t = __ldg(reinterpret_cast<const uint4*>(idx_row) + kb);
+            f[0] = t.x; f[1] = t.y; f[2] = t.z; f[3] = t.w;
+        } else if constexpr (kIdxBits == 64) {
+            const uint2 t = __ldg(reinterpret_cast<const uint2*>(idx_row) + kb);
+            f[0] = t.x; f[1] = t.y;
+        } else {
 #pragma unroll
-        for (int i = 0; i < kIdxWords; ++i) f[i] = __ldg(idx_row + (bit0 >> 5) + i);
+            for (int i = 0; i < kIdxWords; ++i) f[i] = __ldg(idx_row + (bit0 >> 5) + i);
+        }
         if constexpr (kIdxBits % 32 != 0) {      // 48 bits from bit 0 or 16 on
             f[0] = __funnelshift_r(f[0], f[1], bit0 & 31);
             f[1] >>= bit0 & 31;
