@@ -628,7 +628,7 @@ elsa_status launch_attention(const uint16_t* qkv, int images, int tokens, int he
     if (window_attention_suits(tokens, heads, dim))
         return launch_window_attention(qkv, images, tokens, heads, dim, dtype, out, dev_status, stream, bias, mask, n_masks, bias_pitch, dev);
     // A call whose items leave SMs idle is bound by the chain of one: sixteen query rows a CTA instead of 128.
-    if (bias == nullptr && attention_rows_suits(images, tokens, heads, dev.sm_count))
+    if (bias == nullptr && attention_rows_suits(images, tokens, heads, head_dim, dev.sm_count))
         return launch_attention_rows(qkv, images, tokens, heads, dim, dtype, out, dev_status, stream, dev);
     AttnParams p;
     p.out = out;

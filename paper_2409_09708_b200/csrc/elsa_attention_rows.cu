@@ -86,7 +86,6 @@ __global__ void __launch_bounds__(kThreads) attention_rows_kernel(const __grid_c
         tma_load_3d(tile_v, &p.map_kv, v_bar, 2 * p.dim + head * kD, 0, img);
     }
     constexpr float kScale = (kD == 64 ? 0.125f : 0.17677669529663687f) * 1.4426950408889634f;   // log2(e) / sqrt(kD)
-    const int key_tiles = p.tk / 16;
     float s[kMostTiles][2][4], o[kD / 8][4];
     float top0 = -INFINITY, top1 = -INFINITY, sum0 = 0.f, sum1 = 0.f;      // rows g and g + 8
 #pragma unroll
@@ -225,13 +224,16 @@ elsa_status launch(const RowsParams& p, int images, cudaStream_t stream, const D
 
 }  // namespace
 
-// Up to three CTAs an SM, which run together.  Us in a chain of its own kind (5.3 is what a launch takes the host there), this
-// kernel and elsa_attention.cu's: 12 heads of 197 tokens, 2 images (312 CTAs) 5.4, 7.5, 3 images (468) 5.7, 5.6, 4 images 6.4, 5.7,
-// 8 images 9.6, 6.6; 16 heads, 2 images (416) 5.4, 5.6.  In the encoder of DeiT-B an image's twelve take 36 of the 72 us they took
-// (one image 499 -> 468 us, two images 593 -> 578).
-bool attention_rows_suits(int images, int tokens, int heads, int sm_count)
+// Up to three CTAs an SM, which run together; heads of 64 and more than 208 tokens leave room for two, and there up to two and a half.  Us
+// in a chain of its own kind, this kernel and elsa_attention.cu's: 12 heads of 197 tokens, 1 image (156 CTAs) 2.6, 5.2, 2 images (312)
+// 3.6, 5.2, 3 images (468) 5.7, 5.6, 4 images 6.4, 5.7, 8 images 9.6, 6.6; of 65 tokens, 6 images (360) 3.0, 3.9, 7 images (420) 3.6, 3.9; of
+// 145 tokens, 3 images (360) 3.4, 4.8; 6 heads of 224 tokens, 4 images (336) 5.0, 5.1, 5 images (420) 5.3, 5.2.  In the encoder of
+// DeiT-B an image's twelve take 36 of the 72 us they took (one image 499 -> 468 us, two images 593 -> 578).
+bool attention_rows_suits(int images, int tokens, int heads, int head_dim, int sm_count)
 {
-    return (long long)images * heads * ((tokens + kRows - 1) / kRows) <= 3LL * sm_count;
+    const int tk = (tokens + 15) / 16 * 16, smem = head_dim == 64 ? rows_smem<64>(tk) : rows_smem<32>(tk);
+    const bool three = 3 * (smem + 1024 /* reserved for each CTA */) <= 228 * 1024;
+    return 2LL * images * heads * ((tokens + kRows - 1) / kRows) <= (three ? 6LL : 5LL) * sm_count;
 }
 
 elsa_status launch_attention_rows(const uint16_t* qkv, int images, int tokens, int heads, int dim, elsa_dtype dtype, uint16_t* out,

@@ -235,7 +235,7 @@ elsa_status launch_attention(const uint16_t* qkv, int images, int tokens, int he
                              const float* mask = nullptr, int n_masks = 0, int bias_pitch = 0);
 // The same without tables for calls of few items, sixteen query rows a CTA; arguments as checked by launch_attention, which
 // calls it.
-bool attention_rows_suits(int images, int tokens, int heads, int sm_count);
+bool attention_rows_suits(int images, int tokens, int heads, int head_dim, int sm_count);
 elsa_status launch_attention_rows(const uint16_t* qkv, int images, int tokens, int heads, int dim, elsa_dtype dtype, uint16_t* out,
                                   uint32_t* dev_status, cudaStream_t stream, const DeviceInfo& dev);
 // The same for windows that fit a warp's registers (head dimension 32, at most 64 tokens); arguments as checked by

@@ -29,3 +29,10 @@ def test_few_images(images, tokens, heads, d, dtype, spread):
     assert int(status.item()) == 0
     assert bool(((got - ref).abs() <= bound).all())
     assert bool((guard[images * tokens:] == 7.0).all())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("images,tokens,heads", [(4, 208, 8), (4, 224, 6), (5, 224, 6), (10, 209, 3), (3, 256, 9)])
+def test_either_side_of_the_rule(images, tokens, heads):
+    """Heads of 64: up to 208 tokens 444 row tiles of sixteen, beyond 370 (of 148 SMs)."""
+    test_few_images(images, tokens, heads, 64, torch.bfloat16, 1.0)
