@@ -1647,7 +1647,7 @@ elsa_status elsa_nm_linear_backward(const void* dY, const void* X, int rows, con
         // dW = dY^T X, reduction over the token rows: both operands are read as they are stored (reduction index
         // outermost), then the mask
         // when tiles alone leave SM pairs idle, the rows are cut into ranges summed afterwards
-        const TnShape shape = linear_tc_pair_tn_shape(out, in, rows, wgrad_splits_bound(in, out), db ? plan.parts : 1 << 30, dev.sm_count);
+        const TnShape shape = linear_tc_pair_tn_shape(out, in, rows, wgrad_splits_bound(in, out), db ? plan.parts : 0, dev.sm_count);
         float* sums = (float*)(ws + plan.sums);
         const bool db_here = db && linear_tc_pair_tn_sums_parts(in, shape) <= plan.parts;
         if ((st = launch_linear_tc_pair_tn(dy, (const uint16_t*)X, out, in, rows, dtype, (uint16_t*)dW, shape, sums,

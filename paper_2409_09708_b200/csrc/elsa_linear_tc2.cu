@@ -826,17 +826,20 @@ elsa_status launch_linear_tc_pair_group(const PairJob* jobs, int n, elsa_dtype d
 // Compress, forward and backward of a block, us, 256 columns in as many ranges as fit the pairs and like this: dim 192, 25216 rows
 // 259 -> 228, 1576 rows 134 -> 124 (138 with sums of A that found no room); dim 256, 19700 rows 249 -> 225; dim 384, 3152 rows
 // 176 -> 156; dim 512, 985 rows 156 -> 132; dim 768, 3152 rows 249 -> 231; 768 at 25216 rows chooses what it had.
-TnShape linear_tc_pair_tn_shape(int m, int n, int k, int splits_most, int parts_most, int sm_count)
+TnShape linear_tc_pair_tn_shape(int m, int n, int k, int splits_most, int sums_parts, int sm_count)
 {
     const long long pairs = sm_count / 2 > 0 ? sm_count / 2 : 1;
     const long long row_tiles = (m + kPairRows - 1) / kPairRows, k_blocks = (k + kBlockK - 1) / kBlockK;
+    // Sums of A come with the product while there are at most as many tiles as pairs.  A shape that gives that up makes them a pass of
+    // its own over A, two launches more: dim 1088 -> 1088 at 10000 rows 46 us in 2 ranges, 60 in 5; 704 -> 3136 74, 95.
+    const bool sums_fit = sums_parts > 0 && row_tiles * ((n + 255) / 256) <= pairs;
     TnShape best = {256, 1};
     long long best_cost = -1;
     for (int bn = 256; bn >= 128; bn -= 128) {
         const long long tiles = row_tiles * ((n + bn - 1) / bn);
         for (int s = 1; s <= splits_most && s <= k_blocks; ++s) {
-            // more sums of A than there is room for would be a pass of their own, two launches more
-            if (bn < 256 && s * ((n + bn - 1) / bn) > parts_most) break;
+            if (sums_fit && tiles * s > pairs) break;
+            if (sums_parts > 0 && bn < 256 && s * ((n + bn - 1) / bn) > sums_parts) break;      // more of them than there is room for
             const long long cost = (tiles * s + pairs - 1) / pairs * ((k_blocks + s - 1) / s) * (bn == 256 ? 288 : 216) + (s > 1 ? (long long)s * m * n / 1000 : 0);
             if (best_cost < 0 || cost < best_cost) { best.columns = bn; best.splits = s; best_cost = cost; }
         }

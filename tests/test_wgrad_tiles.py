@@ -21,3 +21,26 @@ def test_exact_sums(rows, out, in_, N, M, dtype):
     keep = lib.elsa_nm_unpack(torch.ones_like(vals), idx, out, in_, N, M) != 0
     assert torch.equal(dW, torch.where(keep, dY.double().t() @ X.double(), 0.0).to(dtype))
     assert torch.equal(db.view(-1), dY.double().sum(0).to(dtype))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("rows,out,in_", [(4000, 1216, 1280), (3000, 3136, 704), (5000, 704, 3136), (6000, 1984, 1152)])
+def test_bias_gradient_comes_with_the_product(rows, out, in_):
+    """Shapes whose tiles fit the SM pairs in fewer ranges than dW alone would take: the bias gradient is no pass of its own (one launch more
+    at most, which adds its parts), and right."""
+    from paper_2409_09708_b200 import binding as lib
+    gen = torch.Generator().manual_seed(rows)
+    ints = lambda *s: torch.randint(-1, 2, s, generator=gen).to(torch.bfloat16).cuda()
+    vals, idx = lib.elsa_nm_compress(torch.randn(out, in_, generator=gen).to(torch.bfloat16).cuda(), 2, 8)
+    X, dY = ints(rows, in_), ints(rows, out)
+
+    def launches(want):
+        before = lib.elsa_launch_count()
+        lib.elsa_nm_linear_backward(dY, X, vals, idx, out, in_, 2, 8, want=want)
+        return lib.elsa_launch_count() - before
+
+    assert launches(("dW", "db")) <= launches(("dW",)) + 1
+    _, dW, db = lib.elsa_nm_linear_backward(dY, X, vals, idx, out, in_, 2, 8)
+    keep = lib.elsa_nm_unpack(torch.ones_like(vals), idx, out, in_, 2, 8) != 0
+    assert torch.equal(dW, torch.where(keep, dY.double().t() @ X.double(), 0.0).to(torch.bfloat16))
+    assert torch.equal(db.view(-1), dY.double().sum(0).to(torch.bfloat16))
