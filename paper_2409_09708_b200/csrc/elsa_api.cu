@@ -224,7 +224,7 @@ private:
 // KIND_SMALL expands a packed weight itself; KIND_SMALL_IMAGE is the same kernel on the dense image of the weight.
 enum LinearKind { KIND_SIMT, KIND_SMALL, KIND_SMALL_IMAGE, KIND_DENSE_ONE, KIND_DENSE_PAIR, KIND_SPARSE_ONE, KIND_SPARSE_PAIR, KIND_SPARSE_WS, KIND_SPARSE_ST };
 
-// Form of the 2-of-4 weight image each sparse kernel reads.
+// Form of the 2-of-4 weight image each sparse kernel reads (the weight-stationary one in the masked form only).
 int sp24_layout_of(LinearKind kind)
 {
     return kind == KIND_SPARSE_WS ? SP24_PERMUTED : kind == KIND_SPARSE_ST ? SP24_TILED : SP24_ROWS;
@@ -235,7 +235,7 @@ ImageJob image_job(LinearKind kind, const void* vals, const uint32_t* idx, int o
 {
     ImageJob j;
     j.src = (const uint16_t*)vals; j.idx = idx; j.dst = (uint16_t*)region; j.out = out; j.in = in; j.N = N; j.M = M;
-    if (kind == KIND_SPARSE_PAIR || kind == KIND_SPARSE_WS || kind == KIND_SPARSE_ST) {
+    if (kind == KIND_SPARSE_PAIR || kind == KIND_SPARSE_ST) {
         j.kind = IMAGE_SP24;
         j.meta = (uint8_t*)region + sp24_meta_offset(out, in);
         j.layout = sp24_layout_of(kind);
@@ -1649,9 +1649,9 @@ elsa_status elsa_nm_linear_backward(const void* dY, const void* X, int rows, con
         // when tiles alone leave SM pairs idle, the rows are cut into ranges summed afterwards
         const TnShape shape = linear_tc_pair_tn_shape(out, in, rows, wgrad_splits_bound(in, out), db ? plan.parts : 0, dev.sm_count);
         float* sums = (float*)(ws + plan.sums);
-        const bool db_here = db && linear_tc_pair_tn_sums_parts(in, shape) <= plan.parts;
+        // (the sums of dY find room: plan.parts covers 256 columns in every number of ranges, and the shape's choice minds it at 128)
         if ((st = launch_linear_tc_pair_tn(dy, (const uint16_t*)X, out, in, rows, dtype, (uint16_t*)dW, shape, sums,
-                                           db_here ? db_sums : nullptr, &db_parts, dev_status, stream)) != ELSA_OK)
+                                           db ? db_sums : nullptr, &db_parts, dev_status, stream)) != ELSA_OK)
             return st;
         if (shape.splits > 1) {
             st = launch_wgrad_finish(sums, shape.splits, idx, out, in, N, M, dtype, (uint16_t*)dW, db_sums, db_parts, (uint16_t*)db, stream);

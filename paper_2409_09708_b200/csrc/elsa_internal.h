@@ -124,15 +124,15 @@ elsa_status launch_linear_tc_pair(const uint16_t* X, int rows, const uint16_t* W
                                   cudaStream_t stream);
 // Y [m][n] = A^T B on the same kernel with both operands stored reduction-outermost, A [k][m] and B [k][n]
 // (m, n multiples of 8): the weight-gradient product dY^T X without transposed copies.
-// shape: columns of a tile (256 or 128) and ranges the reduction is cut into, by linear_tc_pair_tn_shape with at most
-// splits_most ranges, and with at most sums_parts rows of sums (0: none are asked for); with several their fp32 sums go to partial [splits][m][n] (Y is then not written).  Where sums_a is not
-// NULL, there are no more tiles than SM pairs and no part has too many rows for the running sums, *sums_parts rows of m floats
-// that add up to the sums of A over the reduction go there (linear_tc_pair_tn_sums_parts(n, shape) of them); else *sums_parts is 0.
+// shape: columns of a tile (256 or 128) and ranges the reduction is cut into, by linear_tc_pair_tn_shape with at most splits_most
+// ranges, and with at most sums_parts rows of sums (0: none are asked for); with several ranges their fp32 sums go to
+// partial [splits][m][n] (Y is then not written).  Where sums_a is not NULL, there are no more tiles than SM pairs and no part has
+// too many rows for the running sums, *sums_parts rows of m floats that add up to the sums of A over the reduction go there, one
+// a range and tile column; else *sums_parts is 0.
 struct TnShape {
     int columns, splits;
 };
 TnShape linear_tc_pair_tn_shape(int m, int n, int k, int splits_most, int sums_parts, int sm_count);
-int linear_tc_pair_tn_sums_parts(int n, const TnShape& shape);
 elsa_status launch_linear_tc_pair_tn(const uint16_t* A, const uint16_t* B, int m, int n, int k, elsa_dtype dtype,
                                      uint16_t* Y, const TnShape& shape, float* partial, float* sums_a, int* sums_parts,
                                      uint32_t* dev_status, cudaStream_t stream);

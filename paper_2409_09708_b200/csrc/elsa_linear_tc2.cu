@@ -847,9 +847,6 @@ TnShape linear_tc_pair_tn_shape(int m, int n, int k, int splits_most, int sums_p
     return best;
 }
 
-// The most parts the sums of A come in: one a range and tile column.
-int linear_tc_pair_tn_sums_parts(int n, const TnShape& shape) { return shape.splits * ((n + shape.columns - 1) / shape.columns); }
-
 // Y [m][n] = A^T B with A [k][m] and B [k][n] (the reduction index outermost in both), no bias: one launch.
 // shape.splits > 1: nothing is written to Y; partial [splits][m][n] receives the fp32 sums of each range of the reduction.
 elsa_status launch_linear_tc_pair_tn(const uint16_t* A, const uint16_t* B, int m, int n, int k, elsa_dtype dtype,
