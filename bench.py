@@ -38,8 +38,8 @@ METRIC = "sparse-GEMM dense-equivalent TFLOP/s over the ViT linear stack"
 UNIT = "TFLOP/s"
 GEMM_KERNELS = ("linear_small", "linear_tc_dense", "linear_tc_pair", "linear_tc_sp24", "linear_tc_sp24_pair", "linear_tc_sp24_ws", "linear_tc_sp24_st")   # forms of the tcgen05 GEMM
 
-# Recorded DRAM traffic (ncu, one-pass captures) lives in profiles/dram_traffic.json: per workload and kernel
-# the bytes of one step, the command that captured them and a hash of the kernel sources at that time.
+# Recorded DRAM traffic lives in profiles/dram_traffic.json: per workload and kernel the bytes of one step, how they were
+# captured and a hash of the kernel sources at that time; it is reported only for those sources.
 DRAM_TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic.json")
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 

@@ -1,15 +1,11 @@
-"""Writes profiles/dram_traffic.json from an ncu capture of bench.py's DRAM counters.
+"""Writes profiles/dram_traffic.json from an ncu capture of bench.py's DRAM counters, read from its CSV.
 
-    python bench.py --steps 2 --warmup 3 --no-e2e --no-cpu-baseline --secondary "" --no-block-chain      # must exit 0 first
-    ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none -k regex:linear_tc_ \
-        --csv --log-file dram_stack.csv \
-        python bench.py --steps 2 --warmup 3 --no-e2e --no-cpu-baseline --secondary "" --no-block-chain
-    python bench_traffic.py dram_stack.csv --workload deit_b_stack_b256
+    python bench_traffic.py dram.csv --workload <name>
 
-The two counters are one pass, so the full-size workload is captured directly.  Only the launches that carry several
-layers (the launches of the timed steps) are counted: per kernel family, bytes read + written summed over those
-launches and divided by the number of steps seen.  The record carries the SHA-256 of the kernel sources
-(bench.kernel_source_hash); bench.py reports the traffic only while that hash matches the tree.
+The capture: the two metrics dram__bytes_read.sum and dram__bytes_write.sum of the linear_tc_ kernels, few launches, on a workload that holds
+a few GB on the device at most.  Only the launches that carry several layers (the launches of the timed steps) are counted: per kernel
+family, bytes read + written summed over those launches and divided by the number of steps seen.  The record carries the SHA-256 of
+the kernel sources (bench.kernel_source_hash); bench.py reports the traffic only while that hash matches the tree.
 """
 from __future__ import annotations
 
@@ -21,10 +17,6 @@ import os
 import re
 
 import bench
-
-COMMAND = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none -k regex:linear_tc_ --csv "
-           "--log-file dram_stack.csv python bench.py --workload %s --steps 2 --warmup 3 --no-e2e --no-cpu-baseline "
-           "--secondary \"\" --no-block-chain")
 
 
 def family_bytes(csv_path):
@@ -56,7 +48,8 @@ def family_bytes(csv_path):
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("csv")
-    ap.add_argument("--workload", default="deit_b_stack_b256")
+    ap.add_argument("--workload", required=True)
+    ap.add_argument("--command", default="", help="how the capture was taken, for the record")
     ap.add_argument("--out", default=os.path.join(bench.ROOT, "profiles", "dram_traffic.json"))
     args = ap.parse_args()
     fam = family_bytes(args.csv)
@@ -65,7 +58,7 @@ def main():
     for name, f in fam.items():
         captures.append({"workload": args.workload, "kernel": name, "dram_bytes_per_step": f["bytes"] / steps,
                          "launches_per_step": f["launches"] / steps, "steps_captured": steps,
-                         "csrc_sha256": bench.kernel_source_hash(), "command": COMMAND % args.workload})
+                         "csrc_sha256": bench.kernel_source_hash(), "command": args.command})
     try:
         with open(args.out) as fh:
             old = [c for c in json.load(fh).get("captures", []) if c.get("workload") != args.workload]
